@@ -150,6 +150,7 @@ struct AdjWs {
   float *a[kMaxLevels], *cr[kMaxLevels], *cz[kMaxLevels], *cn[kMaxLevels], *cnp;   // gate coefficients: fp32 engine
   __nv_bfloat16 *crb[kMaxLevels], *czb[kMaxLevels], *cnb[kMaxLevels], *cnpb;       // ... tensor-core engine (bf16)
   float *dA_h, *dA_i, *lam_tmp; double* res_acc; UmmaAdjWs um; Tf32Ws tf;
+  float* grad_scratch;      // fp32 engine: partial weight gradients
   __nv_bfloat16* chain_dAb; unsigned* chain_bar; uint4* chain_xw; size_t chain_xw_bytes;
   float* chain_dA32;        // fp32 chain: [2][B][3H] operand exchange
 };
@@ -201,7 +202,7 @@ void plan_adj(const mgrit_gru_cfg* c, const Hier& hr, Ws& w, AdjWs* o) {
   else { o->cnpb = nullptr; o->cnp = w.take<float>((size_t)hr.N[0] * BH); }
   o->res_acc = w.take<double>((size_t)(c->iters > 0 ? c->iters : 1));
   if (c->operands == MGRIT_OPERANDS_BF16) {
-    o->dA_h = o->dA_i = o->lam_tmp = nullptr;
+    o->dA_h = o->dA_i = o->lam_tmp = o->grad_scratch = nullptr;
     umma_plan_adj(c, hr.N, hr.L, w.base, &w.off, &o->um);
     o->chain_dA32 = nullptr;
     o->chain_dAb = w.take<__nv_bfloat16>(6 * BH);
@@ -212,9 +213,14 @@ void plan_adj(const mgrit_gru_cfg* c, const Hier& hr, Ws& w, AdjWs* o) {
     o->chain_dAb = nullptr; o->chain_xw = nullptr; o->chain_xw_bytes = 0;
     o->chain_bar = w.take<unsigned>((size_t)c->B / 16 + 64);
     o->chain_dA32 = w.take<float>(6 * BH);
-    o->dA_h = w.take<float>((size_t)c->T * BH * 3);
-    o->dA_i = w.take<float>((size_t)c->T * BH * 3);
-    o->lam_tmp = w.take<float>((size_t)c->T * BH);     // lambda in forward order when the caller wants no dh
+    o->dA_h = o->dA_i = o->lam_tmp = o->grad_scratch = nullptr;
+    if (is_tf32(c)) {
+      o->dA_h = w.take<float>((size_t)c->T * BH * 3);
+      o->dA_i = w.take<float>((size_t)c->T * BH * 3);
+      o->lam_tmp = w.take<float>((size_t)c->T * BH);     // lambda in forward order when the caller wants no dh
+    } else {
+      o->grad_scratch = w.take<float>(simt_gradients_scratch(c->T * c->B, 3 * c->H, c->H, c->I));
+    }
   }
   if (is_tf32(c)) tf32_plan_adj(c, hr.N, hr.L, w.base, &w.off, &o->tf);
 }
@@ -636,25 +642,22 @@ int adjoint_impl(const mgrit_gru_cfg* cfg_in, bool serial, const gru_params* p, 
     if (rc) return rc;
   } else {
     i64 M = (i64)T * c.B;
-    const float* lam = dh;
-    if (!lam) {   // no dh output requested: gather lambda in forward order into workspace scratch
-      lam = aw.lam_tmp;
-      stream_gather_rows(aw.lam_tmp, (i64)BH, aw.U[0] + (size_t)(T - 1) * BH, -(i64)BH, T, (i64)BH, s);
-    }
-    stream_form_dA(lam, aw.cr[0], aw.cz[0], aw.cn[0], aw.cnp, aw.dA_h, aw.dA_i, M, c.H, s);
-    if (tf32) {
+    if (!tf32) {
+      simt_gradients((int)M, c.B, c.H, c.I, aw.U[0] + (size_t)(T - 1) * BH, -(i64)BH, aw.cr[0], aw.cz[0], aw.cn[0], aw.cnp, h0, h, x, p->W_ih, dx, g,
+                     aw.grad_scratch, s);
+    } else {
+      const float* lam = dh;
+      if (!lam) {   // no dh output requested: gather lambda in forward order into workspace scratch
+        lam = aw.lam_tmp;
+        stream_gather_rows(aw.lam_tmp, (i64)BH, aw.U[0] + (size_t)(T - 1) * BH, -(i64)BH, T, (i64)BH, s);
+      }
+      stream_form_dA(lam, aw.cr[0], aw.cz[0], aw.cn[0], aw.cnp, aw.dA_h, aw.dA_i, M, c.H, s);
       rc = tf32_wgrad(aw.dA_h, (int)M, 3 * c.H, h0, c.B, h, c.H, g->dW_hh, &aw.tf, s);
       if (!rc) rc = tf32_wgrad(aw.dA_i, (int)M, 3 * c.H, nullptr, 0, x, c.I, g->dW_ih, &aw.tf, s);
       if (rc) return rc;
-    } else {
-      simt_wgrad(aw.dA_h, (int)M, 3 * c.H, h0, c.B, h, c.H, g->dW_hh, s);
-      simt_wgrad(aw.dA_i, (int)M, 3 * c.H, nullptr, 0, x, c.I, g->dW_ih, s);
-    }
-    stream_colsum(aw.dA_h, M, 3 * c.H, g->db_hh, s);
-    stream_colsum(aw.dA_i, M, 3 * c.H, g->db_ih, s);
-    if (dx) {
-      if (tf32) { rc = tf32_dgrad(aw.dA_i, (int)M, 3 * c.H, c.I, dx, &aw.tf, s); if (rc) return rc; }
-      else simt_dgrad(aw.dA_i, (int)M, 3 * c.H, p->W_ih, c.I, dx, s);
+      stream_colsum(aw.dA_h, M, 3 * c.H, g->db_hh, s);
+      stream_colsum(aw.dA_i, M, 3 * c.H, g->db_ih, s);
+      if (dx) { rc = tf32_dgrad(aw.dA_i, (int)M, 3 * c.H, c.I, dx, &aw.tf, s); if (rc) return rc; }
     }
   }
   if (resnorm && hr.L > 1 && c.iters > 0) {
@@ -805,7 +808,7 @@ struct StackLayerAdj {
 };
 struct StackAdjWs {
   float* U[kMaxLevels]; float* G[kMaxLevels]; double* res_acc;
-  float *tmpLin, *tmpDx, *lamk, *dxk, *dA_h, *dA_i; size_t maxM;
+  float *tmpLin, *tmpDx, *lamk, *dxk, *grad_scratch; size_t maxM;
   StackLayerAdj L[kMaxStack];
 };
 
@@ -822,8 +825,11 @@ void plan_stack_adj(const mgrit_gru_cfg* c, int nl, const Hier& hr, Ws& w, Stack
   o->tmpDx = w.take<float>(o->maxM * c->H);
   o->lamk = w.take<float>(TB * c->H);
   o->dxk = w.take<float>(TB * c->H);
-  if (bf16) { o->dA_h = o->dA_i = nullptr; }
-  else { o->dA_h = w.take<float>(TB * 3 * c->H); o->dA_i = w.take<float>(TB * 3 * c->H); }
+  o->grad_scratch = nullptr;
+  if (!bf16) {
+    const size_t n0 = simt_gradients_scratch((int)TB, 3 * c->H, c->H, c->I), n1 = simt_gradients_scratch((int)TB, 3 * c->H, c->H, c->H);
+    o->grad_scratch = w.take<float>(n0 > n1 ? n0 : n1);
+  }
   for (int k = 0; k < nl; ++k) {
     StackLayerAdj& L = o->L[k];
     for (int l = 0; l < hr.L; ++l) {
@@ -885,12 +891,7 @@ int stack_layer_gradients(const mgrit_gru_cfg& ck, const gru_params* pk, const f
   const i64 bh = (i64)ck.B * ck.H, M = (i64)ck.T * ck.B;
   if (ck.operands == MGRIT_OPERANDS_BF16)
     return umma_gradients(&ck, pk, xk, h0k, L.hk, w.lamk, bh, L.crb[0], L.czb[0], L.cnb[0], L.cnpb[0], dx, g, &L.um, false, s);
-  stream_form_dA(w.lamk, L.cr[0], L.cz[0], L.cn[0], L.cnp[0], w.dA_h, w.dA_i, M, ck.H, s);
-  simt_wgrad(w.dA_h, (int)M, 3 * ck.H, h0k, ck.B, L.hk, ck.H, g->dW_hh, s);
-  simt_wgrad(w.dA_i, (int)M, 3 * ck.H, nullptr, 0, xk, ck.I, g->dW_ih, s);
-  stream_colsum(w.dA_h, M, 3 * ck.H, g->db_hh, s);
-  stream_colsum(w.dA_i, M, 3 * ck.H, g->db_ih, s);
-  if (dx) simt_dgrad(w.dA_i, (int)M, 3 * ck.H, pk->W_ih, ck.I, dx, s);
+  simt_gradients((int)M, ck.B, ck.H, ck.I, w.lamk, bh, L.cr[0], L.cz[0], L.cn[0], L.cnp[0], h0k, L.hk, xk, pk->W_ih, dx, g, w.grad_scratch, s);
   return MGRIT_OK;
 }
 
@@ -994,7 +995,7 @@ struct LstmAdjWs {
   float* U[kMaxLevels]; float* G[kMaxLevels]; double* res_acc;
   float *a[kMaxLevels], *p[kMaxLevels], *ci[kMaxLevels], *cf[kMaxLevels], *cg[kMaxLevels], *co[kMaxLevels];
   __nv_bfloat16 *cib[kMaxLevels], *cfb[kMaxLevels], *cgb[kMaxLevels], *cob[kMaxLevels];    // bf16 operands: the gate coefficients as bf16 instead
-  float *tmpC, *tmpH, *hk, *dA; size_t maxM; Tf32Ws tf; LstmBfWs bf;
+  float *tmpC, *tmpH, *hk, *dA, *grad_scratch; size_t maxM; Tf32Ws tf; LstmBfWs bf;
   uint4* chain_xw; size_t chain_xw_bytes;
 };
 
@@ -1039,6 +1040,7 @@ void plan_lstm_adj(const mgrit_gru_cfg* c, const Hier& hr, Ws& w, LstmAdjWs* o) 
   o->tmpH = w.take<float>(o->maxM * c->H);
   o->hk = w.take<float>(TB * c->H);
   o->dA = w.take<float>(TB * 4 * c->H);
+  o->grad_scratch = c->operands == MGRIT_OPERANDS_FP32 ? w.take<float>(simt_gradients_scratch((int)TB, 4 * c->H, c->H, c->I)) : nullptr;
   if (is_tf32(c)) tf32_plan_adj(c, hr.N, hr.L, w.base, &w.off, &o->tf, 4);
   if (c->operands == MGRIT_OPERANDS_BF16) lstmbf_plan_adj(c, o->maxM, w.base, &w.off, &o->bf);
   o->chain_xw = nullptr; o->chain_xw_bytes = 0;
@@ -1230,15 +1232,11 @@ int lstm_adjoint_impl(const mgrit_gru_cfg* cfg, const gru_params* p, const float
       rc = tf32_wgrad(aw.dA, (int)M, 4 * c.H, u0 + bh, c.B, aw.hk, c.H, g->dW_hh, &aw.tf, s);
       if (!rc) rc = tf32_wgrad(aw.dA, (int)M, 4 * c.H, nullptr, 0, x, c.I, g->dW_ih, &aw.tf, s);
       if (rc) return rc;
+      stream_colsum(aw.dA, M, 4 * c.H, g->db_hh, s);
+      cudaMemcpyAsync(g->db_ih, g->db_hh, sizeof(float) * 4 * c.H, cudaMemcpyDeviceToDevice, s);
+      if (dx) { rc = tf32_dgrad(aw.dA, (int)M, 4 * c.H, c.I, dx, &aw.tf, s); if (rc) return rc; }
     } else {
-      simt_wgrad(aw.dA, (int)M, 4 * c.H, u0 + bh, c.B, aw.hk, c.H, g->dW_hh, s);
-      simt_wgrad(aw.dA, (int)M, 4 * c.H, nullptr, 0, x, c.I, g->dW_ih, s);
-    }
-    stream_colsum(aw.dA, M, 4 * c.H, g->db_hh, s);
-    cudaMemcpyAsync(g->db_ih, g->db_hh, sizeof(float) * 4 * c.H, cudaMemcpyDeviceToDevice, s);
-    if (dx) {
-      if (tf32) { rc = tf32_dgrad(aw.dA, (int)M, 4 * c.H, c.I, dx, &aw.tf, s); if (rc) return rc; }
-      else simt_dgrad(aw.dA, (int)M, 4 * c.H, p->W_ih, c.I, dx, s);
+      simt_lstm_gradients((int)M, c.B, c.H, c.I, aw.dA, u0 + bh, aw.hk, x, p->W_ih, dx, g, aw.grad_scratch, s);
     }
   }
   if (resnorm && hr.L > 1 && c.iters > 0) {

@@ -203,10 +203,14 @@ void simt_project(const float* x, const float* W_ih, const float* b_ih, float* g
 void simt_fwd_step(const FwdStepArgs& a, cudaStream_t s);
 void simt_linearise(const LinArgs& a, cudaStream_t s);
 void simt_adj_step(const AdjStepArgs& a, cudaStream_t s);
-// dW[n3, c] = sum_m dA[m, n3] * R[m, c],  R rows: m < B ? first[m] : rest[m-B]   (first may be nullptr with B = 0)
-void simt_wgrad(const float* dA, int M, int H3, const float* first, int Bfirst, const float* rest, int C, float* dW, cudaStream_t s);
-// dx[m, c] = sum_n3 dA[m, n3] * W[n3, c]
-void simt_dgrad(const float* dA, int M, int H3, const float* W, int C, float* dx, cudaStream_t s);
+// Gradient pass: dW_hh, dW_ih, both bias gradients and (dx != nullptr) the input gradient from the coefficients and the
+// sensitivities lam of all M = T*B rows (row (t, b) at lam + t*lam_ts + b*H); h_prev rows: h0 for t = 0, then h.
+// scratch: simt_gradients_scratch() floats.  The LSTM takes its dA[M, 4H] as given.
+size_t simt_gradients_scratch(int M, int GH, int H, int I);
+void simt_gradients(int M, int B, int H, int I, const float* lam, i64 lam_ts, const float* cr, const float* cz, const float* cn, const float* cnp,
+                    const float* h0, const float* h, const float* x, const float* W_ih, float* dx, const gru_grads* g, float* scratch, cudaStream_t s);
+void simt_lstm_gradients(int M, int B, int H, int I, const float* dA, const float* h0, const float* h, const float* x, const float* W_ih, float* dx,
+                         const gru_grads* g, float* scratch, cudaStream_t s);
 // out[m, c] = sum_{g,i} (c_g * lam)[m, i] W_ih[g*H + i, c]: what the step described by `a` (its cn slot holding c_n') sends to
 // the input of its cell, contiguous rows [M, C]
 void simt_adj_dx(const AdjStepArgs& a, const float* W_ih, int C, float* out, cudaStream_t s);
