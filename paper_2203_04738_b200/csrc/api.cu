@@ -9,6 +9,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "f32_solve.cuh"
 #include "serial_engine.cuh"
 #include "umma_engine.cuh"
 
@@ -458,6 +459,117 @@ struct AdjCycle : Cycle {
   }
 };
 
+// The whole solve of an fp32-state GRU recurrence as phases of the persistent kernels in f32_solve.cu.  The same cycle as
+// Cycle::cycle, phase by phase; what differs is where C-points travel: a C-relaxation of level l leaves its results in the
+// coarse array U[l+1] (which the restriction would fill with them anyway) and the next one back in U[l], so that no row of
+// a phase overwrites what another row of the same phase still reads; the correction is the start of the closing F-relaxation.
+struct F32Cycle {
+  const mgrit_gru_cfg* c; const Hier* hr; bool adjoint; cudaStream_t s;
+  float** U; float** G; double* res_acc; F32Args a;
+  bool ok = true, fcycle_leg = true;
+  int cycle_idx = 0;
+  i64 bh() const { return (i64)c->B * c->H; }
+  void flush() {
+    if (a.nph > 0 && ok) ok = f32_solve(adjoint, a, s);
+    a.nph = 0;
+  }
+  void add(const F32Phase& p) {
+    if (a.nph == kF32MaxPhases) flush();
+    a.ph[a.nph++] = p;
+  }
+  // rows start at slot s0 of their interval of level l; their first step arrives at slot s0 + 1
+  F32Phase phase(int l, const float* src, i64 src_ks, int s0) {
+    const i64 BH = bh(), st = hr->stride_t[l], ks = (i64)c->cf * BH;
+    F32Phase p;
+    memset(&p, 0, sizeof(p));
+    p.level = l; p.gamma = hr->gamma[l];
+    p.src = src; p.src_ks = src_ks;
+    p.out = U[l] + (s0 + 1) * BH; p.out_ks = ks; p.out_ss = BH;
+    p.g = G[l] ? G[l] + (s0 + 1) * BH : nullptr; p.g_ks = ks; p.g_ss = BH;
+    if (adjoint) { p.op = ((i64)hr->N[l] - (s0 + 1)) * BH; p.op_ss = -BH; p.op_ks = -ks; }
+    else { p.op = (st * (s0 + 1) - 1) * BH * 3; p.op_ss = st * BH * 3; p.op_ks = st * ks * 3; }
+    return p;
+  }
+  void cycle(int l, bool skip_first_f, bool record) {
+    const i64 BH = bh();
+    const int cf = c->cf, N = hr->N[l];
+    if (l == hr->L - 1) {
+      F32Phase p = phase(l, U[l], 0, 0);
+      p.nk = p.nfull = 1; p.n = N;
+      add(p);
+      return;
+    }
+    const int nc = hr->N[l + 1], tail = N % cf, relax = l == 0 ? c->relax_fine : c->relax_coarse;
+    float* cp = U[l]; i64 cp_ks = (i64)cf * BH;          // where slot 0 of the intervals is: here or in the coarse array
+    for (int r = 0; r <= relax; ++r) {
+      const bool skip = r == 0 && skip_first_f;          // the F-points are there already: only the closing step
+      const int s0 = skip ? cf - 1 : 0;
+      F32Phase p = skip ? phase(l, U[l] + (cf - 1) * BH, (i64)cf * BH, s0) : phase(l, cp, cp_ks, 0);
+      p.n = skip ? 0 : cf - 1; p.nfull = nc; p.ntail = skip ? 0 : tail; p.nk = nc + (p.ntail > 0 ? 1 : 0);
+      if (r < relax) {
+        p.last_kind = kLastStore;
+        float* dst = cp == U[l] ? U[l + 1] + BH : U[l] + (i64)cf * BH;
+        const i64 dst_ks = cp == U[l] ? BH : (i64)cf * BH;
+        p.last = dst; p.last_ks = dst_ks;
+        add(p);
+        cp = dst - dst_ks; cp_ks = dst_ks;
+      } else {
+        p.last_kind = kLastCoarse;
+        p.last = G[l + 1] + BH; p.last_ks = BH;
+        p.src2 = cp; p.src2_ks = cp_ks;
+        p.uc = cp + cp_ks; p.uc_ks = cp_ks;
+        p.ucd = cp == U[l + 1] ? nullptr : U[l + 1] + BH; p.ucd_ks = BH;
+        p.gamma2 = hr->gamma[l + 1];
+        const i64 st2 = hr->stride_t[l + 1];
+        if (adjoint) { p.op2 = ((i64)nc - 1) * BH; p.op2_ks = -BH; }
+        else { p.op2 = (st2 - 1) * BH * 3; p.op2_ks = st2 * BH * 3; }
+        p.acc = l == 0 && record ? res_acc + cycle_idx : nullptr;
+        add(p);
+      }
+    }
+    cycle(l + 1, false, false);
+    F32Phase p = phase(l, U[l + 1], BH, 0);
+    p.copy = U[l]; p.copy_ks = (i64)cf * BH;
+    p.nk = nc + 1; p.nfull = nc; p.n = cf - 1; p.ntail = tail;
+    add(p);
+    if ((c->flags & MGRIT_FLAG_F_CYCLE) && fcycle_leg) {
+      fcycle_leg = false;
+      cycle(l, true, false);
+      fcycle_leg = true;
+    }
+  }
+  bool solve() {
+    a.nph = 0;
+    if (hr->L == 1) cycle(0, false, false);
+    else {
+      cudaMemsetAsync(res_acc, 0, sizeof(double) * (size_t)(c->iters > 0 ? c->iters : 1), s);
+      for (cycle_idx = 0; cycle_idx < c->iters; ++cycle_idx)
+        cycle(0, cycle_idx > 0 && (c->flags & MGRIT_FLAG_SKIP_DUPLICATE_FRELAX), true);
+    }
+    flush();
+    return ok;
+  }
+};
+
+// Which fp32-state solves run there: every one of the fp32 mode whose weights fit, and those of the tf32 split whose steps are
+// too small for the tensor cores (rows of the largest step x H^2).
+constexpr double kF32TfStep = 2.5e8, kF32TfLin = 6e8;
+bool use_f32_solve(const mgrit_gru_cfg* c, const Hier& hr) {
+  if (!f32_solve_fits(c->H)) return false;
+  if (c->operands == MGRIT_OPERANDS_FP32) return true;
+  if (c->operands != MGRIT_OPERANDS_TF32) return false;
+  const double rows = hr.L == 1 ? c->B : (double)(c->T / c->cf + 1) * c->B;
+  return rows * c->H * c->H <= kF32TfStep;
+}
+bool use_f32_lin(const mgrit_gru_cfg* c, const Hier& hr) {
+  if (!f32_solve_fits(c->H)) return false;
+  if (c->operands == MGRIT_OPERANDS_FP32) return true;
+  if (c->operands != MGRIT_OPERANDS_TF32) return false;
+  double rows = 0;
+  for (int l = 0; l < hr.L; ++l) rows += (double)hr.N[l] * c->B;
+  return rows * c->H * c->H <= kF32TfLin;
+}
+
 // Zero initial guess of a level-0 array [T + 1 slots of `slot` elements] behind its fixed slot 0.  In a multigrid solve
 // with at least one cycle only the C-points are read before they are written (the first F-relaxation fills every
 // F-point from them), so only those slots are cleared: 1 / cf of the memory traffic.
@@ -474,7 +586,7 @@ int finish(cudaStream_t s, bool sync) {
   if (sync && cudaStreamSynchronize(s) != cudaSuccess) return MGRIT_CUDA_ERROR;
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) { fprintf(stderr, "mgrit_gru: CUDA error: %s\n", cudaGetErrorString(e)); return MGRIT_CUDA_ERROR; }
-  if (sync && (umma_device_status() != 0 || serial_device_status() != 0)) return MGRIT_DEVICE_TIMEOUT;
+  if (sync && (umma_device_status() != 0 || serial_device_status() != 0 || f32_device_status() != 0)) return MGRIT_DEVICE_TIMEOUT;
   return MGRIT_OK;
 }
 
@@ -540,8 +652,15 @@ int forward_impl(const mgrit_gru_cfg* cfg_in, bool serial, const gru_params* p, 
   cy.Ub = shadows ? fw.Ub : nullptr;
   cy.gib = shadows ? fw.um.gib : nullptr;
   cy.gi_f32 = gi_f32;
-  rc = cy.solve();
-  if (rc) return rc;
+  if (use_f32_solve(&c, hr)) {
+    F32Cycle fc;
+    fc.c = &c; fc.hr = &hr; fc.adjoint = false; fc.s = s; fc.U = fw.U; fc.G = fw.G; fc.res_acc = fw.res_acc;
+    fc.a.B = c.B; fc.a.H = c.H; fc.a.cell = c.cell; fc.a.W = p->W_hh; fc.a.gi = gi; fc.a.b_hh = p->b_hh; fc.a.bar = fw.chain_bar;
+    if (!fc.solve()) return MGRIT_CUDA_ERROR;
+  } else {
+    rc = cy.solve();
+    if (rc) return rc;
+  }
   if (!h_in_place) cudaMemcpyAsync(h, fw.U[0] + BH, sizeof(float) * (size_t)c.T * BH, cudaMemcpyDeviceToDevice, s);
   if (resnorm && hr.L > 1 && c.iters > 0) {
     rc = fetch_resnorm(fw.res_acc, resnorm, c.iters, s);
@@ -590,14 +709,18 @@ int adjoint_impl(const mgrit_gru_cfg* cfg_in, bool serial, const gru_params* p, 
     if (rc) return rc;
   }
   // adjoint coefficients of every level's steps at the given states (restricted by injection)
+  const bool lin32 = use_f32_lin(&c, hr);
+  LinArgs lins[kMaxLevels];
   for (int l = 0; l < hr.L; ++l) {
-    LinArgs a{};
+    LinArgs& a = lins[l];
+    a = LinArgs{};
     a.M = hr.N[l] * c.B; a.B = c.B; a.H = c.H; a.h0 = h0; a.h = h; a.stride_t = hr.stride_t[l]; a.gi = gi;
     a.t0 = hr.rem[l];     // the level's reversed grid is anchored at T: its forward steps arrive at t0 + stride * j
     a.W_hh = p->W_hh; a.b_hh = p->b_hh; a.gamma = hr.gamma[l]; a.cell = c.cell;
     a.a = aw.a[l]; a.cr = aw.cr[l]; a.cz = aw.cz[l]; a.cn = aw.cn[l]; a.cnp = l == 0 ? aw.cnp : nullptr;
     a.crb = aw.crb[l]; a.czb = aw.czb[l]; a.cnb = aw.cnb[l]; a.cnpb = l == 0 ? aw.cnpb : nullptr;
     a.gi_b = (bf16 && copies) ? aw.um.gib : nullptr;
+    if (lin32) continue;
     if (bf16) {
       rc = umma_linearise(a, &aw.um, s);
       if (rc) return rc;
@@ -608,6 +731,7 @@ int adjoint_impl(const mgrit_gru_cfg* cfg_in, bool serial, const gru_params* p, 
       simt_linearise(a, s);
     }
   }
+  if (lin32 && !f32_linearise(lins, hr.L, s)) return MGRIT_CUDA_ERROR;
   // mu_0 = lambda_T; zero initial guess elsewhere; fine-level source = reversed dh_seed
   zero_guess(aw.U[0], c, hr, BH, s);        // (slot 0 is set below)
   if (dh_seed) {
@@ -627,8 +751,16 @@ int adjoint_impl(const mgrit_gru_cfg* cfg_in, bool serial, const gru_params* p, 
   AdjCycle cy;
   cy.c = &c; cy.hr = hr; cy.s = s; cy.U = aw.U; cy.G = Gl; cy.res_acc = aw.res_acc; cy.BH = BH;
   cy.p = p; cy.w = &aw;
-  rc = cy.solve();
-  if (rc) return rc;
+  if (use_f32_solve(&c, hr)) {
+    F32Cycle fc;
+    fc.c = &c; fc.hr = &hr; fc.adjoint = true; fc.s = s; fc.U = aw.U; fc.G = Gl; fc.res_acc = aw.res_acc;
+    fc.a.B = c.B; fc.a.H = c.H; fc.a.cell = c.cell; fc.a.W = p->W_hh; fc.a.bar = aw.chain_bar;
+    for (int l = 0; l < hr.L; ++l) { fc.a.coef[l][0] = aw.a[l]; fc.a.coef[l][1] = aw.cr[l]; fc.a.coef[l][2] = aw.cz[l]; fc.a.coef[l][3] = aw.cn[l]; }
+    if (!fc.solve()) return MGRIT_CUDA_ERROR;
+  } else {
+    rc = cy.solve();
+    if (rc) return rc;
+  }
 
   // dh[k] = lambda_{k+1} = mu_{T-1-k} (optional output);  dh0 = lambda_0 = mu_T
   if (dh) stream_gather_rows(dh, (i64)BH, aw.U[0] + (size_t)(T - 1) * BH, -(i64)BH, T, (i64)BH, s);
@@ -1464,12 +1596,12 @@ int adam_update(float* p, const float* g, float* m, float* v, size_t n, float lr
 
 int mgrit_gru_last_device_status(void) {
   if (cudaDeviceSynchronize() != cudaSuccess) return MGRIT_CUDA_ERROR;
-  return (umma_device_status() != 0 || serial_device_status() != 0) ? MGRIT_DEVICE_TIMEOUT : MGRIT_OK;
+  return (umma_device_status() != 0 || serial_device_status() != 0 || f32_device_status() != 0) ? MGRIT_DEVICE_TIMEOUT : MGRIT_OK;
 }
 
 int mgrit_gru_clear_device_status(void) {
   if (cudaDeviceSynchronize() != cudaSuccess) return MGRIT_CUDA_ERROR;
-  return (umma_clear_device_status() == 0 && serial_clear_device_status() == 0) ? MGRIT_OK : MGRIT_CUDA_ERROR;
+  return (umma_clear_device_status() == 0 && serial_clear_device_status() == 0 && f32_clear_device_status() == 0) ? MGRIT_OK : MGRIT_CUDA_ERROR;
 }
 
 int mgrit_gru_selftest_bounded_wait(int32_t limit_ms, mgrit_stream_t stream) { return umma_selftest_wait(limit_ms, (cudaStream_t)stream); }
