@@ -552,8 +552,10 @@ struct F32Cycle {
 };
 
 // Which fp32-state solves run there: every one of the fp32 mode whose weights fit, and those of the tf32 split whose steps are
-// too small for the tensor cores (rows of the largest step x H^2).
-constexpr double kF32TfStep = 2.5e8, kF32TfLin = 6e8;
+// too small for the tensor cores (rows of the largest step x H^2).  At H = 256 a step of 500 rows takes 14.6 us forward and
+// 11.8 us adjoint there, 2000 rows 65 and 39 us; the tensor-core step takes 27 + 6 and 24 + 4 us (product and operand split, one
+// wave of tiles) at 512 rows and hardly more at 2000: they meet at about 1200 rows.  Linearisation of 2560 rows: 51 against 58 us.
+constexpr double kF32TfStep = 8e7, kF32TfLin = 1.7e8;
 bool use_f32_solve(const mgrit_gru_cfg* c, const Hier& hr) {
   if (!f32_solve_fits(c->H)) return false;
   if (c->operands == MGRIT_OPERANDS_FP32) return true;

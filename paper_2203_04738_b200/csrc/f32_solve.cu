@@ -11,8 +11,13 @@
 //   adjoint: CTA c owns the SAME gate rows, now as its slice of the reduction: it forms [c_r|c_z|c_n]*mu for its own units,
 //     multiplies with its rows of W_hh and sends partial sums to the unit's owner (a third of the bytes that exchanging the
 //     formed operand would take); mu itself never leaves its thread.
-// Products are FFMA (packed in pairs along the reduction, fma.rn.f32x2, in the forward direction): a thread holds 8 rows x 3
-// gates (forward) or 8 x 4 outputs (adjoint); KP lanes share the sums of 4 rows when there are too few rows to fill the CTA.
+// Products are FFMA (packed in pairs along the reduction, fma.rn.f32x2, in the forward direction): a thread holds 4 rows x 3
+// gates (forward) or 8 x 4 outputs (adjoint); KP lanes share the sums of 4 rows when few rows would not fill the CTA.
+// Measured (B200, whole training steps launched from the host, before -> now): 64 steps x 2 rows, H = 32: 489 -> 262 us; two
+// layers of 128 x 100 rows, H = 104: 4801 -> 2093 us; 128 x 16 rows, H = 256 (tf32 split): 1935 -> 1356 us.  A dependent step
+// of the coarsest level takes 1.4 / 1.9 us at H = 32 (forward / adjoint) and 3.3 / 3.2 us at H = 256, a step of 3300 rows at
+// H = 104 15 / 16 us (14 TFLOP/s): bound by the delivery of operands from shared memory and, with few rows, by the latency of a
+// step's parts.
 #include "cell.cuh"
 #include "f32_solve.cuh"
 
@@ -20,7 +25,7 @@ namespace mg {
 namespace {
 
 typedef unsigned long long u64;
-constexpr int kMaxThreads = 512;
+constexpr int kMaxThreads = 512, kFwdThreads = 640;
 constexpr int kMaxRows = 64;
 constexpr size_t kSmemMax = 227 * 1024 - 2048;     // dynamic part: the kernels hold under 1 KiB of static shared memory
 constexpr uint64_t kWaitLimitNs = 2000000000ull;
@@ -78,18 +83,21 @@ __device__ bool grid_barrier(unsigned* bar, unsigned target, int nc, int* status
 }
 
 // A shared-memory load delivers 32 words a cycle however they are shared, so a sum over r rows and c weight rows runs at
-// r c / (r + c) multiply-adds per word against the 4 that keep the FFMA pipe busy: 8 rows where a lane has a sum to itself
-// (2.2 per word), 4 where KP lanes share one and latency counts.
+// r c / (r + c) multiply-adds per word against the 4 that keep the FFMA pipe busy.  Adjoint: 8 rows where a lane has a sum to
+// itself (2.7 per word), 4 where KP lanes share one and latency counts.  Forward: 4 (1.7); with 8 the gate operands of the
+// rows do not fit the registers next to the sums (256 units x 2000 rows: 64 us a step spilled).
 template <int KP> struct Tile { static constexpr int RT = KP == 1 ? 8 : 4, NR = KP >= 4 ? 1 : RT / KP; };
-// Items: KP lanes per sum (fastest), 8 units, RG groups of RT rows, unit blocks.
+template <int KP> struct FTile { static constexpr int RT = 4, NR = KP >= 4 ? 1 : RT / KP; };
+// Items: 8 units (fastest: the eight lanes that a 16-byte load serves together then read eight different weight rows, which
+// never share a bank), KP lanes per sum, RG groups of RT rows, unit blocks.
 struct Item { int rg, u, kp; bool live; };
 template <int KP>
 __device__ __forceinline__ Item item_of(int it, int RG, int n) {
   Item x;
-  x.kp = it % KP;
-  int q = it / KP;
-  const int ul = q & 7;
-  q >>= 3;
+  const int ul = it & 7;
+  int q = it >> 3;
+  x.kp = q % KP;
+  q /= KP;
   x.rg = q % RG;
   const int u = (q / RG) * 8 + ul;
   x.live = u < n;
@@ -98,8 +106,8 @@ __device__ __forceinline__ Item item_of(int it, int RG, int n) {
 }
 // pre[gate][q] of this lane's rows = sum_k S[row][k] Ws[gate*U + u][k]
 template <int KP>
-__device__ __forceinline__ void fwd_sums(const float* S, const float* Ws, int ld, int H, int U, const Item& x, float (&pre)[3][Tile<KP>::NR]) {
-  constexpr int RT = Tile<KP>::RT, NR = Tile<KP>::NR;
+__device__ __forceinline__ void fwd_sums(const float* S, const float* Ws, int ld, int H, int U, const Item& x, float (&pre)[3][FTile<KP>::NR]) {
+  constexpr int RT = FTile<KP>::RT, NR = FTile<KP>::NR;
   u64 acc[3][RT];
 #pragma unroll
   for (int g = 0; g < 3; ++g)
@@ -126,18 +134,18 @@ __device__ __forceinline__ void fwd_sums(const float* S, const float* Ws, int ld
       const float2 f = unpack2(acc[g][r]);
       float v = f.x + f.y;
 #pragma unroll
-      for (int o = 1; o < KP; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+      for (int o = 1; o < KP; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, 8 * o);
       if (r / NR == x.kp) pre[g][r % NR] = v;
     }
 }
 
 struct FwdShared { float *S[2], *Ws, *bh; int ld, U, Un, u0, rank, NC; int *rk, *rb; };
 
-// What a step of one item needs from global memory.  Where every thread has one item (ONE) the next step's values are
-// requested as soon as the current ones are used, straight into the same registers (a copy would wait for them), and used
-// behind the next sums, so their latency hides behind the exchange; with several items per thread the other warps hide it.
+// What a step needs from global memory (every thread has at most one item).  The next step's values are requested as soon as
+// the current ones are used, straight into the same registers (a copy would wait for them), and used behind the next sums, so
+// their latency hides behind the exchange.
 template <int KP> struct FwdOps {
-  static constexpr int NR = Tile<KP>::NR;
+  static constexpr int NR = FTile<KP>::NR;
   float gi[3][NR], ad[NR];
   bool on[NR];
 };
@@ -147,7 +155,7 @@ __device__ __forceinline__ void fwd_load(const F32Args& a, const F32Phase& p, co
   const int H = a.H, c = sh.u0 + x.u;
 #pragma unroll
   for (int q = 0; q < NR; ++q) {
-    const int row = x.rg * Tile<KP>::RT + x.kp * NR + q, k = sh.rk[row], b = sh.rb[row];
+    const int row = x.rg * FTile<KP>::RT + x.kp * NR + q, k = sh.rk[row], b = sh.rb[row];
     o.on[q] = x.live && k >= 0 && (j < (k < p.nfull ? p.n : p.ntail) || (j >= p.n && k < p.nfull));
     o.ad[q] = o.gi[0][q] = o.gi[1][q] = o.gi[2][q] = 0.f;
     if (o.on[q]) {
@@ -168,7 +176,7 @@ __device__ __forceinline__ float fwd_finish(const F32Args& a, const F32Phase& p,
   if (!x.live) return norm;
 #pragma unroll
   for (int q = 0; q < NR; ++q) {
-    const int row = x.rg * Tile<KP>::RT + x.kp * NR + q;
+    const int row = x.rg * FTile<KP>::RT + x.kp * NR + q;
     const float hp = sh.S[cur][row * sh.ld + c];
     const float phi = cell_forward(o.gi[0][q], o.gi[1][q], o.gi[2][q], pre[0][q] + sh.bh[x.u], pre[1][q] + sh.bh[sh.U + x.u],
                                    pre[2][q] + sh.bh[2 * sh.U + x.u], hp, mode == 2 ? p.gamma2 : p.gamma, a.cell);
@@ -195,32 +203,23 @@ __device__ __forceinline__ float fwd_finish(const F32Args& a, const F32Phase& p,
 }
 
 // All steps of one row block; S[0] holds the start.  load(dst, src, ks, ...): the block's rows from global memory.
-template <bool MULTI, int KP, bool ONE, class Load>
+template <bool MULTI, int KP, class Load>
 __device__ __forceinline__ float fwd_block(const F32Args& a, const F32Phase& p, const FwdShared& sh, float norm, Load load) {
-  const int H = a.H, RG = p.R / Tile<KP>::RT, items = (((sh.Un + 7) / 8) * 8 * RG * KP + 31) & ~31, steps = p.n + (p.last_kind != kLastNone ? 1 : 0);
-  const bool works = (int)threadIdx.x < min(p.nt, items);        // whole warps: the sums are shared by shuffles
+  const int H = a.H, RG = p.R / FTile<KP>::RT, items = (((sh.Un + 7) / 8) * 8 * RG * KP + 31) & ~31, steps = p.n + (p.last_kind != kLastNone ? 1 : 0);
+  const bool works = (int)threadIdx.x < items;                  // whole warps: the sums are shared by shuffles
   const bool coarse = p.last_kind == kLastCoarse;
   FwdOps<KP> o;
   float pre[3][FwdOps<KP>::NR];
-  const Item x1 = item_of<KP>(threadIdx.x, RG, sh.Un);
-  if (ONE && works) fwd_load<KP>(a, p, sh, x1, 0, false, o);
+  const Item x = item_of<KP>(threadIdx.x, RG, sh.Un);
+  if (works) fwd_load<KP>(a, p, sh, x, 0, false, o);
   int cur = 0;
   for (int j = 0; j < steps; ++j) {
     const int mode = j == p.n && coarse ? 1 : 0;
     if (works) {
-      if (ONE) {
-        fwd_sums<KP>(sh.S[cur], sh.Ws, sh.ld, H, sh.U, x1, pre);
-        norm = fwd_finish<KP>(a, p, sh, x1, cur, j, mode, o, pre, norm);
-        if (j + 1 < steps) fwd_load<KP>(a, p, sh, x1, j + 1, false, o);
-        else if (coarse) fwd_load<KP>(a, p, sh, x1, p.n, true, o);
-      } else {
-        for (int it = threadIdx.x; it < items; it += p.nt) {
-          const Item x = item_of<KP>(it, RG, sh.Un);
-          fwd_load<KP>(a, p, sh, x, j, false, o);
-          fwd_sums<KP>(sh.S[cur], sh.Ws, sh.ld, H, sh.U, x, pre);
-          norm = fwd_finish<KP>(a, p, sh, x, cur, j, mode, o, pre, norm);
-        }
-      }
+      fwd_sums<KP>(sh.S[cur], sh.Ws, sh.ld, H, sh.U, x, pre);
+      norm = fwd_finish<KP>(a, p, sh, x, cur, j, mode, o, pre, norm);
+      if (j + 1 < steps) fwd_load<KP>(a, p, sh, x, j + 1, false, o);
+      else if (coarse) fwd_load<KP>(a, p, sh, x, p.n, true, o);
     }
     if (j + 1 == steps) break;
     __syncthreads();
@@ -240,17 +239,8 @@ __device__ __forceinline__ float fwd_block(const F32Args& a, const F32Phase& p, 
     load(sh.S[cur], p.src2, p.src2_ks, nullptr, 0);
     __syncthreads();
     if (works) {
-      if (ONE) {
-        fwd_sums<KP>(sh.S[cur], sh.Ws, sh.ld, H, sh.U, x1, pre);
-        norm = fwd_finish<KP>(a, p, sh, x1, cur, p.n, 2, o, pre, norm);
-      } else {
-        for (int it = threadIdx.x; it < items; it += p.nt) {
-          const Item x = item_of<KP>(it, RG, sh.Un);
-          fwd_load<KP>(a, p, sh, x, p.n, true, o);
-          fwd_sums<KP>(sh.S[cur], sh.Ws, sh.ld, H, sh.U, x, pre);
-          norm = fwd_finish<KP>(a, p, sh, x, cur, p.n, 2, o, pre, norm);
-        }
-      }
+      fwd_sums<KP>(sh.S[cur], sh.Ws, sh.ld, H, sh.U, x, pre);
+      norm = fwd_finish<KP>(a, p, sh, x, cur, p.n, 2, o, pre, norm);
     }
   }
   return norm;
@@ -271,7 +261,7 @@ __device__ __forceinline__ void add_norm(float norm, double* acc) {
 }
 
 template <bool MULTI>
-__global__ void __launch_bounds__(kMaxThreads, 1) f32_fwd_kernel(const __grid_constant__ F32Args a, int NC, int U, int rmax, int* status) {
+__global__ void __launch_bounds__(kFwdThreads, 1) f32_fwd_kernel(const __grid_constant__ F32Args a, int NC, int U, int rmax, int* status) {
   extern __shared__ __align__(16) float fsm[];
   __shared__ int rk[kMaxRows], rb[kMaxRows], verdict;
   const int H = a.H, ld = H + 4, rank = MULTI ? (int)ctarank() : 0;
@@ -307,11 +297,9 @@ __global__ void __launch_bounds__(kMaxThreads, 1) f32_fwd_kernel(const __grid_co
       };
       load(sh.S[0], p.src, p.src_ks, p.copy, p.copy_ks);
       block_sync<MULTI>();       // the peers are done with the previous block before anything is pushed into S[1]
-      const bool one = p.nt >= ((((sh.Un + 7) / 8) * 8 * (p.R / Tile<1>::RT) + 31) & ~31);
-      if (p.KP == 4) norm = fwd_block<MULTI, 4, true>(a, p, sh, norm, load);       // (lanes share a sum only where every item has a thread)
-      else if (p.KP == 2) norm = fwd_block<MULTI, 2, true>(a, p, sh, norm, load);
-      else if (one) norm = fwd_block<MULTI, 1, true>(a, p, sh, norm, load);
-      else norm = fwd_block<MULTI, 1, false>(a, p, sh, norm, load);
+      if (p.KP == 4) norm = fwd_block<MULTI, 4>(a, p, sh, norm, load);
+      else if (p.KP == 2) norm = fwd_block<MULTI, 2>(a, p, sh, norm, load);
+      else norm = fwd_block<MULTI, 1>(a, p, sh, norm, load);
     }
     if (p.acc) add_norm(norm, p.acc);
     if (ip + 1 < a.nph) {
@@ -323,24 +311,27 @@ __global__ void __launch_bounds__(kMaxThreads, 1) f32_fwd_kernel(const __grid_co
 
 // ---- adjoint
 // shared: Ws[3U][H] (this CTA's gate rows), Ad[R][3U + 4] (the formed operand),
-// Pb[2][NC][R][U] (partial sums for this CTA's units by producer)
+// Pb[2][NC or 3 NC][R][U] (partial sums for this CTA's units by producer, and by gate where the gates are split)
+constexpr int kSplitKP = 12, kSplitRows = 8;        // (split: blocks of at most 8 rows, KP = 4)
 struct AdjVals { float4 m, a, g; };                 // four units of one row: mu, and of the step in flight a and the source
 struct AdjNext { float4 cr, cz, cn, a, g; };        // ... the next step's coefficients, requested before the product in front of it
 
-template <int KP>
+// SPLIT: the three gates' sums go to three groups of threads, each with partial results of its own (few rows: more warps)
+template <int KP, bool SPLIT>
 __device__ __forceinline__ void adj_product(const F32Args& a, const F32Phase& p, const float* Ws, const float* Ad, float* Pb, int lda, int U, int Un, int NC,
                                             int rank, bool multi) {
   constexpr int RT = Tile<KP>::RT, NR = Tile<KP>::NR;
-  const int H = a.H, RG = p.R / RT, n4 = H / 4, items = ((n4 + 7) / 8) * 8 * RG * KP;
+  const int H = a.H, RG = p.R / RT, n4 = H / 4, items = (((n4 + 7) / 8) * 8 * RG * KP + 31) & ~31;
   if ((int)threadIdx.x >= p.nt) return;
-  for (int it = threadIdx.x; it < ((items + 31) & ~31); it += p.nt) {
+  for (int it0 = threadIdx.x; it0 < (SPLIT ? 3 : 1) * items; it0 += p.nt) {
+    const int gs = SPLIT ? it0 / items : 0, it = it0 - gs * items;
     const Item x = item_of<KP>(it, RG, n4);
     float acc[RT][4];
 #pragma unroll
     for (int r = 0; r < RT; ++r) acc[r][0] = acc[r][1] = acc[r][2] = acc[r][3] = 0.f;
     const float* a0 = Ad + x.rg * RT * lda;
     // the operand rows are [gate][own units]: the reduction runs over 3 Un values
-    for (int g = 0; g < 3; ++g) {
+    for (int g = SPLIT ? gs : 0; g < (SPLIT ? gs + 1 : 3); ++g) {
       const float* ag = a0 + g * U;
       const float* wg = Ws + (i64)g * U * H + 4 * x.u;
 #pragma unroll 1
@@ -361,14 +352,14 @@ __device__ __forceinline__ void adj_product(const F32Args& a, const F32Phase& p,
       }
     }
     const int n = 4 * x.u, d = n / U;
-    float* dst0 = Pb + ((i64)rank * p.R) * U + (n - d * U);
+    float* dst0 = Pb + ((i64)(SPLIT ? rank * 3 + gs : rank) * p.R) * U + (n - d * U);
 #pragma unroll
     for (int r = 0; r < RT; ++r) {
       float4 v = make_float4(acc[r][0], acc[r][1], acc[r][2], acc[r][3]);
 #pragma unroll
       for (int o = 1; o < KP; o <<= 1) {
-        v.x += __shfl_xor_sync(0xffffffffu, v.x, o); v.y += __shfl_xor_sync(0xffffffffu, v.y, o);
-        v.z += __shfl_xor_sync(0xffffffffu, v.z, o); v.w += __shfl_xor_sync(0xffffffffu, v.w, o);
+        v.x += __shfl_xor_sync(0xffffffffu, v.x, 8 * o); v.y += __shfl_xor_sync(0xffffffffu, v.y, 8 * o);
+        v.z += __shfl_xor_sync(0xffffffffu, v.z, 8 * o); v.w += __shfl_xor_sync(0xffffffffu, v.w, 8 * o);
       }
       if (r / NR == x.kp && x.live) {
         float* q = dst0 + (x.rg * RT + r) * U;
@@ -386,10 +377,13 @@ __global__ void __launch_bounds__(kMaxThreads, 1) f32_adj_kernel(const __grid_co
   __shared__ int rk[kMaxRows], rb[kMaxRows], verdict;
   const int H = a.H, rank = MULTI ? (int)ctarank() : 0, u0 = rank * U, Un = max(0, min(U, H - u0)), lda = 3 * U + 4, U4 = Un / 4;
   const int cid = blockIdx.x / NC, ncl = gridDim.x / NC;
+  // with one quadruple the next step's coefficients are requested in front of the product; two of them do not fit the registers
+  // next to its sums, and such launches have enough work per step to bear the wait
+  constexpr bool kAhead = kQ == 1;
   float* Ws = fsm;
   float* Ad = Ws + 3 * U * H;
   float* Pbuf = Ad + rmax * lda;
-  const int pstride = NC * rmax * U;
+  const int pstride = 3 * NC * kSplitRows * U > NC * rmax * U ? 3 * NC * kSplitRows * U : NC * rmax * U;
   for (int e = threadIdx.x; e < 3 * Un * (H / 4); e += blockDim.x) {
     const int r = e / (H / 4), c = e % (H / 4), g = r / Un, i = r % Un;
     *reinterpret_cast<float4*>(Ws + (i64)(g * U + i) * H + 4 * c) = __ldg(reinterpret_cast<const float4*>(a.W + ((i64)g * H + u0 + i) * H) + c);
@@ -449,9 +443,10 @@ __global__ void __launch_bounds__(kMaxThreads, 1) f32_adj_kernel(const __grid_co
       auto product = [&]() {
         float* Pb = Pbuf + par * pstride;
         switch (p.KP) {
-          case 1: adj_product<1>(a, p, Ws, Ad, Pb, lda, U, Un, NC, rank, MULTI); break;
-          case 2: adj_product<2>(a, p, Ws, Ad, Pb, lda, U, Un, NC, rank, MULTI); break;
-          default: adj_product<4>(a, p, Ws, Ad, Pb, lda, U, Un, NC, rank, MULTI); break;
+          case 1: adj_product<1, false>(a, p, Ws, Ad, Pb, lda, U, Un, NC, rank, MULTI); break;
+          case 2: adj_product<2, false>(a, p, Ws, Ad, Pb, lda, U, Un, NC, rank, MULTI); break;
+          case 4: adj_product<4, false>(a, p, Ws, Ad, Pb, lda, U, Un, NC, rank, MULTI); break;
+          default: adj_product<4, true>(a, p, Ws, Ad, Pb, lda, U, Un, NC, rank, MULTI); break;
         }
         block_sync<MULTI>();
       };
@@ -460,7 +455,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1) f32_adj_kernel(const __grid_co
         float4 s = z4;
         if (!where(q, &row, &u)) return s;
         const float* Pb = Pbuf + par * pstride + row * U + u;
-        for (int c = 0; c < NC; ++c) {
+        for (int c = 0; c < (p.KP == kSplitKP ? 3 * NC : NC); ++c) {
           const float4 t = *reinterpret_cast<const float4*>(Pb + (i64)c * p.R * U);
           s.x += t.x; s.y += t.y; s.z += t.z; s.w += t.w;
         }
@@ -474,6 +469,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1) f32_adj_kernel(const __grid_co
         __syncthreads();
 #pragma unroll
         for (int q = 0; q < kQ; ++q) {
+          if (!kAhead) continue;
           if (j + 1 < steps) coefs(q, j + 1, false);
           else if (coarse) { coefs(q, p.n, true); m2[q] = start(q, p.src2, p.src2_ks, nullptr, 0); }
         }
@@ -488,6 +484,10 @@ __global__ void __launch_bounds__(kMaxThreads, 1) f32_adj_kernel(const __grid_co
             const i64 bo = (i64)rb[row] * H + u0 + u;
             if (last) { if (k < p.nfull) *reinterpret_cast<float4*>(p.last + k * p.last_ks + bo) = x[q].m; }
             else if (j < (k < p.nfull ? p.n : p.ntail)) *reinterpret_cast<float4*>(p.out + k * p.out_ks + j * p.out_ss + bo) = x[q].m;
+          }
+          if (!kAhead) {
+            if (j + 1 < steps) coefs(q, j + 1, false);
+            else if (coarse) { coefs(q, p.n, true); m2[q] = start(q, p.src2, p.src2_ks, nullptr, 0); }
           }
           if (vstep) { v[q] = x[q].m; x[q].m = m2[q]; }
           if (j + 1 < steps || coarse) form(q);
@@ -524,7 +524,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1) f32_adj_kernel(const __grid_co
 
 // ---- linearisation: the forward product of every level's rows with the transposed-Jacobian epilogue; no exchange
 struct LinSet { LinArgs l[kF32Levels]; int n, blk0[kF32Levels + 1]; };
-__global__ void __launch_bounds__(kMaxThreads, 1) f32_lin_kernel(const __grid_constant__ LinSet ls, int U, int R) {
+__global__ void __launch_bounds__(kFwdThreads, 1) f32_lin_kernel(const __grid_constant__ LinSet ls, int U, int R) {
   extern __shared__ __align__(16) float fsm[];
   const int H = ls.l[0].H, B = ls.l[0].B, ld = H + 4, u0 = blockIdx.x * U, Un = min(U, H - u0);
   float* Ws = fsm;
@@ -550,7 +550,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1) f32_lin_kernel(const __grid_co
       *reinterpret_cast<float4*>(S + r * ld + 4 * c) = v;
     }
     __syncthreads();
-    constexpr int RT = Tile<1>::RT;
+    constexpr int RT = FTile<1>::RT;
     const int RG = R / RT, items = ((Un + 7) / 8) * 8 * RG;
     for (int it = threadIdx.x; it < items; it += blockDim.x) {
       const Item x = item_of<1>(it, RG, Un);
@@ -589,7 +589,7 @@ int* status_ptr() {
 // CTAs per cluster, units per CTA and the shared memory of `R` rows per block
 struct Shape { int NC, U; };
 size_t fwd_bytes(int H, int U, int R) { return (size_t)((3 * U + 2 * R) * (H + 4) + 3 * U) * 4; }
-size_t adj_bytes(int H, int U, int NC, int R) { return (size_t)(3 * U * H + R * (3 * U + 4) + 2 * NC * R * U) * 4; }
+size_t adj_bytes(int H, int U, int NC, int R) { return (size_t)(3 * U * H + R * (3 * U + 4) + 2 * NC * (R > 3 * kSplitRows ? R : 3 * kSplitRows) * U) * 4; }
 size_t shape_bytes(bool adj, int H, Shape q, int R) { return adj ? adj_bytes(H, q.U, q.NC, R) : fwd_bytes(H, q.U, R); }
 bool pick_shape(int H, Shape* q) {
   for (int nc = 1; nc <= 8; nc *= 2) {
@@ -611,14 +611,17 @@ void tune(bool adj, F32Phase& p, int H, Shape q, int ncl, int M, int fixed_kp) {
     if (adj && (i64)R * q.U / 4 > (i64)kMaxQ * kMaxThreads) break;
     const int cols = (((adj ? H / 4 : q.U) + 7) / 8) * 8;
     int KP = fixed_kp > 0 ? fixed_kp : 1;
-    while (fixed_kp == 0 && KP < 4 && cols * (R / 4) * KP * 2 <= kMaxThreads) KP *= 2;
-    if (KP == 1 && R % Tile<1>::RT != 0) continue;
-    const int base = cols * (R / (KP == 1 ? Tile<1>::RT : 4));
-    if (KP > 1 && base * KP > kMaxThreads) continue;      // lanes share a sum only where every item has a thread
-    const int items = base * KP, passes = (items + kMaxThreads - 1) / kMaxThreads, nt = ((items + passes - 1) / passes + 31) / 32 * 32;
+    const int most = adj ? kMaxThreads : kFwdThreads;
+    while (fixed_kp == 0 && KP < 4 && cols * (R / 4) * KP * 2 <= most) KP *= 2;
+    if (fixed_kp == 0 && adj && KP == 4 && R <= kSplitRows && cols * (R / 4) * kSplitKP <= kMaxThreads) KP = kSplitKP;
+    if (KP == kSplitKP && R > kSplitRows) continue;
+    const int rt = adj && KP == 1 ? Tile<1>::RT : 4, base = cols * (R / rt);
+    if (R % rt != 0) continue;
+    if ((KP > 1 || !adj) && base * KP > most) continue;   // lanes share a sum only where every item has a thread; forward: always
+    const int items = base * KP, passes = (items + most - 1) / most, nt = ((items + passes - 1) / passes + 31) / 32 * 32;
     const int waves = ((M + R - 1) / R + ncl - 1) / ncl;
     // cycles of one item's operand delivery, with one warp on each of the four schedulers
-    const double rt = KP == 1 ? 8 : 4, per = adj ? (rt + 4.0) * 4 * 3.0 * q.U : (rt + 3.0) * 4 * H;
+    const double per = adj ? (rt + 4.0) * 4 * 3.0 * q.U : (rt + 3.0) * 4 * H;
     const double t = waves * (1500.0 + passes * ((nt / 32 + 3) / 4) * per / KP);
     if (t < best - 1e-9) { best = t; p.R = R; p.KP = KP; p.nt = nt; }
     if (R >= M && best < 1e30) break;
@@ -626,9 +629,9 @@ void tune(bool adj, F32Phase& p, int H, Shape q, int ncl, int M, int fixed_kp) {
 }
 
 template <class K>
-int max_clusters(K kern, int nc, size_t smem) {      // co-resident clusters of this shape on the current device
+int max_clusters(K kern, int nc, int threads, size_t smem) {      // co-resident clusters of this shape on the current device
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(nc); cfg.blockDim = dim3(kMaxThreads); cfg.dynamicSmemBytes = smem;
+  cfg.gridDim = dim3(nc); cfg.blockDim = dim3(threads); cfg.dynamicSmemBytes = smem;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = nc; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
@@ -645,7 +648,7 @@ bool launch_solve(bool adj, const F32Args& a, Shape q, int blocks, int rmax, cud
   if (!st || !set_smem_once(kern, (int)kSmemMax, attr)) return false;
   if (cudaMemsetAsync(a.bar, 0, sizeof(unsigned), s) != cudaSuccess) return false;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(blocks * q.NC); cfg.blockDim = dim3(kMaxThreads); cfg.dynamicSmemBytes = shape_bytes(adj, a.H, q, rmax); cfg.stream = s;
+  cfg.gridDim = dim3(blocks * q.NC); cfg.blockDim = dim3(adj ? kMaxThreads : kFwdThreads); cfg.dynamicSmemBytes = shape_bytes(adj, a.H, q, rmax); cfg.stream = s;
   cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeCooperative;       // the grid barrier needs every CTA resident
   at[0].val.cooperative = 1;
@@ -673,7 +676,7 @@ bool f32_solve(bool adjoint, F32Args& a, cudaStream_t s) {
   if (ncl == 0) {
     auto count = [&](auto kern) {
       if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax) != cudaSuccess) { cudaGetLastError(); return 0; }
-      return max_clusters(kern, q.NC, kSmemMax);
+      return max_clusters(kern, q.NC, adjoint ? kMaxThreads : kFwdThreads, kSmemMax);
     };
     ncl = adjoint ? count(f32_adj_kernel<true, 2>) : count(f32_fwd_kernel<true>);
   }
@@ -710,7 +713,7 @@ bool f32_linearise(const LinArgs* levels, int n, cudaStream_t s) {
   for (int l = 0; l < n; ++l) ls.blk0[l + 1] = ls.blk0[l] + (levels[l].M + R - 1) / R;
   const int gx = (H + q.U - 1) / q.U, gy = ls.blk0[n] < 148 / gx ? ls.blk0[n] : 148 / gx;
   ProfScope prof(KC_LINEARISE, flops, s);
-  f32_lin_kernel<<<dim3(gx, gy), kMaxThreads, (size_t)(3 * q.U + R) * (H + 4) * 4, s>>>(ls, q.U, R);
+  f32_lin_kernel<<<dim3(gx, gy), kFwdThreads, (size_t)(3 * q.U + R) * (H + 4) * 4, s>>>(ls, q.U, R);
   count_launch();
   return true;
 }
