@@ -128,9 +128,9 @@ GiTail gi_tail(const mgrit_gru_cfg* c, float* gi) {
   t.total_bytes = off;
   return t;
 }
-// the copies exist when the tensor-core engine keeps bf16 shadows of the level states (B divides 128) in an MGRIT solve
+// the copies exist when the tensor-core engine keeps bf16 shadows of the level states (B <= 128) in an MGRIT solve
 bool carries_copies(const mgrit_gru_cfg* c, bool serial) {
-  return !serial && (c->flags & MGRIT_FLAG_GI_CARRIES_COPIES) && c->operands == MGRIT_OPERANDS_BF16 && 128 % c->B == 0 && c->levels > 1;
+  return !serial && (c->flags & MGRIT_FLAG_GI_CARRIES_COPIES) && c->operands == MGRIT_OPERANDS_BF16 && c->B <= 128 && c->levels > 1;
 }
 
 // MGRIT_GRU_GI_BF16=0 in the environment keeps the fused kernels on the fp32 input projection (A/B measurements).
@@ -352,14 +352,43 @@ struct FwdCycle : Cycle {
     if (!gi_f32) { a.gi_b = gib + (st - 1) * (i64)BH * 3; a.gi = nullptr; }
     a.g = G[l]; a.W = um->W_hh; a.b_hh = p->b_hh; a.gamma = hr.gamma[l]; a.cell = c->cell; a.bar = fw->chain_bar;
     a.xw = fw->chain_xw; a.xw_bytes = fw->chain_xw_bytes;
-    return serial_fwd_solve(a, s);
+    return serial_fwd_solve(a, s) || chain_by_sweeps(l);
+  }
+  // The dependent steps of a level whose rows and weights do not fit the chain kernel (many batch rows at a large width): sweeps
+  // over ONE interval of N_l points, up to kMaxFwdSweepSteps steps per launch (100 rows at H = 1024: 34 -> 13 us a step).
+  bool chain_by_sweeps(int l) {
+    const int N = hr.N[l], kMax = kMaxFwdSweepSteps;
+    if (!Ub || c->B > 128 || N < 2 || !fw->sweep_ctr || fw->sweep_ctr_used + N > fw->sweep_ctr_n) return false;
+    const i64 st = hr.stride_t[l];
+    for (int j0 = 1; j0 <= N && rc == MGRIT_OK; j0 += kMax) {
+      FwdSweepArgs a{};
+      a.B = c->B; a.H = c->H; a.nk = 1; a.cf = N; a.n = N - j0 + 1 < kMax ? N - j0 + 1 : kMax;
+      a.U = U[l]; a.Ub = Ub[l];
+      a.gi = gi + (st - 1) * (i64)BH * 3; a.gi_ss = st * (i64)BH * 3; a.gi_ks = st * N * (i64)BH * 3;
+      a.gi_b = gib ? gib + (st - 1) * (i64)BH * 3 : nullptr;
+      a.g = G[l] ? G[l] + BH : nullptr;
+      a.b_hh = p->b_hh; a.gamma = hr.gamma[l]; a.cell = c->cell; a.ctr = fw->sweep_ctr + fw->sweep_ctr_used;
+      for (int i = 0; i < a.n; ++i) {
+        FwdSweepStep& q = a.st[i];
+        const int j = j0 + i;
+        q.in_s = q.tgt_s = j - 1; q.nk = 1; q.dep = 1;
+        q.out = U[l] + (size_t)j * BH; q.out_ks = (i64)N * BH; q.out_b = Ub[l] + (size_t)j * BH;
+      }
+      const int r = umma_fwd_sweep(a, um, s);
+      if (r == MGRIT_UNSUPPORTED && j0 == 1) return false;
+      fw->sweep_ctr_used += a.n;
+      if (r != MGRIT_OK) rc = r;
+    }
+    return true;
   }
   bool launch_sweep(int l, const int* kinds, int n) override {
     const int cf = c->cf;
-    if (c->operands != MGRIT_OPERANDS_BF16 || !Ub || hr.N[l] % cf != 0 || n > kMaxFwdSweepSteps) return false;
+    const int tail = hr.N[l] % cf;      // F-points behind the last C-point (ragged levels): a shorter last interval
+    if (c->operands != MGRIT_OPERANDS_BF16 || !Ub || c->B > 128 || hr.N[l] < cf || n > kMaxFwdSweepSteps) return false;
     FwdSweepArgs a{};
     a.B = c->B; a.H = c->H; a.nk = hr.N[l] / cf; a.cf = cf; a.n = n;
-    const size_t need = (size_t)n * (((size_t)a.nk * c->B + 127) / 128);
+    const int kt = 128 / c->B;
+    const size_t need = (size_t)n * ((a.nk + (tail > 0 ? 1 : 0) + kt - 1) / kt);
     if (!fw->sweep_ctr || fw->sweep_ctr_used + need > fw->sweep_ctr_n) return false;
     a.U = U[l]; a.Ub = Ub[l];
     const i64 st = hr.stride_t[l];
@@ -371,6 +400,7 @@ struct FwdCycle : Cycle {
     for (int i = 0; i < n; ++i) {
       FwdSweepStep& q = a.st[i];
       const int kd = kinds[i], prev = i ? kinds[i - 1] : 0;
+      q.nk = a.nk + (kd < cf && kd <= tail ? 1 : 0);
       if (kd < cf) {             // F-step to slot kd
         q.in_s = kd - 1; q.tgt_s = kd - 1;
         q.out = U[l] + (size_t)kd * BH; q.out_ks = (i64)cf * BH; q.out_b = Ub[l] + (size_t)kd * BH;
@@ -628,7 +658,8 @@ int forward_impl(const mgrit_gru_cfg* cfg_in, bool serial, const gru_params* p, 
   }
   if (!gi_bf16_enabled()) fw.um.gib = nullptr;
   // the caller does not read the fp32 projection and every kernel of this solve reads its bf16 copy: do not write it
-  const bool gi_f32 = !((c.flags & MGRIT_FLAG_GI_F32_UNUSED) && carries_copies(&c, serial) && fw.um.gib);
+  // (where B divides 128, as the flag's contract says)
+  const bool gi_f32 = !((c.flags & MGRIT_FLAG_GI_F32_UNUSED) && carries_copies(&c, serial) && 128 % c.B == 0 && fw.um.gib);
 
   if (c.operands == MGRIT_OPERANDS_BF16) {
     rc = umma_prepare_fwd(&c, p, x, gi_f32 ? gi : nullptr, &fw.um, s);
@@ -641,7 +672,7 @@ int forward_impl(const mgrit_gru_cfg* cfg_in, bool serial, const gru_params* p, 
   }
   zero_guess(fw.U[0], c, hr, BH, s);
   for (int l = 0; l < hr.L; ++l) cudaMemcpyAsync(fw.U[l], h0, sizeof(float) * BH, cudaMemcpyDeviceToDevice, s);
-  const bool shadows = c.operands == MGRIT_OPERANDS_BF16 && 128 % c.B == 0;
+  const bool shadows = c.operands == MGRIT_OPERANDS_BF16 && c.B <= 128;
   if (shadows && fw.sweep_ctr) cudaMemsetAsync(fw.sweep_ctr, 0, sizeof(int) * fw.sweep_ctr_n, s);
   if (shadows) {
     zero_guess(fw.Ub[0], c, hr, BH, s);
@@ -699,7 +730,8 @@ int adjoint_impl(const mgrit_gru_cfg* cfg_in, bool serial, const gru_params* p, 
     aw.um.xb = t.xb;
     aw.um.hb0 = t.hb0;
     aw.um.hb = t.hb0 + BH;
-    aw.um.gib = gi_bf16_enabled() ? t.gib : nullptr;
+    // (where B does not divide 128 the flags change no bit: the linearisation stays on the fp32 projection)
+    aw.um.gib = gi_bf16_enabled() && 128 % c.B == 0 ? t.gib : nullptr;
   }
   if (bf16) {
     rc = umma_prepare_adj(&c, p, h0, h, &aw.um, copies, s);

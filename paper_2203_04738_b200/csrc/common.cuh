@@ -109,18 +109,19 @@ struct FwdStepArgs {
 struct FwdSweepStep {
   int in_s, tgt_s;
   float* out; i64 out_ks; __nv_bfloat16* out_b;
+  int nk;        // intervals that take the step: FwdSweepArgs::nk, or one more where the ragged last interval takes it too
   int dep;       // 0: first step; 1: follows a step on the same intervals; 2: follows a step that advanced the C-points
                  // (reads what the neighbouring interval wrote); 3: advances the C-points (must not overtake their readers)
 };
 constexpr int kMaxFwdSweepSteps = 20;
 struct FwdSweepArgs {
-  int B, H, nk, cf, n;
+  int B, H, nk, cf, n;                       // nk complete intervals of cf points
   const float* U; const __nv_bfloat16* Ub;   // level state and its bf16 copy, from slot 0
   const float* gi; i64 gi_ss, gi_ks;         // input projection of target coordinate 0 of interval 0; element strides per slot / interval
   const __nv_bfloat16* gi_b;                 // its bf16 copy (same indexing) or nullptr
   const float* g;                            // FAS term of target coordinate 0 of interval 0 (slots like U), or nullptr
   const float* b_hh; float gamma; int cell;
-  int* ctr;                                  // n * ceil(nk*B / 128) zeroed ints
+  int* ctr;                                  // n * ceil(intervals / floor(128 / B)) zeroed ints
   FwdSweepStep st[kMaxFwdSweepSteps];
 };
 

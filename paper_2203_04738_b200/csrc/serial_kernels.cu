@@ -204,6 +204,9 @@ __device__ __forceinline__ void warp_gemm_regs(const bf16* As, int ldk, int kbeg
   }
 }
 
+// first reduction index of warp `w`: the K / 16 steps of sixteen split as evenly as they go over the warps (K % 16 == 0)
+__device__ __forceinline__ int warp_k(int K, int w) { return (K / 16 * w / kWarps) * 16; }
+
 // warp partial sums -> red[warp][row][col]   (col < NT*8)
 template <int NT>
 __device__ __forceinline__ void store_partials(float* red, float (*acc)[4]) {
@@ -301,7 +304,7 @@ __global__ void __launch_bounds__(kThreads, 1) serial_fwd_kernel(SerialFwdArgs a
 #pragma unroll
     for (int nt = 0; nt < NT; ++nt) acc[nt][0] = acc[nt][1] = acc[nt][2] = acc[nt][3] = 0.f;
     if (KS > 0) warp_gemm_regs<NT, (KS > 0 ? KS : 1)>(As, ldk, warp * kw, wreg, acc);
-    else warp_gemm<NT>(As, Ws, ldk, warp * kw, (warp + 1) * kw, acc);
+    else warp_gemm<NT>(As, Ws, ldk, warp_k(H, warp), warp_k(H, warp + 1), acc);
     store_partials<NT>(red, acc);
     __syncthreads();
     bf16* ub = a.ub + (i64)(j & 1) * BH;
@@ -421,7 +424,7 @@ __global__ void __launch_bounds__(kThreads, 1) serial_adj_kernel(SerialAdjArgs a
 #pragma unroll
     for (int nt = 0; nt < NT; ++nt) acc[nt][0] = acc[nt][1] = acc[nt][2] = acc[nt][3] = 0.f;
     if (KS > 0) warp_gemm_regs<NT, (KS > 0 ? KS : 1)>(As, ldk, warp * kw, wreg, acc);
-    else warp_gemm<NT>(As, Ws, ldk, warp * kw, (warp + 1) * kw, acc);
+    else warp_gemm<NT>(As, Ws, ldk, warp_k(K, warp), warp_k(K, warp + 1), acc);
     store_partials<NT>(red, acc);
     __syncthreads();
     bf16* dAb = a.dAb + (i64)(s & 1) * 3 * BH;
@@ -538,12 +541,11 @@ __global__ void __launch_bounds__(kThreads, 1) lstm_fwd_chain_kernel(LstmChainFw
   }
   __syncthreads();
 
-  const int kw = H / kWarps;
   for (int j = 1; j <= a.nsteps; ++j) {
     float acc[NT][4];
 #pragma unroll
     for (int nt = 0; nt < NT; ++nt) acc[nt][0] = acc[nt][1] = acc[nt][2] = acc[nt][3] = 0.f;
-    warp_gemm<NT>(As, Ws, ldk, warp * kw, (warp + 1) * kw, acc);
+    warp_gemm<NT>(As, Ws, ldk, warp_k(H, warp), warp_k(H, warp + 1), acc);
     store_partials<NT>(red, acc);
     __syncthreads();
 #pragma unroll
@@ -962,7 +964,7 @@ size_t adj_smem(int unc, int H) { return (size_t)(unc + kRows) * (3 * H + 8) * 2
 
 // smallest units-per-CTA whose grid is co-resident (one CTA per SM) and whose slice fits shared memory
 int pick_unc(int B, int H, bool adj) {
-  if (H % 128 != 0) return 0;
+  if (H % 64 != 0) return 0;
   int rgs = (B + kRows - 1) / kRows;
   const int cands[3] = {8, 16, 32};
   for (int c : cands) {
@@ -1110,7 +1112,7 @@ namespace {
 size_t lstm_fwd_smem(int unc, int H) { return (size_t)(4 * unc + kRows) * (H + 8) * 2 + (size_t)kWarps * kRows * 4 * unc * 4; }
 size_t lstm_adj_smem(int unc, int H) { return (size_t)kRows * (4 * H + 8) * 2 + (size_t)kWarps * kRows * unc * 4; }
 int lstm_pick_unc(int B, int H, bool adj) {
-  if (adj ? !(H == 128 || H == 256 || H == 512 || H == 1024) : H % 128 != 0) return 0;
+  if (adj ? !(H == 128 || H == 256 || H == 512 || H == 1024) : H % 64 != 0) return 0;
   const int rgs = (B + kRows - 1) / kRows;
   const int cands[3] = {8, 16, 32};
   for (int c : cands) {

@@ -1,6 +1,7 @@
 // Adjoint step product with TMA-staged epilogue operands, sm_100a:
 //
-//   rows m = (k, b)          k = interval / coarse point, b = batch row, 128 rows per CTA = kt k's x B
+//   rows m = (k, b)          k = interval / coarse point, b = batch row; a CTA tile is kt = floor(128 / B) k's x B rows (the
+//                            operand rows behind them belong to the next tile and are computed there)
 //   D[m, n]   = sum_j dA[m, j] * W_hhT[n, j]           dA = [c_r | c_z | c_n] * lambda as bf16 [M, 3H] (packed beforehand)
 //   out[m, n] = a[m, n] * lambda[m, n] + D[m, n] (+ g[m, n])      or   g - (...)   (mode 1)
 //
@@ -22,7 +23,7 @@ namespace mg {
 namespace umma {
 
 struct AdjKArgs {
-  int M, B, H, kt, nk;                // kt = 128 / B
+  int M, B, H, kt, nk;                // kt = 128 / B, whole k's per CTA tile
   float* lout; i64 lout_ks;           // result rows (k, b)
   int a_rev;                          // 1: the coefficient map runs backwards in k (coordinate nk - 1 - k)
   int mode;
@@ -72,8 +73,9 @@ umma_adj_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
   const int H = p.H;
   const uint32_t rank = PAIR ? cluster_ctarank() : 0u;
   const int cta = PAIR ? (int)(blockIdx.x >> 1) : (int)blockIdx.x, ncta = PAIR ? (int)(gridDim.x >> 1) : (int)gridDim.x;
-  constexpr int kTileRows = PAIR ? 2 * BM : BM;
-  const int m_tiles = (p.M + kTileRows - 1) / kTileRows, n_tiles = (H + BNa - 1) / BNa, tiles = m_tiles * n_tiles;
+  const int tile_k = PAIR ? 2 * p.kt : p.kt, rt = p.kt * p.B;        // k's per tile, rows per CTA
+  const uint32_t epi_tx = (uint32_t)(C::kEpiBytes / BM * rt);
+  const int m_tiles = (p.nk + tile_k - 1) / tile_k, n_tiles = (H + BNa - 1) / BNa, tiles = m_tiles * n_tiles;
   const int k_blocks = (K + BK - 1) / BK;
   // Row tiles from the last to the first: the packing kernel writes the operand rows in ascending order and most of the
   // 100 MB of a 16384-row step have left L2 by the time it ends, except the rows written last (and this kernel's
@@ -127,12 +129,12 @@ umma_adj_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
             // the packed operand is read once: let it leave L2 first
             asm volatile(
                 "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%3, %4}], [%2], %5;"
-                ::"r"(a_dst), "l"(&tmA), "r"(fullL), "r"(kb * BK), "r"(mt * BM), "l"(drop_policy)
+                ::"r"(a_dst), "l"(&tmA), "r"(fullL), "r"(kb * BK), "r"(mt * rt), "l"(drop_policy)
                 : "memory");
             tma_load_2d_pair(b_dst, &tmB, fullL, kb * BK, nt * BNa + (int)rank * (BNa / 2));
           } else {
             mbar_expect_tx(full_bar(stage), kStageBytes);
-            tma_load_2d(a_dst, &tmA, full_bar(stage), kb * BK, mt * BM);
+            tma_load_2d(a_dst, &tmA, full_bar(stage), kb * BK, mt * rt);
             tma_load_2d(b_dst, &tmB, full_bar(stage), kb * BK, nt * BNa);
           }
           if (++stage == C::kStages) { stage = 0; phase ^= 1u; }
@@ -191,7 +193,7 @@ umma_adj_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
           if (n >= H) break;
           if (!mbar_wait(eempty_bar(eb), ephase ^ 1u, abortp, status, 34)) { ok = false; break; }
           const uint32_t dst = epi_base + eb * C::kEpiBytes;
-          mbar_expect_tx(efull_bar(eb), C::kEpiBytes);
+          mbar_expect_tx(efull_bar(eb), epi_tx);
           tma_load_3d(dst, &tmL, efull_bar(eb), n, 0, k0);
           tma_load_3d(dst + kOpB, &tmCa, efull_bar(eb), n, 0, ka);
           if (HAS_G) tma_load_3d(dst + 2 * kOpB, &tmG, efull_bar(eb), n, 0, k0);
@@ -205,7 +207,7 @@ umma_adj_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     const int half = (warp - 3) >> 2;    // which 8 of a chunk's 16 columns
     const int r = q * 32 + lane;         // row inside the CTA's 128 rows
     const int kl = r / p.B, bl = r - kl * p.B;
-    const int ra = p.a_rev ? (p.kt - 1 - kl) * p.B + bl : r;     // where this row's coefficients sit in their tile
+    const int ra = p.a_rev && r < rt ? (p.kt - 1 - kl) * p.B + bl : r;     // where this row's coefficients sit in their tile
     auto swz = [&](int row, uint32_t piece) { return (uint32_t)row * 64u + ((piece ^ ((uint32_t)(row >> 1) & 3u)) << 4); };
     const uint32_t off0 = swz(r, (uint32_t)half * 2u), off1 = swz(r, (uint32_t)half * 2u + 1u);
     const uint32_t oa0 = swz(ra, (uint32_t)half * 2u), oa1 = swz(ra, (uint32_t)half * 2u + 1u);
@@ -215,9 +217,8 @@ umma_adj_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
       const int mt = row_tile(t), nt = t % n_tiles;
       const int as = it & 1;
       const uint32_t aphase = (uint32_t)(it >> 1) & 1u;
-      const int row = mt * BM + r;
-      const bool valid = row < p.M;
       const int k = mt * p.kt + kl;
+      const bool valid = r < rt && k < p.nk;
       if (ok && !mbar_wait(tfull_bar(as), aphase, abortp, status, 35)) ok = false;
       ok = __all_sync(0xffffffffu, ok);
       tc_fence_after();

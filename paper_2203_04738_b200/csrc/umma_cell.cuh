@@ -1,7 +1,10 @@
 // Fused "recurrent GEMM + GRU cell" kernel for sm_100a: every operand of the epilogue is staged through
 // shared memory by TMA, so that the only latency-exposed global accesses of the epilogue are its stores.
 //
-//   rows m = (k, b)      k = interval / coarse point, b = batch row, 128 rows per CTA tile = kt k's x B
+//   rows m = (k, b)      k = interval / coarse point, b = batch row; a CTA tile is kt = floor(128 / B) k's x B rows.  Where B does
+//                        not divide 128 the last 128 - kt*B rows of the tile hold whatever the stage held before: rows never
+//                        meet in the product, and these are never stored (B = 100: 78 % of the MMA rows count, still three
+//                        times the rate of the row-per-thread kernels that gathered their operands; B = 24: 94 %)
 //   D[m, gate, u] = sum_j hb[m, j] * W_hh[gate*H + u, j]          (tcgen05, bf16 x bf16 -> fp32 in TMEM)
 //   forward : out[m, u] = Phi_gamma(gi[m, :, u], D + b_hh, h[m, u]) (+ g[m, u])   or   g - Phi   (mode 1)
 //   linearise: a, c_r, c_z, c_n, c_n'[m, u] = transposed-Jacobian coefficients of that step
@@ -134,7 +137,7 @@ __device__ __forceinline__ float4 lds4(uint32_t addr) {
 }
 
 struct CellArgs {
-  int M, B, H, kt;                                    // kt = 128 / B
+  int M, B, H, kt, nk;                                // kt = 128 / B (whole k's per CTA tile); nk: intervals, the ragged last one included
   float* hout; i64 hout_ks; __nv_bfloat16* hout_b;    // forward: fp32 rows (k, b) and their bf16 copy (or nullptr)
   float* a;                                           // linearise: row-major [M, H]; a in fp32,
   __nv_bfloat16 *cr, *cz, *cn, *cnp;                  // the gate coefficients in bf16 (cnp may be nullptr)
@@ -152,6 +155,8 @@ struct SweepStep {
   float* hout; i64 hout_ks; __nv_bfloat16* hout_b;   // destination rows (k, b): fp32 state and its bf16 copy (or nullptr)
   int in_s;     // slot coordinate of the state the step starts from (maps A and HP)
   int tgt_s;    // slot coordinate of the point it arrives at (maps GI and G)
+  int nk;       // complete k's: rows of later k's are not stored (ragged levels: the last, shorter interval)
+  int ext;      // 1: the maps that include the last, shorter interval (tmCR, tmCZ, tmCN, tmCP instead of A, GI, HP, G)
   int dep;      // row tiles of the previous step that must be complete: 0 none, 1 {mt}, 2 {mt - 1, mt}, 3 {mt, mt + 1}
 };
 struct SweepArgs {
@@ -264,9 +269,10 @@ umma_cell_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   // PAIR: a tile is 256 rows; CTA `rank` of the pair owns its rows [128 rank, 128 rank + 128).
   const uint32_t rank = PAIR ? cluster_ctarank() : 0u;
   const int cta = PAIR ? (int)(blockIdx.x >> 1) : (int)blockIdx.x, ncta = PAIR ? (int)(gridDim.x >> 1) : (int)gridDim.x;
-  constexpr int kTileRows = PAIR ? 2 * BM : BM;
-  const int m_tiles = (p.M + kTileRows - 1) / kTileRows, n_tiles = (H + UN - 1) / UN, tiles = m_tiles * n_tiles;
+  const int tile_k = PAIR ? 2 * p.kt : p.kt, rt = p.kt * p.B;        // k's per tile, rows per CTA
+  const int m_tiles = (p.nk + tile_k - 1) / tile_k, n_tiles = (H + UN - 1) / UN, tiles = m_tiles * n_tiles;
   const int k_blocks = (H + BK - 1) / BK;
+  const uint32_t stage_tx = (uint32_t)(rt * BK * 2 + G::kBBytes), epi_tx = (uint32_t)(C::kEpiBytes / BM * rt);   // bytes that really arrive
   auto row_tile = [&](int t) { return PAIR ? 2 * (t / n_tiles) + (int)rank : t / n_tiles; };
   // forward: items (step, tile); the linearisation is a single step
   const int n_items = LIN ? tiles : tiles * swp.n_steps;
@@ -321,6 +327,7 @@ umma_cell_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         const int sg = LIN ? 0 : w / tiles, t = w - sg * tiles;
         const int mt = row_tile(t), nt = t % n_tiles;
         const int in_s = LIN ? 0 : swp.st[sg].in_s;
+        const CUtensorMap* mapA = !LIN && swp.st[sg].ext ? &tmCR : &tmA;
         if (!deps_ready(sg, t / n_tiles, 17)) { ok = false; break; }
         for (int kb = 0; kb < k_blocks; ++kb) {
           if (!mbar_wait(empty_bar(stage), phase ^ 1u, abortp, status, 11)) { ok = false; break; }
@@ -329,18 +336,18 @@ umma_cell_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             // The accumulator columns r | z | n (80 each) split into two halves of 120: CTA 0 stages the weight rows
             // of r and of the first 40 units of z, CTA 1 the rest -- six 40-row boxes, three per CTA.
             const uint32_t fullL = mapa_shared(full_bar(stage), 0);
-            if (rank == 0) mbar_expect_tx(full_bar(stage), 2 * kStageBytes);
+            if (rank == 0) mbar_expect_tx(full_bar(stage), 2 * stage_tx);
             if (LIN) tma_load_3d_pair(a_dst, &tmA, fullL, kb * BK, 0, mt * p.kt);
-            else tma_load_4d_pair(a_dst, &tmA, fullL, kb * BK, 0, in_s, mt * p.kt);
+            else tma_load_4d_pair(a_dst, mapA, fullL, kb * BK, 0, in_s, mt * p.kt);
 #pragma unroll
             for (int j = 0; j < 3; ++j) {
               const int piece = 3 * (int)rank + j;
               tma_load_2d_pair(b_dst + j * (G::kBox * BK * 2), &tmB, fullL, kb * BK, (piece >> 1) * H + nt * UN + (piece & 1) * G::kBox);
             }
           } else {
-            mbar_expect_tx(full_bar(stage), kStageBytes);
+            mbar_expect_tx(full_bar(stage), stage_tx);
             if (LIN) tma_load_3d(a_dst, &tmA, full_bar(stage), kb * BK, 0, mt * p.kt);
-            else tma_load_4d(a_dst, &tmA, full_bar(stage), kb * BK, 0, in_s, mt * p.kt);
+            else tma_load_4d(a_dst, mapA, full_bar(stage), kb * BK, 0, in_s, mt * p.kt);
 #pragma unroll
             for (int g = 0; g < 3; ++g) tma_load_2d(b_dst + g * (G::kBBytes / 3), &tmB, full_bar(stage), kb * BK, g * H + nt * UN);
           }
@@ -395,24 +402,26 @@ umma_cell_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         const int sg = LIN ? 0 : w / tiles, t = w - sg * tiles;
         const int mt = row_tile(t), nt = t % n_tiles;
         const int in_s = LIN ? 0 : swp.st[sg].in_s, tgt_s = LIN ? 0 : swp.st[sg].tgt_s;
+        const bool ext = !LIN && swp.st[sg].ext;
+        const CUtensorMap *mapGI = ext ? &tmCZ : &tmGI, *mapHP = ext ? &tmCN : &tmHP, *mapG = ext ? &tmCP : &tmG;
         if (!deps_ready(sg, t / n_tiles, 18)) { ok = false; break; }
         for (int c = 0; c < NCH; ++c) {
           const int u = nt * UN + c * CH, k0 = mt * p.kt;
           if (u >= H) break;                       // ragged last unit tile: these columns are never stored
           if (!mbar_wait(eempty_bar(eb), ephase ^ 1u, abortp, status, 14)) { ok = false; break; }
           const uint32_t dst = epi_base + eb * C::kEpiBytes;
-          mbar_expect_tx(efull_bar(eb), C::kEpiBytes);
+          mbar_expect_tx(efull_bar(eb), epi_tx);
           if (LIN) {
             tma_load_3d(dst, &tmGI, efull_bar(eb), u, 0, k0);
             tma_load_3d(dst + kGi, &tmGI, efull_bar(eb), H + u, 0, k0);
             tma_load_3d(dst + 2 * kGi, &tmGI, efull_bar(eb), 2 * H + u, 0, k0);
             tma_load_3d(dst + 3 * kGi, &tmHP, efull_bar(eb), u, 0, k0);
           } else {
-            tma_load_4d(dst, &tmGI, efull_bar(eb), u, 0, tgt_s, k0);
-            tma_load_4d(dst + kGi, &tmGI, efull_bar(eb), H + u, 0, tgt_s, k0);
-            tma_load_4d(dst + 2 * kGi, &tmGI, efull_bar(eb), 2 * H + u, 0, tgt_s, k0);
-            tma_load_4d(dst + 3 * kGi, &tmHP, efull_bar(eb), u, 0, in_s, k0);
-            if (HAS_G) tma_load_4d(dst + 3 * kGi + kOpBytes, &tmG, efull_bar(eb), u, 0, tgt_s, k0);
+            tma_load_4d(dst, mapGI, efull_bar(eb), u, 0, tgt_s, k0);
+            tma_load_4d(dst + kGi, mapGI, efull_bar(eb), H + u, 0, tgt_s, k0);
+            tma_load_4d(dst + 2 * kGi, mapGI, efull_bar(eb), 2 * H + u, 0, tgt_s, k0);
+            tma_load_4d(dst + 3 * kGi, mapHP, efull_bar(eb), u, 0, in_s, k0);
+            if (HAS_G) tma_load_4d(dst + 3 * kGi + kOpBytes, mapG, efull_bar(eb), u, 0, tgt_s, k0);
           }
           if (++eb == C::kEpiBufs) { eb = 0; ephase ^= 1u; }
         }
@@ -429,6 +438,7 @@ umma_cell_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     // bf16 coefficient tiles, 32-byte swizzle: rows of 32 bytes, 16-byte piece index XOR ((row >> 2) & 1)
     const uint32_t offb = (uint32_t)r * 32u + ((((uint32_t)half) ^ ((uint32_t)(r >> 2) & 1u)) << 4);
     const bool storer = threadIdx.x == 96;   // the epilogue thread that issues the TMA stores
+    const int kl = r / p.B, b = r - kl * p.B;     // this row's k inside the tile and its batch row
     int it = 0, eb = 0, ob = 0; uint32_t ephase = 0;
     // A thread whose wait ran out (ok = false) keeps walking the loops without touching data, so that the named
     // barrier of the linearisation's store hand-over still sees all 256 epilogue threads.
@@ -438,9 +448,8 @@ umma_cell_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       const int mt = row_tile(t), nt = t % n_tiles;
       const int as = it & 1;
       const uint32_t aphase = (uint32_t)(it >> 1) & 1u;
-      const int row = mt * BM + r;
-      const bool valid = row < p.M;
-      const int k = valid ? row / p.B : 0, b = valid ? row % p.B : 0;
+      const int k = mt * p.kt + kl;
+      const bool valid = r < rt && k < (LIN ? p.nk : swp.st[sg].nk);
       if (ok && !mbar_wait(tfull_bar(as), aphase, abortp, status, 15)) ok = false;
       ok = __all_sync(0xffffffffu, ok);      // warp-uniform: the accumulator loads below are warp-collective
       tc_fence_after();
@@ -515,7 +524,7 @@ umma_cell_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
               CellLin L = cell_linearise<true>(gr[e], gz[e], gn[e], ar[e] + br[e], az[e] + bz[e], an[e] + bn[e], hp[e], p.gamma, p.cell);
               oa[e] = L.a; ocr[e] = L.cr; ocz[e] = L.cz; ocn[e] = L.cn; ocp[e] = L.cnp;
             }
-            const i64 idx = (i64)row * H + u;
+            const i64 idx = ((i64)k * p.B + b) * H + u;
             if (GIB) {      // `a` leaves through shared memory like the coefficients (64-byte rows, 64-byte swizzle)
               const uint32_t da = out_base + ob * C::kOutBytes + 4 * kCoefBytes;
               asm volatile("st.shared.v4.f32 [%0], {%1,%2,%3,%4};" ::"r"(da + off0), "f"(oa[0]), "f"(oa[1]), "f"(oa[2]), "f"(oa[3]) : "memory");
@@ -538,9 +547,9 @@ umma_cell_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
           asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
           if (storer) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
           asm volatile("bar.sync 1, 256;" ::: "memory");
-          if (storer && ok && mt * BM < p.M) {
+          if (storer && ok && mt * rt < p.M) {
             const uint32_t srcb = out_base + ob * C::kOutBytes;
-            const int u = nt * UN + c * CH, row0 = mt * BM;
+            const int u = nt * UN + c * CH, row0 = mt * rt;
             tma_store_2d(&tmCR, srcb, u, row0);
             tma_store_2d(&tmCZ, srcb + kCoefBytes, u, row0);
             tma_store_2d(&tmCN, srcb + 2 * kCoefBytes, u, row0);

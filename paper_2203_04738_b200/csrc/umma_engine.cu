@@ -227,7 +227,7 @@ bool launch_lin_geo(int kc, const bf16* A, i64 a_ks, const void* gi, i64 gi_ks, 
   auto kern = umma_cell_kernel<true, false, PAIR, GIB>;
   if (!set_smem_once(kern, C::kSmemBytes, attr_set)) return false;
   const int B = ca.B, H = ca.H, kt = 128 / B;
-  ca.kt = kt; ca.M = nk * B;
+  ca.kt = kt; ca.nk = nk; ca.M = nk * B;
   CUtensorMap ta, tb, tgi, thp;
   if (!make_map3(&ta, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, A, H, B, nk, H, a_ks, BK, kt, CU_TENSOR_MAP_SWIZZLE_128B)) return false;
   if (!make_map(&tb, W, (uint64_t)H, (uint64_t)3 * H, (uint64_t)H, G::kBox)) return false;
@@ -238,14 +238,14 @@ bool launch_lin_geo(int kc, const bf16* A, i64 a_ks, const void* gi, i64 gi_ks, 
   // the four bf16 coefficient arrays [M, H] are written by TMA stores of [128 x 16] tiles
   CUtensorMap tcr = thp, tcz = thp, tcn = thp, tcp = thp;
   auto cmap = [&](CUtensorMap* m, const bf16* base) {
-    return make_map2(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, base, H, (uint64_t)ca.M, H, cellk::CH, BM, CU_TENSOR_MAP_SWIZZLE_32B);
+    return make_map2(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, base, H, (uint64_t)ca.M, H, cellk::CH, kt * B, CU_TENSOR_MAP_SWIZZLE_32B);
   };
   if (!cmap(&tcr, ca.cr) || !cmap(&tcz, ca.cz) || !cmap(&tcn, ca.cn) || (ca.cnp && !cmap(&tcp, ca.cnp))) return false;
   CUtensorMap taout = thp;      // with the bf16-staged projection `a` is written by TMA stores too ([128 x 16] fp32 tiles)
-  if (GIB && !make_map2(&taout, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, ca.a, H, (uint64_t)ca.M, H, cellk::CH, BM, CU_TENSOR_MAP_SWIZZLE_64B))
+  if (GIB && !make_map2(&taout, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, ca.a, H, (uint64_t)ca.M, H, cellk::CH, kt * B, CU_TENSOR_MAP_SWIZZLE_64B))
     return false;
-  constexpr int kTileRows = PAIR ? 2 * BM : BM;
-  const int tiles = ((ca.M + kTileRows - 1) / kTileRows) * ((H + G::UN - 1) / G::UN);
+  const int tile_k = PAIR ? 2 * kt : kt;
+  const int tiles = ((nk + tile_k - 1) / tile_k) * ((H + G::UN - 1) / G::UN);
   SweepArgs sw{};
   sw.n_steps = 1;
   ProfScope prof_(kc, 2.0 * ca.M * 3.0 * H * H, s);
@@ -280,7 +280,7 @@ struct CellFwdOperands {
   const bf16* gi_b;      // bf16 copy of gi (same element indexing) or nullptr: staged instead of the fp32 rows
 };
 template <bool HAS_G, bool PAIR, bool GIB>
-bool launch_fwd_geo(int kc, const CellFwdOperands& o, int nk, const bf16* W, CellArgs ca, const SweepArgs& sw, cudaStream_t s) {
+bool launch_fwd_geo(int kc, const CellFwdOperands& o, int nk, int nk_ext, const bf16* W, CellArgs ca, const SweepArgs& sw, cudaStream_t s) {
   using C = cellk::CellCfg<HAS_G, false, PAIR, GIB>;
   using G = cellk::Geo<PAIR>;
   if (nk <= 0) return true;
@@ -290,42 +290,49 @@ bool launch_fwd_geo(int kc, const CellFwdOperands& o, int nk, const bf16* W, Cel
   auto kern = umma_cell_kernel<false, HAS_G, PAIR, GIB>;
   if (!set_smem_once(kern, C::kSmemBytes, attr_set)) return false;
   const int B = ca.B, H = ca.H, kt = 128 / B;
-  ca.kt = kt; ca.M = nk * B;
-  CUtensorMap ta, tb, tgi, thp, tg;
+  ca.kt = kt; ca.nk = nk_ext; ca.M = nk_ext * B;
+  // maps over the complete intervals, and (ragged levels) over all of them for the steps that the last one takes too
+  CUtensorMap ta, tb, tgi, thp, tg, xa, xgi, xhp, xg;
   const auto f32 = CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
-  if (!make_map4(&ta, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, o.A, H, B, o.in_slots, nk, H, o.in_ss, o.in_ks, BK, kt, CU_TENSOR_MAP_SWIZZLE_128B)) return false;
   if (!make_map(&tb, W, (uint64_t)H, (uint64_t)3 * H, (uint64_t)H, G::kBox)) return false;
-  if (GIB ? !make_map4(&tgi, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, o.gi_b, 3 * H, B, o.tgt_slots, nk, 3 * H, o.gi_ss, o.gi_ks, cellk::CH, kt,
-                       CU_TENSOR_MAP_SWIZZLE_32B)
-          : !make_map4(&tgi, f32, 4, o.gi, 3 * H, B, o.tgt_slots, nk, 3 * H, o.gi_ss, o.gi_ks, cellk::CH, kt, CU_TENSOR_MAP_SWIZZLE_64B))
-    return false;
-  if (!make_map4(&thp, f32, 4, o.hp, H, B, o.in_slots, nk, H, o.in_ss, o.in_ks, cellk::CH, kt, CU_TENSOR_MAP_SWIZZLE_64B)) return false;
-  if (HAS_G) {
-    if (!make_map4(&tg, f32, 4, o.g, H, B, o.tgt_slots, nk, H, o.g_ss, o.g_ks, cellk::CH, kt, CU_TENSOR_MAP_SWIZZLE_64B)) return false;
+  auto maps = [&](int n, CUtensorMap* a, CUtensorMap* gi, CUtensorMap* hp, CUtensorMap* g) {
+    return make_map4(a, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, o.A, H, B, o.in_slots, n, H, o.in_ss, o.in_ks, BK, kt, CU_TENSOR_MAP_SWIZZLE_128B) &&
+           (GIB ? make_map4(gi, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, o.gi_b, 3 * H, B, o.tgt_slots, n, 3 * H, o.gi_ss, o.gi_ks, cellk::CH, kt,
+                            CU_TENSOR_MAP_SWIZZLE_32B)
+                : make_map4(gi, f32, 4, o.gi, 3 * H, B, o.tgt_slots, n, 3 * H, o.gi_ss, o.gi_ks, cellk::CH, kt, CU_TENSOR_MAP_SWIZZLE_64B)) &&
+           make_map4(hp, f32, 4, o.hp, H, B, o.in_slots, n, H, o.in_ss, o.in_ks, cellk::CH, kt, CU_TENSOR_MAP_SWIZZLE_64B) &&
+           (!HAS_G || make_map4(g, f32, 4, o.g, H, B, o.tgt_slots, n, H, o.g_ss, o.g_ks, cellk::CH, kt, CU_TENSOR_MAP_SWIZZLE_64B));
+  };
+  if (!maps(nk, &ta, &tgi, &thp, &tg)) return false;
+  if (!HAS_G) tg = thp;
+  if (nk_ext > nk) {
+    if (!maps(nk_ext, &xa, &xgi, &xhp, &xg)) return false;
+    if (!HAS_G) xg = xhp;
   } else {
-    tg = thp;
+    xa = ta; xgi = tgi; xhp = thp; xg = tg;
   }
-  constexpr int kTileRows = PAIR ? 2 * BM : BM;
-  const int tiles = ((ca.M + kTileRows - 1) / kTileRows) * ((H + G::UN - 1) / G::UN);
+  const int tile_k = PAIR ? 2 * kt : kt;
+  const int tiles = ((nk_ext + tile_k - 1) / tile_k) * ((H + G::UN - 1) / G::UN);
   const i64 items = (i64)tiles * sw.n_steps;
   ProfScope prof_(kc, 2.0 * ca.M * 3.0 * H * H * sw.n_steps, s);
   cudaError_t e;
   if (PAIR) {
     const int grid = 2 * (int)(items < kSMs / 2 ? items : kSMs / 2);
-    e = launch_pdl_cluster(kern, 2, dim3(grid), dim3(cellk::kThreads), C::kSmemBytes, s, ta, tb, tgi, thp, tg, thp, thp, thp, thp, ca, sw, status);
+    e = launch_pdl_cluster(kern, 2, dim3(grid), dim3(cellk::kThreads), C::kSmemBytes, s, ta, tb, tgi, thp, tg, xa, xgi, xhp, xg, ca, sw, status);
   } else {
     const int grid = (int)(items < kSMs ? items : kSMs);
-    e = launch_pdl(kern, dim3(grid), dim3(cellk::kThreads), C::kSmemBytes, s, ta, tb, tgi, thp, tg, thp, thp, thp, thp, ca, sw, status);
+    e = launch_pdl(kern, dim3(grid), dim3(cellk::kThreads), C::kSmemBytes, s, ta, tb, tgi, thp, tg, xa, xgi, xhp, xg, ca, sw, status);
   }
   if (e != cudaSuccess) return false;
   count_launch();
   return true;
 }
+// nk complete intervals; nk_ext = nk, or nk + 1 on a ragged level whose last interval takes some of the steps
 template <bool HAS_G>
-bool launch_fwd(int kc, const CellFwdOperands& o, int nk, const bf16* W, const CellArgs& ca, const SweepArgs& sw, cudaStream_t s) {
+bool launch_fwd(int kc, const CellFwdOperands& o, int nk, int nk_ext, const bf16* W, const CellArgs& ca, const SweepArgs& sw, cudaStream_t s) {
   const bool pair = cell_pair_enabled(nk * ca.B, ca.H);
-  if (o.gi_b) return pair ? launch_fwd_geo<HAS_G, true, true>(kc, o, nk, W, ca, sw, s) : launch_fwd_geo<HAS_G, false, true>(kc, o, nk, W, ca, sw, s);
-  return pair ? launch_fwd_geo<HAS_G, true, false>(kc, o, nk, W, ca, sw, s) : launch_fwd_geo<HAS_G, false, false>(kc, o, nk, W, ca, sw, s);
+  if (o.gi_b) return pair ? launch_fwd_geo<HAS_G, true, true>(kc, o, nk, nk_ext, W, ca, sw, s) : launch_fwd_geo<HAS_G, false, true>(kc, o, nk, nk_ext, W, ca, sw, s);
+  return pair ? launch_fwd_geo<HAS_G, true, false>(kc, o, nk, nk_ext, W, ca, sw, s) : launch_fwd_geo<HAS_G, false, false>(kc, o, nk, nk_ext, W, ca, sw, s);
 }
 
 // ---------------------------------------------------------------- epilogues (one output row per thread)
@@ -796,21 +803,21 @@ int umma_prepare_adj(const mgrit_gru_cfg* c, const gru_params* p, const float* h
 
 int umma_fwd_step(const FwdStepArgs& a, UmmaFwdWs* w, cudaStream_t s) {
   bool ok;
-  if (a.hin_b && 128 % a.B == 0) {
+  if (a.hin_b && a.B <= BM) {
     // operands through strided tensor maps, bf16 copy of the new state written by the epilogue
     CellArgs ca{};
     ca.B = a.B; ca.H = a.H; ca.b_hh = a.b_hh; ca.gamma = a.gamma; ca.cell = a.cell; ca.mode = a.mode;
     const int nk = a.M / a.B;
     SweepArgs sw{};
     sw.n_steps = 1;
-    sw.st[0].hout = a.hout; sw.st[0].hout_ks = a.hout_ks; sw.st[0].hout_b = a.hout_b;
+    sw.st[0].hout = a.hout; sw.st[0].hout_ks = a.hout_ks; sw.st[0].hout_b = a.hout_b; sw.st[0].nk = nk;
     CellFwdOperands o{};
     o.A = a.hin_b; o.hp = a.hin; o.in_ks = a.hin_ks; o.in_slots = 1;
     o.gi = a.gi; o.gi_b = a.gi_b; o.gi_ks = a.gi_ks; o.tgt_slots = 1;
     // in mode 1 the previous content of the destination plays the role of the additive term
     if (a.mode == 1) { o.g = a.hout; o.g_ks = a.hout_ks; }
     else { o.g = a.gadd; o.g_ks = a.gadd_ks; }
-    ok = o.g ? launch_fwd<true>(KC_FWD_STEP, o, nk, w->W_hh, ca, sw, s) : launch_fwd<false>(KC_FWD_STEP, o, nk, w->W_hh, ca, sw, s);
+    ok = o.g ? launch_fwd<true>(KC_FWD_STEP, o, nk, nk, w->W_hh, ca, sw, s) : launch_fwd<false>(KC_FWD_STEP, o, nk, nk, w->W_hh, ca, sw, s);
     return ok ? MGRIT_OK : MGRIT_CUDA_ERROR;
   }
   if (launch_pdl(pack_rows_kernel, dim3(pgrid((i64)a.M * (a.H / 4))), dim3(kPT), 0, s, a.hin, a.hin_ks, a.B, a.H / 4, (i64)a.M,
@@ -829,22 +836,25 @@ static bool sweep_enabled() {
 }
 
 int umma_fwd_sweep(const FwdSweepArgs& a, UmmaFwdWs* w, cudaStream_t s) {
-  if (!sweep_enabled() || 128 % a.B != 0 || !a.Ub || a.n < 1 || a.n > kMaxSweepSteps || a.n > kMaxFwdSweepSteps || !a.ctr)
+  if (!sweep_enabled() || a.B > BM || !a.Ub || a.n < 1 || a.n > kMaxSweepSteps || a.n > kMaxFwdSweepSteps || !a.ctr)
     return MGRIT_UNSUPPORTED;
   const i64 BH = (i64)a.B * a.H;
   CellArgs ca{};
   ca.B = a.B; ca.H = a.H; ca.b_hh = a.b_hh; ca.gamma = a.gamma; ca.cell = a.cell; ca.mode = 0;
   SweepArgs sw{};
   sw.n_steps = a.n; sw.ctr = a.ctr;
+  int nk_ext = a.nk;
   for (int i = 0; i < a.n; ++i) {
     sw.st[i].hout = a.st[i].out; sw.st[i].hout_ks = a.st[i].out_ks; sw.st[i].hout_b = a.st[i].out_b;
     sw.st[i].in_s = a.st[i].in_s; sw.st[i].tgt_s = a.st[i].tgt_s; sw.st[i].dep = i == 0 ? 0 : a.st[i].dep;
+    sw.st[i].nk = a.st[i].nk; sw.st[i].ext = a.st[i].nk > a.nk ? 1 : 0;
+    if (sw.st[i].ext) nk_ext = a.st[i].nk;
   }
   CellFwdOperands o{};
-  o.A = a.Ub; o.hp = a.U; o.in_ss = BH; o.in_ks = (i64)a.cf * BH; o.in_slots = a.cf;
+  o.A = a.Ub; o.hp = a.U; o.in_ss = BH; o.in_ks = (i64)a.cf * BH; o.in_slots = a.cf;      // (cf slots per interval)
   o.gi = a.gi; o.gi_b = a.gi_b; o.gi_ss = a.gi_ss; o.gi_ks = a.gi_ks; o.tgt_slots = a.cf;
   o.g = a.g; o.g_ss = BH; o.g_ks = (i64)a.cf * BH;
-  const bool ok = a.g ? launch_fwd<true>(KC_FWD_STEP, o, a.nk, w->W_hh, ca, sw, s) : launch_fwd<false>(KC_FWD_STEP, o, a.nk, w->W_hh, ca, sw, s);
+  const bool ok = a.g ? launch_fwd<true>(KC_FWD_STEP, o, a.nk, nk_ext, w->W_hh, ca, sw, s) : launch_fwd<false>(KC_FWD_STEP, o, a.nk, nk_ext, w->W_hh, ca, sw, s);
   return ok ? MGRIT_OK : MGRIT_CUDA_ERROR;
 }
 
@@ -855,7 +865,7 @@ int umma_linearise(const LinArgs& a, UmmaAdjWs* w, cudaStream_t s) {
   const int N = a.M / a.B;
   const float* gi0 = a.gi + (a.t0 + a.stride_t - 1) * BH * 3;       // input of the fine step that arrives with step 1
   const bf16* gib0 = a.gi_b ? a.gi_b + (a.t0 + a.stride_t - 1) * BH * 3 : nullptr;   // ... in the bf16 copy
-  if (128 % a.B == 0) {
+  if (a.B <= BM) {
     CellArgs ca{};
     ca.B = a.B; ca.H = a.H; ca.b_hh = a.b_hh; ca.gamma = a.gamma; ca.cell = a.cell;
     ca.a = a.a; ca.cr = a.crb; ca.cz = a.czb; ca.cn = a.cnb; ca.cnp = a.cnpb;
@@ -904,7 +914,7 @@ static bool adj_staged_enabled() {
   return v == 1;
 }
 
-// The adjoint product with TMA-staged epilogue operands (rows (k, b), 128 % B == 0).
+// The adjoint product with TMA-staged epilogue operands (rows (k, b), B <= 128).
 template <bool HAS_G, bool PAIR>
 static bool launch_adj_staged(const AdjStepArgs& a, const bf16* Apack, const bf16* W_hhT, const float* g, i64 g_ks, cudaStream_t s) {
   using C = adjk::ACfg<HAS_G, PAIR>;
@@ -929,8 +939,8 @@ static bool launch_adj_staged(const AdjStepArgs& a, const bf16* Apack, const bf1
   } else {
     tg = tl;
   }
-  constexpr int kTileRows = PAIR ? 2 * BM : BM;
-  const int tiles = ((a.M + kTileRows - 1) / kTileRows) * ((H + adjk::ABN - 1) / adjk::ABN);
+  const int tile_k = PAIR ? 2 * kt : kt;
+  const int tiles = ((nk + tile_k - 1) / tile_k) * ((H + adjk::ABN - 1) / adjk::ABN);
   cudaError_t e;
   if (PAIR) {
     const int grid = 2 * (tiles < kSMs / 2 ? tiles : kSMs / 2);
@@ -955,7 +965,7 @@ int umma_adj_step(const AdjStepArgs& a, UmmaAdjWs* w, cudaStream_t s) {
   const int tiles256 = ((a.M + BM - 1) / BM) * ((a.H + 255) / 256);
   bool ok;
   // strides of the staged operands: positive for the sensitivities, any sign for the coefficient rows
-  const bool staged = adj_staged_enabled() && 128 % a.B == 0 && tiles256 * 2 > kSMs && a.lin_ks > 0 && a.lout_ks > 0 &&
+  const bool staged = adj_staged_enabled() && a.B <= BM && tiles256 * 2 > kSMs && a.lin_ks > 0 && a.lout_ks > 0 &&
                       (a.mode == 1 || !a.gadd || a.gadd_ks > 0);
   if (staged) {
     const float* g = a.mode == 1 ? a.lout : a.gadd;
