@@ -9,6 +9,7 @@
 #include "umma_adj.cuh"
 #include "umma_gemm.cuh"
 #include "umma_gemm_pair.cuh"
+#include "umma_split.cuh"
 
 namespace mg {
 
@@ -133,6 +134,44 @@ bool launch_gemm_pair(int kc, const bf16* A, i64 lda, const bf16* Bm, i64 ldb, i
     return false;
   count_launch();
   return true;
+}
+
+// The few-row product with the reduction split over a cluster of S CTAs (umma_split.cuh).
+template <int BN, int S, class Epi>
+bool launch_split(int kc, const bf16* A, i64 lda, const bf16* Bm, i64 ldb, int M, int N, int K, int b_rows, Epi epi, cudaStream_t s) {
+  using C = SplitCfg<BN, S>;
+  if (M <= 0 || N <= 0) return true;
+  int* const status = status_ptr();
+  if (!status) return false;
+  static bool attr_set[kMaxDevices] = {false};
+  auto kern = umma_split_kernel<BN, S, Epi>;
+  if (!set_smem_once(kern, C::kSmemBytes, attr_set)) return false;
+  CUtensorMap ta, tb;
+  if (!make_map(&ta, A, (uint64_t)K, (uint64_t)M, (uint64_t)lda, BM)) return false;
+  if (!make_map(&tb, Bm, (uint64_t)K, (uint64_t)b_rows, (uint64_t)ldb, BN)) return false;
+  const int tiles = ((M + BM - 1) / BM) * ((N + BN - 1) / BN);
+  ProfScope prof_(kc, 2.0 * M * (double)N * K, s);
+  if (launch_pdl_cluster(kern, S, dim3(tiles * S), dim3(kThreads), C::kSmemBytes, s, ta, tb, N, K, epi, status) != cudaSuccess) return false;
+  count_launch();
+  return true;
+}
+// Which split: code 100 * BN + S, or 0 for the unsplit product on 64-column tiles.  Measured (B200, us per launch behind its
+// packing kernel): a fixed 4.6 unsplit, 4.9 split on 64 and 6.7 on 128 columns (launch, first loads, exchange) plus 0.245 per
+// k-block and CTA; one wave holds 148 CTAs, 74 clusters of two, 33 of four, 15 of eight.  128 rows at H = 1024 (48 k-blocks):
+// 16.6 unsplit, 10.8 / 8.0 / 12.0 with S = 2 / 4 / 8 (eight: two waves); 512 rows: 17, 11.7 / 15.3 with S = 2 / 4 on 64 columns,
+// 9.7 with S = 4 on 128; 128 rows at H = 512: 12, 5.6 with S = 8.
+int pick_split(int M, int N, int K) {
+  const int mt = (M + BM - 1) / BM, kb = (K + BK - 1) / BK;
+  double best = 1e30;
+  int code = 0;
+  const int bn[6] = {64, 64, 64, 64, 128, 128}, sp[6] = {1, 2, 4, 8, 4, 8}, resident[9] = {0, 148, 74, 0, 33, 0, 0, 0, 15};
+  for (int i = 0; i < 6; ++i) {
+    if (kb < sp[i]) continue;            // every CTA of a cluster has something to reduce
+    const int tiles = mt * ((N + bn[i] - 1) / bn[i]), waves = (tiles + resident[sp[i]] - 1) / resident[sp[i]];
+    const double t = waves * ((sp[i] == 1 ? 4.6 : bn[i] == 64 ? 4.9 : 6.7) + 0.245 * ((kb + sp[i] - 1) / sp[i]));
+    if (t < best) { best = t; code = sp[i] == 1 ? 0 : 100 * bn[i] + sp[i]; }
+  }
+  return code;
 }
 
 // D[m, n] = sum_k A[k, m] * B[k, n]: both operands stored with the reduction index as the ROW index
@@ -591,6 +630,39 @@ struct EpiAdj {  // lambda_prev = a*lambda + acc (+ source); each epilogue warp 
   }
 };
 
+// ... for the split product: NW columns per thread, operands requested before the sums are there
+template <int NW>
+struct EpiAdjSplit {
+  AdjStepArgs a;
+  struct Ops { float l[NW], ac[NW], g[NW]; };
+  __device__ __forceinline__ static void ld(const float* p, float* v) {
+#pragma unroll
+    for (int i = 0; i < NW; i += 4) *reinterpret_cast<float4*>(v + i) = ld4(p + i);
+  }
+  __device__ void load(int row, int n, Ops& o) const {
+#pragma unroll
+    for (int i = 0; i < NW; ++i) o.g[i] = 0.f;
+    if (row >= a.M || n >= a.H) return;
+    const int k = row / a.B, b = row % a.B;
+    const i64 bo = (i64)b * a.H + n;
+    ld(a.lin + (i64)k * a.lin_ks + bo, o.l);
+    ld(a.a + (i64)k * a.coef_ks + bo, o.ac);
+    const float* ga = a.mode == 1 ? a.lout + (i64)k * a.lout_ks + bo : (a.gadd ? a.gadd + (i64)k * a.gadd_ks + bo : nullptr);
+    if (ga) ld(ga, o.g);
+  }
+  __device__ void finish(int row, int n, float* v, const Ops& o) const {
+    if (row >= a.M || n >= a.H) return;
+    float* lo = a.lout + (i64)(row / a.B) * a.lout_ks + (i64)(row % a.B) * a.H + n;
+#pragma unroll
+    for (int i = 0; i < NW; ++i) {
+      const float t = o.ac[i] * o.l[i] + v[i];
+      v[i] = a.mode == 1 ? o.g[i] - t : t + o.g[i];
+    }
+#pragma unroll
+    for (int i = 0; i < NW; i += 4) st4(lo + i, v[i], v[i + 1], v[i + 2], v[i + 3]);
+  }
+};
+
 // ---------------------------------------------------------------- operand packing (HBM streams)
 constexpr int kPT = 256;
 inline int pgrid(i64 items) {
@@ -954,6 +1026,24 @@ static bool launch_adj_staged(const AdjStepArgs& a, const bf16* Apack, const bf1
   return true;
 }
 
+// MGRIT_GRU_ADJ_SPLIT=0 in the environment keeps few-row adjoint products unsplit.
+static bool adj_split_enabled() {
+  static int v = -1;
+  if (v < 0) { const char* e = getenv("MGRIT_GRU_ADJ_SPLIT"); v = (e && e[0] == '0') ? 0 : 1; }
+  return v == 1;
+}
+static bool few_row_adj(const AdjStepArgs& a, const bf16* Apack, const bf16* WT, cudaStream_t s) {
+  const int K = 3 * a.H;
+  switch (adj_split_enabled() ? pick_split(a.M, a.H, K) : 0) {
+    case 6402: return launch_split<64, 2>(KC_ADJ_STEP, Apack, K, WT, K, a.M, a.H, K, a.H, EpiAdjSplit<16>{a}, s);
+    case 6404: return launch_split<64, 4>(KC_ADJ_STEP, Apack, K, WT, K, a.M, a.H, K, a.H, EpiAdjSplit<8>{a}, s);
+    case 6408: return launch_split<64, 8>(KC_ADJ_STEP, Apack, K, WT, K, a.M, a.H, K, a.H, EpiAdjSplit<4>{a}, s);
+    case 12804: return launch_split<128, 4>(KC_ADJ_STEP, Apack, K, WT, K, a.M, a.H, K, a.H, EpiAdjSplit<16>{a}, s);
+    case 12808: return launch_split<128, 8>(KC_ADJ_STEP, Apack, K, WT, K, a.M, a.H, K, a.H, EpiAdjSplit<8>{a}, s);
+    default: return launch_gemm<64, 0>(KC_ADJ_STEP, Apack, K, WT, K, a.M, a.H, K, 0, a.H, EpiAdj<64>{a}, s);
+  }
+}
+
 int umma_adj_step(const AdjStepArgs& a, UmmaAdjWs* w, cudaStream_t s) {
   ProfScope prof(KC_ADJ_STEP, 2.0 * a.M * 3.0 * a.H * a.H, s);     // operand packing + product, timed together
   if (launch_pdl(pack_adj_kernel, dim3(pgrid((i64)a.M * (a.H / 4))), dim3(kPT), 0, s, a.lin, a.lin_ks, a.crb, a.czb, a.cnb, a.coef_ks,
@@ -976,7 +1066,7 @@ int umma_adj_step(const AdjStepArgs& a, UmmaAdjWs* w, cudaStream_t s) {
     return ok ? MGRIT_OK : MGRIT_CUDA_ERROR;
   }
   if (tiles256 * 2 <= kSMs)
-    ok = launch_gemm<64, 0>(KC_ADJ_STEP, w->Apack, 3 * a.H, w->W_hhT, 3 * a.H, a.M, a.H, 3 * a.H, 0, a.H, EpiAdj<64>{a}, s);
+    ok = few_row_adj(a, w->Apack, w->W_hhT, s);
   else if (gemm_pair_enabled(a.M, a.H))
     ok = launch_gemm_pair(KC_ADJ_STEP, w->Apack, 3 * a.H, w->W_hhT, 3 * a.H, a.M, a.H, 3 * a.H, a.H, EpiAdj<256>{a}, s);
   else
