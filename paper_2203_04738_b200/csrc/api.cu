@@ -268,40 +268,56 @@ struct Cycle {
   }
   virtual ~Cycle() {}
 
-  // F-relaxation: from every C-point the cf - 1 F-points of its interval, one dependent step per launch over all
-  // intervals; a ragged level has one more, shorter interval of N % cf F-points behind its last C-point.
-  void frelax(int l) {
-    int cf = c->cf, nki = hr.N[l] / cf, tail = hr.N[l] % cf;
-    for (int sI = 1; sI < cf; ++sI)
-      step(StepDesc{l, nki + (sI <= tail ? 1 : 0), sI - 1, cf, U[l], sI, cf, G[l], sI, cf, sI, cf, 0});
+  // A recurrence without source terms that starts from a zero guess (the adjoint of a loss on the last state alone) is zero
+  // behind its first points until the first coarse solve has spread the start: on the way down of the first cycle only the
+  // intervals that can be non-zero are stepped (`homog`; zero_levels() clears what is then never written).  A level whose
+  // unknowns and right-hand sides vanish behind point P has P / cf + 1 such intervals, one more after every C-relaxation.
+  bool homog = false;
+  void zero_levels() {
+    for (int l = 1; l < hr.L; ++l) {
+      if (l + 1 < hr.L) cudaMemsetAsync(U[l] + BH, 0, sizeof(float) * (size_t)hr.N[l] * BH, s);
+      cudaMemsetAsync(G[l] + BH, 0, sizeof(float) * (size_t)hr.N[l] * BH, s);
+    }
   }
-  void crelax(int l) {
+  // F-relaxation: from every C-point (of the first kz intervals) the cf - 1 F-points of its interval, one dependent step per
+  // launch over all intervals; a ragged level has one more, shorter interval of N % cf F-points behind its last C-point.
+  void frelax(int l, int kz = INT_MAX) {
+    int cf = c->cf, nki = hr.N[l] / cf, tail = hr.N[l] % cf;
+    for (int sI = 1; sI < cf; ++sI) {
+      const int nk = nki + (sI <= tail ? 1 : 0);
+      step(StepDesc{l, nk < kz ? nk : kz, sI - 1, cf, U[l], sI, cf, G[l], sI, cf, sI, cf, 0});
+    }
+  }
+  void crelax(int l, int kz = INT_MAX) {
     int cf = c->cf, nki = hr.N[l] / cf;
-    step(StepDesc{l, nki, cf - 1, cf, U[l], cf, cf, G[l], cf, cf, cf, cf, 0});
+    step(StepDesc{l, nki < kz ? nki : kz, cf - 1, cf, U[l], cf, cf, G[l], cf, cf, cf, cf, 0});
   }
   // One cycle from level l down.  skip_first_f: the state of level l was F-relaxed last and no C-point has changed
   // since, so the opening F-relaxation would reproduce it bit for bit.  record: store the level-0 residual norm.
-  void cycle(int l, bool skip_first_f, bool record) {
+  // live: the last point with a non-zero unknown or right-hand side while `homog`.
+  void cycle(int l, bool skip_first_f, bool record, int live = 0) {
     int cf = c->cf, N = hr.N[l];
     if (l == hr.L - 1) {  // coarsest level: serial propagation
+      homog = false;
       if (chain(l)) return;
       for (int j = 1; j <= N; ++j) step(StepDesc{l, 1, j - 1, 1, U[l], j, 1, G[l], j, 1, j, 1, 0});
       return;
     }
     int relax = l == 0 ? c->relax_fine : c->relax_coarse;       // n: F (CF)^n
-    int nc = hr.N[l + 1];
-    if (!relax_sweep(l, !skip_first_f, relax, true)) {
-      if (!skip_first_f) frelax(l);
-      for (int n = 0; n < relax; ++n) { crelax(l); frelax(l); }
+    int nc = hr.N[l + 1], kz = homog ? live / cf + 1 : INT_MAX;
+    if (homog || !relax_sweep(l, !skip_first_f, relax, true)) {
+      if (!skip_first_f) frelax(l, kz);
+      for (int n = 0; n < relax; ++n) { crelax(l, kz); if (homog) ++kz; frelax(l, kz); }
       // v_k = step_l(u_{cf k - 1}) + g_{cf k}  ->  G[l+1][k]
-      step(StepDesc{l, nc, cf - 1, cf, G[l + 1], 1, 1, G[l], cf, cf, cf, cf, 0});
+      step(StepDesc{l, nc < kz ? nc : kz, cf - 1, cf, G[l + 1], 1, 1, G[l], cf, cf, cf, cf, 0});
     }
+    const int np = nc < kz ? nc : kz;
     // r_k = u_{cf k} - v_k ; U'_k = u_{cf k}
-    stream_restrict_residual(U[l], cf, G[l + 1], U[l + 1], Ub ? Ub[l + 1] : nullptr, nc, (i64)BH,
+    stream_restrict_residual(U[l], cf, G[l + 1], U[l + 1], Ub ? Ub[l + 1] : nullptr, np, (i64)BH,
                              (l == 0 && record) ? res_acc + cycle_idx : nullptr, s);
     // G_k = v_k - step_{l+1}(U'_{k-1})
-    step(StepDesc{l + 1, nc, 0, 1, G[l + 1], 1, 1, nullptr, 0, 0, 1, 1, 1});
-    cycle(l + 1, false, false);
+    step(StepDesc{l + 1, np, 0, 1, G[l + 1], 1, 1, nullptr, 0, 0, 1, 1, 1});
+    cycle(l + 1, false, false, np);
     stream_correct(U[l], Ub ? Ub[l] : nullptr, cf, U[l + 1], nc, (i64)BH, s);
     if (!relax_sweep(l, true, 0, false)) frelax(l);
     // F-cycle: one more V-cycle from this level down on the corrected state (on the last two levels: a second
@@ -315,7 +331,9 @@ struct Cycle {
   }
   bool fcycle_leg = true;     // false while a trailing V-cycle of an F-cycle runs (it does not spawn further ones)
   int solve() {
-    if (hr.L == 1) { cycle(0, false, false); return rc; }
+    if (hr.L == 1) { homog = false; cycle(0, false, false); return rc; }
+    if (c->iters <= 0) homog = false;
+    if (homog) zero_levels();
     cudaMemsetAsync(res_acc, 0, sizeof(double) * (size_t)(c->iters > 0 ? c->iters : 1), s);
     for (cycle_idx = 0; cycle_idx < c->iters && rc == MGRIT_OK; ++cycle_idx) {
       // the previous cycle ended with an F-relaxation of level 0: the caller may ask not to repeat it
@@ -497,6 +515,7 @@ struct F32Cycle {
   const mgrit_gru_cfg* c; const Hier* hr; bool adjoint; cudaStream_t s;
   float** U; float** G; double* res_acc; F32Args a;
   bool ok = true, fcycle_leg = true;
+  bool homog = false;      // as Cycle::homog
   int cycle_idx = 0;
   i64 bh() const { return (i64)c->B * c->H; }
   void flush() {
@@ -520,22 +539,25 @@ struct F32Cycle {
     else { p.op = (st * (s0 + 1) - 1) * BH * 3; p.op_ss = st * BH * 3; p.op_ks = st * ks * 3; }
     return p;
   }
-  void cycle(int l, bool skip_first_f, bool record) {
+  void cycle(int l, bool skip_first_f, bool record, int live = 0) {
     const i64 BH = bh();
     const int cf = c->cf, N = hr->N[l];
     if (l == hr->L - 1) {
       F32Phase p = phase(l, U[l], 0, 0);
       p.nk = p.nfull = 1; p.n = N;
       add(p);
+      homog = false;
       return;
     }
     const int nc = hr->N[l + 1], tail = N % cf, relax = l == 0 ? c->relax_fine : c->relax_coarse;
+    int kz = homog ? live / cf + 1 : INT_MAX;
     float* cp = U[l]; i64 cp_ks = (i64)cf * BH;          // where slot 0 of the intervals is: here or in the coarse array
     for (int r = 0; r <= relax; ++r) {
       const bool skip = r == 0 && skip_first_f;          // the F-points are there already: only the closing step
       const int s0 = skip ? cf - 1 : 0;
       F32Phase p = skip ? phase(l, U[l] + (cf - 1) * BH, (i64)cf * BH, s0) : phase(l, cp, cp_ks, 0);
       p.n = skip ? 0 : cf - 1; p.nfull = nc; p.ntail = skip ? 0 : tail; p.nk = nc + (p.ntail > 0 ? 1 : 0);
+      if (p.nk > kz) p.nk = kz;
       if (r < relax) {
         p.last_kind = kLastStore;
         float* dst = cp == U[l] ? U[l + 1] + BH : U[l] + (i64)cf * BH;
@@ -543,6 +565,7 @@ struct F32Cycle {
         p.last = dst; p.last_ks = dst_ks;
         add(p);
         cp = dst - dst_ks; cp_ks = dst_ks;
+        if (homog) ++kz;
       } else {
         p.last_kind = kLastCoarse;
         p.last = G[l + 1] + BH; p.last_ks = BH;
@@ -557,7 +580,7 @@ struct F32Cycle {
         add(p);
       }
     }
-    cycle(l + 1, false, false);
+    cycle(l + 1, false, false, nc < kz ? nc : kz);
     F32Phase p = phase(l, U[l + 1], BH, 0);
     p.copy = U[l]; p.copy_ks = (i64)cf * BH;
     p.nk = nc + 1; p.nfull = nc; p.n = cf - 1; p.ntail = tail;
@@ -573,6 +596,11 @@ struct F32Cycle {
     if (hr->L == 1) cycle(0, false, false);
     else {
       cudaMemsetAsync(res_acc, 0, sizeof(double) * (size_t)(c->iters > 0 ? c->iters : 1), s);
+      if (c->iters <= 0) homog = false;
+      for (int l = 1; homog && l < hr->L; ++l) {      // what the first way down then never writes
+        cudaMemsetAsync(U[l] + bh(), 0, sizeof(float) * (size_t)hr->N[l] * bh(), s);
+        cudaMemsetAsync(G[l] + bh(), 0, sizeof(float) * (size_t)hr->N[l] * bh(), s);
+      }
       for (cycle_idx = 0; cycle_idx < c->iters; ++cycle_idx)
         cycle(0, cycle_idx > 0 && (c->flags & MGRIT_FLAG_SKIP_DUPLICATE_FRELAX), true);
     }
@@ -607,7 +635,8 @@ bool use_f32_lin(const mgrit_gru_cfg* c, const Hier& hr) {
 // F-point from them), so only those slots are cleared: 1 / cf of the memory traffic.
 template <class T>
 void zero_guess(T* U0, const mgrit_gru_cfg& c, const Hier& hr, size_t slot, cudaStream_t s) {
-  if (hr.L > 1 && c.iters > 0 && c.cf > 1 && c.T / c.cf > 0) {
+  if (hr.L == 1) return;      // the sweep writes every point
+  if (c.iters > 0 && c.cf > 1 && c.T / c.cf > 0) {
     cudaMemset2DAsync(U0 + (size_t)c.cf * slot, (size_t)c.cf * slot * sizeof(T), 0, slot * sizeof(T), (size_t)(c.T / c.cf), s);
   } else {
     cudaMemsetAsync(U0 + slot, 0, sizeof(T) * (size_t)c.T * slot, s);
@@ -785,8 +814,10 @@ int adjoint_impl(const mgrit_gru_cfg* cfg_in, bool serial, const gru_params* p, 
   AdjCycle cy;
   cy.c = &c; cy.hr = hr; cy.s = s; cy.U = aw.U; cy.G = Gl; cy.res_acc = aw.res_acc; cy.BH = BH;
   cy.p = p; cy.w = &aw;
+  cy.homog = !dh_seed;
   if (use_f32_solve(&c, hr)) {
     F32Cycle fc;
+    fc.homog = !dh_seed;
     fc.c = &c; fc.hr = &hr; fc.adjoint = true; fc.s = s; fc.U = aw.U; fc.G = Gl; fc.res_acc = aw.res_acc;
     fc.a.B = c.B; fc.a.H = c.H; fc.a.cell = c.cell; fc.a.W = p->W_hh; fc.a.bar = aw.chain_bar;
     for (int l = 0; l < hr.L; ++l) { fc.a.coef[l][0] = aw.a[l]; fc.a.coef[l][1] = aw.cr[l]; fc.a.coef[l][2] = aw.cz[l]; fc.a.coef[l][3] = aw.cn[l]; }
@@ -948,7 +979,7 @@ int stack_forward_impl(const mgrit_gru_cfg* cfg, int nl, const gru_params* p, co
   } else {
     simt_project(x, p[0].W_ih, p[0].b_ih, gi0, c.T * c.B, c.I, 3 * c.H, s);
   }
-  cudaMemsetAsync(fw.U[0] + slot, 0, sizeof(float) * (size_t)c.T * slot, s);
+  zero_guess(fw.U[0], c, hr, slot, s);
   for (int l = 0; l < hr.L; ++l) cudaMemcpyAsync(fw.U[l], h0, sizeof(float) * slot, cudaMemcpyDeviceToDevice, s);
   StackFwdCycle cy;
   cy.c = &c; cy.hr = hr; cy.s = s; cy.U = fw.U; cy.G = fw.G; cy.res_acc = fw.res_acc; cy.BH = slot;
@@ -1114,17 +1145,22 @@ int stack_adjoint_impl(const mgrit_gru_cfg* cfg, int nl, const gru_params* p, co
     }
   }
   // mu_0 = lambda_T (all layers); zero initial guess elsewhere; fine-level source = reversed dh_seed
-  cudaMemsetAsync(aw.U[0], 0, sizeof(float) * (size_t)(T + 1) * slot, s);
-  cudaMemsetAsync(aw.G[0], 0, sizeof(float) * (size_t)(T + 1) * slot, s);
+  cudaMemsetAsync(aw.U[0], 0, sizeof(float) * slot, s);
+  zero_guess(aw.U[0], c, hr, slot, s);
+  float* Gl[kMaxLevels];
+  for (int l = 0; l < hr.L; ++l) Gl[l] = aw.G[l];
+  if (!dh_seed) Gl[0] = nullptr;
   if (dh_seed) {
     cudaMemcpyAsync(aw.U[0], dh_seed + (size_t)(T - 1) * slot, sizeof(float) * slot, cudaMemcpyDeviceToDevice, s);
+    cudaMemsetAsync(aw.G[0] + (size_t)T * slot, 0, sizeof(float) * slot, s);
     if (T > 1) stream_gather_rows(aw.G[0] + slot, (i64)slot, dh_seed + (size_t)(T - 2) * slot, -(i64)slot, T - 1, (i64)slot, s);
   }
   if (dhT) stream_add_rows(aw.U[0] + (size_t)(nl - 1) * bh, dhT, (i64)bh, s);       // loss on the top layer's last state
   for (int l = 1; l < hr.L; ++l) cudaMemcpyAsync(aw.U[l], aw.U[0], sizeof(float) * slot, cudaMemcpyDeviceToDevice, s);
 
   StackAdjCycle cy;
-  cy.c = &c; cy.hr = hr; cy.s = s; cy.U = aw.U; cy.G = aw.G; cy.res_acc = aw.res_acc; cy.BH = slot;
+  cy.homog = !dh_seed;
+  cy.c = &c; cy.hr = hr; cy.s = s; cy.U = aw.U; cy.G = Gl; cy.res_acc = aw.res_acc; cy.BH = slot;
   cy.nl = nl; cy.p = p; cy.w = &aw;
   rc = cy.solve();
   if (rc) return rc;
@@ -1321,7 +1357,7 @@ int lstm_forward_impl(const mgrit_gru_cfg* cfg, const gru_params* p, const float
   if (is_tf32(&c)) { rc = tf32_prepare_fwd(&c, p, x, gi, &fw.tf, s); if (rc) return rc; }
   else if (c.operands == MGRIT_OPERANDS_BF16) { rc = lstmbf_prepare_fwd(&c, p, x, gi, &fw.bf, s); if (rc) return rc; }
   else simt_project(x, p->W_ih, p->b_ih, gi, c.T * c.B, c.I, 4 * c.H, s);
-  cudaMemsetAsync(fw.U[0] + slot, 0, sizeof(float) * (size_t)c.T * slot, s);
+  zero_guess(fw.U[0], c, hr, slot, s);
   for (int l = 0; l < hr.L; ++l) cudaMemcpyAsync(fw.U[l], u0, sizeof(float) * slot, cudaMemcpyDeviceToDevice, s);
   LstmFwdCycle cy;
   cy.c = &c; cy.hr = hr; cy.s = s; cy.U = fw.U; cy.G = fw.G; cy.res_acc = fw.res_acc; cy.BH = slot;
@@ -1368,16 +1404,21 @@ int lstm_adjoint_impl(const mgrit_gru_cfg* cfg, const gru_params* p, const float
     else if (bf) { rc = lstmbf_linearise(a, &aw.bf, s); if (rc) return rc; }
     else simt_lstm_linearise(a, s);
   }
-  cudaMemsetAsync(aw.U[0], 0, sizeof(float) * (size_t)(T + 1) * slot, s);
-  cudaMemsetAsync(aw.G[0], 0, sizeof(float) * (size_t)(T + 1) * slot, s);
+  cudaMemsetAsync(aw.U[0], 0, sizeof(float) * slot, s);
+  zero_guess(aw.U[0], c, hr, slot, s);
+  float* Gl[kMaxLevels];
+  for (int l = 0; l < hr.L; ++l) Gl[l] = aw.G[l];
+  if (!du_seed) Gl[0] = nullptr;
   if (du_seed) {
     cudaMemcpyAsync(aw.U[0], du_seed + (size_t)(T - 1) * slot, sizeof(float) * slot, cudaMemcpyDeviceToDevice, s);
+    cudaMemsetAsync(aw.G[0] + (size_t)T * slot, 0, sizeof(float) * slot, s);
     if (T > 1) stream_gather_rows(aw.G[0] + slot, (i64)slot, du_seed + (size_t)(T - 2) * slot, -(i64)slot, T - 1, (i64)slot, s);
   }
   if (dhT) stream_add_rows(aw.U[0] + bh, dhT, (i64)bh, s);      // loss on the last hidden state
   for (int l = 1; l < hr.L; ++l) cudaMemcpyAsync(aw.U[l], aw.U[0], sizeof(float) * slot, cudaMemcpyDeviceToDevice, s);
   LstmAdjCycle cy;
-  cy.c = &c; cy.hr = hr; cy.s = s; cy.U = aw.U; cy.G = aw.G; cy.res_acc = aw.res_acc; cy.BH = slot;
+  cy.homog = !du_seed;
+  cy.c = &c; cy.hr = hr; cy.s = s; cy.U = aw.U; cy.G = Gl; cy.res_acc = aw.res_acc; cy.BH = slot;
   cy.p = p; cy.w = &aw;
   rc = cy.solve();
   if (rc) return rc;
