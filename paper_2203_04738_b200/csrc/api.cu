@@ -348,13 +348,18 @@ struct FwdCycle : Cycle {
   const gru_params* p; const float* gi; UmmaFwdWs* um; FwdWs* fw;
   const __nv_bfloat16* gib = nullptr;   // bf16 copy of gi: what every kernel of the solve reads when the state copies exist
   bool gi_f32 = true;                   // false: the fp32 projection was not written (MGRIT_FLAG_GI_F32_UNUSED); gib is set
+  // stacked layers: the input of a layer above the first is the layer below's newest result, so its projection is kept per
+  // level, one row block per point (arrays by level); null: the fine-grid projection, strided
+  float* const* gi_lv = nullptr;
+  i64 gi_stride(int l) const { return gi_lv ? 1 : hr.stride_t[l]; }
+  const float* gi_of(int l) const { return gi_lv ? gi_lv[l] : gi; }
 
   bool chain(int l) override {
     if (c->operands != MGRIT_OPERANDS_BF16) {     // fp32 and tf32 modes: the chain in FFMA arithmetic
       if (!fw->chain_bar) return false;
       Serial32FwdArgs a;
       a.B = c->B; a.H = c->H; a.nsteps = hr.N[l]; a.u = U[l];
-      const i64 st = hr.stride_t[l];
+      const i64 st = gi_stride(l); const float* gi = gi_of(l);
       a.gi = gi + (st - 1) * (i64)BH * 3; a.gi_step = st * (i64)BH * 3;
       a.g = G[l]; a.W = p->W_hh; a.b_hh = p->b_hh; a.gamma = hr.gamma[l]; a.cell = c->cell; a.bar = fw->chain_bar;
       return serial32_fwd_solve(a, s);
@@ -363,7 +368,7 @@ struct FwdCycle : Cycle {
     SerialFwdArgs a{};
     a.B = c->B; a.H = c->H; a.nsteps = hr.N[l];
     a.u = U[l]; a.ub = fw->chain_ub;
-    i64 st = hr.stride_t[l];
+    const i64 st = gi_stride(l); const float* gi = gi_of(l);
     a.gi = gi + (st - 1) * (i64)BH * 3; a.gi_step = st * (i64)BH * 3;
     // (the plain serial sweep has no other level to stay consistent with: it uses the fp32 projection as it is)
     a.gi_as_bf16 = (gib && hr.L > 1) ? 1 : 0;
@@ -377,7 +382,7 @@ struct FwdCycle : Cycle {
   bool chain_by_sweeps(int l) {
     const int N = hr.N[l], kMax = kMaxFwdSweepSteps;
     if (!Ub || c->B > 128 || N < 2 || !fw->sweep_ctr || fw->sweep_ctr_used + N > fw->sweep_ctr_n) return false;
-    const i64 st = hr.stride_t[l];
+    const i64 st = gi_stride(l); const float* gi = gi_of(l);
     for (int j0 = 1; j0 <= N && rc == MGRIT_OK; j0 += kMax) {
       FwdSweepArgs a{};
       a.B = c->B; a.H = c->H; a.nk = 1; a.cf = N; a.n = N - j0 + 1 < kMax ? N - j0 + 1 : kMax;
@@ -409,7 +414,7 @@ struct FwdCycle : Cycle {
     const size_t need = (size_t)n * ((a.nk + (tail > 0 ? 1 : 0) + kt - 1) / kt);
     if (!fw->sweep_ctr || fw->sweep_ctr_used + need > fw->sweep_ctr_n) return false;
     a.U = U[l]; a.Ub = Ub[l];
-    const i64 st = hr.stride_t[l];
+    const i64 st = gi_stride(l); const float* gi = gi_of(l);
     a.gi = gi + (st - 1) * (i64)BH * 3; a.gi_ss = st * (i64)BH * 3; a.gi_ks = st * cf * (i64)BH * 3;
     a.gi_b = gib ? gib + (st - 1) * (i64)BH * 3 : nullptr;
     a.g = G[l] ? G[l] + BH : nullptr;
@@ -446,7 +451,7 @@ struct FwdCycle : Cycle {
     a.hout = d.out + (size_t)d.out_slot * BH; a.hout_ks = (i64)d.out_stride * BH;
     a.hin_b = Ub ? Ub[d.l] + (size_t)d.in_slot * BH : nullptr;
     a.hout_b = (Ub && d.out == U[d.l]) ? Ub[d.l] + (size_t)d.out_slot * BH : nullptr;
-    i64 st = hr.stride_t[d.l];
+    const i64 st = gi_stride(d.l); const float* gi = gi_of(d.l);
     a.gi = gi + ((i64)st * d.tgt_slot - 1) * (i64)BH * 3; a.gi_ks = st * d.tgt_stride * (i64)BH * 3;
     a.gi_b = gib ? gib + ((i64)st * d.tgt_slot - 1) * (i64)BH * 3 : nullptr;
     a.gadd = d.gadd ? d.gadd + (size_t)d.gadd_slot * BH : nullptr; a.gadd_ks = (i64)d.gadd_stride * BH;
@@ -460,32 +465,37 @@ struct FwdCycle : Cycle {
 
 struct AdjCycle : Cycle {
   const gru_params* p; AdjWs* w;
-  bool chain(int l) override {
+  // stacked layers: what the layer above sends to its input joins the incoming sensitivities (rows ladd + k*ladd_ks; the sums
+  // go to lsum)
+  const float* ladd = nullptr; i64 ladd_ks = 0; float* lsum = nullptr;
+  bool chain(int l) override { return chain_on(l, U[l], G[l]); }
+  bool chain_on(int l, float* mu, const float* g) {
     if (c->operands != MGRIT_OPERANDS_BF16) {
       if (!w->chain_bar || !w->chain_dA32) return false;
       Serial32AdjArgs a;
-      a.B = c->B; a.H = c->H; a.nsteps = hr.N[l]; a.mu = U[l]; a.dA = w->chain_dA32;
+      a.B = c->B; a.H = c->H; a.nsteps = hr.N[l]; a.mu = mu; a.dA = w->chain_dA32;
       const i64 row0 = (i64)(hr.N[l] - 1) * BH;    // step s = 1 applies forward step N_l, stored at row N_l - 1
       a.a = w->a[l] + row0; a.cr = w->cr[l] + row0; a.cz = w->cz[l] + row0; a.cn = w->cn[l] + row0;
       a.coef_step = -(i64)BH;
-      a.g = G[l]; a.W = p->W_hh; a.bar = w->chain_bar;
+      a.g = g; a.W = p->W_hh; a.bar = w->chain_bar;
       return serial32_adj_solve(a, s);
     }
     if (!w->chain_dAb) return false;
     SerialAdjArgs a;
     a.B = c->B; a.H = c->H; a.nsteps = hr.N[l];
-    a.mu = U[l]; a.dAb = w->chain_dAb;
+    a.mu = mu; a.dAb = w->chain_dAb;
     i64 row0 = (i64)(hr.N[l] - 1) * BH;        // step s = 1 applies forward step N_l, stored at row N_l - 1
     a.a = w->a[l] + row0; a.cr = w->crb[l] + row0; a.cz = w->czb[l] + row0; a.cn = w->cnb[l] + row0;
     a.coef_step = -(i64)BH;
-    a.g = G[l]; a.WT = w->um.W_hhT; a.bar = w->chain_bar;
+    a.g = g; a.WT = w->um.W_hhT; a.bar = w->chain_bar;
     a.xw = w->chain_xw; a.xw_bytes = w->chain_xw_bytes;
     return serial_adj_solve(a, s);
   }
   int launch_step(const StepDesc& d) override {
-    AdjStepArgs a;
+    AdjStepArgs a{};
     a.M = d.nk * c->B; a.B = c->B; a.H = c->H;
     a.lin = U[d.l] + (size_t)d.in_slot * BH; a.lin_ks = (i64)d.in_stride * BH;
+    a.ladd = ladd; a.ladd_ks = ladd_ks; a.lsum = lsum;
     a.lout = d.out + (size_t)d.out_slot * BH; a.lout_ks = (i64)d.out_stride * BH;
     a.gadd = d.gadd ? d.gadd + (size_t)d.gadd_slot * BH : nullptr; a.gadd_ks = (i64)d.gadd_stride * BH;
     // the step arriving at reversed point s applies forward step j = N_l - s + 1, stored at row N_l - s
@@ -502,6 +512,10 @@ struct AdjCycle : Cycle {
     a.W_hh = p->W_hh; a.mode = d.mode;
     if (c->operands == MGRIT_OPERANDS_BF16) return umma_adj_step(a, &w->um, s);
     if (is_tf32(c)) return tf32_adj_step(a, &w->tf, s);
+    if (ladd) {
+      stream_sum_rows(lsum, a.lin, a.lin_ks, ladd, ladd_ks, d.nk, (i64)BH, s);
+      a.lin = lsum; a.lin_ks = (i64)BH;
+    }
     simt_adj_step(a, s);
     return MGRIT_OK;
   }
@@ -685,7 +699,8 @@ int forward_impl(const mgrit_gru_cfg* cfg_in, bool serial, const gru_params* p, 
     fw.Ub[0] = t.hb0;
     fw.um.gib = t.gib;
   }
-  if (!gi_bf16_enabled()) fw.um.gib = nullptr;
+  // (the projection is staged as bf16 where B divides 128; other batch sizes keep its fp32 values, as they always have)
+  if (!gi_bf16_enabled() || 128 % c.B != 0) fw.um.gib = nullptr;
   // the caller does not read the fp32 projection and every kernel of this solve reads its bf16 copy: do not write it
   // (where B divides 128, as the flag's contract says)
   const bool gi_f32 = !((c.flags & MGRIT_FLAG_GI_F32_UNUSED) && carries_copies(&c, serial) && 128 % c.B == 0 && fw.um.gib);
@@ -869,8 +884,7 @@ int adjoint_impl(const mgrit_gru_cfg* cfg_in, bool serial, const gru_params* p, 
 // ======================================================================================================
 // Stacked layers in one state: the state of a time point is the stack of all layers' hidden states, layer k's input
 // at a step is layer k-1's NEW state of the same step, and ONE multigrid cycle advances the whole stack.  Level
-// arrays are [N_l + 1][n_layers][B][H]; the cycle logic (Cycle) is the same, a "step" becomes a short sequence of
-// launches per layer: cell step on the raw result, FAS combination, input projection for the layer above.
+// arrays are kept per layer ([N_l + 1][B][H] each); StackCycle below runs the same cycle operation by operation.
 constexpr int kMaxStack = 8;
 
 size_t stack_max_rows(const mgrit_gru_cfg* c, const Hier& hr) {
@@ -882,68 +896,179 @@ size_t stack_max_rows(const mgrit_gru_cfg* c, const Hier& hr) {
   return m;
 }
 
-struct StackFwdWs {
-  float* U[kMaxLevels]; float* G[kMaxLevels]; double* res_acc;
-  float* tmpPhi; float* gi_tmp; size_t maxM;
-  UmmaFwdWs um[kMaxStack];
-};
-
 mgrit_gru_cfg layer_cfg(const mgrit_gru_cfg& c, int k) {
   mgrit_gru_cfg ck = c;
   if (k > 0) ck.I = c.H;
   return ck;
 }
 
-void plan_stack_fwd(const mgrit_gru_cfg* c, int nl, const Hier& hr, Ws& w, StackFwdWs* o) {
-  const size_t slot = (size_t)nl * c->B * c->H;
-  for (int l = 0; l < hr.L; ++l) {
-    o->U[l] = w.take<float>((size_t)(hr.N[l] + 1) * slot);
-    o->G[l] = l == 0 ? nullptr : w.take<float>((size_t)(hr.N[l] + 1) * slot);
-  }
-  o->res_acc = w.take<double>((size_t)(c->iters > 0 ? c->iters : 1));
-  o->maxM = stack_max_rows(c, hr);
-  o->tmpPhi = w.take<float>(o->maxM * c->H);
-  o->gi_tmp = w.take<float>(o->maxM * 3 * c->H);
-  if (c->operands == MGRIT_OPERANDS_BF16)
+// The cycle of the stack, operation by operation.  Within one relaxation segment -- every point visited at most once -- a layer
+// never waits for the layer above it (forward) or below it (adjoint), so an operation runs layer by layer on the single-layer
+// kernels: a whole sweep, chain or coarse step of one layer, then ONE product that forms every point's input for the next.
+// (Step by step the two-layer solve of 512 points took about 1700 launches of few rows.)
+struct StackCycle {
+  const mgrit_gru_cfg* c; Hier hr; cudaStream_t s; int nl;
+  double* res_acc; int cycle_idx = 0; int rc = MGRIT_OK;
+  bool homog = false, fcycle_leg = true;      // as in Cycle
+  enum { kNone, kC, kV };
+  // F-relaxation (optional) of the first kz intervals of level l, then nothing, the C-step or the evaluation of v
+  virtual void segment(int l, int kz, bool f, int last) = 0;
+  virtual void coarse_rhs(int l, int np) = 0;      // G_k = v_k - step_l(U'_{k-1}), k = 1..np
+  virtual void coarsest(int l) = 0;
+  virtual Cycle& layer(int k) = 0;
+  virtual ~StackCycle() {}
+  void cycle(int l, bool skip_first_f, bool record, int live = 0) {
+    const int cf = c->cf;
+    if (l == hr.L - 1) { homog = false; coarsest(l); return; }
+    const int relax = l == 0 ? c->relax_fine : c->relax_coarse, nc = hr.N[l + 1];
+    int kz = homog ? live / cf + 1 : INT_MAX;
+    for (int r = 0; r < relax; ++r) { segment(l, kz, !(r == 0 && skip_first_f), kC); if (homog) ++kz; }
+    segment(l, kz, !(relax == 0 && skip_first_f), kV);
+    const int np = nc < kz ? nc : kz;
     for (int k = 0; k < nl; ++k) {
-      mgrit_gru_cfg ck = layer_cfg(*c, k);
-      umma_plan_fwd(&ck, hr.N, hr.L, w.base, &w.off, &o->um[k]);
+      Cycle& y = layer(k);
+      stream_restrict_residual(y.U[l], cf, y.G[l + 1], y.U[l + 1], y.Ub ? y.Ub[l + 1] : nullptr, np, (i64)y.BH,
+                               (l == 0 && record) ? res_acc + cycle_idx : nullptr, s);
     }
+    coarse_rhs(l + 1, np);
+    cycle(l + 1, false, false, np);
+    for (int k = 0; k < nl; ++k) {
+      Cycle& y = layer(k);
+      stream_correct(y.U[l], y.Ub ? y.Ub[l] : nullptr, cf, y.U[l + 1], nc, (i64)y.BH, s);
+    }
+    segment(l, INT_MAX, true, kNone);
+    if ((c->flags & MGRIT_FLAG_F_CYCLE) && fcycle_leg) {
+      fcycle_leg = false;
+      cycle(l, true, false);
+      fcycle_leg = true;
+    }
+  }
+  int solve() {
+    if (hr.L == 1) { homog = false; coarsest(0); return status(); }
+    cudaMemsetAsync(res_acc, 0, sizeof(double) * (size_t)(c->iters > 0 ? c->iters : 1), s);
+    if (c->iters <= 0) homog = false;
+    if (homog) for (int k = 0; k < nl; ++k) layer(k).zero_levels();
+    for (cycle_idx = 0; cycle_idx < c->iters && status() == MGRIT_OK; ++cycle_idx)
+      cycle(0, cycle_idx > 0 && (c->flags & MGRIT_FLAG_SKIP_DUPLICATE_FRELAX), true);
+    return status();
+  }
+  int status() {
+    for (int k = 0; k < nl && rc == MGRIT_OK; ++k) rc = layer(k).rc;
+    return rc;
+  }
+  // the steps of a segment on layer y, one launch per step
+  static void steps(Cycle& y, int l, int kz, bool f, int last) {
+    const int cf = y.c->cf;
+    if (f) y.frelax(l, kz);
+    if (last == kC) y.crelax(l, kz);
+    if (last == kV) {
+      const int nc = y.hr.N[l + 1];
+      y.step(StepDesc{l, nc < kz ? nc : kz, cf - 1, cf, y.G[l + 1], 1, 1, y.G[l], cf, cf, cf, cf, 0});
+    }
+  }
+};
+
+struct StackFwdWs {
+  FwdWs L[kMaxStack];
+  float* gi_l[kMaxStack][kMaxLevels];      // layers >= 1: projections by level
+  float *phi, *raw;        // raw results of a coarse step; of a segment as fp32 rows (fp32 engine)
+  double* res_acc;
+};
+// the fused kernels and the state copies they need
+bool stack_fused(const mgrit_gru_cfg* c) { return c->operands == MGRIT_OPERANDS_BF16 && c->B <= 128; }
+
+void plan_stack_fwd(const mgrit_gru_cfg* c, int nl, const Hier& hr, Ws& w, StackFwdWs* o) {
+  const size_t bh = (size_t)c->B * c->H;
+  for (int k = 0; k < nl; ++k) {
+    mgrit_gru_cfg ck = layer_cfg(*c, k);
+    plan_fwd(&ck, hr, w, &o->L[k]);
+    for (int l = 0; l < hr.L; ++l) {
+      o->gi_l[k][l] = k > 0 ? w.take<float>((size_t)hr.N[l] * bh * 3) : nullptr;
+    }
+  }
+  o->phi = hr.L > 1 ? w.take<float>((size_t)hr.N[1] * bh) : nullptr;
+  o->raw = c->operands == MGRIT_OPERANDS_BF16 ? nullptr : w.take<float>((size_t)c->T * bh);
+  o->res_acc = w.take<double>((size_t)(c->iters > 0 ? c->iters : 1));
 }
 
-struct StackFwdCycle : Cycle {
-  int nl; const gru_params* p; const float* gi0; StackFwdWs* fw;
-  int launch_step(const StepDesc& d) override {
-    const size_t bh = (size_t)c->B * c->H, slot = (size_t)nl * bh;
-    const int M = d.nk * c->B;
-    const bool bf16 = c->operands == MGRIT_OPERANDS_BF16;
-    const i64 st = hr.stride_t[d.l];
-    for (int k = 0; k < nl; ++k) {
-      FwdStepArgs a{};
-      a.M = M; a.B = c->B; a.H = c->H;
-      a.hin = U[d.l] + ((size_t)d.in_slot * nl + k) * bh; a.hin_ks = (i64)d.in_stride * slot;
-      a.hout = fw->tmpPhi; a.hout_ks = (i64)bh;            // the raw step result, rows (k, b) contiguous
-      a.hin_b = nullptr; a.hout_b = nullptr;
-      if (k == 0) { a.gi = gi0 + ((i64)st * d.tgt_slot - 1) * (i64)bh * 3; a.gi_ks = st * d.tgt_stride * (i64)bh * 3; }
-      else { a.gi = fw->gi_tmp; a.gi_ks = (i64)bh * 3; }
-      a.gadd = nullptr; a.gadd_ks = 0;
-      a.W_hh = p[k].W_hh; a.b_hh = p[k].b_hh; a.gamma = hr.gamma[d.l]; a.cell = c->cell; a.mode = 0;
-      if (bf16) { int r = umma_fwd_step(a, &fw->um[k], s); if (r) return r; }
-      else simt_fwd_step(a, s);
-      // level unknown = raw result + FAS term (mode 0), or right-hand side -= raw result (mode 1)
-      const float* g = d.gadd ? d.gadd + ((size_t)d.gadd_slot * nl + k) * bh : nullptr;
-      stream_combine_rows(fw->tmpPhi, g, (i64)d.gadd_stride * slot, d.out + ((size_t)d.out_slot * nl + k) * bh, (i64)d.out_stride * slot,
-                          c->B, c->H, (i64)M, d.mode, s);
-      if (k + 1 < nl) {   // input projection of the layer above: its input is this layer's raw new state
-        if (bf16) {
-          int r = umma_project_rows(fw->tmpPhi, fw->um[k + 1].xb, fw->um[k + 1].W_ih, p[k + 1].b_ih, fw->gi_tmp, M, c->H, 3 * c->H, s);
-          if (r) return r;
-        } else {
-          simt_project(fw->tmpPhi, p[k + 1].W_ih, p[k + 1].b_ih, fw->gi_tmp, M, c->H, 3 * c->H, s);
-        }
-      }
+struct StackFwdCycle : StackCycle {
+  FwdCycle y[kMaxStack]; const gru_params* p; StackFwdWs* fw;
+  Cycle& layer(int k) override { return y[k]; }
+  // projection of n points of layer k (rows raw[n, B, H], fp32 rows or already bf16 in the upper layer's xb) for layer k + 1
+  void project(int k, int l, const float* raw, int n) {
+    const int M = n * c->B;
+    if (rc != MGRIT_OK) return;
+    if (c->operands == MGRIT_OPERANDS_BF16)
+      rc = umma_project_packed(fw->L[k + 1].um.xb, fw->L[k + 1].um.W_ih, p[k + 1].b_ih, fw->gi_l[k + 1][l], nullptr, M, c->H, 3 * c->H, s);
+    else
+      simt_project(raw, p[k + 1].W_ih, p[k + 1].b_ih, fw->gi_l[k + 1][l], M, c->H, 3 * c->H, s);
+  }
+  // raw results (before the FAS term) of every point of level l: its unknown, at the C-points v where the segment evaluated it
+  void feed(int k, int l, bool v) {
+    if (k + 1 >= nl) return;
+    const bool bf = c->operands == MGRIT_OPERANDS_BF16;
+    stream_raw_rows(y[k].U[l], y[k].G[l], v ? y[k].G[l + 1] : nullptr, c->cf, hr.N[l], (i64)y[k].BH, bf ? nullptr : fw->raw,
+                    bf ? fw->L[k + 1].um.xb : nullptr, s);
+    project(k, l, fw->raw, hr.N[l]);
+  }
+  bool run_fp32(FwdCycle& q, int k, int l, int kz, bool f, int last) {
+    if (c->operands != MGRIT_OPERANDS_FP32 || !f32_solve_fits(c->H)) return false;
+    F32Cycle fc;
+    fc.c = c; fc.hr = &hr; fc.adjoint = false; fc.s = s; fc.U = q.U; fc.G = q.G; fc.res_acc = res_acc;
+    fc.a.B = c->B; fc.a.H = c->H; fc.a.cell = c->cell; fc.a.W = p[k].W_hh; fc.a.gi = q.gi_of(l); fc.a.b_hh = p[k].b_hh; fc.a.bar = fw->L[k].chain_bar;
+    fc.a.nph = 0;
+    const int cf = c->cf, N = hr.N[l];
+    const i64 BH = (i64)q.BH, st = q.gi_stride(l);
+    const bool chain = l == hr.L - 1 && last == kNone && !f;
+    const int s0 = chain || f ? 0 : cf - 1;
+    F32Phase ph = fc.phase(l, q.U[l] + s0 * BH, (i64)cf * BH, s0);
+    ph.op = (st * (s0 + 1) - 1) * BH * 3; ph.op_ss = st * BH * 3; ph.op_ks = st * cf * BH * 3;
+    if (chain) { ph.nk = ph.nfull = 1; ph.n = N; }
+    else {
+      const int nc = N / cf, tail = f ? N % cf : 0;
+      ph.n = f ? cf - 1 : 0; ph.nfull = nc; ph.ntail = tail; ph.nk = nc + (tail > 0 ? 1 : 0);
+      if (ph.nk > kz) ph.nk = kz;
+      if (last == kV) { ph.last_kind = kLastStore; ph.last = q.G[l + 1] + BH; ph.last_ks = BH; }
     }
-    return MGRIT_OK;
+    fc.add(ph);
+    fc.flush();
+    if (!fc.ok) rc = MGRIT_CUDA_ERROR;
+    return true;
+  }
+  void segment(int l, int kz, bool f, int last) override {
+    int kinds[32], n = 0;
+    const int cf = c->cf;
+    if (f) for (int i = 1; i < cf && n < 31; ++i) kinds[n++] = i;
+    if (last == kC) kinds[n++] = cf;
+    if (last == kV) kinds[n++] = cf + 1;
+    for (int k = 0; k < nl && status() == MGRIT_OK; ++k) {
+      if (!(cf <= kMaxFwdSweepSteps && y[k].launch_sweep(l, kinds, n))) {
+        // (fp32 phases: the C-step overwrites what other rows of a phase read, so it is a launch of its own)
+        const bool part = last == kC && f;
+        if (part && run_fp32(y[k], k, l, kz, true, kNone)) steps(y[k], l, kz, false, kC);
+        else if (last == kC || !run_fp32(y[k], k, l, kz, f, last)) steps(y[k], l, kz, f, last);
+      }
+      feed(k, l, last == kV);
+    }
+  }
+  void coarse_rhs(int l, int np) override {
+    for (int k = 0; k < nl && status() == MGRIT_OK; ++k) {
+      FwdCycle& q = y[k];
+      if (k + 1 == nl) { q.step(StepDesc{l, np, 0, 1, q.G[l], 1, 1, nullptr, 0, 0, 1, 1, 1}); continue; }
+      // the layer above reads the raw step result: keep it, then form the right-hand side
+      q.step(StepDesc{l, np, 0, 1, fw->phi, 0, 1, nullptr, 0, 0, 1, 1, 0});
+      const bool bf = c->operands == MGRIT_OPERANDS_BF16;
+      stream_subtract_rows(q.G[l] + q.BH, fw->phi, (i64)np * (i64)q.BH, bf ? fw->L[k + 1].um.xb : nullptr, s);
+      project(k, l, fw->phi, np);
+    }
+  }
+  void coarsest(int l) override {
+    for (int k = 0; k < nl && status() == MGRIT_OK; ++k) {
+      FwdCycle& q = y[k];
+      if (!run_fp32(q, k, l, 1, false, kNone) && !q.chain(l))
+        for (int j = 1; j <= hr.N[l]; ++j) q.step(StepDesc{l, 1, j - 1, 1, q.U[l], j, 1, q.G[l], j, 1, j, 1, 0});
+      feed(k, l, false);
+    }
   }
 };
 
@@ -969,24 +1094,40 @@ int stack_forward_impl(const mgrit_gru_cfg* cfg, int nl, const gru_params* p, co
   plan_stack_fwd(&c, nl, hr, w, &fw);
   if (!w.fits()) return MGRIT_WORKSPACE_TOO_SMALL;
   const size_t bh = (size_t)c.B * c.H, slot = (size_t)nl * bh;
-  if (c.operands == MGRIT_OPERANDS_BF16) {
-    rc = umma_prepare_fwd(&c, &p[0], x, gi0, &fw.um[0], s);
+  const bool bf = c.operands == MGRIT_OPERANDS_BF16, fused = stack_fused(&c);
+  if (bf) {
+    for (int k = 0; k < nl; ++k) fw.L[k].um.gib = nullptr;      // stacked layers: fp32 projections throughout
+    rc = umma_prepare_fwd(&c, &p[0], x, gi0, &fw.L[0].um, s);
     if (rc) return rc;
     for (int k = 1; k < nl; ++k) {
-      umma_convert(p[k].W_hh, fw.um[k].W_hh, (i64)3 * c.H * c.H, s);
-      umma_convert(p[k].W_ih, fw.um[k].W_ih, (i64)3 * c.H * c.H, s);
+      umma_convert(p[k].W_hh, fw.L[k].um.W_hh, (i64)3 * c.H * c.H, s);
+      umma_convert(p[k].W_ih, fw.L[k].um.W_ih, (i64)3 * c.H * c.H, s);
     }
   } else {
     simt_project(x, p[0].W_ih, p[0].b_ih, gi0, c.T * c.B, c.I, 3 * c.H, s);
   }
-  zero_guess(fw.U[0], c, hr, slot, s);
-  for (int l = 0; l < hr.L; ++l) cudaMemcpyAsync(fw.U[l], h0, sizeof(float) * slot, cudaMemcpyDeviceToDevice, s);
   StackFwdCycle cy;
-  cy.c = &c; cy.hr = hr; cy.s = s; cy.U = fw.U; cy.G = fw.G; cy.res_acc = fw.res_acc; cy.BH = slot;
-  cy.nl = nl; cy.p = p; cy.gi0 = gi0; cy.fw = &fw;
+  cy.c = &c; cy.hr = hr; cy.s = s; cy.nl = nl; cy.res_acc = fw.res_acc; cy.p = p; cy.fw = &fw;
+  mgrit_gru_cfg ck[kMaxStack];
+  for (int k = 0; k < nl; ++k) {
+    FwdWs& q = fw.L[k];
+    ck[k] = layer_cfg(c, k);
+    zero_guess(q.U[0], c, hr, bh, s);
+    for (int l = 0; l < hr.L; ++l) cudaMemcpyAsync(q.U[l], h0 + k * bh, sizeof(float) * bh, cudaMemcpyDeviceToDevice, s);
+    if (fused) {
+      cudaMemsetAsync(q.sweep_ctr, 0, sizeof(int) * q.sweep_ctr_n, s);
+      zero_guess(q.Ub[0], c, hr, bh, s);
+      for (int l = 0; l < hr.L; ++l) umma_convert(h0 + k * bh, q.Ub[l], (i64)bh, s);
+    }
+    FwdCycle& y = cy.y[k];
+    y.c = &ck[k]; y.hr = hr; y.s = s; y.U = q.U; y.G = q.G; y.res_acc = fw.res_acc; y.BH = bh; y.p = &p[k]; y.um = &q.um; y.fw = &q;
+    y.Ub = fused ? q.Ub : nullptr;
+    y.gi = gi0;
+    if (k > 0) y.gi_lv = fw.gi_l[k];
+  }
   rc = cy.solve();
   if (rc) return rc;
-  cudaMemcpyAsync(h, fw.U[0] + slot, sizeof(float) * (size_t)c.T * slot, cudaMemcpyDeviceToDevice, s);
+  for (int k = 0; k < nl; ++k) stream_gather_rows(h + k * bh, (i64)slot, fw.L[k].U[0] + bh, (i64)bh, c.T, (i64)bh, s);
   if (resnorm && hr.L > 1 && c.iters > 0) {
     rc = fetch_resnorm(fw.res_acc, resnorm, c.iters, s);
     if (rc) return rc;
@@ -996,99 +1137,166 @@ int stack_forward_impl(const mgrit_gru_cfg* cfg, int nl, const gru_params* p, co
 }
 
 struct StackLayerAdj {
-  float *a[kMaxLevels], *cr[kMaxLevels], *cz[kMaxLevels], *cn[kMaxLevels], *cnp[kMaxLevels];                 // fp32 engine
-  __nv_bfloat16 *crb[kMaxLevels], *czb[kMaxLevels], *cnb[kMaxLevels], *cnpb[kMaxLevels];                     // tensor-core engine
+  AdjWs w;
+  float* cnp[kMaxLevels]; __nv_bfloat16* cnpb[kMaxLevels];     // c_n' of every level: what a cell sends to its input
   float* hk;                 // this layer's given states [T, B, H], contiguous
   float* gik;                // layers >= 1: input projection of the layer below's given states [T, B, 3H]
   __nv_bfloat16* Wihb;       // layers >= 1, tensor-core engine: W_ih as bf16 [3H, H]
-  UmmaAdjWs um;
 };
 struct StackAdjWs {
-  float* U[kMaxLevels]; float* G[kMaxLevels]; double* res_acc;
-  float *tmpLin, *tmpDx, *lamk, *dxk, *grad_scratch; size_t maxM;
+  double* res_acc;
+  float *dx, *lsum, *nu, *gnu, *lamk, *dxk;
   StackLayerAdj L[kMaxStack];
 };
 
 void plan_stack_adj(const mgrit_gru_cfg* c, int nl, const Hier& hr, Ws& w, StackAdjWs* o) {
-  const size_t bh = (size_t)c->B * c->H, slot = (size_t)nl * bh, TB = (size_t)c->T * c->B;
+  const size_t bh = (size_t)c->B * c->H, TB = (size_t)c->T * c->B;
   const bool bf16 = c->operands == MGRIT_OPERANDS_BF16;
-  for (int l = 0; l < hr.L; ++l) {
-    o->U[l] = w.take<float>((size_t)(hr.N[l] + 1) * slot);
-    o->G[l] = w.take<float>((size_t)(hr.N[l] + 1) * slot);
-  }
   o->res_acc = w.take<double>((size_t)(c->iters > 0 ? c->iters : 1));
-  o->maxM = stack_max_rows(c, hr);
-  o->tmpLin = w.take<float>(o->maxM * c->H);
-  o->tmpDx = w.take<float>(o->maxM * c->H);
+  o->dx = w.take<float>(TB * c->H);                                          // rows sent to the layer below, by incoming point
+  o->lsum = w.take<float>(stack_max_rows(c, hr) * c->H);
+  o->nu = w.take<float>((size_t)(hr.N[hr.L - 1] + 1) * bh);
+  o->gnu = w.take<float>((size_t)(hr.N[hr.L - 1] + 1) * bh);
   o->lamk = w.take<float>(TB * c->H);
   o->dxk = w.take<float>(TB * c->H);
-  o->grad_scratch = nullptr;
-  if (!bf16) {
-    const size_t n0 = simt_gradients_scratch((int)TB, 3 * c->H, c->H, c->I), n1 = simt_gradients_scratch((int)TB, 3 * c->H, c->H, c->H);
-    o->grad_scratch = w.take<float>(n0 > n1 ? n0 : n1);
-  }
   for (int k = 0; k < nl; ++k) {
     StackLayerAdj& L = o->L[k];
+    mgrit_gru_cfg ck = layer_cfg(*c, k);
+    plan_adj(&ck, hr, w, &L.w);
     for (int l = 0; l < hr.L; ++l) {
       const size_t n = (size_t)hr.N[l] * bh;
-      L.a[l] = w.take<float>(n);
-      if (bf16) {
-        L.cr[l] = L.cz[l] = L.cn[l] = L.cnp[l] = nullptr;
-        L.crb[l] = w.take<__nv_bfloat16>(n); L.czb[l] = w.take<__nv_bfloat16>(n);
-        L.cnb[l] = w.take<__nv_bfloat16>(n); L.cnpb[l] = w.take<__nv_bfloat16>(n);
-      } else {
-        L.crb[l] = L.czb[l] = L.cnb[l] = L.cnpb[l] = nullptr;
-        L.cr[l] = w.take<float>(n); L.cz[l] = w.take<float>(n); L.cn[l] = w.take<float>(n); L.cnp[l] = w.take<float>(n);
-      }
+      L.cnp[l] = bf16 ? nullptr : l == 0 ? L.w.cnp : w.take<float>(n);
+      L.cnpb[l] = !bf16 ? nullptr : l == 0 ? L.w.cnpb : w.take<__nv_bfloat16>(n);
     }
     L.hk = w.take<float>(TB * c->H);
     L.gik = k > 0 ? w.take<float>(TB * 3 * c->H) : nullptr;
     L.Wihb = (bf16 && k > 0) ? w.take<__nv_bfloat16>((size_t)3 * c->H * c->H) : nullptr;
-    if (bf16) { mgrit_gru_cfg ck = layer_cfg(*c, k); umma_plan_adj(&ck, hr.N, hr.L, w.base, &w.off, &L.um); }
   }
 }
 
-struct StackAdjCycle : Cycle {
-  int nl; const gru_params* p; StackAdjWs* w;
-  int launch_step(const StepDesc& d) override {
-    const size_t bh = (size_t)c->B * c->H, slot = (size_t)nl * bh;
-    const int M = d.nk * c->B;
+struct StackAdjCycle : StackCycle {
+  AdjCycle y[kMaxStack]; const gru_params* p; StackAdjWs* w;
+  Cycle& layer(int k) override { return y[k]; }
+  // what layer k (>= 1) sends to its input in the n steps that leave points j0, j0 + js, ... of level l  ->  w->dx[n, B, H]
+  void send(int k, int l, int j0, int js, int n) {
+    if (k == 0 || status() != MGRIT_OK) return;
+    const i64 bh = (i64)y[k].BH;
+    StackLayerAdj& L = w->L[k];
+    AdjStepArgs a{};
+    a.B = c->B; a.H = c->H; a.lin_ks = js * bh; a.coef_ks = -js * bh; a.W_hh = p[k].W_hh;
     const bool bf16 = c->operands == MGRIT_OPERANDS_BF16;
-    // the step arriving at reversed point s applies the level's forward step stored at coefficient row N_l - s
-    const i64 row0 = (i64)(hr.N[d.l] - d.tgt_slot) * (i64)bh, coef_ks = -(i64)d.tgt_stride * (i64)bh;
-    for (int k = nl - 1; k >= 0; --k) {       // top layer first: what it sends to its input joins the layer below
-      StackLayerAdj& L = w->L[k];
-      AdjStepArgs a;
-      a.M = M; a.B = c->B; a.H = c->H;
-      if (k == nl - 1) { a.lin = U[d.l] + ((size_t)d.in_slot * nl + k) * bh; a.lin_ks = (i64)d.in_stride * slot; }
-      else { a.lin = w->tmpLin; a.lin_ks = (i64)bh; }
-      a.lout = d.out + ((size_t)d.out_slot * nl + k) * bh; a.lout_ks = (i64)d.out_stride * slot;
-      a.gadd = d.gadd ? d.gadd + ((size_t)d.gadd_slot * nl + k) * bh : nullptr; a.gadd_ks = (i64)d.gadd_stride * slot;
-      a.a = L.a[d.l] + row0; a.coef_ks = coef_ks; a.W_hh = p[k].W_hh; a.mode = d.mode;
-      if (bf16) { a.cr = a.cz = a.cn = nullptr; a.crb = L.crb[d.l] + row0; a.czb = L.czb[d.l] + row0; a.cnb = L.cnb[d.l] + row0; }
-      else { a.crb = a.czb = a.cnb = nullptr; a.cr = L.cr[d.l] + row0; a.cz = L.cz[d.l] + row0; a.cn = L.cn[d.l] + row0; }
-      if (bf16) { int r = umma_adj_step(a, &L.um, s); if (r) return r; }
-      else simt_adj_step(a, s);
-      if (k > 0) {
-        // total output sensitivity of the layer below = its own entry of the incoming unknown + [c_r|c_z|c_n'] * lin W_ih
-        AdjStepArgs b = a;
-        if (bf16) { b.cnb = L.cnpb[d.l] + row0; int r = umma_adj_dx(b, L.um.W_ihT, c->H, w->tmpDx, &L.um, s); if (r) return r; }
-        else { b.cn = L.cnp[d.l] + row0; simt_adj_dx(b, p[k].W_ih, c->H, w->tmpDx, s); }
-        stream_gather_rows(w->tmpLin, (i64)bh, U[d.l] + ((size_t)d.in_slot * nl + (k - 1)) * bh, (i64)d.in_stride * slot, d.nk, (i64)bh, s);
-        stream_add_rows(w->tmpLin, w->tmpDx, (i64)M * c->H, s);
+    // (the operand buffer holds so many points at a time)
+    const int step = bf16 ? (int)(L.w.um.apack_elems / ((size_t)3 * bh)) : n;
+    for (int i0 = 0; i0 < n; i0 += step) {
+      const int m = n - i0 < step ? n - i0 : step;
+      const i64 row0 = ((i64)hr.N[l] - 1 - j0 - (i64)i0 * js) * bh;      // the step leaving point j is stored at row N - 1 - j
+      a.M = m * c->B;
+      a.lin = y[k].U[l] + ((i64)j0 + (i64)i0 * js) * bh;
+      float* out = w->dx + (i64)i0 * bh;
+      // (a middle layer's incoming sensitivities include what the layer above sent, which these rows still hold)
+      const bool mid = k < nl - 1;
+      if (bf16) {
+        if (mid) { a.ladd = out; a.ladd_ks = bh; }
+        a.crb = L.w.crb[l] + row0; a.czb = L.w.czb[l] + row0; a.cnb = L.cnpb[l] + row0;
+        rc = umma_adj_dx(a, L.w.um.W_ihT, c->H, out, &L.w.um, s);
+        if (rc) return;
+      } else {
+        a.cr = L.w.cr[l] + row0; a.cz = L.w.cz[l] + row0; a.cn = L.cnp[l] + row0;
+        if (mid) {
+          stream_sum_rows(w->lamk, a.lin, a.lin_ks, out, bh, m, bh, s);
+          a.lin = w->lamk; a.lin_ks = bh;
+        }
+        simt_adj_dx(a, p[k].W_ih, c->H, out, s);
       }
     }
-    return MGRIT_OK;
+  }
+  void part(int l, int kz, bool f, int last) {      // F-steps and v leave the points as they were sent; a C-step is a part of its own
+    const int cf = c->cf, N = hr.N[l], nc = N / cf;
+    for (int k = nl - 1; k >= 0 && status() == MGRIT_OK; --k) {
+      AdjCycle& q = y[k];
+      const i64 bh = (i64)q.BH;
+      q.lsum = w->lsum;
+      if (f) {
+        const int nki = nc, tail = N % cf;
+        for (int sI = 1; sI < cf; ++sI) {
+          q.ladd = k == nl - 1 ? nullptr : w->dx + (i64)(sI - 1) * bh; q.ladd_ks = (i64)cf * bh;
+          const int nk = nki + (sI <= tail ? 1 : 0);
+          q.step(StepDesc{l, nk < kz ? nk : kz, sI - 1, cf, q.U[l], sI, cf, q.G[l], sI, cf, sI, cf, 0});
+        }
+      }
+      if (last != kNone) {
+        q.ladd = k == nl - 1 ? nullptr : f ? w->dx + (i64)(cf - 1) * bh : w->dx; q.ladd_ks = f ? (i64)cf * bh : bh;
+        float* out = last == kV ? q.G[l + 1] : q.U[l];
+        q.step(StepDesc{l, nc < kz ? nc : kz, cf - 1, cf, out, last == kV ? 1 : cf, last == kV ? 1 : cf, q.G[l], cf, cf, cf, cf, 0});
+      }
+      q.ladd = nullptr;
+      if (f) send(k, l, 0, 1, kz < nc ? kz * cf : N);
+      else send(k, l, cf - 1, cf, nc < kz ? nc : kz);
+    }
+  }
+  void segment(int l, int kz, bool f, int last) override {
+    if (last == kC) {        // (the C-step overwrites points that F-steps left from)
+      if (f) part(l, kz, true, kNone);
+      part(l, kz, false, kC);
+    } else {
+      part(l, kz, f, last);
+    }
+  }
+  void coarse_rhs(int l, int np) override {
+    for (int k = nl - 1; k >= 0 && status() == MGRIT_OK; --k) {
+      AdjCycle& q = y[k];
+      q.lsum = w->lsum; q.ladd = k == nl - 1 ? nullptr : w->dx; q.ladd_ks = (i64)q.BH;
+      q.step(StepDesc{l, np, 0, 1, q.G[l], 1, 1, nullptr, 0, 0, 1, 1, 1});
+      q.ladd = nullptr;
+      send(k, l, 0, 1, np);
+    }
+  }
+  bool chain(int k, int l, float* mu, const float* g) {
+    if (c->operands != MGRIT_OPERANDS_FP32 || !f32_solve_fits(c->H)) return y[k].chain_on(l, mu, g);
+    float* Us[kMaxLevels] = {}; float* Gs[kMaxLevels] = {};
+    Us[l] = mu; Gs[l] = const_cast<float*>(g);
+    AdjWs& q = w->L[k].w;
+    F32Cycle fc;
+    fc.c = c; fc.hr = &hr; fc.adjoint = true; fc.s = s; fc.U = Us; fc.G = Gs; fc.res_acc = res_acc;
+    fc.a.B = c->B; fc.a.H = c->H; fc.a.cell = c->cell; fc.a.W = p[k].W_hh; fc.a.bar = q.chain_bar;
+    fc.a.coef[l][0] = q.a[l]; fc.a.coef[l][1] = q.cr[l]; fc.a.coef[l][2] = q.cz[l]; fc.a.coef[l][3] = q.cn[l];
+    fc.a.nph = 0;
+    fc.cycle(l, false, false);       // (the coarsest level: one phase)
+    fc.flush();
+    if (!fc.ok) rc = MGRIT_CUDA_ERROR;
+    return true;
+  }
+  // Below the top layer mu_s = step(mu_{s-1} + d_{s-1}) + g_s: a chain in nu_s = mu_s + d_s with the source g_s + d_s.
+  void coarsest(int l) override {
+    const int N = hr.N[l];
+    for (int k = nl - 1; k >= 0 && status() == MGRIT_OK; --k) {
+      AdjCycle& q = y[k];
+      const i64 bh = (i64)q.BH;
+      if (k == nl - 1) {
+        if (!chain(k, l, q.U[l], q.G[l]))
+          for (int j = 1; j <= N; ++j) q.step(StepDesc{l, 1, j - 1, 1, q.U[l], j, 1, q.G[l], j, 1, j, 1, 0});
+      } else {
+        stream_nu_start(w->nu, w->gnu, q.U[l], q.G[l], w->dx, N, bh, s);
+        if (chain(k, l, w->nu, w->gnu)) {
+          stream_nu_finish(q.U[l], w->nu, w->dx, N, bh, s);
+        } else {
+          q.lsum = w->lsum; q.ladd_ks = bh;
+          for (int j = 1; j <= N; ++j) { q.ladd = w->dx + (i64)(j - 1) * bh; q.step(StepDesc{l, 1, j - 1, 1, q.U[l], j, 1, q.G[l], j, 1, j, 1, 0}); }
+          q.ladd = nullptr;
+        }
+      }
+      send(k, l, 0, 1, N);
+    }
   }
 };
 
-// time-parallel gradient pass of one layer given its total output sensitivities lam[T, B, H] (forward order, contiguous)
+// time-parallel gradient pass of one layer given its total output sensitivities (row (t, b) at lam + t*lam_ts + b*H)
 int stack_layer_gradients(const mgrit_gru_cfg& ck, const gru_params* pk, const float* xk, const float* h0k, StackLayerAdj& L,
-                          StackAdjWs& w, float* dx, const gru_grads* g, cudaStream_t s) {
-  const i64 bh = (i64)ck.B * ck.H, M = (i64)ck.T * ck.B;
+                          const float* lam, i64 lam_ts, float* dx, const gru_grads* g, cudaStream_t s) {
+  const i64 M = (i64)ck.T * ck.B;
   if (ck.operands == MGRIT_OPERANDS_BF16)
-    return umma_gradients(&ck, pk, xk, h0k, L.hk, w.lamk, bh, L.crb[0], L.czb[0], L.cnb[0], L.cnpb[0], dx, g, &L.um, false, s);
-  simt_gradients((int)M, ck.B, ck.H, ck.I, w.lamk, bh, L.cr[0], L.cz[0], L.cn[0], L.cnp[0], h0k, L.hk, xk, pk->W_ih, dx, g, w.grad_scratch, s);
+    return umma_gradients(&ck, pk, xk, h0k, L.hk, lam, lam_ts, L.w.crb[0], L.w.czb[0], L.w.cnb[0], L.cnpb[0], dx, g, &L.w.um, false, s);
+  simt_gradients((int)M, ck.B, ck.H, ck.I, lam, lam_ts, L.w.cr[0], L.w.cz[0], L.w.cn[0], L.cnp[0], h0k, L.hk, xk, pk->W_ih, dx, g, L.w.grad_scratch, s);
   return MGRIT_OK;
 }
 
@@ -1121,13 +1329,13 @@ int stack_adjoint_impl(const mgrit_gru_cfg* cfg, int nl, const gru_params* p, co
     StackLayerAdj& L = aw.L[k];
     mgrit_gru_cfg ck = layer_cfg(c, k);
     if (bf16) {
-      rc = umma_prepare_adj(&ck, &p[k], h0 + (size_t)k * bh, L.hk, &L.um, false, s);
+      rc = umma_prepare_adj(&ck, &p[k], h0 + (size_t)k * bh, L.hk, &L.w.um, false, s);
       if (rc) return rc;
     }
     if (k > 0) {
       if (bf16) {
         umma_convert(p[k].W_ih, L.Wihb, (i64)3 * c.H * c.H, s);
-        rc = umma_project_rows(aw.L[k - 1].hk, L.um.xb, L.Wihb, p[k].b_ih, L.gik, T * c.B, c.H, 3 * c.H, s);
+        rc = umma_project_rows(aw.L[k - 1].hk, L.w.um.xb, L.Wihb, p[k].b_ih, L.gik, T * c.B, c.H, 3 * c.H, s);
         if (rc) return rc;
       } else {
         simt_project(aw.L[k - 1].hk, p[k].W_ih, p[k].b_ih, L.gik, T * c.B, c.H, 3 * c.H, s);
@@ -1138,43 +1346,54 @@ int stack_adjoint_impl(const mgrit_gru_cfg* cfg, int nl, const gru_params* p, co
       a.M = hr.N[l] * c.B; a.B = c.B; a.H = c.H; a.h0 = h0 + (size_t)k * bh; a.h = L.hk; a.stride_t = hr.stride_t[l];
       a.t0 = hr.rem[l]; a.gi = k == 0 ? gi0 : L.gik;
       a.W_hh = p[k].W_hh; a.b_hh = p[k].b_hh; a.gamma = hr.gamma[l]; a.cell = c.cell;
-      a.a = L.a[l]; a.cr = L.cr[l]; a.cz = L.cz[l]; a.cn = L.cn[l]; a.cnp = L.cnp[l];
-      a.crb = L.crb[l]; a.czb = L.czb[l]; a.cnb = L.cnb[l]; a.cnpb = L.cnpb[l];
-      if (bf16) { rc = umma_linearise(a, &L.um, s); if (rc) return rc; }
+      a.a = L.w.a[l]; a.cr = L.w.cr[l]; a.cz = L.w.cz[l]; a.cn = L.w.cn[l]; a.cnp = L.cnp[l];
+      a.crb = L.w.crb[l]; a.czb = L.w.czb[l]; a.cnb = L.w.cnb[l]; a.cnpb = L.cnpb[l];
+      if (bf16) { rc = umma_linearise(a, &L.w.um, s); if (rc) return rc; }
       else simt_linearise(a, s);
     }
   }
   // mu_0 = lambda_T (all layers); zero initial guess elsewhere; fine-level source = reversed dh_seed
-  cudaMemsetAsync(aw.U[0], 0, sizeof(float) * slot, s);
-  zero_guess(aw.U[0], c, hr, slot, s);
-  float* Gl[kMaxLevels];
-  for (int l = 0; l < hr.L; ++l) Gl[l] = aw.G[l];
-  if (!dh_seed) Gl[0] = nullptr;
-  if (dh_seed) {
-    cudaMemcpyAsync(aw.U[0], dh_seed + (size_t)(T - 1) * slot, sizeof(float) * slot, cudaMemcpyDeviceToDevice, s);
-    cudaMemsetAsync(aw.G[0] + (size_t)T * slot, 0, sizeof(float) * slot, s);
-    if (T > 1) stream_gather_rows(aw.G[0] + slot, (i64)slot, dh_seed + (size_t)(T - 2) * slot, -(i64)slot, T - 1, (i64)slot, s);
-  }
-  if (dhT) stream_add_rows(aw.U[0] + (size_t)(nl - 1) * bh, dhT, (i64)bh, s);       // loss on the top layer's last state
-  for (int l = 1; l < hr.L; ++l) cudaMemcpyAsync(aw.U[l], aw.U[0], sizeof(float) * slot, cudaMemcpyDeviceToDevice, s);
-
   StackAdjCycle cy;
   cy.homog = !dh_seed;
-  cy.c = &c; cy.hr = hr; cy.s = s; cy.U = aw.U; cy.G = Gl; cy.res_acc = aw.res_acc; cy.BH = slot;
-  cy.nl = nl; cy.p = p; cy.w = &aw;
+  cy.c = &c; cy.hr = hr; cy.s = s; cy.nl = nl; cy.res_acc = aw.res_acc; cy.p = p; cy.w = &aw;
+  mgrit_gru_cfg ck[kMaxStack];
+  float* Gl[kMaxStack][kMaxLevels];
+  for (int k = 0; k < nl; ++k) {
+    AdjWs& q = aw.L[k].w;
+    ck[k] = layer_cfg(c, k);
+    zero_guess(q.U[0], c, hr, bh, s);
+    for (int l = 0; l < hr.L; ++l) Gl[k][l] = q.G[l];
+    if (!dh_seed) Gl[k][0] = nullptr;
+    if (dh_seed) {
+      cudaMemcpyAsync(q.U[0], dh_seed + (size_t)(T - 1) * slot + k * bh, sizeof(float) * bh, cudaMemcpyDeviceToDevice, s);
+      cudaMemsetAsync(q.G[0] + (size_t)T * bh, 0, sizeof(float) * bh, s);
+      if (T > 1) stream_gather_rows(q.G[0] + bh, (i64)bh, dh_seed + (size_t)(T - 2) * slot + k * bh, -(i64)slot, T - 1, (i64)bh, s);
+    } else {
+      cudaMemsetAsync(q.U[0], 0, sizeof(float) * bh, s);
+    }
+    if (dhT && k == nl - 1) stream_add_rows(q.U[0], dhT, (i64)bh, s);       // loss on the top layer's last state
+    for (int l = 1; l < hr.L; ++l) cudaMemcpyAsync(q.U[l], q.U[0], sizeof(float) * bh, cudaMemcpyDeviceToDevice, s);
+    AdjCycle& y = cy.y[k];
+    y.c = &ck[k]; y.hr = hr; y.s = s; y.U = q.U; y.G = Gl[k]; y.res_acc = aw.res_acc; y.BH = bh; y.p = &p[k]; y.w = &q;
+  }
   rc = cy.solve();
   if (rc) return rc;
 
-  if (dh) stream_gather_rows(dh, (i64)slot, aw.U[0] + (size_t)(T - 1) * slot, -(i64)slot, T, (i64)slot, s);
-  cudaMemcpyAsync(dh0, aw.U[0] + (size_t)T * slot, sizeof(float) * slot, cudaMemcpyDeviceToDevice, s);
-
+  for (int k = 0; k < nl; ++k) {
+    const float* U0 = aw.L[k].w.U[0];
+    if (dh) stream_gather_rows(dh + k * bh, (i64)slot, U0 + (size_t)(T - 1) * bh, -(i64)bh, T, (i64)bh, s);
+    cudaMemcpyAsync(dh0 + k * bh, U0 + (size_t)T * bh, sizeof(float) * bh, cudaMemcpyDeviceToDevice, s);
+  }
   // gradient pass, top layer first: a layer's total output sensitivity is its entry of the unknown plus what the layer
   // above sends to its input (that layer's input gradient)
   for (int k = nl - 1; k >= 0; --k) {
-    stream_gather_rows(aw.lamk, (i64)bh, aw.U[0] + (size_t)(T - 1) * slot + (size_t)k * bh, -(i64)slot, T, (i64)bh, s);
-    if (k < nl - 1) stream_add_rows(aw.lamk, aw.dxk, (i64)T * (i64)bh, s);
-    mgrit_gru_cfg ck = layer_cfg(c, k);
-    rc = stack_layer_gradients(ck, &p[k], k == 0 ? x : aw.L[k - 1].hk, h0 + (size_t)k * bh, aw.L[k], aw, k > 0 ? aw.dxk : dx, &g[k], s);
+    const float* lam = aw.L[k].w.U[0] + (size_t)(T - 1) * bh;
+    i64 lam_ts = -(i64)bh;
+    if (k < nl - 1) {
+      stream_sum_rows(aw.lamk, lam, lam_ts, aw.dxk, (i64)bh, T, (i64)bh, s);
+      lam = aw.lamk; lam_ts = (i64)bh;
+    }
+    rc = stack_layer_gradients(ck[k], &p[k], k == 0 ? x : aw.L[k - 1].hk, h0 + (size_t)k * bh, aw.L[k], lam, lam_ts, k > 0 ? aw.dxk : dx, &g[k], s);
     if (rc) return rc;
   }
   if (resnorm && hr.L > 1 && c.iters > 0) {

@@ -152,6 +152,8 @@ struct AdjStepArgs {
   const float* gadd; i64 gadd_ks;   // optional source / FAS term, same shape as lout
   const float *a, *cr, *cz, *cn; i64 coef_ks;   // coefficient rows (+k*coef_ks + b*H), already offset to k = 0
   const __nv_bfloat16 *crb, *czb, *cnb;         // the same rows in bf16 (tensor-core engine; same indexing)
+  // stacked layers, optional: rows ladd (+k*ladd_ks + b*H) join the incoming rows; the sums go to lsum (contiguous [M, H])
+  const float* ladd; i64 ladd_ks; float* lsum;
   const float* W_hh;                // [3H,H] fp32
   int mode;                         // as FwdStepArgs
 };
@@ -225,6 +227,16 @@ void stream_correct(float* uf, __nv_bfloat16* ufb, int cf, const float* uc, int 
 // dst[k] = src[k*src_ks], k = 0..nk-1, rows of rowlen floats (src_ks in elements, may be negative)
 void stream_gather_rows(float* dst, i64 dst_ks, const float* src, i64 src_ks, int nk, i64 rowlen, cudaStream_t s);
 void stream_add_rows(float* dst, const float* src, i64 n, cudaStream_t s);
+// dst[k] = a[k*a_ks] + b[k*b_ks], k = 0..nk-1, rows of rowlen floats (dst contiguous)
+void stream_sum_rows(float* dst, const float* a, i64 a_ks, const float* b, i64 b_ks, int nk, i64 rowlen, cudaStream_t s);
+// stacked layers.  Row j - 1 = U[j] (V[j / cf] at the C-points when V is given) minus G[j] (when G is given), j = 1..N, to
+// exactly one of out32 / out16 (bf16).
+void stream_raw_rows(const float* U, const float* G, const float* V, int cf, int N, i64 rowlen, float* out32, __nv_bfloat16* out16, cudaStream_t s);
+// G -= phi (n floats); phi as bf16 to out16 when given
+void stream_subtract_rows(float* G, const float* phi, i64 n, __nv_bfloat16* out16, cudaStream_t s);
+// nu[0] = U[0] + d[0]; gnu[s] = (G ? G[s] : 0) + (s < N ? d[s] : 0);   U[s] = nu[s] - (s < N ? d[s] : 0), s = 1..N
+void stream_nu_start(float* nu, float* gnu, const float* U, const float* G, const float* d, int N, i64 rowlen, cudaStream_t s);
+void stream_nu_finish(float* U, const float* nu, const float* d, int N, i64 rowlen, cudaStream_t s);
 // tmp[M, H] contiguous (rows (k, b)) -> dst rows at dst + k*dst_ks + b*H: mode 0 dst = tmp (+ g rows, same indexing with g_ks),
 // mode 1 dst = dst - tmp
 void stream_combine_rows(const float* tmp, const float* g, i64 g_ks, float* dst, i64 dst_ks, int B, int H, i64 M, int mode, cudaStream_t s);

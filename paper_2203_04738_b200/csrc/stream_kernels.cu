@@ -118,6 +118,50 @@ __global__ void __launch_bounds__(kThreads) add_rows_kernel(float4* __restrict__
   }
 }
 
+__device__ __forceinline__ float4 sub4(float4 a, float4 b) { return make_float4(a.x - b.x, a.y - b.y, a.z - b.z, a.w - b.w); }
+__device__ __forceinline__ float4 sum4(float4 a, float4 b) { return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); }
+__global__ void __launch_bounds__(kThreads) sum_rows_kernel(float4* __restrict__ dst, const float4* __restrict__ a, i64 a_ks4, const float4* __restrict__ b,
+                                                            i64 b_ks4, int nk, i64 row4) {
+  for (i64 e = (i64)blockIdx.x * blockDim.x + threadIdx.x; e < (i64)nk * row4; e += (i64)gridDim.x * blockDim.x) {
+    const i64 k = e / row4, c = e % row4;
+    dst[e] = sum4(a[k * a_ks4 + c], b[k * b_ks4 + c]);
+  }
+}
+__global__ void __launch_bounds__(kThreads) raw_rows_kernel(const float4* __restrict__ U, const float4* __restrict__ G, const float4* __restrict__ V, int cf,
+                                                            int N, i64 row4, float4* __restrict__ out32, uint2* __restrict__ out16) {
+  pdl_wait();
+  pdl_trigger();
+  for (i64 e = (i64)blockIdx.x * blockDim.x + threadIdx.x; e < (i64)N * row4; e += (i64)gridDim.x * blockDim.x) {
+    const int j = (int)(e / row4) + 1;
+    const i64 c = e % row4;
+    float4 v = V && j % cf == 0 ? V[(j / cf) * row4 + c] : U[j * row4 + c];
+    if (G) v = sub4(v, G[j * row4 + c]);
+    if (out16) out16[e] = pack_bf16x4(v);
+    else out32[e] = v;
+  }
+}
+__global__ void __launch_bounds__(kThreads) subtract_rows_kernel(float4* __restrict__ G, const float4* __restrict__ phi, i64 n4, uint2* __restrict__ out16) {
+  pdl_wait();
+  pdl_trigger();
+  for (i64 e = (i64)blockIdx.x * blockDim.x + threadIdx.x; e < n4; e += (i64)gridDim.x * blockDim.x) {
+    const float4 v = phi[e];
+    G[e] = sub4(G[e], v);
+    if (out16) out16[e] = pack_bf16x4(v);
+  }
+}
+__global__ void __launch_bounds__(kThreads) nu_start_kernel(float4* __restrict__ nu, float4* __restrict__ gnu, const float4* __restrict__ U,
+                                                            const float4* __restrict__ G, const float4* __restrict__ d, int N, i64 row4) {
+  for (i64 e = (i64)blockIdx.x * blockDim.x + threadIdx.x; e < (i64)(N + 1) * row4; e += (i64)gridDim.x * blockDim.x) {
+    const float4 z = make_float4(0.f, 0.f, 0.f, 0.f), dv = e < (i64)N * row4 ? d[e] : z;
+    if (e < row4) nu[e] = sum4(U[e], dv);
+    else gnu[e] = sum4(G ? G[e] : z, dv);
+  }
+}
+__global__ void __launch_bounds__(kThreads) nu_finish_kernel(float4* __restrict__ U, const float4* __restrict__ nu, const float4* __restrict__ d, int N, i64 row4) {
+  for (i64 e = row4 + (i64)blockIdx.x * blockDim.x + threadIdx.x; e < (i64)(N + 1) * row4; e += (i64)gridDim.x * blockDim.x)
+    U[e] = e < (i64)N * row4 ? sub4(nu[e], d[e]) : nu[e];
+}
+
 __global__ void __launch_bounds__(kThreads) form_dA_kernel(const float4* __restrict__ lam, const float4* __restrict__ cr,
                                                            const float4* __restrict__ cz, const float4* __restrict__ cn,
                                                            const float4* __restrict__ cnp, float4* __restrict__ dA_h,
@@ -337,6 +381,30 @@ void stream_combine_rows(const float* tmp, const float* g, i64 g_ks, float* dst,
 
 void stream_add_rows(float* dst, const float* src, i64 n, cudaStream_t s) {
   add_rows_kernel<<<stream_grid(n / 4), kThreads, 0, s>>>(reinterpret_cast<float4*>(dst), reinterpret_cast<const float4*>(src), n / 4);
+  count_launch();
+}
+
+void stream_sum_rows(float* dst, const float* a, i64 a_ks, const float* b, i64 b_ks, int nk, i64 rowlen, cudaStream_t s) {
+  if (nk <= 0) return;
+  sum_rows_kernel<<<stream_grid((i64)nk * (rowlen / 4)), kThreads, 0, s>>>((float4*)dst, (const float4*)a, a_ks / 4, (const float4*)b, b_ks / 4, nk, rowlen / 4);
+  count_launch();
+}
+void stream_raw_rows(const float* U, const float* G, const float* V, int cf, int N, i64 rowlen, float* out32, __nv_bfloat16* out16, cudaStream_t s) {
+  launch_pdl(raw_rows_kernel, dim3(stream_grid((i64)N * (rowlen / 4))), dim3(kThreads), 0, s, (const float4*)U, (const float4*)G, (const float4*)V, cf, N,
+             rowlen / 4, (float4*)out32, (uint2*)out16);
+  count_launch();
+}
+void stream_subtract_rows(float* G, const float* phi, i64 n, __nv_bfloat16* out16, cudaStream_t s) {
+  launch_pdl(subtract_rows_kernel, dim3(stream_grid(n / 4)), dim3(kThreads), 0, s, (float4*)G, (const float4*)phi, n / 4, (uint2*)out16);
+  count_launch();
+}
+void stream_nu_start(float* nu, float* gnu, const float* U, const float* G, const float* d, int N, i64 rowlen, cudaStream_t s) {
+  nu_start_kernel<<<stream_grid((i64)(N + 1) * (rowlen / 4)), kThreads, 0, s>>>((float4*)nu, (float4*)gnu, (const float4*)U, (const float4*)G, (const float4*)d, N,
+                                                                               rowlen / 4);
+  count_launch();
+}
+void stream_nu_finish(float* U, const float* nu, const float* d, int N, i64 rowlen, cudaStream_t s) {
+  nu_finish_kernel<<<stream_grid((i64)N * (rowlen / 4)), kThreads, 0, s>>>((float4*)U, (const float4*)nu, (const float4*)d, N, rowlen / 4);
   count_launch();
 }
 

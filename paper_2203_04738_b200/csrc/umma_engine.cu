@@ -690,7 +690,8 @@ __global__ void __launch_bounds__(kPT) pack_rows_kernel(const float* __restrict_
 // dst[m, g*H + i] = bf16(c_g[m, i] * lam[m, i])
 __global__ void __launch_bounds__(kPT) pack_adj_kernel(const float* __restrict__ lin, i64 lin_ks, const bf16* __restrict__ cr,
                                                        const bf16* __restrict__ cz, const bf16* __restrict__ cn, i64 coef_ks,
-                                                       int B, int H4, i64 M, uint2* __restrict__ dst) {
+                                                       int B, int H4, i64 M, uint2* __restrict__ dst, const float* __restrict__ ladd,
+                                                       i64 ladd_ks, float4* __restrict__ lsum) {
   pdl_wait();
   pdl_trigger();
   i64 total = M * H4;
@@ -705,6 +706,11 @@ __global__ void __launch_bounds__(kPT) pack_adj_kernel(const float* __restrict__
     i64 k = m / B; int b = (int)(m % B);
     i64 ro = ((i64)b * H4 + c) * 4;
     float4 l = *reinterpret_cast<const float4*>(lin + k * lin_ks + ro);
+    if (ladd) {
+      const float4 t = *reinterpret_cast<const float4*>(ladd + k * ladd_ks + ro);
+      l = make_float4(l.x + t.x, l.y + t.y, l.z + t.z, l.w + t.w);
+      if (lsum) lsum[e] = l;
+    }
     float4 r = unpack4(ldc(cr + k * coef_ks + ro));
     float4 z = unpack4(ldc(cz + k * coef_ks + ro));
     float4 n = unpack4(ldc(cn + k * coef_ks + ro));
@@ -1044,12 +1050,14 @@ static bool few_row_adj(const AdjStepArgs& a, const bf16* Apack, const bf16* WT,
   }
 }
 
-int umma_adj_step(const AdjStepArgs& a, UmmaAdjWs* w, cudaStream_t s) {
-  ProfScope prof(KC_ADJ_STEP, 2.0 * a.M * 3.0 * a.H * a.H, s);     // operand packing + product, timed together
-  if (launch_pdl(pack_adj_kernel, dim3(pgrid((i64)a.M * (a.H / 4))), dim3(kPT), 0, s, a.lin, a.lin_ks, a.crb, a.czb, a.cnb, a.coef_ks,
-                 a.B, a.H / 4, (i64)a.M, reinterpret_cast<uint2*>(w->Apack)) != cudaSuccess)
+int umma_adj_step(const AdjStepArgs& in, UmmaAdjWs* w, cudaStream_t s) {
+  ProfScope prof(KC_ADJ_STEP, 2.0 * in.M * 3.0 * in.H * in.H, s);     // operand packing + product, timed together
+  if (launch_pdl(pack_adj_kernel, dim3(pgrid((i64)in.M * (in.H / 4))), dim3(kPT), 0, s, in.lin, in.lin_ks, in.crb, in.czb, in.cnb, in.coef_ks,
+                 in.B, in.H / 4, (i64)in.M, reinterpret_cast<uint2*>(w->Apack), in.ladd, in.ladd_ks, reinterpret_cast<float4*>(in.lsum)) != cudaSuccess)
     return MGRIT_CUDA_ERROR;
   count_launch();
+  AdjStepArgs a = in;
+  if (a.ladd) { a.lin = a.lsum; a.lin_ks = (i64)a.B * a.H; }
   // Few-row launches (coarse levels, short prefixes) cannot fill the SMs with 256-column tiles and are
   // bound by one CTA streaming all of K; 64-column tiles spread that stream over four times the CTAs.
   const int tiles256 = ((a.M + BM - 1) / BM) * ((a.H + 255) / 256);
@@ -1159,13 +1167,18 @@ void umma_convert(const float* src, __nv_bfloat16* dst, i64 n, cudaStream_t s) {
 // out[M, 3H] = X[M, K] W^T + bias with X fp32 contiguous (converted into xb first) and W already bf16 [3H, K]
 int umma_project_rows(const float* X, bf16* xb, const bf16* Wb, const float* bias, float* out, int M, int K, int H3, cudaStream_t s) {
   convert(X, xb, (i64)M * K, s);
-  return launch_gemm<256, 0>(KC_PROJ, xb, K, Wb, K, M, H3, K, 0, H3, EpiBias{out, H3, bias, M, H3}, s) ? MGRIT_OK : MGRIT_CUDA_ERROR;
+  return umma_project_packed(xb, Wb, bias, out, nullptr, M, K, H3, s);
+}
+int umma_project_packed(const bf16* xb, const bf16* Wb, const float* bias, float* out, bf16* outb, int M, int K, int H3, cudaStream_t s) {
+  const EpiBias epi{out, H3, bias, M, H3, outb};
+  return (gemm_pair_enabled(M, H3) ? launch_gemm_pair(KC_PROJ, xb, K, Wb, K, M, H3, K, H3, epi, s)
+                                   : launch_gemm<256, 0>(KC_PROJ, xb, K, Wb, K, M, H3, K, 0, H3, epi, s)) ? MGRIT_OK : MGRIT_CUDA_ERROR;
 }
 
 // out[M, C] = ([cr|cz|cn]*lam of the step `a`) W_ihT^T: the sensitivity a cell sends to its input (a.cnb holding c_n')
 int umma_adj_dx(const AdjStepArgs& a, const bf16* W_ihT, int C, float* out, UmmaAdjWs* w, cudaStream_t s) {
   if (launch_pdl(pack_adj_kernel, dim3(pgrid((i64)a.M * (a.H / 4))), dim3(kPT), 0, s, a.lin, a.lin_ks, a.crb, a.czb, a.cnb, a.coef_ks,
-                 a.B, a.H / 4, (i64)a.M, reinterpret_cast<uint2*>(w->Apack)) != cudaSuccess)
+                 a.B, a.H / 4, (i64)a.M, reinterpret_cast<uint2*>(w->Apack), a.ladd, a.ladd_ks, (float4*)nullptr) != cudaSuccess)
     return MGRIT_CUDA_ERROR;
   count_launch();
   return launch_gemm<256, 0>(KC_ADJ_STEP, w->Apack, 3 * a.H, W_ihT, 3 * a.H, a.M, C, 3 * a.H, 0, C, EpiStore{out, C, a.M, C, 0}, s)

@@ -86,6 +86,9 @@ int umma_prepare_fwd(const mgrit_gru_cfg* c, const gru_params* p, const float* x
 int umma_prepare_adj(const mgrit_gru_cfg* c, const gru_params* p, const float* h0, const float* h, UmmaAdjWs* w, bool have_hb,
                      cudaStream_t s);
 void umma_convert(const float* src, __nv_bfloat16* dst, i64 n, cudaStream_t s);
+// out / outb [M, 3H] = xb[M, K] W^T + bias, rows already bf16; one of the outputs may be null
+int umma_project_packed(const __nv_bfloat16* xb, const __nv_bfloat16* Wb, const float* bias, float* out, __nv_bfloat16* outb, int M, int K, int H3,
+                        cudaStream_t s);
 int umma_project_rows(const float* X, __nv_bfloat16* xb, const __nv_bfloat16* Wb, const float* bias, float* out, int M, int K, int H3,
                       cudaStream_t s);
 int umma_adj_dx(const AdjStepArgs& a, const __nv_bfloat16* W_ihT, int C, float* out, UmmaAdjWs* w, cudaStream_t s);
