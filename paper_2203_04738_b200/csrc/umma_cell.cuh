@@ -200,19 +200,21 @@ constexpr int kOpBytes = BM * CH * 4;   // one epilogue operand chunk: 128 rows 
 // the same 20 us of a 118 us step and one stage of the operand ring; what a store costs here is the number of
 // row pieces that reach L2, not the path they take (rows of 128 bytes instead of 64 halve it).
 constexpr int kCoefBytes = BM * CH * 2;   // one coefficient chunk: 128 rows x 16 bf16
-template <bool PAIR> struct Geo {
-  static constexpr int UN = PAIR ? 80 : 64;         // hidden units per tile
+// SMALL: 32 units per tile, for steps whose 64-unit tiles would leave half of the SMs without one: a step is then bound by what
+// one CTA takes in (28 instead of 40 KiB per k-block) and by its epilogue (half the chunks).
+template <bool PAIR, bool SMALL = false> struct Geo {
+  static constexpr int UN = PAIR ? 80 : (SMALL ? 32 : 64);   // hidden units per tile
   static constexpr int BN = 3 * UN;                 // accumulator columns: r | z | n
   static constexpr int NCH = UN / CH;
-  static constexpr int kBox = PAIR ? 40 : 64;       // weight rows per TMA box
+  static constexpr int kBox = PAIR ? 40 : UN;       // weight rows per TMA box
   static constexpr int kBBytes = (PAIR ? BN / 2 : BN) * BK * 2;   // weight bytes staged per CTA and k-block
   static constexpr int kStageBytes = kABytes + kBBytes;           // 31 KiB / 40 KiB (multiples of 1 KiB)
 };
 // GIB: the input projection is staged from its bf16 copy (rows of 32 bytes, 32-byte swizzle) instead of fp32: 10 instead of
 // 16 bytes per element of epilogue operands, and a third operand buffer fits.  What hides the latency of those loads is
 // the bytes in flight, and shared memory bounds them: a tile needs 128 x UN x (bytes per element) per main-loop time.
-template <bool HAS_G, bool LIN = false, bool PAIR = false, bool GIB = false> struct CellCfg {
-  using G = Geo<PAIR>;
+template <bool HAS_G, bool LIN = false, bool PAIR = false, bool GIB = false, bool SMALL = false> struct CellCfg {
+  using G = Geo<PAIR, SMALL>;
 #ifndef CELL_PAIR_STAGES_PLAIN
 #define CELL_PAIR_STAGES_PLAIN 5
 #endif
@@ -222,11 +224,11 @@ template <bool HAS_G, bool LIN = false, bool PAIR = false, bool GIB = false> str
 #ifndef CELL_PAIR_EBUFS
 #define CELL_PAIR_EBUFS 2
 #endif
-  static constexpr int kStages = PAIR ? CELL_PAIR_STAGES : ((HAS_G || LIN) ? 3 : 4);
+  static constexpr int kStages = PAIR ? CELL_PAIR_STAGES : SMALL ? 5 : ((HAS_G || LIN) ? 3 : 4);
 #ifndef CELL_GIB_EBUFS
 #define CELL_GIB_EBUFS 3
 #endif
-  static constexpr int kEpiBufs = GIB ? ((PAIR && !HAS_G && !LIN) ? CELL_GIB_EBUFS : (LIN ? 2 : 3)) : (PAIR ? CELL_PAIR_EBUFS : 2);     // epilogue-operand chunks in flight
+  static constexpr int kEpiBufs = SMALL ? 2 : GIB ? ((PAIR && !HAS_G && !LIN) ? CELL_GIB_EBUFS : (LIN ? 2 : 3)) : (PAIR ? CELL_PAIR_EBUFS : 2);     // epilogue-operand chunks in flight
   static constexpr int kGiBytes = GIB ? BM * CH * 2 : kOpBytes;   // one gate's chunk of the input projection
   static constexpr int kEpiBytes = 3 * kGiBytes + (HAS_G ? 2 : 1) * kOpBytes;   // gi r | z | n, previous state, additive term
   // per buffer: four bf16 coefficient tiles and (with GIB, where shared memory allows it) the fp32 tile of `a`
@@ -236,7 +238,7 @@ template <bool HAS_G, bool LIN = false, bool PAIR = false, bool GIB = false> str
 };
 }  // namespace cellk
 
-template <bool LIN, bool HAS_G, bool PAIR, bool GIB = false>
+template <bool LIN, bool HAS_G, bool PAIR, bool GIB = false, bool SMALL = false>
 __global__ void __launch_bounds__(cellk::kThreads, 1)
 umma_cell_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                  const __grid_constant__ CUtensorMap tmGI, const __grid_constant__ CUtensorMap tmHP,
@@ -244,9 +246,9 @@ umma_cell_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                  const __grid_constant__ CUtensorMap tmCZ, const __grid_constant__ CUtensorMap tmCN,
                  const __grid_constant__ CUtensorMap tmCP, CellArgs p, const __grid_constant__ SweepArgs swp, int* status) {
   using namespace cellk;
-  using C = CellCfg<HAS_G, LIN, PAIR, GIB>;
+  using C = CellCfg<HAS_G, LIN, PAIR, GIB, SMALL>;
   constexpr int kGi = C::kGiBytes;
-  using G = Geo<PAIR>;
+  using G = Geo<PAIR, SMALL>;
   constexpr int UN = G::UN, BN = G::BN, NCH = G::NCH, kStageBytes = G::kStageBytes;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
@@ -328,29 +330,50 @@ umma_cell_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         const int mt = row_tile(t), nt = t % n_tiles;
         const int in_s = LIN ? 0 : swp.st[sg].in_s;
         const CUtensorMap* mapA = !LIN && swp.st[sg].ext ? &tmCR : &tmA;
-        if (!deps_ready(sg, t / n_tiles, 17)) { ok = false; break; }
-        for (int kb = 0; kb < k_blocks; ++kb) {
-          if (!mbar_wait(empty_bar(stage), phase ^ 1u, abortp, status, 11)) { ok = false; break; }
-          const uint32_t a_dst = tiles_base + stage * kStageBytes, b_dst = a_dst + kABytes;
+        // The weight tiles of the first stages do not depend on the step before: they are requested before the wait for it.
+        const int ahead = k_blocks < C::kStages ? k_blocks : C::kStages;
+        auto load_w = [&](int st, int kb) {
+          const uint32_t b_dst = tiles_base + st * kStageBytes + kABytes;
           if (PAIR) {
             // The accumulator columns r | z | n (80 each) split into two halves of 120: CTA 0 stages the weight rows
             // of r and of the first 40 units of z, CTA 1 the rest -- six 40-row boxes, three per CTA.
-            const uint32_t fullL = mapa_shared(full_bar(stage), 0);
-            if (rank == 0) mbar_expect_tx(full_bar(stage), 2 * stage_tx);
-            if (LIN) tma_load_3d_pair(a_dst, &tmA, fullL, kb * BK, 0, mt * p.kt);
-            else tma_load_4d_pair(a_dst, mapA, fullL, kb * BK, 0, in_s, mt * p.kt);
+            const uint32_t fullL = mapa_shared(full_bar(st), 0);
+            if (rank == 0) mbar_expect_tx(full_bar(st), 2 * stage_tx);
 #pragma unroll
             for (int j = 0; j < 3; ++j) {
               const int piece = 3 * (int)rank + j;
               tma_load_2d_pair(b_dst + j * (G::kBox * BK * 2), &tmB, fullL, kb * BK, (piece >> 1) * H + nt * UN + (piece & 1) * G::kBox);
             }
           } else {
-            mbar_expect_tx(full_bar(stage), stage_tx);
-            if (LIN) tma_load_3d(a_dst, &tmA, full_bar(stage), kb * BK, 0, mt * p.kt);
-            else tma_load_4d(a_dst, mapA, full_bar(stage), kb * BK, 0, in_s, mt * p.kt);
+            mbar_expect_tx(full_bar(st), stage_tx);
 #pragma unroll
-            for (int g = 0; g < 3; ++g) tma_load_2d(b_dst + g * (G::kBBytes / 3), &tmB, full_bar(stage), kb * BK, g * H + nt * UN);
+            for (int g = 0; g < 3; ++g) tma_load_2d(b_dst + g * (G::kBBytes / 3), &tmB, full_bar(st), kb * BK, g * H + nt * UN);
           }
+        };
+        auto load_state = [&](int st, int kb) {
+          const uint32_t a_dst = tiles_base + st * kStageBytes;
+          if (PAIR) {
+            const uint32_t fullL = mapa_shared(full_bar(st), 0);
+            if (LIN) tma_load_3d_pair(a_dst, &tmA, fullL, kb * BK, 0, mt * p.kt);
+            else tma_load_4d_pair(a_dst, mapA, fullL, kb * BK, 0, in_s, mt * p.kt);
+          } else {
+            if (LIN) tma_load_3d(a_dst, &tmA, full_bar(st), kb * BK, 0, mt * p.kt);
+            else tma_load_4d(a_dst, mapA, full_bar(st), kb * BK, 0, in_s, mt * p.kt);
+          }
+        };
+        int st = stage; uint32_t ph = phase;
+        for (int kb = 0; kb < ahead && ok; ++kb) {
+          ok = mbar_wait(empty_bar(st), ph ^ 1u, abortp, status, 11);
+          if (ok) load_w(st, kb);
+          if (++st == C::kStages) { st = 0; ph ^= 1u; }
+        }
+        if (!ok || !deps_ready(sg, t / n_tiles, 17)) { ok = false; break; }
+        for (int kb = 0; kb < k_blocks; ++kb) {
+          if (kb >= ahead) {
+            if (!mbar_wait(empty_bar(stage), phase ^ 1u, abortp, status, 11)) { ok = false; break; }
+            load_w(stage, kb);
+          }
+          load_state(stage, kb);
           if (++stage == C::kStages) { stage = 0; phase ^= 1u; }
         }
       }
@@ -404,25 +427,37 @@ umma_cell_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         const int in_s = LIN ? 0 : swp.st[sg].in_s, tgt_s = LIN ? 0 : swp.st[sg].tgt_s;
         const bool ext = !LIN && swp.st[sg].ext;
         const CUtensorMap *mapGI = ext ? &tmCZ : &tmGI, *mapHP = ext ? &tmCN : &tmHP, *mapG = ext ? &tmCP : &tmG;
-        if (!deps_ready(sg, t / n_tiles, 18)) { ok = false; break; }
-        for (int c = 0; c < NCH; ++c) {
-          const int u = nt * UN + c * CH, k0 = mt * p.kt;
-          if (u >= H) break;                       // ragged last unit tile: these columns are never stored
-          if (!mbar_wait(eempty_bar(eb), ephase ^ 1u, abortp, status, 14)) { ok = false; break; }
-          const uint32_t dst = epi_base + eb * C::kEpiBytes;
-          mbar_expect_tx(efull_bar(eb), epi_tx);
-          if (LIN) {
-            tma_load_3d(dst, &tmGI, efull_bar(eb), u, 0, k0);
-            tma_load_3d(dst + kGi, &tmGI, efull_bar(eb), H + u, 0, k0);
-            tma_load_3d(dst + 2 * kGi, &tmGI, efull_bar(eb), 2 * H + u, 0, k0);
-            tma_load_3d(dst + 3 * kGi, &tmHP, efull_bar(eb), u, 0, k0);
-          } else {
-            tma_load_4d(dst, mapGI, efull_bar(eb), u, 0, tgt_s, k0);
-            tma_load_4d(dst + kGi, mapGI, efull_bar(eb), H + u, 0, tgt_s, k0);
-            tma_load_4d(dst + 2 * kGi, mapGI, efull_bar(eb), 2 * H + u, 0, tgt_s, k0);
-            tma_load_4d(dst + 3 * kGi, mapHP, efull_bar(eb), u, 0, in_s, k0);
-            if (HAS_G) tma_load_4d(dst + 3 * kGi + kOpBytes, mapG, efull_bar(eb), u, 0, tgt_s, k0);
+        const int k0 = mt * p.kt;
+        const int chunks = H - nt * UN >= UN ? NCH : (H - nt * UN + CH - 1) / CH;      // (a ragged last unit tile has fewer)
+        // the projection and the additive term do not depend on the step before either; the state does
+        const int ahead = chunks < C::kEpiBufs ? chunks : C::kEpiBufs;
+        auto load_gi = [&](int e, int c) {
+          const int u = nt * UN + c * CH;
+          const uint32_t dst = epi_base + e * C::kEpiBytes;
+          mbar_expect_tx(efull_bar(e), epi_tx);
+#pragma unroll
+          for (int g = 0; g < 3; ++g) {
+            if (LIN) tma_load_3d(dst + g * kGi, &tmGI, efull_bar(e), g * H + u, 0, k0);
+            else tma_load_4d(dst + g * kGi, mapGI, efull_bar(e), g * H + u, 0, tgt_s, k0);
           }
+          if (HAS_G) tma_load_4d(dst + 3 * kGi + kOpBytes, mapG, efull_bar(e), u, 0, tgt_s, k0);
+        };
+        int e = eb; uint32_t ph = ephase;
+        for (int c = 0; c < ahead && ok; ++c) {
+          ok = mbar_wait(eempty_bar(e), ph ^ 1u, abortp, status, 14);
+          if (ok) load_gi(e, c);
+          if (++e == C::kEpiBufs) { e = 0; ph ^= 1u; }
+        }
+        if (!ok || !deps_ready(sg, t / n_tiles, 18)) { ok = false; break; }
+        for (int c = 0; c < chunks; ++c) {
+          const int u = nt * UN + c * CH;
+          if (c >= ahead) {
+            if (!mbar_wait(eempty_bar(eb), ephase ^ 1u, abortp, status, 14)) { ok = false; break; }
+            load_gi(eb, c);
+          }
+          const uint32_t dst = epi_base + eb * C::kEpiBytes + 3 * kGi;
+          if (LIN) tma_load_3d(dst, &tmHP, efull_bar(eb), u, 0, k0);
+          else tma_load_4d(dst, mapHP, efull_bar(eb), u, 0, in_s, k0);
           if (++eb == C::kEpiBufs) { eb = 0; ephase ^= 1u; }
         }
       }

@@ -236,6 +236,13 @@ static bool cell_pair_enabled(int M, int H) {
   return v == 1 && (i64)(M / (2 * BM)) * ((H + 79) / 80) >= kSMs / 2;
 }
 
+// MGRIT_GRU_CELL_SMALL=0 in the environment keeps few-row forward steps on 64-unit tiles.
+static bool cell_small_enabled() {
+  static int v = -1;
+  if (v < 0) { const char* e = getenv("MGRIT_GRU_CELL_SMALL"); v = (e && e[0] == '0') ? 0 : 1; }
+  return v == 1;
+}
+
 // 4-D map {column, batch row, slot, interval}: element (c, b, sl, k) at base + k*ks + sl*ss + b*ld + c
 bool make_map4(CUtensorMap* m, CUtensorMapDataType dt, size_t esize, const void* base, uint64_t inner, uint64_t B, uint64_t nslots,
                uint64_t nk, uint64_t ld, i64 ss, i64 ks, uint32_t box_inner, uint32_t box_k, CUtensorMapSwizzle sw) {
@@ -318,15 +325,15 @@ struct CellFwdOperands {
   const float* gi; i64 gi_ss, gi_ks; const float* g; i64 g_ss, g_ks; int tgt_slots;
   const bf16* gi_b;      // bf16 copy of gi (same element indexing) or nullptr: staged instead of the fp32 rows
 };
-template <bool HAS_G, bool PAIR, bool GIB>
+template <bool HAS_G, bool PAIR, bool GIB, bool SMALL = false>
 bool launch_fwd_geo(int kc, const CellFwdOperands& o, int nk, int nk_ext, const bf16* W, CellArgs ca, const SweepArgs& sw, cudaStream_t s) {
-  using C = cellk::CellCfg<HAS_G, false, PAIR, GIB>;
-  using G = cellk::Geo<PAIR>;
+  using C = cellk::CellCfg<HAS_G, false, PAIR, GIB, SMALL>;
+  using G = cellk::Geo<PAIR, SMALL>;
   if (nk <= 0) return true;
   int* const status = status_ptr();
   if (!status) return false;
   static bool attr_set[kMaxDevices] = {false};
-  auto kern = umma_cell_kernel<false, HAS_G, PAIR, GIB>;
+  auto kern = umma_cell_kernel<false, HAS_G, PAIR, GIB, SMALL>;
   if (!set_smem_once(kern, C::kSmemBytes, attr_set)) return false;
   const int B = ca.B, H = ca.H, kt = 128 / B;
   ca.kt = kt; ca.nk = nk_ext; ca.M = nk_ext * B;
@@ -359,7 +366,9 @@ bool launch_fwd_geo(int kc, const CellFwdOperands& o, int nk, int nk_ext, const 
     const int grid = 2 * (int)(items < kSMs / 2 ? items : kSMs / 2);
     e = launch_pdl_cluster(kern, 2, dim3(grid), dim3(cellk::kThreads), C::kSmemBytes, s, ta, tb, tgi, thp, tg, xa, xgi, xhp, xg, ca, sw, status);
   } else {
-    const int grid = (int)(items < kSMs ? items : kSMs);
+    // (a multiple of the tiles where they are few: a CTA then keeps its tile from step to step, and the CTAs of the next step
+    // request its weights and projections while this step runs)
+    const int grid = (int)(items < kSMs ? items : tiles < kSMs ? kSMs / tiles * tiles : kSMs);
     e = launch_pdl(kern, dim3(grid), dim3(cellk::kThreads), C::kSmemBytes, s, ta, tb, tgi, thp, tg, xa, xgi, xhp, xg, ca, sw, status);
   }
   if (e != cudaSuccess) return false;
@@ -370,6 +379,10 @@ bool launch_fwd_geo(int kc, const CellFwdOperands& o, int nk, int nk_ext, const 
 template <bool HAS_G>
 bool launch_fwd(int kc, const CellFwdOperands& o, int nk, int nk_ext, const bf16* W, const CellArgs& ca, const SweepArgs& sw, cudaStream_t s) {
   const bool pair = cell_pair_enabled(nk * ca.B, ca.H);
+  // 32-unit tiles where 64-unit tiles would use at most half of the SMs
+  const int kt = 128 / ca.B;
+  if (!pair && cell_small_enabled() && ((nk_ext + kt - 1) / kt) * ((ca.H + 63) / 64) <= kSMs / 2)
+    return o.gi_b ? launch_fwd_geo<HAS_G, false, true, true>(kc, o, nk, nk_ext, W, ca, sw, s) : launch_fwd_geo<HAS_G, false, false, true>(kc, o, nk, nk_ext, W, ca, sw, s);
   if (o.gi_b) return pair ? launch_fwd_geo<HAS_G, true, true>(kc, o, nk, nk_ext, W, ca, sw, s) : launch_fwd_geo<HAS_G, false, true>(kc, o, nk, nk_ext, W, ca, sw, s);
   return pair ? launch_fwd_geo<HAS_G, true, false>(kc, o, nk, nk_ext, W, ca, sw, s) : launch_fwd_geo<HAS_G, false, false>(kc, o, nk, nk_ext, W, ca, sw, s);
 }
