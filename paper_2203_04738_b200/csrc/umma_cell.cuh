@@ -278,7 +278,9 @@ umma_cell_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   auto row_tile = [&](int t) { return PAIR ? 2 * (t / n_tiles) + (int)rank : t / n_tiles; };
   // forward: items (step, tile); the linearisation is a single step
   const int n_items = LIN ? tiles : tiles * swp.n_steps;
-  constexpr int kCtrTarget = PAIR ? 16 : 8;       // epilogue warps that finish one item (both CTAs of a pair)
+  // what one item adds to its row tile's counter: its epilogue warps (of both CTAs of a pair); small tiles count once per item,
+  // because many of them share a counter and adds to one address are served one after another
+  constexpr int kCtrTarget = SMALL ? 1 : PAIR ? 16 : 8;
   // the row tiles of step sg - 1 that item (sg, row tile mtile) depends on are complete (true also when there are none)
   auto deps_ready = [&](int sg, int mtile, int code) {
     if (LIN || sg == 0 || swp.st[sg].dep == 0) return true;
@@ -602,13 +604,16 @@ umma_cell_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         if (lane == 0) {
           if (PAIR) mbar_arrive_cluster(mapa_shared(tempty_bar(as), 0));
           else mbar_arrive(tempty_bar(as));
-          // sweep: this warp's rows of the item are written (the warp barrier above ordered every lane's stores before
-          // this lane; the fence makes them visible before the count)
-          if (!LIN && swp.ctr) {
-            __threadfence();
+          // sweep: this warp's rows of the item are written (the warp barrier above ordered every lane's stores before this
+          // lane's release, which makes them visible before the count)
+          if (!LIN && !SMALL && swp.ctr) {
             asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(swp.ctr + sg * m_tiles + t / n_tiles) : "memory");
           }
         }
+      }
+      if (SMALL && swp.ctr) {        // (every epilogue warp comes here, aborting or not)
+        asm volatile("bar.sync 1, 256;" ::: "memory");
+        if (storer && ok) asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(swp.ctr + sg * m_tiles + t / n_tiles) : "memory");
       }
     }
     if (LIN && storer) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");   // coefficients are in global memory before exit
