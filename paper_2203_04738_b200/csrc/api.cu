@@ -1433,7 +1433,7 @@ void plan_lstm_fwd(const mgrit_gru_cfg* c, const Hier& hr, Ws& w, LstmFwdWs* o) 
   if (is_tf32(c)) tf32_plan_fwd(c, hr.N, hr.L, w.base, &w.off, &o->tf, 4);
   if (c->operands == MGRIT_OPERANDS_BF16) lstmbf_plan_fwd(c, o->maxM, w.base, &w.off, &o->bf);
   o->chain_xw = nullptr; o->chain_xw_bytes = 0;
-  if (c->operands == MGRIT_OPERANDS_BF16 && c->H % 128 == 0) {
+  if (c->operands == MGRIT_OPERANDS_BF16) {
     o->chain_xw_bytes = serial_xw_bytes(c->B, c->H, 1);
     o->chain_xw = reinterpret_cast<uint4*>(w.take<char>(o->chain_xw_bytes));
   }
@@ -1465,7 +1465,7 @@ void plan_lstm_adj(const mgrit_gru_cfg* c, const Hier& hr, Ws& w, LstmAdjWs* o) 
   if (is_tf32(c)) tf32_plan_adj(c, hr.N, hr.L, w.base, &w.off, &o->tf, 4);
   if (c->operands == MGRIT_OPERANDS_BF16) lstmbf_plan_adj(c, o->maxM, w.base, &w.off, &o->bf);
   o->chain_xw = nullptr; o->chain_xw_bytes = 0;
-  if (c->operands == MGRIT_OPERANDS_BF16 && c->H % 128 == 0) {
+  if (c->operands == MGRIT_OPERANDS_BF16) {
     o->chain_xw_bytes = serial_xw_bytes(c->B, c->H, 4);
     o->chain_xw = reinterpret_cast<uint4*>(w.take<char>(o->chain_xw_bytes));
   }

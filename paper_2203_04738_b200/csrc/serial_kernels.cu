@@ -9,6 +9,8 @@
 // status leaves at its next barrier, so the launch always terminates.
 #include <stdlib.h>
 
+#include <type_traits>
+
 #include "cell.cuh"
 #include "serial_engine.cuh"
 
@@ -101,13 +103,13 @@ __device__ __forceinline__ void publish_block(const bf16* stage, int nvals, uint
     st_word(dst + w, v);
   }
 }
-// All producers' blocks of step `step` -> the CTA's operand rows in shared memory.  A block holds GATES x 16 x UNC
-// values in the order [gate][row][unit]; value (g, r, i) of producer x goes to As[r][g*H + x*UNC + i].
+// All producers' blocks of step `step` -> the CTA's operand rows in shared memory.  A block holds GATES x RL x UNC
+// values (RL: the rows that travel) in the order [gate][row][unit]; value (g, r, i) of producer x goes to As[r][g*H + x*UNC + i].
 // Every round a thread issues the loads of all its words that are still missing together and then looks at what
 // came back, so a round costs one trip to L2 however many words are outstanding.
-template <int UNC, int GATES>
+template <int UNC, int GATES, int RL = kRows>
 __device__ __forceinline__ bool gather_blocks(const uint4* src, int nprod, unsigned step, bf16* As, int ldk, int H, int* status) {
-  constexpr int kBlockVals = GATES * kRows * UNC, kBlockWords = (kBlockVals + kValsPerWord - 1) / kValsPerWord;
+  constexpr int kBlockVals = GATES * RL * UNC, kBlockWords = (kBlockVals + kValsPerWord - 1) / kValsPerWord;
   constexpr int kBatch = GATES == 1 ? 12 : 16;
   const int total = nprod * kBlockWords;
   for (int base = threadIdx.x; base < total; base += kThreads * kBatch) {
@@ -132,7 +134,7 @@ __device__ __forceinline__ bool gather_blocks(const uint4* src, int nprod, unsig
           for (int t = 0; t < 3; ++t) {
             const int vv = kValsPerWord * w + 2 * t;
             if (vv < kBlockVals) {
-              const int g = vv / (kRows * UNC), r = (vv / UNC) % kRows, i = vv % UNC;
+              const int g = vv / (RL * UNC), r = (vv / UNC) % RL, i = vv % UNC;
               *reinterpret_cast<uint32_t*>(As + r * ldk + g * H + x * UNC + i) = d[t];
             }
           }
@@ -245,10 +247,10 @@ __device__ __forceinline__ float use_gi(const SerialFwdArgs& a, float raw) {
 // ------------------------------------------------------------------------------------------------
 // forward chain:  u_j = Phi_gamma(gi_j, u_{j-1}) + g_j ,  j = 1..nsteps
 // KS > 0: the weight fragments live in registers (KS = k-steps of 16 per warp = H / 128; see warp_gemm_regs).
-template <int UNC, bool LL, int KS = 0>
+template <int UNC, bool LL, int RL, int KS = 0>
 __global__ void __launch_bounds__(kThreads, 1) serial_fwd_kernel(SerialFwdArgs a, int* status) {
-  constexpr int NW = 3 * UNC, NT = NW / 8, OPT = (kRows * UNC + kThreads - 1) / kThreads;
-  constexpr int kBlockVals = kRows * UNC, kBlockWords = (kBlockVals + kValsPerWord - 1) / kValsPerWord;
+  constexpr int NW = 3 * UNC, NT = NW / 8, OPT = (RL * UNC + kThreads - 1) / kThreads;
+  constexpr int kBlockVals = RL * UNC, kBlockWords = (kBlockVals + kValsPerWord - 1) / kValsPerWord;
   __shared__ __align__(16) bf16 xstage[kRows * 32];
   extern __shared__ __align__(16) uint8_t smem[];
   const int H = a.H, ldk = H + 8;
@@ -287,7 +289,7 @@ __global__ void __launch_bounds__(kThreads, 1) serial_fwd_kernel(SerialFwdArgs a
 #pragma unroll
   for (int o = 0; o < OPT; ++o) {
     int idx = tid + o * kThreads, r = idx / UNC, i = idx % UNC;
-    bool v = idx < kRows * UNC && r < nrows;
+    bool v = idx < RL * UNC && r < nrows;
     hp[o] = v ? __ldcg(a.u + (i64)(row0 + r) * H + u0 + i) : 0.f;
     br[o] = a.b_hh[u0 + i]; bz[o] = a.b_hh[H + u0 + i]; bn[o] = a.b_hh[2 * H + u0 + i];
     const i64 go = (i64)(row0 + r) * 3 * H + u0 + i;
@@ -312,7 +314,7 @@ __global__ void __launch_bounds__(kThreads, 1) serial_fwd_kernel(SerialFwdArgs a
     for (int o = 0; o < OPT; ++o) {
       int idx = tid + o * kThreads, r = idx / UNC, i = idx % UNC;
       float val = 0.f;
-      if (idx < kRows * UNC && r < nrows) {
+      if (idx < RL * UNC && r < nrows) {
         float ghr = sum_partials<NW>(red, r, i) + br[o];
         float ghz = sum_partials<NW>(red, r, UNC + i) + bz[o];
         float ghn = sum_partials<NW>(red, r, 2 * UNC + i) + bn[o];
@@ -323,7 +325,7 @@ __global__ void __launch_bounds__(kThreads, 1) serial_fwd_kernel(SerialFwdArgs a
         a.u[(i64)j * BH + off] = val;
         if (!LL) ub[off] = __float2bfloat16(val);
       }
-      if (LL && idx < kRows * UNC) xstage[idx] = __float2bfloat16(val);      // rows beyond the batch travel as zeros
+      if (LL && idx < RL * UNC) xstage[idx] = __float2bfloat16(val);      // rows beyond the batch travel as zeros
     }
     if (j == a.nsteps) break;
     if (LL) {
@@ -334,7 +336,7 @@ __global__ void __launch_bounds__(kThreads, 1) serial_fwd_kernel(SerialFwdArgs a
 #pragma unroll
     for (int o = 0; o < OPT; ++o) {
       int idx = tid + o * kThreads, r = idx / UNC, i = idx % UNC;
-      if (idx < kRows * UNC && r < nrows) {
+      if (idx < RL * UNC && r < nrows) {
         const i64 go = (i64)j * a.gi_step + (i64)(row0 + r) * 3 * H + u0 + i;
         // (loaded now, rounded where they are used: an instruction that depends on these loads here would wait for them
         // in front of the exchange)
@@ -344,7 +346,7 @@ __global__ void __launch_bounds__(kThreads, 1) serial_fwd_kernel(SerialFwdArgs a
     }
     if (LL) {
       // the full new state of this row group, as the bf16 A operand: every producer's words, polled in place
-      const bool ok = gather_blocks<UNC, 1>(a.xw + (i64)(rg * 2 + (j & 1)) * gridDim.x * kBlockWords, (int)gridDim.x, (unsigned)j, As, ldk,
+      const bool ok = gather_blocks<UNC, 1, RL>(a.xw + (i64)(rg * 2 + (j & 1)) * gridDim.x * kBlockWords, (int)gridDim.x, (unsigned)j, As, ldk,
                                             H, status);
       if (!ok) ok_smem = 0;
       __syncthreads();
@@ -365,10 +367,10 @@ __global__ void __launch_bounds__(kThreads, 1) serial_fwd_kernel(SerialFwdArgs a
 // ------------------------------------------------------------------------------------------------
 // adjoint chain:  mu_s = a_s * mu_{s-1} + [cr_s|cz_s|cn_s]*mu_{s-1} W_hh + g_s ,  s = 1..nsteps
 // The bf16 operand copy carries dA_{s+1} = [cr|cz|cn]_{s+1} * mu_s, formed by the CTA that produced mu_s.
-template <int UNC, bool LL, int KS = 0>     // KS > 0: weight fragments in registers, KS = 3H / 128
+template <int UNC, bool LL, int RL, int KS = 0>     // KS > 0: weight fragments in registers, KS = 3H / 128
 __global__ void __launch_bounds__(kThreads, 1) serial_adj_kernel(SerialAdjArgs a, int* status) {
-  constexpr int NT = UNC / 8, OPT = (kRows * UNC + kThreads - 1) / kThreads;
-  constexpr int kBlockVals = 3 * kRows * UNC, kBlockWords = (kBlockVals + kValsPerWord - 1) / kValsPerWord;
+  constexpr int NT = UNC / 8, OPT = (RL * UNC + kThreads - 1) / kThreads;
+  constexpr int kBlockVals = 3 * RL * UNC, kBlockWords = (kBlockVals + kValsPerWord - 1) / kValsPerWord;
   __shared__ __align__(16) bf16 xstage[3 * kRows * 32];
   extern __shared__ __align__(16) uint8_t smem[];
   const int H = a.H, K = 3 * H, ldk = K + 8;
@@ -403,7 +405,7 @@ __global__ void __launch_bounds__(kThreads, 1) serial_adj_kernel(SerialAdjArgs a
 #pragma unroll
   for (int o = 0; o < OPT; ++o) {
     int idx = tid + o * kThreads, r = idx / UNC, i = idx % UNC;
-    bool v = idx < kRows * UNC && r < nrows;
+    bool v = idx < RL * UNC && r < nrows;
     i64 off = (i64)(row0 + r) * H + u0 + i;
     mp[o] = v ? __ldcg(a.mu + off) : 0.f;
     pa[o] = v ? a.a[off] : 0.f;
@@ -432,7 +434,7 @@ __global__ void __launch_bounds__(kThreads, 1) serial_adj_kernel(SerialAdjArgs a
     for (int o = 0; o < OPT; ++o) {
       int idx = tid + o * kThreads, r = idx / UNC, i = idx % UNC;
       float val = 0.f;
-      const bool live = idx < kRows * UNC && r < nrows;
+      const bool live = idx < RL * UNC && r < nrows;
       if (live) {
         val = pa[o] * mp[o] + sum_partials<UNC>(red, r, i) + pg[o];
         mp[o] = val;
@@ -445,10 +447,10 @@ __global__ void __launch_bounds__(kThreads, 1) serial_adj_kernel(SerialAdjArgs a
           d[2 * H] = __float2bfloat16(__bfloat162float(ncn[o]) * val);
         }
       }
-      if (LL && idx < kRows * UNC) {     // block order [gate][row][unit]; rows beyond the batch travel as zeros
+      if (LL && idx < RL * UNC) {     // block order [gate][row][unit]; rows beyond the batch travel as zeros
         xstage[idx] = __float2bfloat16(live ? __bfloat162float(ncr[o]) * val : 0.f);
-        xstage[kRows * UNC + idx] = __float2bfloat16(live ? __bfloat162float(ncz[o]) * val : 0.f);
-        xstage[2 * kRows * UNC + idx] = __float2bfloat16(live ? __bfloat162float(ncn[o]) * val : 0.f);
+        xstage[RL * UNC + idx] = __float2bfloat16(live ? __bfloat162float(ncz[o]) * val : 0.f);
+        xstage[2 * RL * UNC + idx] = __float2bfloat16(live ? __bfloat162float(ncn[o]) * val : 0.f);
       }
     }
     if (s == a.nsteps) break;
@@ -459,7 +461,7 @@ __global__ void __launch_bounds__(kThreads, 1) serial_adj_kernel(SerialAdjArgs a
 #pragma unroll
     for (int o = 0; o < OPT; ++o) {
       int idx = tid + o * kThreads, r = idx / UNC, i = idx % UNC;
-      if (idx < kRows * UNC && r < nrows) {
+      if (idx < RL * UNC && r < nrows) {
         i64 off = (i64)(row0 + r) * H + u0 + i;
         pa[o] = a.a[(i64)s * a.coef_step + off];
         if (a.g) pg[o] = a.g[(i64)(s + 1) * BH + off];
@@ -470,7 +472,7 @@ __global__ void __launch_bounds__(kThreads, 1) serial_adj_kernel(SerialAdjArgs a
       }
     }
     if (LL) {
-      const bool ok = gather_blocks<UNC, 3>(a.xw + (i64)(rg * 2 + (s & 1)) * gridDim.x * kBlockWords, (int)gridDim.x, (unsigned)s, As, ldk,
+      const bool ok = gather_blocks<UNC, 3, RL>(a.xw + (i64)(rg * 2 + (s & 1)) * gridDim.x * kBlockWords, (int)gridDim.x, (unsigned)s, As, ldk,
                                             H, status);
       if (!ok) ok_smem = 0;
       __syncthreads();
@@ -492,10 +494,10 @@ __global__ void __launch_bounds__(kThreads, 1) serial_adj_kernel(SerialAdjArgs a
 // time point's state is (c, h): the cell state never leaves the thread that owns its (row, unit), only h crosses CTAs.
 //
 // forward:  gates from gi_j and h_{j-1} W_hh^T (four gate rows per unit in shared memory), (c, h)_j = cell + g_j
-template <int UNC>
+template <int UNC, int RL>
 __global__ void __launch_bounds__(kThreads, 1) lstm_fwd_chain_kernel(LstmChainFwdArgs a, int* status) {
-  constexpr int NW = 4 * UNC, NT = NW / 8, OPT = (kRows * UNC + kThreads - 1) / kThreads;
-  constexpr int kBlockVals = kRows * UNC, kBlockWords = (kBlockVals + kValsPerWord - 1) / kValsPerWord;
+  constexpr int NW = 4 * UNC, NT = NW / 8, OPT = (RL * UNC + kThreads - 1) / kThreads;
+  constexpr int kBlockVals = RL * UNC, kBlockWords = (kBlockVals + kValsPerWord - 1) / kValsPerWord;
   __shared__ __align__(16) bf16 xstage[kRows * 32];
   extern __shared__ __align__(16) uint8_t smem[];
   const int H = a.H, ldk = H + 8;
@@ -528,7 +530,7 @@ __global__ void __launch_bounds__(kThreads, 1) lstm_fwd_chain_kernel(LstmChainFw
 #pragma unroll
   for (int o = 0; o < OPT; ++o) {
     int idx = tid + o * kThreads, r = idx / UNC, i = idx % UNC;
-    bool v = idx < kRows * UNC && r < nrows;
+    bool v = idx < RL * UNC && r < nrows;
     const i64 off = (i64)(row0 + r) * H + u0 + i;
     cp[o] = v ? __ldcg(a.u + off) : 0.f;
 #pragma unroll
@@ -552,7 +554,7 @@ __global__ void __launch_bounds__(kThreads, 1) lstm_fwd_chain_kernel(LstmChainFw
     for (int o = 0; o < OPT; ++o) {
       int idx = tid + o * kThreads, r = idx / UNC, i = idx % UNC;
       float hv = 0.f;
-      if (idx < kRows * UNC && r < nrows) {
+      if (idx < RL * UNC && r < nrows) {
         float gh[4];
 #pragma unroll
         for (int g = 0; g < 4; ++g) gh[g] = sum_partials<NW>(red, r, g * UNC + i) + bia[o][g];
@@ -564,7 +566,7 @@ __global__ void __launch_bounds__(kThreads, 1) lstm_fwd_chain_kernel(LstmChainFw
         a.u[(i64)j * slot + off] = cv;
         a.u[(i64)j * slot + BH + off] = hv;
       }
-      if (idx < kRows * UNC) xstage[idx] = __float2bfloat16(hv);      // rows beyond the batch travel as zeros
+      if (idx < RL * UNC) xstage[idx] = __float2bfloat16(hv);      // rows beyond the batch travel as zeros
     }
     if (j == a.nsteps) break;
     __syncthreads();
@@ -573,7 +575,7 @@ __global__ void __launch_bounds__(kThreads, 1) lstm_fwd_chain_kernel(LstmChainFw
 #pragma unroll
     for (int o = 0; o < OPT; ++o) {
       int idx = tid + o * kThreads, r = idx / UNC, i = idx % UNC;
-      if (idx < kRows * UNC && r < nrows) {
+      if (idx < RL * UNC && r < nrows) {
         const float* gi = a.gi + (i64)j * a.gi_step + (i64)(row0 + r) * 4 * H + u0 + i;
 #pragma unroll
         for (int g = 0; g < 4; ++g) pgi[o][g] = gi[g * H];
@@ -583,7 +585,7 @@ __global__ void __launch_bounds__(kThreads, 1) lstm_fwd_chain_kernel(LstmChainFw
         }
       }
     }
-    const bool ok = gather_blocks<UNC, 1>(a.xw + (i64)(rg * 2 + (j & 1)) * gridDim.x * kBlockWords, (int)gridDim.x, (unsigned)j, As, ldk, H,
+    const bool ok = gather_blocks<UNC, 1, RL>(a.xw + (i64)(rg * 2 + (j & 1)) * gridDim.x * kBlockWords, (int)gridDim.x, (unsigned)j, As, ldk, H,
                                           status);
     if (!ok) ok_smem = 0;
     __syncthreads();
@@ -596,10 +598,10 @@ __global__ void __launch_bounds__(kThreads, 1) lstm_fwd_chain_kernel(LstmChainFw
 // for the whole chain: warp w reduces k in [w*K/8, (w+1)*K/8) and a lane keeps exactly the B fragments of its
 // m16n8k16 products there (KS k-steps x UNC/8 column tiles x 2 words; 128 registers at H = 1024, UNC = 16).
 // The bf16 operand [ci*dc | cf*dc | cg*dc | co*Lh] of the NEXT step is formed by the CTA that produced (Lc, Lh).
-template <int UNC, int KS>
+template <int UNC, int RL, int KS>
 __global__ void __launch_bounds__(kThreads, 1) lstm_adj_chain_kernel(LstmChainAdjArgs a, int* status) {
-  constexpr int NT = UNC / 8, OPT = (kRows * UNC + kThreads - 1) / kThreads;
-  constexpr int kBlockVals = 4 * kRows * UNC, kBlockWords = (kBlockVals + kValsPerWord - 1) / kValsPerWord;
+  constexpr int NT = UNC / 8, OPT = (RL * UNC + kThreads - 1) / kThreads;
+  constexpr int kBlockVals = 4 * RL * UNC, kBlockWords = (kBlockVals + kValsPerWord - 1) / kValsPerWord;
   __shared__ __align__(16) bf16 xstage[4 * kRows * 16];
   extern __shared__ __align__(16) uint8_t smem[];
   const int H = a.H, K = 4 * H, ldk = K + 8;
@@ -643,7 +645,7 @@ __global__ void __launch_bounds__(kThreads, 1) lstm_adj_chain_kernel(LstmChainAd
 #pragma unroll
   for (int o = 0; o < OPT; ++o) {
     int idx = tid + o * kThreads, r = idx / UNC, i = idx % UNC;
-    bool v = idx < kRows * UNC && r < nrows;
+    bool v = idx < RL * UNC && r < nrows;
     const i64 off = (i64)(row0 + r) * H + u0 + i;
     dcur[o] = v ? __ldcg(a.mu + off) + a.p[off] * __ldcg(a.mu + BH + off) : 0.f;
     pa[o] = v ? a.a[off] : 0.f;
@@ -676,7 +678,7 @@ __global__ void __launch_bounds__(kThreads, 1) lstm_adj_chain_kernel(LstmChainAd
 #pragma unroll
     for (int o = 0; o < OPT; ++o) {
       int idx = tid + o * kThreads, r = idx / UNC, i = idx % UNC;
-      const bool live = idx < kRows * UNC && r < nrows;
+      const bool live = idx < RL * UNC && r < nrows;
       float x4[4] = {0.f, 0.f, 0.f, 0.f};
       if (live) {
         const float lc = pa[o] * dcur[o] + pgc[o];
@@ -689,9 +691,9 @@ __global__ void __launch_bounds__(kThreads, 1) lstm_adj_chain_kernel(LstmChainAd
         x4[0] = __bfloat162float(nci[o]) * dn; x4[1] = __bfloat162float(ncf[o]) * dn; x4[2] = __bfloat162float(ncg[o]) * dn;
         x4[3] = __bfloat162float(nco[o]) * lh;
       }
-      if (idx < kRows * UNC) {                  // block order [gate][row][unit]; rows beyond the batch travel as zeros
+      if (idx < RL * UNC) {                  // block order [gate][row][unit]; rows beyond the batch travel as zeros
 #pragma unroll
-        for (int g = 0; g < 4; ++g) xstage[g * kRows * UNC + idx] = __float2bfloat16(x4[g]);
+        for (int g = 0; g < 4; ++g) xstage[g * RL * UNC + idx] = __float2bfloat16(x4[g]);
       }
     }
     if (s == a.nsteps) break;
@@ -700,7 +702,7 @@ __global__ void __launch_bounds__(kThreads, 1) lstm_adj_chain_kernel(LstmChainAd
 #pragma unroll
     for (int o = 0; o < OPT; ++o) {             // operands of the steps to come that do not depend on other CTAs
       int idx = tid + o * kThreads, r = idx / UNC, i = idx % UNC;
-      if (idx < kRows * UNC && r < nrows) {
+      if (idx < RL * UNC && r < nrows) {
         const i64 off = (i64)(row0 + r) * H + u0 + i;
         pa[o] = a.a[(i64)s * a.coef_step + off];
         if (a.g) { pgc[o] = a.g[(i64)(s + 1) * slot + off]; pgh[o] = a.g[(i64)(s + 1) * slot + BH + off]; }
@@ -712,11 +714,181 @@ __global__ void __launch_bounds__(kThreads, 1) lstm_adj_chain_kernel(LstmChainAd
         }
       }
     }
-    const bool ok = gather_blocks<UNC, 4>(a.xw + (i64)(rg * 2 + (s & 1)) * gridDim.x * kBlockWords, (int)gridDim.x, (unsigned)s, As, ldk, H,
+    const bool ok = gather_blocks<UNC, 4, RL>(a.xw + (i64)(rg * 2 + (s & 1)) * gridDim.x * kBlockWords, (int)gridDim.x, (unsigned)s, As, ldk, H,
                                           status);
     if (!ok) ok_smem = 0;
     __syncthreads();
     if (ok_smem == 0) return;
+  }
+}
+
+// ================================================================================================
+// Adjoint chains with the reduction split by gate (GRU: NG = 3, LSTM: NG = 4; bf16 operands, flag-in-data exchange).
+// In the kernels above a CTA reduces over all NG gate blocks of the operand, so every CTA polls NG x 16 x H values per step: at
+// H = 1024, two row groups and 64 CTAs each that is 17 MB of L2 reads per round and what bounds the step.  Here the NG CTAs of a
+// cluster share NG x UF output units: CTA g reduces over gate block g alone (a third or a quarter of the polling), partial sums
+// change hands through distributed shared memory, and CTA g finishes units [g UF, (g + 1) UF) of the cluster's.
+// A CTA whose wait ran out goes on without waiting until the last step: its peers may still write into its shared memory.
+__device__ __forceinline__ void cluster_barrier() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+template <int NG> struct AdjChainArgs;
+template <> struct AdjChainArgs<3> { typedef SerialAdjArgs type; };
+template <> struct AdjChainArgs<4> { typedef LstmChainAdjArgs type; };
+
+template <int NG, int UF, int RL, int KS = 0>      // KS > 0: weight fragments in registers, KS = H / 128
+__global__ void __launch_bounds__(kThreads, 1) adj_split_chain_kernel(typename AdjChainArgs<NG>::type a, int* status) {
+  constexpr int U = NG * UF, NT = U / 8, OPT = (RL * UF + kThreads - 1) / kThreads;
+  constexpr int kBlockVals = RL * UF, kBlockWords = (kBlockVals + kValsPerWord - 1) / kValsPerWord;
+  constexpr bool LSTM = NG == 4;
+  __shared__ __align__(16) bf16 xstage[NG][(kBlockVals + 7) / 8 * 8];
+  __shared__ float pb[2][NG][RL * UF];                      // partial sums of this CTA's units by gate
+  extern __shared__ __align__(16) uint8_t smem[];
+  const int H = a.H, ldk = H + 8;
+  bf16* Ws = reinterpret_cast<bf16*>(smem);                 // [U][ldk]: W_hh^T rows of the cluster's units, gate block g
+  bf16* As = Ws + U * ldk;                                  // [16][ldk]
+  float* red = reinterpret_cast<float*>(As + kRows * ldk);  // [8][16][U]
+  __shared__ int ok_smem;
+  const int tid = threadIdx.x, warp = tid >> 5;
+  const int g = blockIdx.x % NG, c0 = (blockIdx.x / NG) * U, u0 = c0 + g * UF, rg = blockIdx.y, row0 = rg * kRows;
+  const int nrows = min(kRows, a.B - row0), nprod = gridDim.x;
+  const i64 BH = (i64)a.B * H, slot = (LSTM ? 2 : 1) * BH;
+
+  for (int e = tid; e < U * (H / 8); e += kThreads) {
+    const int r = e / (H / 8), c = e % (H / 8);
+    uint4 v = make_uint4(0, 0, 0, 0);
+    if (c0 + r < H) v = __ldg(reinterpret_cast<const uint4*>(a.WT + (i64)(c0 + r) * NG * H + g * H + c * 8));
+    *reinterpret_cast<uint4*>(Ws + r * ldk + c * 8) = v;
+  }
+  for (int e = tid; e < kRows * ldk / 2; e += kThreads) reinterpret_cast<uint32_t*>(As)[e] = 0u;
+  if (tid == 0) ok_smem = 1;
+  __syncthreads();
+  // step 1: gate block g of the operand from the given sensitivities
+  const bf16* cg;
+  if constexpr (LSTM) cg = g == 0 ? a.ci : g == 1 ? a.cf : g == 2 ? a.cg : a.co;
+  else cg = g == 0 ? a.cr : g == 1 ? a.cz : a.cn;
+  for (int e = tid; e < nrows * H; e += kThreads) {
+    const int r = e / H, i = e % H;
+    const i64 off = (i64)(row0 + r) * H + i;
+    float m = __ldcg(a.mu + off);
+    if constexpr (LSTM) { const float lh = __ldcg(a.mu + BH + off); m = g == 3 ? lh : m + a.p[off] * lh; }
+    As[r * ldk + i] = __float2bfloat16(__bfloat162float(cg[off]) * m);
+  }
+  // per owned (row, unit): mu (LSTM: dc) of the step in flight, its a and source terms; the coefficients of the step after it, kept
+  // raw until they are used (a conversion behind the load would wait for it in front of the exchange)
+  float mp[OPT], pa[OPT], pg[OPT], pgh[OPT], np_[OPT];
+  bf16 nc[OPT][NG];
+  auto live_of = [&](int o, int* r, int* i) {
+    const int idx = tid + o * kThreads;
+    *r = idx / UF; *i = idx % UF;
+    return idx < RL * UF && *r < nrows && u0 + *i < H;
+  };
+  auto load_coefs = [&](int o, i64 at, bool more) {
+#pragma unroll
+    for (int q = 0; q < NG; ++q) nc[o][q] = __float2bfloat16(0.f);
+    np_[o] = 0.f;
+    if (!more) return;
+    if constexpr (LSTM) { np_[o] = a.p[at]; nc[o][0] = a.ci[at]; nc[o][1] = a.cf[at]; nc[o][2] = a.cg[at]; nc[o][3] = a.co[at]; }
+    else { nc[o][0] = a.cr[at]; nc[o][1] = a.cz[at]; nc[o][2] = a.cn[at]; }
+  };
+#pragma unroll
+  for (int o = 0; o < OPT; ++o) {
+    int r, i;
+    const bool v = live_of(o, &r, &i);
+    const i64 off = (i64)(row0 + r) * H + u0 + i;
+    mp[o] = v ? __ldcg(a.mu + off) : 0.f;
+    if constexpr (LSTM) { if (v) mp[o] += a.p[off] * __ldcg(a.mu + BH + off); }
+    pa[o] = v ? a.a[off] : 0.f;
+    pg[o] = v && a.g ? a.g[slot + off] : 0.f;
+    pgh[o] = LSTM && v && a.g ? a.g[slot + BH + off] : 0.f;
+    load_coefs(o, a.coef_step + off, v && a.nsteps > 1);
+  }
+  __syncthreads();
+  cluster_barrier();       // every CTA of the cluster runs before anything is written into its shared memory
+
+  uint32_t wreg[KS > 0 ? KS : 1][NT][2];
+  if (KS > 0) load_wregs<NT, (KS > 0 ? KS : 1)>(Ws, ldk, warp * (H / kWarps), wreg);
+  bool waits = true;
+  for (int s = 1; s <= a.nsteps; ++s) {
+    float acc[NT][4];
+#pragma unroll
+    for (int nt = 0; nt < NT; ++nt) acc[nt][0] = acc[nt][1] = acc[nt][2] = acc[nt][3] = 0.f;
+    if (KS > 0) warp_gemm_regs<NT, (KS > 0 ? KS : 1)>(As, ldk, warp * (H / kWarps), wreg, acc);
+    else warp_gemm<NT>(As, Ws, ldk, warp_k(H, warp), warp_k(H, warp + 1), acc);
+    store_partials<NT>(red, acc);
+    __syncthreads();
+#pragma unroll
+    for (int e = tid; e < RL * U; e += kThreads) {          // this gate's sums to the units' owners
+      const int r = e / U, col = e % U, owner = col / UF;
+      const float v = sum_partials<U>(red, r, col);
+      const uint32_t mine = (uint32_t)__cvta_generic_to_shared(&pb[s & 1][g][r * UF + col % UF]);
+      uint32_t dst;
+      asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(dst) : "r"(mine), "r"(owner));
+      asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(dst), "f"(v) : "memory");
+    }
+    cluster_barrier();
+#pragma unroll
+    for (int o = 0; o < OPT; ++o) {
+      int r, i;
+      const bool live = live_of(o, &r, &i);
+      const int idx = tid + o * kThreads;
+      float x[NG] = {};
+      if (live) {
+        float sum = 0.f;
+#pragma unroll
+        for (int q = 0; q < NG; ++q) sum += pb[s & 1][q][idx];
+        const i64 off = (i64)s * slot + (i64)(row0 + r) * H + u0 + i;
+        if constexpr (LSTM) {
+          const float lc = pa[o] * mp[o] + pg[o], lh = sum + pgh[o], dn = lc + np_[o] * lh;
+          a.mu[off] = lc;
+          a.mu[off + BH] = lh;
+          mp[o] = dn;      // the next step's dc (its coefficients are zero behind the last step)
+#pragma unroll
+          for (int q = 0; q < NG; ++q) x[q] = __bfloat162float(nc[o][q]) * (q == 3 ? lh : dn);
+        } else {
+          const float val = pa[o] * mp[o] + sum + pg[o];
+          a.mu[off] = val;
+          mp[o] = val;
+#pragma unroll
+          for (int q = 0; q < NG; ++q) x[q] = __bfloat162float(nc[o][q]) * val;
+        }
+      }
+      if (idx < RL * UF) {                                  // rows beyond the batch travel as zeros
+#pragma unroll
+        for (int q = 0; q < NG; ++q) xstage[q][idx] = __float2bfloat16(x[q]);
+      }
+    }
+    if (s == a.nsteps) break;
+    __syncthreads();
+    const i64 xbase = (i64)(rg * 2 + (s & 1)) * NG * nprod * kBlockWords;
+    if (u0 < H) {
+      for (int w = tid; w < NG * kBlockWords; w += kThreads) {
+        const int q = w / kBlockWords, k = w % kBlockWords;
+        const uint32_t* s32 = reinterpret_cast<const uint32_t*>(xstage[q]) + 3 * k;
+        uint4 v;
+        v.x = 6 * k < kBlockVals ? s32[0] : 0u;
+        v.y = 6 * k + 2 < kBlockVals ? s32[1] : 0u;
+        v.z = 6 * k + 4 < kBlockVals ? s32[2] : 0u;
+        v.w = (unsigned)s;
+        st_word(a.xw + xbase + ((i64)q * nprod + blockIdx.x) * kBlockWords + k, v);
+      }
+    }
+#pragma unroll
+    for (int o = 0; o < OPT; ++o) {                         // operands of the steps to come that do not depend on other CTAs
+      int r, i;
+      const bool v = live_of(o, &r, &i);
+      if (!v) continue;
+      const i64 off = (i64)(row0 + r) * H + u0 + i;
+      pa[o] = a.a[(i64)s * a.coef_step + off];
+      if (a.g) {
+        pg[o] = a.g[(i64)(s + 1) * slot + off];
+        if (LSTM) pgh[o] = a.g[(i64)(s + 1) * slot + BH + off];
+      }
+      load_coefs(o, (i64)(s + 1) * a.coef_step + off, s + 1 < a.nsteps);
+    }
+    if (waits && !gather_blocks<UF, 1, RL>(a.xw + xbase + (i64)g * nprod * kBlockWords, H / UF, (unsigned)s, As, ldk, H, status)) ok_smem = 0;
+    __syncthreads();
+    waits = ok_smem != 0;
   }
 }
 
@@ -985,12 +1157,12 @@ bool chain_ll_enabled() {
 }
 
 template <class Args, class Kern>
-bool launch_coop(Kern kern, const Args& a, int unc, size_t smem, bool ll, int gates, cudaStream_t s) {
+bool launch_coop(Kern kern, const Args& a, int unc, int RL, size_t smem, bool ll, int gates, cudaStream_t s) {
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return false;
   int rgs = (a.B + kRows - 1) / kRows;
   if (cudaMemsetAsync(a.bar, 0, sizeof(unsigned) * rgs, s) != cudaSuccess) return false;
   if (ll) {   // no word may carry a step number of an earlier launch
-    const size_t words = (size_t)rgs * 2 * (a.H / unc) * ((size_t)(gates * kRows * unc + kValsPerWord - 1) / kValsPerWord);
+    const size_t words = (size_t)rgs * 2 * (a.H / unc) * ((size_t)(gates * RL * unc + kValsPerWord - 1) / kValsPerWord);
     if (words * sizeof(uint4) > a.xw_bytes) return false;
     if (cudaMemsetAsync(a.xw, 0, words * sizeof(uint4), s) != cudaSuccess) return false;
   }
@@ -1044,7 +1216,8 @@ bool launch_coop32(Kern kern, const Args& a, int unc, size_t smem, cudaStream_t 
 size_t serial_xw_bytes(int B, int H, int gates) {
   // the smallest unit slice (8) has the most words: 2 parities x row groups x (H / 8) producers x ceil(gates*16*8 / 6)
   const size_t rgs = (size_t)(B + kRows - 1) / kRows;
-  return rgs * 2 * (size_t)(H / 8) * (size_t)((gates * kRows * 8 + kValsPerWord - 1) / kValsPerWord) * sizeof(uint4) + 256;
+  // (split by gate: one block per gate, producers rounded up to whole clusters)
+  return rgs * 2 * (size_t)(H / 8 + 8) * (size_t)gates * (size_t)((kRows * 8 + kValsPerWord - 1) / kValsPerWord) * sizeof(uint4) + 256;
 }
 
 bool serial_fwd_supported(int B, int H) { return pick_unc(B, H, false) != 0; }
@@ -1057,52 +1230,127 @@ static bool chain_wreg_enabled() {
   return v == 1;
 }
 
+namespace {
+// Rows that travel between the CTAs of a row group: with few batch rows most of a sixteen-row block would be zeros, and every
+// CTA polls every block (8 rows at H = 1024: forward 2.05 -> 1.88 us a step, adjoint 3.43 -> 2.00).
+template <class F> bool by_rows(int B, F f) {
+  if (B <= 4) return f(std::integral_constant<int, 4>());
+  if (B <= 8) return f(std::integral_constant<int, 8>());
+  return f(std::integral_constant<int, kRows>());
+}
+}  // namespace
+
 bool serial_fwd_solve(const SerialFwdArgs& a, cudaStream_t s) {
-  int unc = pick_unc(a.B, a.H, false);
+  const int unc = pick_unc(a.B, a.H, false);
   if (unc == 0 || a.nsteps <= 0 || !status_ptr()) return false;
-  size_t smem = fwd_smem(unc, a.H);
+  const size_t smem = fwd_smem(unc, a.H);
+  const bool ll = chain_ll_enabled() && a.xw != nullptr, wreg = ll && chain_wreg_enabled();
   prof_begin(KC_FWD_SERIAL, 2.0 * a.B * 3.0 * a.H * a.H * a.nsteps, s);
-  const bool ll = chain_ll_enabled() && a.xw != nullptr;
-  if (ll && chain_wreg_enabled() && (unc == 8 || unc == 16) && (a.H == 512 || a.H == 1024)) {
-    bool okr;
-    if (a.H == 1024) okr = unc == 8 ? launch_coop(serial_fwd_kernel<8, true, 8>, a, unc, smem, true, 1, s)
-                                    : launch_coop(serial_fwd_kernel<16, true, 8>, a, unc, smem, true, 1, s);
-    else okr = unc == 8 ? launch_coop(serial_fwd_kernel<8, true, 4>, a, unc, smem, true, 1, s)
-                        : launch_coop(serial_fwd_kernel<16, true, 4>, a, unc, smem, true, 1, s);
-    prof_end(s);
-    return okr;
+  bool ok;
+  if (!ll) {
+    auto go = [&](auto kern) { return launch_coop(kern, a, unc, kRows, smem, false, 1, s); };
+    ok = unc == 8 ? go(serial_fwd_kernel<8, false, kRows>) : unc == 16 ? go(serial_fwd_kernel<16, false, kRows>) : go(serial_fwd_kernel<32, false, kRows>);
+  } else {
+    ok = by_rows(a.B, [&](auto rl) {
+      constexpr int RL = decltype(rl)::value;
+      auto go = [&](auto kern) { return launch_coop(kern, a, unc, RL, smem, true, 1, s); };
+      if (wreg && a.H == 1024 && unc == 8) return go(serial_fwd_kernel<8, true, RL, 8>);
+      if (wreg && a.H == 1024 && unc == 16) return go(serial_fwd_kernel<16, true, RL, 8>);
+      if (wreg && a.H == 512 && unc == 8) return go(serial_fwd_kernel<8, true, RL, 4>);
+      if (wreg && a.H == 512 && unc == 16) return go(serial_fwd_kernel<16, true, RL, 4>);
+      return unc == 8 ? go(serial_fwd_kernel<8, true, RL>) : unc == 16 ? go(serial_fwd_kernel<16, true, RL>) : go(serial_fwd_kernel<32, true, RL>);
+    });
   }
-  bool ok = ll ? (unc == 8 ? launch_coop(serial_fwd_kernel<8, true>, a, unc, smem, true, 1, s)
-                  : unc == 16 ? launch_coop(serial_fwd_kernel<16, true>, a, unc, smem, true, 1, s)
-                              : launch_coop(serial_fwd_kernel<32, true>, a, unc, smem, true, 1, s))
-               : (unc == 8 ? launch_coop(serial_fwd_kernel<8, false>, a, unc, smem, false, 1, s)
-                  : unc == 16 ? launch_coop(serial_fwd_kernel<16, false>, a, unc, smem, false, 1, s)
-                              : launch_coop(serial_fwd_kernel<32, false>, a, unc, smem, false, 1, s));
   prof_end(s);
   return ok;
 }
 
-bool serial_adj_solve(const SerialAdjArgs& a, cudaStream_t s) {
-  int unc = pick_unc(a.B, a.H, true);
-  if (unc == 0 || a.nsteps <= 0 || !status_ptr()) return false;
-  size_t smem = adj_smem(unc, a.H);
-  prof_begin(KC_ADJ_SERIAL, 2.0 * a.B * 3.0 * a.H * a.H * a.nsteps, s);
-  const bool ll = chain_ll_enabled() && a.xw != nullptr;
-  if (ll && chain_wreg_enabled() && (unc == 8 || unc == 16) && (a.H == 512 || a.H == 1024)) {
-    bool okr;
-    if (a.H == 1024) okr = unc == 8 ? launch_coop(serial_adj_kernel<8, true, 24>, a, unc, smem, true, 3, s)
-                                    : launch_coop(serial_adj_kernel<16, true, 24>, a, unc, smem, true, 3, s);
-    else okr = unc == 8 ? launch_coop(serial_adj_kernel<8, true, 12>, a, unc, smem, true, 3, s)
-                        : launch_coop(serial_adj_kernel<16, true, 12>, a, unc, smem, true, 3, s);
-    prof_end(s);
-    return okr;
+namespace {
+// Units finished per CTA of the gate-split adjoint chain, 0 = not available: H / (NG UF) clusters of NG CTAs per row group, all of
+// them resident, and the widest slice that fits.
+template <int NG> size_t adj_split_smem(int uf, int H) { return (size_t)(NG * uf + kRows) * (H + 8) * 2 + (size_t)kWarps * kRows * NG * uf * 4; }
+template <int NG, int UF, int RL, int KS = 0>
+bool launch_adj_split(const typename AdjChainArgs<NG>::type& a, cudaStream_t s) {
+  auto kern = adj_split_chain_kernel<NG, UF, RL, KS>;
+  const size_t smem = adj_split_smem<NG>(UF, a.H);
+  const int rgs = (a.B + kRows - 1) / kRows, clusters = (a.H + NG * UF - 1) / (NG * UF);
+  static int attr_ok[kMaxDevices] = {0}, resident[kMaxDevices] = {0};
+  const int dev = current_device_slot();
+  if (dev < 0 || smem > kSmemLimit - 8192) return false;
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = NG; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+  at[1].id = cudaLaunchAttributeCooperative;      // CTAs wait for one another: all of them resident
+  at[1].val.cooperative = 1;
+  cfg.blockDim = dim3(kThreads); cfg.attrs = at; cfg.numAttrs = 1;
+  if (!attr_ok[dev]) {
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kSmemLimit - 8192)) != cudaSuccess) { cudaGetLastError(); return false; }
+    cfg.gridDim = dim3(NG); cfg.dynamicSmemBytes = kSmemLimit - 8192;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess) { cudaGetLastError(); n = 0; }
+    resident[dev] = n;
+    attr_ok[dev] = 1;
   }
-  bool ok = ll ? (unc == 8 ? launch_coop(serial_adj_kernel<8, true>, a, unc, smem, true, 3, s)
-                  : unc == 16 ? launch_coop(serial_adj_kernel<16, true>, a, unc, smem, true, 3, s)
-                              : launch_coop(serial_adj_kernel<32, true>, a, unc, smem, true, 3, s))
-               : (unc == 8 ? launch_coop(serial_adj_kernel<8, false>, a, unc, smem, false, 3, s)
-                  : unc == 16 ? launch_coop(serial_adj_kernel<16, false>, a, unc, smem, false, 3, s)
-                              : launch_coop(serial_adj_kernel<32, false>, a, unc, smem, false, 3, s));
+  if (clusters * rgs > resident[dev]) return false;
+  const size_t words = (size_t)rgs * 2 * NG * NG * clusters * ((size_t)(RL * UF + kValsPerWord - 1) / kValsPerWord);
+  if (words * sizeof(uint4) > a.xw_bytes) return false;
+  int* st = status_ptr();
+  if (!st || cudaMemsetAsync(a.xw, 0, words * sizeof(uint4), s) != cudaSuccess) return false;
+  cfg.gridDim = dim3(NG * clusters, rgs); cfg.dynamicSmemBytes = smem; cfg.stream = s; cfg.numAttrs = 2;
+  if (cudaLaunchKernelEx(&cfg, kern, a, st) != cudaSuccess) { cudaGetLastError(); return false; }
+  count_launch();
+  return true;
+}
+template <int NG, int RL>
+bool adj_split_solve(const typename AdjChainArgs<NG>::type& a, bool wreg, cudaStream_t s) {
+  if (wreg && a.H == 1024) return launch_adj_split<NG, 8, RL, 8>(a, s) || launch_adj_split<NG, 16, RL, 8>(a, s);
+  if (wreg && a.H == 512) return launch_adj_split<NG, 8, RL, 4>(a, s) || launch_adj_split<NG, 16, RL, 4>(a, s);
+  return launch_adj_split<NG, 8, RL>(a, s) || launch_adj_split<NG, 16, RL>(a, s);
+}
+// Splitting costs a cluster barrier and the exchange of the sums (about 0.6 us a step) and pays where the unsplit kernel's words
+// of a step exceed one batch of polls (16 per thread): us a step unsplit / split (B200)  H = 1024: B = 32 4.13 / 3.18, B = 8
+// 2.00 / 2.35;  H = 640, B = 16 3.15 / 2.56;  H = 512, B = 32 1.79 / 2.36;  LSTM  H = 1024: B = 32 8.93 / 4.29;  H = 512:
+// B = 32 4.47 / 2.71;  H = 256, B = 64 2.14 / 2.71.  unc: units per CTA of the unsplit kernel, 0 where it does not fit.
+bool split_pays(int gates, int B, int H, int unc) {
+  const int rl = B <= 4 ? 4 : B <= 8 ? 8 : kRows;
+  return unc == 0 || (H / unc) * ((gates * rl * unc + kValsPerWord - 1) / kValsPerWord) > 16 * kThreads;
+}
+// MGRIT_GRU_CHAIN_SPLIT=0 in the environment keeps the adjoint chains unsplit.
+bool chain_split_enabled() {
+  static int v = -1;
+  if (v < 0) { const char* e = getenv("MGRIT_GRU_CHAIN_SPLIT"); v = (e && e[0] == '0') ? 0 : 1; }
+  return v == 1;
+}
+}  // namespace
+
+bool serial_adj_solve(const SerialAdjArgs& a, cudaStream_t s) {
+  if (chain_split_enabled() && chain_ll_enabled() && a.xw && a.H % 64 == 0 && a.nsteps > 0 && split_pays(3, a.B, a.H, pick_unc(a.B, a.H, true))) {
+    prof_begin(KC_ADJ_SERIAL, 2.0 * a.B * 3.0 * a.H * a.H * a.nsteps, s);
+    const bool ok = by_rows(a.B, [&](auto rl) { return adj_split_solve<3, decltype(rl)::value>(a, chain_wreg_enabled(), s); });
+    prof_end(s);
+    if (ok) return true;
+  }
+  const int unc = pick_unc(a.B, a.H, true);
+  if (unc == 0 || a.nsteps <= 0 || !status_ptr()) return false;
+  const size_t smem = adj_smem(unc, a.H);
+  const bool ll = chain_ll_enabled() && a.xw != nullptr, wreg = ll && chain_wreg_enabled();
+  prof_begin(KC_ADJ_SERIAL, 2.0 * a.B * 3.0 * a.H * a.H * a.nsteps, s);
+  bool ok;
+  if (!ll) {
+    auto go = [&](auto kern) { return launch_coop(kern, a, unc, kRows, smem, false, 3, s); };
+    ok = unc == 8 ? go(serial_adj_kernel<8, false, kRows>) : unc == 16 ? go(serial_adj_kernel<16, false, kRows>) : go(serial_adj_kernel<32, false, kRows>);
+  } else {
+    ok = by_rows(a.B, [&](auto rl) {
+      constexpr int RL = decltype(rl)::value;
+      auto go = [&](auto kern) { return launch_coop(kern, a, unc, RL, smem, true, 3, s); };
+      if (wreg && a.H == 1024 && unc == 8) return go(serial_adj_kernel<8, true, RL, 24>);
+      if (wreg && a.H == 1024 && unc == 16) return go(serial_adj_kernel<16, true, RL, 24>);
+      if (wreg && a.H == 512 && unc == 8) return go(serial_adj_kernel<8, true, RL, 12>);
+      if (wreg && a.H == 512 && unc == 16) return go(serial_adj_kernel<16, true, RL, 12>);
+      return unc == 8 ? go(serial_adj_kernel<8, true, RL>) : unc == 16 ? go(serial_adj_kernel<16, true, RL>) : go(serial_adj_kernel<32, true, RL>);
+    });
+  }
   prof_end(s);
   return ok;
 }
@@ -1124,11 +1372,11 @@ int lstm_pick_unc(int B, int H, bool adj) {
   return 0;
 }
 template <class Args, class Kern>
-bool launch_lstm_chain(Kern kern, const Args& a, int unc, size_t smem, int gates, cudaStream_t s) {
+bool launch_lstm_chain(Kern kern, const Args& a, int unc, int RL, size_t smem, int gates, cudaStream_t s) {
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return false;
   const int rgs = (a.B + kRows - 1) / kRows;
   // no exchange word may carry a step number of an earlier launch
-  const size_t words = (size_t)rgs * 2 * (a.H / unc) * ((size_t)(gates * kRows * unc + kValsPerWord - 1) / kValsPerWord);
+  const size_t words = (size_t)rgs * 2 * (a.H / unc) * ((size_t)(gates * RL * unc + kValsPerWord - 1) / kValsPerWord);
   if (words * sizeof(uint4) > a.xw_bytes) return false;
   if (cudaMemsetAsync(a.xw, 0, words * sizeof(uint4), s) != cudaSuccess) return false;
   Args args = a;
@@ -1142,13 +1390,13 @@ bool launch_lstm_chain(Kern kern, const Args& a, int unc, size_t smem, int gates
   count_launch();
   return true;
 }
-template <int UNC>
+template <int UNC, int RL>
 bool launch_lstm_adj(const LstmChainAdjArgs& a, size_t smem, cudaStream_t s) {
   switch (a.H) {
-    case 128: return launch_lstm_chain(lstm_adj_chain_kernel<UNC, 4>, a, UNC, smem, 4, s);
-    case 256: return launch_lstm_chain(lstm_adj_chain_kernel<UNC, 8>, a, UNC, smem, 4, s);
-    case 512: return launch_lstm_chain(lstm_adj_chain_kernel<UNC, 16>, a, UNC, smem, 4, s);
-    case 1024: return launch_lstm_chain(lstm_adj_chain_kernel<UNC, 32>, a, UNC, smem, 4, s);
+    case 128: return launch_lstm_chain(lstm_adj_chain_kernel<UNC, RL, 4>, a, UNC, RL, smem, 4, s);
+    case 256: return launch_lstm_chain(lstm_adj_chain_kernel<UNC, RL, 8>, a, UNC, RL, smem, 4, s);
+    case 512: return launch_lstm_chain(lstm_adj_chain_kernel<UNC, RL, 16>, a, UNC, RL, smem, 4, s);
+    case 1024: return launch_lstm_chain(lstm_adj_chain_kernel<UNC, RL, 32>, a, UNC, RL, smem, 4, s);
     default: return false;
   }
 }
@@ -1159,19 +1407,30 @@ bool lstm_chain_fwd_solve(const LstmChainFwdArgs& a, cudaStream_t s) {
   if (unc == 0 || a.nsteps <= 0 || !a.xw || !status_ptr()) return false;
   const size_t smem = lstm_fwd_smem(unc, a.H);
   prof_begin(KC_FWD_SERIAL, 2.0 * a.B * 4.0 * a.H * a.H * a.nsteps, s);
-  const bool ok = unc == 8    ? launch_lstm_chain(lstm_fwd_chain_kernel<8>, a, unc, smem, 1, s)
-                  : unc == 16 ? launch_lstm_chain(lstm_fwd_chain_kernel<16>, a, unc, smem, 1, s)
-                              : launch_lstm_chain(lstm_fwd_chain_kernel<32>, a, unc, smem, 1, s);
+  const bool ok = by_rows(a.B, [&](auto rl) {
+    constexpr int RL = decltype(rl)::value;
+    auto go = [&](auto kern) { return launch_lstm_chain(kern, a, unc, RL, smem, 1, s); };
+    return unc == 8 ? go(lstm_fwd_chain_kernel<8, RL>) : unc == 16 ? go(lstm_fwd_chain_kernel<16, RL>) : go(lstm_fwd_chain_kernel<32, RL>);
+  });
   prof_end(s);
   return ok;
 }
 
 bool lstm_chain_adj_solve(const LstmChainAdjArgs& a, cudaStream_t s) {
+  if (chain_split_enabled() && chain_ll_enabled() && a.xw && a.H % 64 == 0 && a.nsteps > 0 && split_pays(4, a.B, a.H, lstm_pick_unc(a.B, a.H, true))) {
+    prof_begin(KC_ADJ_SERIAL, 2.0 * a.B * 4.0 * a.H * a.H * a.nsteps, s);
+    const bool ok = by_rows(a.B, [&](auto rl) { return adj_split_solve<4, decltype(rl)::value>(a, chain_wreg_enabled(), s); });
+    prof_end(s);
+    if (ok) return true;
+  }
   const int unc = chain_ll_enabled() ? lstm_pick_unc(a.B, a.H, true) : 0;
   if (unc == 0 || a.nsteps <= 0 || !a.xw || !status_ptr()) return false;
   const size_t smem = lstm_adj_smem(unc, a.H);
   prof_begin(KC_ADJ_SERIAL, 2.0 * a.B * 4.0 * a.H * a.H * a.nsteps, s);
-  const bool ok = unc == 8 ? launch_lstm_adj<8>(a, smem, s) : launch_lstm_adj<16>(a, smem, s);
+  const bool ok = by_rows(a.B, [&](auto rl) {
+    constexpr int RL = decltype(rl)::value;
+    return unc == 8 ? launch_lstm_adj<8, RL>(a, smem, s) : launch_lstm_adj<16, RL>(a, smem, s);
+  });
   prof_end(s);
   return ok;
 }
