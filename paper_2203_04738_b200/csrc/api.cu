@@ -624,10 +624,11 @@ struct F32Cycle {
 };
 
 // Which fp32-state solves run there: every one of the fp32 mode whose weights fit, and those of the tf32 split whose steps are
-// too small for the tensor cores (rows of the largest step x H^2).  At H = 256 a step of 500 rows takes 14.6 us forward and
-// 11.8 us adjoint there, 2000 rows 65 and 39 us; the tensor-core step takes 27 + 6 and 24 + 4 us (product and operand split, one
-// wave of tiles) at 512 rows and hardly more at 2000: they meet at about 1200 rows.  Linearisation of 2560 rows: 51 against 58 us.
-constexpr double kF32TfStep = 8e7, kF32TfLin = 1.7e8;
+// too small for the tensor cores (rows of the largest step x H^2).  Forward and adjoint us a step there: H = 256 500 rows 11.1 and
+// 8.4, 1200 rows 22 and 18, 1700 rows 32 and 26; H = 320 700 rows 23 and 26, 1100 rows 41 and 44.  The tensor-core step takes
+// 27 + 6 and 24 + 4 us (product and operand split, one wave of tiles) at 512 rows and hardly more at 2000.  They meet at
+// 900 (H = 320) to 1700 rows (H = 256); the line is the lower one.  Linearisation at H = 256: 2560 rows 45 against 58 us, 5120 rows 84.
+constexpr double kF32TfStep = 9e7, kF32TfLin = 2.2e8;
 bool use_f32_solve(const mgrit_gru_cfg* c, const Hier& hr) {
   if (!f32_solve_fits(c->H)) return false;
   if (c->operands == MGRIT_OPERANDS_FP32) return true;

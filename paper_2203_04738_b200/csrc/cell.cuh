@@ -21,12 +21,19 @@ __device__ __forceinline__ float rcp_approx(float x) {
   return y;
 }
 
+// 1 / x for 1 <= x < 2^125 by one Newton-Raphson step on the hardware's approximation (relative error 2^-23 before, below 2^-23
+// after it: the step squares the error, what remains is its rounding).  A division of the language brings a branch for the
+// operands it cannot take; four gates side by side have to be branch-free to hide each other's latency.
+__device__ __forceinline__ float rcp_newton(float x) {
+  const float y = rcp_approx(x);
+  return fmaf(fmaf(-x, y, 1.0f), y, y);
+}
 template <bool FAST> __device__ __forceinline__ float sigmoid_t(float x) {
   if (FAST) return fmaf(tanh_approx(0.5f * x), 0.5f, 0.5f);
-  return 1.0f / (1.0f + __expf(-x));
+  return rcp_newton(1.0f + __expf(fminf(-x, 80.0f)));      // (below -80 the result is 1.8e-35 instead of less)
 }
 template <bool FAST> __device__ __forceinline__ float tanh_t(float x) { return FAST ? tanh_approx(x) : tanhf(x); }
-template <bool FAST> __device__ __forceinline__ float inv_t(float x) { return FAST ? rcp_approx(x) : 1.0f / x; }
+template <bool FAST> __device__ __forceinline__ float inv_t(float x) { return FAST ? rcp_approx(x) : rcp_newton(x); }
 
 // Phi_gamma(x_t, h_{t-1}) given the pre-activations: gi_* = W_i* x + b_i*, gh_* = W_h* h + b_h*.
 // classic  (Eq. "gru-classic"): h + gamma(1-z)(n - h)

@@ -18,7 +18,7 @@ enum { kLastNone = 0, kLastStore = 1, kLastCoarse = 2 };
 struct F32Phase {
   int nk, nfull, n, ntail, last_kind, level;
   float gamma, gamma2;
-  int R, KP, nt;                  // rows per block, lanes per sum, threads: set by the launcher
+  int R;                          // rows per block: set by the launcher
   const float* src; i64 src_ks;
   float* copy; i64 copy_ks;
   float* out; i64 out_ks, out_ss;
