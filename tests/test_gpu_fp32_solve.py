@@ -15,7 +15,9 @@ pytestmark = pytest.mark.gpu
 CASES = [(64, 2, 32, 4, 2, 0, 1, 2, False, 0), (37, 1, 8, 2, 3, 1, 0, 2, False, 0), (50, 5, 104, 4, 2, 2, 1, 2, False, 0),
          (48, 100, 104, 4, 3, 0, 1, 1, False, 0), (40, 3, 136, 2, 3, 1, 1, 2, False, 0), (33, 17, 184, 4, 2, 1, 0, 2, False, 0),
          (36, 2, 248, 3, 3, 3, 2, 2, False, 0), (64, 33, 256, 4, 2, 0, 1, 2, False, 1), (30, 4, 320, 2, 2, 1, 1, 2, False, 1),
-         (96, 2, 64, 2, 5, 1, 1, 4, True, 0), (29, 6, 352, 2, 1, 0, 0, 1, False, 0), (128, 16, 64, 4, 3, 1, 1, 2, False, 1)]
+         (96, 2, 64, 2, 5, 1, 1, 4, True, 0), (29, 6, 352, 2, 1, 0, 0, 1, False, 0), (128, 16, 64, 4, 3, 1, 1, 2, False, 1),
+         (26, 21, 96, 4, 2, 1, 1, 1, False, 0), (24, 40, 128, 2, 2, 1, 1, 1, False, 0), (24, 65, 168, 2, 2, 1, 1, 1, False, 0),
+         (20, 70, 216, 2, 2, 0, 1, 1, False, 0)]
 
 
 @pytest.mark.parametrize("c", CASES, ids=lambda c: "T{}B{}H{}cf{}L{}r{}{}i{}{}o{}".format(*c[:8], "F" if c[8] else "V", c[9]))
@@ -58,3 +60,19 @@ def test_solve_against_the_oracle(c):
         for k in ("dx", "dW_ih", "dW_hh", "db_ih", "db_hh"):
             assert norm(getattr(r, k).cpu().numpy(), g[k]) < (6e-5 if op else 1e-5), k
     assert Bd.last_device_status() == 0
+
+
+@pytest.mark.parametrize("H", [8, 112, 160])
+def test_gates_at_the_ends_of_their_range(H):
+    """Pre-activations from -120 to 120, where e^-x leaves the range of fp32: against the oracle in double precision."""
+    from paper_2203_04738_b200 import binding as Bd
+    T, B, rng = 3, 9, np.random.default_rng(H)
+    W_ih, W_hh = rng.standard_normal((3 * H, 8)).astype(np.float32), (rng.standard_normal((3 * H, H)) * H ** -0.5).astype(np.float32)
+    b_ih, b_hh = rng.permutation(np.linspace(-120, 120, 3 * H)).astype(np.float32), np.zeros(3 * H, np.float32)
+    x, h0 = rng.standard_normal((T, B, 8)).astype(np.float32), np.zeros((B, H), np.float32)
+    p = {k: to_dev(v) for k, v in dict(W_ih=W_ih, W_hh=W_hh, b_ih=b_ih, b_hh=b_hh).items()}
+    h, _ = Bd.gru_serial_forward(Bd.make_cfg(T, B, 8, H, operands=0, levels=1), p, to_dev(x), to_dev(h0))
+    ref = O.serial_forward(*(v.astype(np.float64) for v in (W_ih, W_hh, b_ih, b_hh, x, h0)))
+    # a pre-activation a is rounded to 2^-24 |a|, at most 2^-17 for |a| < 128, and moves its gate by that times e^-|a| / (1 + e^-|a|)^2
+    # or 1 - n^2, that is by at most 2^-24 max |a| sech^2 a < 2^-24; the gates' functions add a few units of 2^-24 each, T = 3 steps
+    assert np.abs(h.cpu().numpy() - ref).max() < 3 * 10 * 2.0 ** -24
