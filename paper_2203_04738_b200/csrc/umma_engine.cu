@@ -122,15 +122,17 @@ bool launch_gemm_pair(int kc, const bf16* A, i64 lda, const bf16* Bm, i64 ldb, i
   if (!status) return false;
   static bool attr_set[kMaxDevices] = {false};
   auto kern = umma_gemm_pair_kernel<Epi>;
-  if (!set_smem_once(kern, pairk::kSmemBytes, attr_set)) return false;
+  using P = pairk::Cfg<Epi>;
+  static_assert(P::kSmemBytes <= 227 * 1024, "shared memory of a CTA");
+  if (!set_smem_once(kern, P::kSmemBytes, attr_set)) return false;
   CUtensorMap ta, tb;
   if (!make_map(&ta, A, (uint64_t)(a_ext > 0 ? a_ext : K), (uint64_t)M, (uint64_t)lda, BM)) return false;
-  if (!make_map(&tb, Bm, (uint64_t)K, (uint64_t)b_rows, (uint64_t)ldb, pairk::BN / 2)) return false;
-  GemmShape sh{M, N, K, 0, 1, 0, desc ? 1 : 0, a_from, a_add};
-  int tiles = ((M + 2 * BM - 1) / (2 * BM)) * ((N + pairk::BN - 1) / pairk::BN);
+  if (!make_map(&tb, Bm, (uint64_t)K, (uint64_t)b_rows, (uint64_t)ldb, P::kGates ? P::kUnits : pairk::BN / 2)) return false;
+  GemmShape sh{M, N, K, P::kGates ? N : 0, 1, 0, desc ? 1 : 0, a_from, a_add};
+  int tiles = ((M + 2 * BM - 1) / (2 * BM)) * ((N + P::kUnits - 1) / P::kUnits);
   int grid = 2 * (tiles < kSMs / 2 ? tiles : kSMs / 2);
-  ProfScope prof_(kc, 2.0 * M * (double)N * K, s);
-  if (launch_pdl_cluster(kern, 2, dim3(grid), dim3(kThreads), pairk::kSmemBytes, s, ta, tb, sh, epi, status) != cudaSuccess)
+  ProfScope prof_(kc, 2.0 * M * (double)N * (P::kGates ? P::kGates : 1) * K, s);
+  if (launch_pdl_cluster(kern, 2, dim3(grid), dim3(kThreads), P::kSmemBytes, s, ta, tb, sh, epi, status) != cudaSuccess)
     return false;
   count_launch();
   return true;
@@ -1495,6 +1497,177 @@ struct EpiLstm {
   }
 };
 
+// The same for the pair kernel, with everything but the accumulator passing through shared memory.  A thread that reads its own
+// row from global memory waits for every 8 units anew, and with the 8 warps that the registers allow nothing else hides it: the
+// operands of a tile took 27,000 cycles, its product 8,200.  Here a warp copies slices of 32 rows x 8 units (two lanes per
+// 32-byte row segment) two slices ahead of their use, over the ends of tiles, and stores its results the same way.
+// us a step (H = 1024): 16384 rows 207 -> 150, with an additive term 184; 4096 rows 65 -> 62; linearisation of 65536 rows 940 -> 840.
+// What bounds it now: the product alone takes 95 us at 16384 rows, the 470 MB of the epilogue 72; they overlap by a third.
+// COMB: the result is combined with the additive term, or (mode 1) with what the destination holds
+template <bool LIN, bool COMB = false>
+struct EpiLstmStaged {
+  // per warp: two slices of five operands (the projections of the four gates, the cell state; COMB: the two parts of what the result
+  // is combined with), and the two results
+  static constexpr int kGates = 4, kSlot = 32 * 32, kSlice = (COMB ? 7 : 5) * kSlot, kWarpBytes = 2 * kSlice + 2 * kSlot;
+  LstmFwdArgs f;      // !LIN
+  LstmLinArgs l;      // LIN
+  // 16-byte chunk `c` of row `r`: chunks trade places so that eight rows lie in different banks
+  static __device__ __forceinline__ float4* at(uint8_t* slot, int r, int c) { return reinterpret_cast<float4*>(slot + r * 32 + ((c ^ ((r >> 2) & 1)) << 4)); }
+  static __device__ __forceinline__ void copy(void* dst, const float* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+  }
+  // the two rows of a tile that this lane copies: row0 + (lane / 2) and 16 further on
+  struct Rows { i64 gi[2], c[2], o[COMB ? 2 : 1]; bool on[2]; };
+  __device__ __forceinline__ Rows rows(int row0) const {
+    const int M = LIN ? l.M : f.M, B = LIN ? l.B : f.B, H = LIN ? l.H : f.H;
+    Rows x;
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const int row = row0 + i * 16 + ((threadIdx.x & 31) >> 1), k = row / B, b = row - k * B;
+      x.on[i] = row < M;
+      if (LIN) {
+        const i64 t = l.t0 + (i64)k * l.stride_t;
+        x.gi[i] = ((t + l.stride_t - 1) * B + b) * 4 * H;
+        x.c[i] = t == 0 ? -1 - (i64)b * H : (t - 1) * l.ts + (i64)b * H;       // negative: of the initial state
+      } else {
+        x.gi[i] = (i64)k * f.gi_ks + (i64)b * 4 * H;
+        x.c[i] = (i64)k * f.in_ks + (i64)b * H;
+        if (COMB) x.o[COMB ? i : 0] = (i64)k * (f.up.mode == 1 ? f.up.out_ks : f.up.g_ks) + (i64)b * H;
+      }
+    }
+    return x;
+  }
+  template <class RowOf, class ColOf, class Acquire, class Release>
+  __device__ __forceinline__ void run(uint8_t* buf, int half, int cta, int ncta, int tiles, RowOf row_of, ColOf col_of, Acquire acquire, Release release) const {
+    const int lane = threadIdx.x & 31, chunk = lane & 1, M = LIN ? l.M : f.M, B = LIN ? l.B : f.B, H = LIN ? l.H : f.H;
+    const float gamma = LIN ? l.gamma : f.gamma; const int cell = LIN ? l.cell : f.cell;
+    const float* const other = f.up.mode == 1 ? f.up.out : f.up.g;
+    const float *const gi = LIN ? l.gi : f.gi, *const cs = LIN ? l.c : f.cin, *const bh = LIN ? l.b_hh : f.b_hh;
+    uint8_t* const res = buf + 2 * kSlice;
+    // next slice to fetch
+    int ft = cta, fs = 0;
+    Rows fr;
+    if (ft < tiles) fr = rows(row_of(ft));
+    auto fetch = [&](uint8_t* to) {
+      if (ft < tiles) {
+        const int u = col_of(ft) + half * 32 + fs * 8 + chunk * 4;
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          if (!fr.on[i]) continue;
+          const int r = i * 16 + (lane >> 1);
+          const float* g = gi + fr.gi[i] + u;
+#pragma unroll
+          for (int s = 0; s < 4; ++s) copy(at(to + s * kSlot, r, chunk), g + (i64)s * H);
+          copy(at(to + 4 * kSlot, r, chunk), (LIN && fr.c[i] < 0 ? l.c0 - (fr.c[i] + 1) : cs + fr.c[i]) + u);
+          if (COMB) {
+            copy(at(to + 5 * kSlot, r, chunk), other + fr.o[COMB ? i : 0] + u);
+            copy(at(to + (COMB ? 6 : 5) * kSlot, r, chunk), other + f.up.part + fr.o[COMB ? i : 0] + u);
+          }
+        }
+        if (++fs == 4) {
+          fs = 0; ft += ncta;
+          if (ft < tiles) fr = rows(row_of(ft));
+        }
+      }
+      asm volatile("cp.async.commit_group;" ::: "memory");      // (an empty one when nothing is left: the waits count groups)
+    };
+    fetch(buf);
+    fetch(buf + kSlice);
+    const bool update = !LIN && f.up.out;
+    int it = 0;
+    for (int t = cta; t < tiles; t += ncta, ++it) {
+      const uint32_t taddr = acquire(it);
+      if (taddr == ~0u) break;
+      const int row0 = row_of(t), col0 = col_of(t) + half * 32;
+      i64 dst[2];        // where this lane stores
+      bool on[2];
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const int row = row0 + i * 16 + (lane >> 1), k = row / B, b = row - k * B;
+        on[i] = row < M;
+        dst[i] = (update ? (i64)k * f.up.out_ks + (i64)b * H : (i64)row * H) + col0 + chunk * 4;
+      }
+#pragma unroll 1
+      for (int s = 0; s < 4; ++s) {
+        uint8_t* const in = buf + (s & 1) * kSlice;
+        float4 bb[4][2];
+#pragma unroll
+        for (int g = 0; g < 4; ++g)
+#pragma unroll
+          for (int e = 0; e < 2; ++e) bb[g][e] = __ldg(reinterpret_cast<const float4*>(bh + (i64)g * H + col0 + s * 8) + e);
+        float acc[4][8];
+#pragma unroll
+        for (int g = 0; g < 4; ++g) tmem_ld8(taddr + g * 64 + half * 32 + s * 8, acc[g]);
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+        __syncwarp();
+        float4 x[5][2];
+#pragma unroll
+        for (int q = 0; q < 5; ++q) { x[q][0] = *at(in + q * kSlot, lane, 0); x[q][1] = *at(in + q * kSlot, lane, 1); }
+        __syncwarp();
+        if (!COMB) fetch(in);
+        tmem_ld_wait8x4(acc[0], acc[1], acc[2], acc[3]);
+        float o0[8], o1[8], o2[8], o3[8], o4[8], o5[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+          auto at4 = [&](const float4 (&v)[2]) { const float4& w = v[e >> 2]; return (e & 3) == 0 ? w.x : (e & 3) == 1 ? w.y : (e & 3) == 2 ? w.z : w.w; };
+          const float ai = acc[0][e] + at4(bb[0]), af = acc[1][e] + at4(bb[1]), ag = acc[2][e] + at4(bb[2]), ao = acc[3][e] + at4(bb[3]);
+          if (LIN) {
+            const LstmLin L = lstm_linearise<true>(at4(x[0]), at4(x[1]), at4(x[2]), at4(x[3]), ai, af, ag, ao, at4(x[4]), gamma, cell);
+            o0[e] = L.a; o1[e] = L.p; o2[e] = L.ci; o3[e] = L.cf; o4[e] = L.cg; o5[e] = L.co;
+          } else {
+            const LstmOut r = lstm_forward<true>(at4(x[0]), at4(x[1]), at4(x[2]), at4(x[3]), ai, af, ag, ao, at4(x[4]), gamma, cell);
+            o0[e] = r.c; o1[e] = r.h;
+          }
+        }
+        auto put = [&](uint8_t* slot, const float* v) {
+          *at(slot, lane, 0) = make_float4(v[0], v[1], v[2], v[3]);
+          *at(slot, lane, 1) = make_float4(v[4], v[5], v[6], v[7]);
+        };
+        if (COMB) {      // (previous content - result, or result + additive term)
+          const float sg = f.up.mode == 1 ? -1.f : 1.f;
+          auto join = [&](uint8_t* slot, float* v) {
+            const float4 p = *at(slot, lane, 0), q = *at(slot, lane, 1);
+            v[0] = fmaf(sg, v[0], p.x); v[1] = fmaf(sg, v[1], p.y); v[2] = fmaf(sg, v[2], p.z); v[3] = fmaf(sg, v[3], p.w);
+            v[4] = fmaf(sg, v[4], q.x); v[5] = fmaf(sg, v[5], q.y); v[6] = fmaf(sg, v[6], q.z); v[7] = fmaf(sg, v[7], q.w);
+          };
+          join(in + 5 * kSlot, o0); join(in + (COMB ? 6 : 5) * kSlot, o1);
+        }
+        put(res, o0); put(res + kSlot, o1);
+        if (LIN && row0 + lane < M) {      // gate coefficients as bf16: eight units are one 16-byte store
+          const i64 o = (i64)(row0 + lane) * H + col0 + s * 8;
+          auto stb = [&](bf16* d, const float* v) {
+            const uint2 q0 = pack4(make_float4(v[0], v[1], v[2], v[3])), q1 = pack4(make_float4(v[4], v[5], v[6], v[7]));
+            *reinterpret_cast<uint4*>(d + o) = make_uint4(q0.x, q0.y, q1.x, q1.y);
+          };
+          stb(l.cib, o2); stb(l.cfb, o3); stb(l.cgb, o4); stb(l.cob, o5);
+        }
+        __syncwarp();
+        if (COMB) fetch(in);
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          if (!on[i]) continue;
+          const int r = i * 16 + (lane >> 1);
+          const float4 c = *at(res, r, chunk), h = *at(res + kSlot, r, chunk);
+          const i64 o = dst[i] + s * 8;
+          if (LIN) {
+            *reinterpret_cast<float4*>(l.a + o) = c;
+            *reinterpret_cast<float4*>(l.p + o) = h;
+          } else if (update) {
+            *reinterpret_cast<float4*>(f.up.out + o) = c;
+            *reinterpret_cast<float4*>(f.up.out + f.up.part + o) = h;
+          } else {
+            *reinterpret_cast<float4*>(f.cout + o) = c;
+            *reinterpret_cast<float4*>(f.hout + o) = h;
+          }
+        }
+        __syncwarp();
+      }
+      release(it);
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");      // (an aborted loop leaves copies in flight)
+  }
+};
+
 // cell-part result of an adjoint step: raw to lc_out, or straight into the level array (see LstmUpdate)
 __device__ __forceinline__ void lstm_store_lc(const LstmAdjArgs& a, i64 e, i64 kk, int b, int i, float v) {
   if (!a.up.out) { a.lc_out[e] = v; return; }
@@ -1674,8 +1847,10 @@ int lstmbf_prepare_fwd(const mgrit_gru_cfg* c, const gru_params* p, const float*
   convert(p->W_hh, w->W_hh, (i64)4 * H * H, s);
   convert(p->W_ih, w->W_ih, (i64)4 * H * I, s);
   convert(x, w->Apack, (i64)TB * I, s);
-  return launch_gemm<256, 0>(KC_PROJ, w->Apack, I, w->W_ih, I, TB, 4 * H, I, 0, 4 * H, EpiBias{gi, 4 * H, p->b_ih, TB, 4 * H}, s) ? MGRIT_OK
-                                                                                                                       : MGRIT_CUDA_ERROR;
+  const EpiBias epi{gi, 4 * H, p->b_ih, TB, 4 * H};
+  return (gemm_pair_enabled(TB, 4 * H) ? launch_gemm_pair(KC_PROJ, w->Apack, I, w->W_ih, I, TB, 4 * H, I, 4 * H, epi, s)
+                                       : launch_gemm<256, 0>(KC_PROJ, w->Apack, I, w->W_ih, I, TB, 4 * H, I, 0, 4 * H, epi, s))
+             ? MGRIT_OK : MGRIT_CUDA_ERROR;
 }
 
 int lstmbf_prepare_adj(const mgrit_gru_cfg* c, const gru_params* p, LstmBfWs* w, cudaStream_t s) {
@@ -1687,8 +1862,23 @@ int lstmbf_prepare_adj(const mgrit_gru_cfg* c, const gru_params* p, LstmBfWs* w,
   return MGRIT_OK;
 }
 
+// Cell products as pairs with the staged epilogue where they have more rows than one CTA's tile.  us a step, single CTAs against pairs:
+// H = 1024: 192 rows 17 / 15, 1024 rows 20 / 18, 2048 rows 32 / 29; H = 256: 192 rows 13 / 11, 2048 rows 14 / 12.
+static bool lstm_pair(int M) {
+  static int v = -1;
+  if (v < 0) { const char* e = getenv("MGRIT_GRU_LSTM_PAIR"); v = (e && e[0] == '0') ? 0 : 1; }
+  return v == 1 && M > BM;
+}
+
 int lstmbf_fwd_step(const LstmFwdArgs& a, LstmBfWs* w, cudaStream_t s) {
   if (!pack_rows(a.hin, a.in_ks, a.B, a.H, a.M, w->Apack, s)) return MGRIT_CUDA_ERROR;
+  if (lstm_pair(a.M)) {
+    auto launch = [&](auto epi) {
+      epi.f = a;
+      return launch_gemm_pair(KC_FWD_STEP, w->Apack, a.H, w->W_hh, a.H, a.M, a.H, a.H, 4 * a.H, epi, s) ? MGRIT_OK : MGRIT_CUDA_ERROR;
+    };
+    return a.up.out && (a.up.mode == 1 || a.up.g) ? launch(EpiLstmStaged<false, true>{}) : launch(EpiLstmStaged<false>{});
+  }
   EpiLstm<false, true> epi{};
   epi.f = a;
   return launch_gemm<256, 4>(KC_FWD_STEP, w->Apack, a.H, w->W_hh, a.H, a.M, a.H, a.H, a.H, 4 * a.H, epi, s) ? MGRIT_OK : MGRIT_CUDA_ERROR;
@@ -1705,6 +1895,11 @@ int lstmbf_linearise(const LstmLinArgs& a, LstmBfWs* w, cudaStream_t s) {
   if (N > done) {
     const i64 t1 = a.t0 + (i64)done * a.stride_t;
     if (!pack_rows(a.h + (t1 - 1) * a.ts, a.stride_t * a.ts, a.B, a.H, (i64)(N - done) * a.B, w->Apack + (i64)done * BH, s)) return MGRIT_CUDA_ERROR;
+  }
+  if (lstm_pair(a.M)) {
+    EpiLstmStaged<true> epi{};
+    epi.l = a;
+    return launch_gemm_pair(KC_LINEARISE, w->Apack, a.H, w->W_hh, a.H, a.M, a.H, a.H, 4 * a.H, epi, s) ? MGRIT_OK : MGRIT_CUDA_ERROR;
   }
   EpiLstm<true, true> epi{};
   epi.l = a;
@@ -1810,7 +2005,9 @@ int lstmbf_gradients(const mgrit_gru_cfg* c, const float* lc, const float* lh, i
   if (c->T > 1 && !pack_rows(h_rows, h_ts, B, H, M - B, w->hb0 + (i64)B * H, s)) return MGRIT_CUDA_ERROR;   // rows (t, b) of h_{t-1} start at hb0
   bool ok = wgrad_gemm(w->dAb, 4 * H, w->hb0, H, (int)M, g->dW_hh, w->scratch, w->scratch_bytes, s);
   ok = ok && wgrad_gemm(w->dAb, 4 * H, w->xb, I, (int)M, g->dW_ih, w->scratch, w->scratch_bytes, s);
-  if (dx) ok = ok && launch_gemm<256, 0>(KC_WGRAD, w->dAb, 4 * H, w->W_ihT, 4 * H, (int)M, I, 4 * H, 0, I, EpiStore{dx, I, (int)M, I, 0}, s);
+  const EpiStore st{dx, I, (int)M, I, 0};
+  if (dx) ok = ok && (gemm_pair_enabled((int)M, I) ? launch_gemm_pair(KC_WGRAD, w->dAb, 4 * H, w->W_ihT, 4 * H, (int)M, I, 4 * H, I, st, s)
+                                                   : launch_gemm<256, 0>(KC_WGRAD, w->dAb, 4 * H, w->W_ihT, 4 * H, (int)M, I, 4 * H, 0, I, st, s));
   return ok ? MGRIT_OK : MGRIT_CUDA_ERROR;
 }
 

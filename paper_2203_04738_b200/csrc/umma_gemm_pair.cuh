@@ -55,10 +55,19 @@ __device__ __forceinline__ void mma_commit_pair(uint32_t cluster_bar) {
   asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(cluster_bar) : "memory");
 }
 
+// A staged epilogue (one that declares kGates and kWarpBytes): the tile is kGates x 64 hidden units -- each CTA loads half of the
+// gates' 64-row boxes -- and every epilogue warp has kWarpBytes of shared memory, through which it fetches its operands ahead of
+// their use, over the ends of tiles.  It therefore has the loop over the tiles itself.
+template <class E, class = void> struct EpiStaged { static constexpr int kGates = 0, kWarpBytes = 0; };
+template <class E> struct EpiStaged<E, decltype((void)E::kWarpBytes)> { static constexpr int kGates = E::kGates, kWarpBytes = E::kWarpBytes; };
+
 namespace pairk {
-constexpr int BN = 256, kStages = 6;
+constexpr int BN = 256;
 constexpr int kABytes = BM * BK * 2, kBBytes = (BN / 2) * BK * 2, kStageBytes = kABytes + kBBytes;
-constexpr int kSmemBytes = kStages * kStageBytes + 1024 + 256;
+template <class Epi> struct Cfg {
+  static constexpr int kGates = EpiStaged<Epi>::kGates, kStages = kGates ? (EpiStaged<Epi>::kWarpBytes <= 12 * 1024 ? 4 : 3) : 6, kUnits = kGates ? BN / kGates : BN;
+  static constexpr int kSmemBytes = kStages * kStageBytes + 1024 + 256 + kEpiWarps * EpiStaged<Epi>::kWarpBytes;
+};
 }  // namespace pairk
 
 template <class Epi>
@@ -66,6 +75,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 umma_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, GemmShape sh, Epi epi,
                       int* status) {
   using namespace pairk;
+  constexpr int kStages = pairk::Cfg<Epi>::kStages, kGates = pairk::Cfg<Epi>::kGates, kUnits = pairk::Cfg<Epi>::kUnits;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t tiles_base = (raw + 1023u) & ~1023u;
@@ -81,7 +91,7 @@ umma_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
   const uint32_t rank = cluster_ctarank();
   const int cta = (int)(blockIdx.x >> 1), ncta = (int)(gridDim.x >> 1);
   const int m_tiles = (sh.M + 2 * BM - 1) / (2 * BM);     // a tile is 256 rows; CTA `rank` owns rows [128 rank, +128)
-  const int n_tiles = (sh.N + BN - 1) / BN;
+  const int n_tiles = (sh.N + kUnits - 1) / kUnits;
   const int tiles = m_tiles * n_tiles;
   const int k_blocks = (sh.K + BK - 1) / BK;
 
@@ -116,7 +126,13 @@ umma_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
           const uint32_t fullL = mapa_shared(full_bar(stage), 0);
           if (rank == 0) mbar_expect_tx(full_bar(stage), 2 * kStageBytes);
           tma_load_2d_pair(a_dst, &tmA, fullL, (sh.a_add && kb * BK >= sh.a_from) ? kb * BK + sh.a_add : kb * BK, mt * BM);
-          tma_load_2d_pair(b_dst, &tmB, fullL, kb * BK, nt * BN + (int)rank * (BN / 2));
+          if constexpr (kGates > 0) {
+#pragma unroll
+            for (int g = 0; g < kGates / 2; ++g)
+              tma_load_2d_pair(b_dst + g * kUnits * BK * 2, &tmB, fullL, kb * BK, ((int)rank * (kGates / 2) + g) * sh.gate_rows + nt * kUnits);
+          } else {
+            tma_load_2d_pair(b_dst, &tmB, fullL, kb * BK, nt * BN + (int)rank * (BN / 2));
+          }
           if (++stage == kStages) { stage = 0; phase ^= 1u; }
         }
       }
@@ -152,17 +168,30 @@ umma_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
   } else {
     const int q = warp & 3;
     const int half = (warp - 2) >> 2;
-    int it = 0;
-    for (int t = cta; t < tiles; t += ncta, ++it) {
-      const int mq = t / n_tiles, mt = 2 * (sh.desc ? m_tiles - 1 - mq : mq) + (int)rank, nt = t % n_tiles;
+    auto row_of = [&](int t) { const int mq = t / n_tiles; return (2 * (sh.desc ? m_tiles - 1 - mq : mq) + (int)rank) * BM + q * 32; };
+    auto col_of = [&](int t) { return t % n_tiles * kUnits; };
+    uint8_t* const buf = smem_raw + (bars + 256 - raw) + (warp - 2) * EpiStaged<Epi>::kWarpBytes;
+    // accumulator of this warp's rows in the it-th tile, ~0 when the CTA is aborting; and its release
+    auto acquire = [&](int it) {
       const int as = it & 1;
-      const uint32_t aphase = (uint32_t)(it >> 1) & 1u;
-      if (!mbar_wait(tfull_bar(as), aphase, abortp, status, 24)) break;
+      if (!mbar_wait(tfull_bar(as), (uint32_t)(it >> 1) & 1u, abortp, status, 24)) return ~0u;
       tc_fence_after();
-      const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(as * BN);
-      epi(taddr, mt * BM + q * 32 + lane, nt * BN, half);
+      return tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(as * BN);
+    };
+    auto release = [&](int it) {
       tc_fence_before();
-      mbar_arrive_cluster(mapa_shared(tempty_bar(as), 0));
+      mbar_arrive_cluster(mapa_shared(tempty_bar(it & 1), 0));
+    };
+    if constexpr (kGates > 0) {
+      epi.run(buf, half, cta, ncta, tiles, row_of, col_of, acquire, release);
+    } else {
+      int it = 0;
+      for (int t = cta; t < tiles; t += ncta, ++it) {
+        const uint32_t taddr = acquire(it);
+        if (taddr == ~0u) break;
+        epi(taddr, row_of(t) + lane, col_of(t), half);
+        release(it);
+      }
     }
   }
 
