@@ -273,10 +273,10 @@ struct Cycle {
   // intervals that can be non-zero are stepped (`homog`; zero_levels() clears what is then never written).  A level whose
   // unknowns and right-hand sides vanish behind point P has P / cf + 1 such intervals, one more after every C-relaxation.
   bool homog = false;
-  void zero_levels() {
+  void zero_levels(Setup* q) {
     for (int l = 1; l < hr.L; ++l) {
-      if (l + 1 < hr.L) cudaMemsetAsync(U[l] + BH, 0, sizeof(float) * (size_t)hr.N[l] * BH, s);
-      cudaMemsetAsync(G[l] + BH, 0, sizeof(float) * (size_t)hr.N[l] * BH, s);
+      if (l + 1 < hr.L) q->zero(U[l] + BH, sizeof(float) * (size_t)hr.N[l] * BH);
+      q->zero(G[l] + BH, sizeof(float) * (size_t)hr.N[l] * BH);
     }
   }
   // F-relaxation: from every C-point (of the first kz intervals) the cf - 1 F-points of its interval, one dependent step per
@@ -330,11 +330,12 @@ struct Cycle {
     }
   }
   bool fcycle_leg = true;     // false while a trailing V-cycle of an F-cycle runs (it does not spawn further ones)
-  int solve() {
-    if (hr.L == 1) { homog = false; cycle(0, false, false); return rc; }
+  int solve(Setup* q) {      // q: what the caller has collected
+    if (hr.L == 1) { homog = false; if (!q->run()) return MGRIT_CUDA_ERROR; cycle(0, false, false); return rc; }
     if (c->iters <= 0) homog = false;
-    if (homog) zero_levels();
-    cudaMemsetAsync(res_acc, 0, sizeof(double) * (size_t)(c->iters > 0 ? c->iters : 1), s);
+    if (homog) zero_levels(q);
+    q->zero(res_acc, sizeof(double) * (size_t)(c->iters > 0 ? c->iters : 1));
+    if (!q->run()) return MGRIT_CUDA_ERROR;
     for (cycle_idx = 0; cycle_idx < c->iters && rc == MGRIT_OK; ++cycle_idx) {
       // the previous cycle ended with an F-relaxation of level 0: the caller may ask not to repeat it
       const bool dup = cycle_idx > 0 && (c->flags & MGRIT_FLAG_SKIP_DUPLICATE_FRELAX);
@@ -532,8 +533,15 @@ struct F32Cycle {
   bool homog = false;      // as Cycle::homog
   int cycle_idx = 0;
   i64 bh() const { return (i64)c->B * c->H; }
+  unsigned* bars = nullptr; int bars_left = 0;      // cleared barrier counters, one per launch
   void flush() {
-    if (a.nph > 0 && ok) ok = f32_solve(adjoint, a, s);
+    if (a.nph > 0 && ok) {
+      unsigned* const own = a.bar;
+      if (bars_left > 0) { a.bar = bars++; --bars_left; }
+      else ok = cudaMemsetAsync(own, 0, sizeof(unsigned), s) == cudaSuccess;
+      ok = ok && f32_solve(adjoint, a, s);
+      a.bar = own;
+    }
     a.nph = 0;
   }
   void add(const F32Phase& p) {
@@ -605,16 +613,21 @@ struct F32Cycle {
       fcycle_leg = true;
     }
   }
-  bool solve() {
+  bool solve(Setup* q) {      // q: what the caller has collected
     a.nph = 0;
-    if (hr->L == 1) cycle(0, false, false);
-    else {
-      cudaMemsetAsync(res_acc, 0, sizeof(double) * (size_t)(c->iters > 0 ? c->iters : 1), s);
+    bars = a.bar + 1; bars_left = 15;
+    q->zero(bars - 1, 16 * sizeof(unsigned));
+    if (hr->L == 1) {
+      ok = q->run();
+      cycle(0, false, false);
+    } else {
+      q->zero(res_acc, sizeof(double) * (size_t)(c->iters > 0 ? c->iters : 1));
       if (c->iters <= 0) homog = false;
       for (int l = 1; homog && l < hr->L; ++l) {      // what the first way down then never writes
-        cudaMemsetAsync(U[l] + bh(), 0, sizeof(float) * (size_t)hr->N[l] * bh(), s);
-        cudaMemsetAsync(G[l] + bh(), 0, sizeof(float) * (size_t)hr->N[l] * bh(), s);
+        q->zero(U[l] + bh(), sizeof(float) * (size_t)hr->N[l] * bh());
+        q->zero(G[l] + bh(), sizeof(float) * (size_t)hr->N[l] * bh());
       }
+      ok = q->run();
       for (cycle_idx = 0; cycle_idx < c->iters; ++cycle_idx)
         cycle(0, cycle_idx > 0 && (c->flags & MGRIT_FLAG_SKIP_DUPLICATE_FRELAX), true);
     }
@@ -649,13 +662,12 @@ bool use_f32_lin(const mgrit_gru_cfg* c, const Hier& hr) {
 // with at least one cycle only the C-points are read before they are written (the first F-relaxation fills every
 // F-point from them), so only those slots are cleared: 1 / cf of the memory traffic.
 template <class T>
-void zero_guess(T* U0, const mgrit_gru_cfg& c, const Hier& hr, size_t slot, cudaStream_t s) {
+void zero_guess(T* U0, const mgrit_gru_cfg& c, const Hier& hr, size_t slot, Setup* q) {
   if (hr.L == 1) return;      // the sweep writes every point
-  if (c.iters > 0 && c.cf > 1 && c.T / c.cf > 0) {
-    cudaMemset2DAsync(U0 + (size_t)c.cf * slot, (size_t)c.cf * slot * sizeof(T), 0, slot * sizeof(T), (size_t)(c.T / c.cf), s);
-  } else {
-    cudaMemsetAsync(U0 + slot, 0, sizeof(T) * (size_t)c.T * slot, s);
-  }
+  if (c.iters > 0 && c.cf > 1 && c.T / c.cf > 0)
+    q->zero(U0 + (size_t)c.cf * slot, slot * sizeof(T), (size_t)(c.T / c.cf), (size_t)c.cf * slot * sizeof(T));
+  else
+    q->zero(U0 + slot, sizeof(T) * (size_t)c.T * slot);
 }
 
 int finish(cudaStream_t s, bool sync) {
@@ -715,13 +727,14 @@ int forward_impl(const mgrit_gru_cfg* cfg_in, bool serial, const gru_params* p, 
   } else {
     simt_project(x, p->W_ih, p->b_ih, gi, c.T * c.B, c.I, 3 * c.H, s);
   }
-  zero_guess(fw.U[0], c, hr, BH, s);
-  for (int l = 0; l < hr.L; ++l) cudaMemcpyAsync(fw.U[l], h0, sizeof(float) * BH, cudaMemcpyDeviceToDevice, s);
+  Setup setup(s);
+  zero_guess(fw.U[0], c, hr, BH, &setup);
+  for (int l = 0; l < hr.L; ++l) setup.copy(fw.U[l], h0, BH);
   const bool shadows = c.operands == MGRIT_OPERANDS_BF16 && c.B <= 128;
-  if (shadows && fw.sweep_ctr) cudaMemsetAsync(fw.sweep_ctr, 0, sizeof(int) * fw.sweep_ctr_n, s);
+  if (shadows && fw.sweep_ctr) setup.zero(fw.sweep_ctr, sizeof(int) * fw.sweep_ctr_n);
   if (shadows) {
-    zero_guess(fw.Ub[0], c, hr, BH, s);
-    for (int l = 0; l < hr.L; ++l) umma_convert(h0, fw.Ub[l], (i64)BH, s);
+    zero_guess(fw.Ub[0], c, hr, BH, &setup);
+    for (int l = 0; l < hr.L; ++l) setup.to_bf16(fw.Ub[l], h0, BH);
   }
 
   FwdCycle cy;
@@ -734,9 +747,9 @@ int forward_impl(const mgrit_gru_cfg* cfg_in, bool serial, const gru_params* p, 
     F32Cycle fc;
     fc.c = &c; fc.hr = &hr; fc.adjoint = false; fc.s = s; fc.U = fw.U; fc.G = fw.G; fc.res_acc = fw.res_acc;
     fc.a.B = c.B; fc.a.H = c.H; fc.a.cell = c.cell; fc.a.W = p->W_hh; fc.a.gi = gi; fc.a.b_hh = p->b_hh; fc.a.bar = fw.chain_bar;
-    if (!fc.solve()) return MGRIT_CUDA_ERROR;
+    if (!fc.solve(&setup)) return MGRIT_CUDA_ERROR;
   } else {
-    rc = cy.solve();
+    rc = cy.solve(&setup);
     if (rc) return rc;
   }
   if (!h_in_place) cudaMemcpyAsync(h, fw.U[0] + BH, sizeof(float) * (size_t)c.T * BH, cudaMemcpyDeviceToDevice, s);
@@ -812,17 +825,15 @@ int adjoint_impl(const mgrit_gru_cfg* cfg_in, bool serial, const gru_params* p, 
   }
   if (lin32 && !f32_linearise(lins, hr.L, s)) return MGRIT_CUDA_ERROR;
   // mu_0 = lambda_T; zero initial guess elsewhere; fine-level source = reversed dh_seed
-  zero_guess(aw.U[0], c, hr, BH, s);        // (slot 0 is set below)
+  Setup setup(s);
+  zero_guess(aw.U[0], c, hr, BH, &setup);        // (slot 0 is set below)
+  const float* const last = dh_seed ? dh_seed + (size_t)(T - 1) * BH : dhT;
+  for (int l = 0; l < hr.L; ++l) setup.copy(aw.U[l], last, BH, dh_seed ? dhT : nullptr);
   if (dh_seed) {
-    cudaMemcpyAsync(aw.U[0], dh_seed + (size_t)(T - 1) * BH, sizeof(float) * BH, cudaMemcpyDeviceToDevice, s);
-    if (dhT) stream_add_rows(aw.U[0], dhT, (i64)BH, s);
-    cudaMemsetAsync(aw.G[0], 0, sizeof(float) * BH, s);
-    cudaMemsetAsync(aw.G[0] + (size_t)T * BH, 0, sizeof(float) * BH, s);
+    setup.zero(aw.G[0], sizeof(float) * BH);
+    setup.zero(aw.G[0] + (size_t)T * BH, sizeof(float) * BH);
     if (T > 1) stream_gather_rows(aw.G[0] + BH, (i64)BH, dh_seed + (size_t)(T - 2) * BH, -(i64)BH, T - 1, (i64)BH, s);
-  } else {
-    cudaMemcpyAsync(aw.U[0], dhT, sizeof(float) * BH, cudaMemcpyDeviceToDevice, s);
   }
-  for (int l = 1; l < hr.L; ++l) cudaMemcpyAsync(aw.U[l], aw.U[0], sizeof(float) * BH, cudaMemcpyDeviceToDevice, s);
 
   float* Gl[kMaxLevels];
   for (int l = 0; l < hr.L; ++l) Gl[l] = aw.G[l];
@@ -837,9 +848,9 @@ int adjoint_impl(const mgrit_gru_cfg* cfg_in, bool serial, const gru_params* p, 
     fc.c = &c; fc.hr = &hr; fc.adjoint = true; fc.s = s; fc.U = aw.U; fc.G = Gl; fc.res_acc = aw.res_acc;
     fc.a.B = c.B; fc.a.H = c.H; fc.a.cell = c.cell; fc.a.W = p->W_hh; fc.a.bar = aw.chain_bar;
     for (int l = 0; l < hr.L; ++l) { fc.a.coef[l][0] = aw.a[l]; fc.a.coef[l][1] = aw.cr[l]; fc.a.coef[l][2] = aw.cz[l]; fc.a.coef[l][3] = aw.cn[l]; }
-    if (!fc.solve()) return MGRIT_CUDA_ERROR;
+    if (!fc.solve(&setup)) return MGRIT_CUDA_ERROR;
   } else {
-    rc = cy.solve();
+    rc = cy.solve(&setup);
     if (rc) return rc;
   }
 
@@ -944,11 +955,12 @@ struct StackCycle {
       fcycle_leg = true;
     }
   }
-  int solve() {
-    if (hr.L == 1) { homog = false; coarsest(0); return status(); }
-    cudaMemsetAsync(res_acc, 0, sizeof(double) * (size_t)(c->iters > 0 ? c->iters : 1), s);
+  int solve(Setup* q) {      // q: what the caller has collected
+    if (hr.L == 1) { homog = false; if (!q->run()) return MGRIT_CUDA_ERROR; coarsest(0); return status(); }
+    q->zero(res_acc, sizeof(double) * (size_t)(c->iters > 0 ? c->iters : 1));
     if (c->iters <= 0) homog = false;
-    if (homog) for (int k = 0; k < nl; ++k) layer(k).zero_levels();
+    if (homog) for (int k = 0; k < nl; ++k) layer(k).zero_levels(q);
+    if (!q->run()) return MGRIT_CUDA_ERROR;
     for (cycle_idx = 0; cycle_idx < c->iters && status() == MGRIT_OK; ++cycle_idx)
       cycle(0, cycle_idx > 0 && (c->flags & MGRIT_FLAG_SKIP_DUPLICATE_FRELAX), true);
     return status();
@@ -1107,18 +1119,19 @@ int stack_forward_impl(const mgrit_gru_cfg* cfg, int nl, const gru_params* p, co
   } else {
     simt_project(x, p[0].W_ih, p[0].b_ih, gi0, c.T * c.B, c.I, 3 * c.H, s);
   }
+  Setup setup(s);
   StackFwdCycle cy;
   cy.c = &c; cy.hr = hr; cy.s = s; cy.nl = nl; cy.res_acc = fw.res_acc; cy.p = p; cy.fw = &fw;
   mgrit_gru_cfg ck[kMaxStack];
   for (int k = 0; k < nl; ++k) {
     FwdWs& q = fw.L[k];
     ck[k] = layer_cfg(c, k);
-    zero_guess(q.U[0], c, hr, bh, s);
-    for (int l = 0; l < hr.L; ++l) cudaMemcpyAsync(q.U[l], h0 + k * bh, sizeof(float) * bh, cudaMemcpyDeviceToDevice, s);
+    zero_guess(q.U[0], c, hr, bh, &setup);
+    for (int l = 0; l < hr.L; ++l) setup.copy(q.U[l], h0 + k * bh, bh);
     if (fused) {
-      cudaMemsetAsync(q.sweep_ctr, 0, sizeof(int) * q.sweep_ctr_n, s);
-      zero_guess(q.Ub[0], c, hr, bh, s);
-      for (int l = 0; l < hr.L; ++l) umma_convert(h0 + k * bh, q.Ub[l], (i64)bh, s);
+      setup.zero(q.sweep_ctr, sizeof(int) * q.sweep_ctr_n);
+      zero_guess(q.Ub[0], c, hr, bh, &setup);
+      for (int l = 0; l < hr.L; ++l) setup.to_bf16(q.Ub[l], h0 + k * bh, bh);
     }
     FwdCycle& y = cy.y[k];
     y.c = &ck[k]; y.hr = hr; y.s = s; y.U = q.U; y.G = q.G; y.res_acc = fw.res_acc; y.BH = bh; y.p = &p[k]; y.um = &q.um; y.fw = &q;
@@ -1126,7 +1139,7 @@ int stack_forward_impl(const mgrit_gru_cfg* cfg, int nl, const gru_params* p, co
     y.gi = gi0;
     if (k > 0) y.gi_lv = fw.gi_l[k];
   }
-  rc = cy.solve();
+  rc = cy.solve(&setup);
   if (rc) return rc;
   for (int k = 0; k < nl; ++k) stream_gather_rows(h + k * bh, (i64)slot, fw.L[k].U[0] + bh, (i64)bh, c.T, (i64)bh, s);
   if (resnorm && hr.L > 1 && c.iters > 0) {
@@ -1357,27 +1370,29 @@ int stack_adjoint_impl(const mgrit_gru_cfg* cfg, int nl, const gru_params* p, co
   StackAdjCycle cy;
   cy.homog = !dh_seed;
   cy.c = &c; cy.hr = hr; cy.s = s; cy.nl = nl; cy.res_acc = aw.res_acc; cy.p = p; cy.w = &aw;
+  Setup setup(s);
   mgrit_gru_cfg ck[kMaxStack];
   float* Gl[kMaxStack][kMaxLevels];
   for (int k = 0; k < nl; ++k) {
     AdjWs& q = aw.L[k].w;
     ck[k] = layer_cfg(c, k);
-    zero_guess(q.U[0], c, hr, bh, s);
+    zero_guess(q.U[0], c, hr, bh, &setup);
     for (int l = 0; l < hr.L; ++l) Gl[k][l] = q.G[l];
     if (!dh_seed) Gl[k][0] = nullptr;
-    if (dh_seed) {
-      cudaMemcpyAsync(q.U[0], dh_seed + (size_t)(T - 1) * slot + k * bh, sizeof(float) * bh, cudaMemcpyDeviceToDevice, s);
-      cudaMemsetAsync(q.G[0] + (size_t)T * bh, 0, sizeof(float) * bh, s);
-      if (T > 1) stream_gather_rows(q.G[0] + bh, (i64)bh, dh_seed + (size_t)(T - 2) * slot + k * bh, -(i64)slot, T - 1, (i64)bh, s);
-    } else {
-      cudaMemsetAsync(q.U[0], 0, sizeof(float) * bh, s);
+    const float* const seed = dh_seed ? dh_seed + (size_t)(T - 1) * slot + k * bh : nullptr;
+    const float* const top = k == nl - 1 ? dhT : nullptr;      // loss on the top layer's last state
+    for (int l = 0; l < hr.L; ++l) {
+      if (seed || top) setup.copy(q.U[l], seed ? seed : top, bh, seed ? top : nullptr);
+      else setup.zero(q.U[l], sizeof(float) * bh);
     }
-    if (dhT && k == nl - 1) stream_add_rows(q.U[0], dhT, (i64)bh, s);       // loss on the top layer's last state
-    for (int l = 1; l < hr.L; ++l) cudaMemcpyAsync(q.U[l], q.U[0], sizeof(float) * bh, cudaMemcpyDeviceToDevice, s);
+    if (dh_seed) {
+      setup.zero(q.G[0] + (size_t)T * bh, sizeof(float) * bh);
+      if (T > 1) stream_gather_rows(q.G[0] + bh, (i64)bh, dh_seed + (size_t)(T - 2) * slot + k * bh, -(i64)slot, T - 1, (i64)bh, s);
+    }
     AdjCycle& y = cy.y[k];
     y.c = &ck[k]; y.hr = hr; y.s = s; y.U = q.U; y.G = Gl[k]; y.res_acc = aw.res_acc; y.BH = bh; y.p = &p[k]; y.w = &q;
   }
-  rc = cy.solve();
+  rc = cy.solve(&setup);
   if (rc) return rc;
 
   for (int k = 0; k < nl; ++k) {
@@ -1577,12 +1592,13 @@ int lstm_forward_impl(const mgrit_gru_cfg* cfg, const gru_params* p, const float
   if (is_tf32(&c)) { rc = tf32_prepare_fwd(&c, p, x, gi, &fw.tf, s); if (rc) return rc; }
   else if (c.operands == MGRIT_OPERANDS_BF16) { rc = lstmbf_prepare_fwd(&c, p, x, gi, &fw.bf, s); if (rc) return rc; }
   else simt_project(x, p->W_ih, p->b_ih, gi, c.T * c.B, c.I, 4 * c.H, s);
-  zero_guess(fw.U[0], c, hr, slot, s);
-  for (int l = 0; l < hr.L; ++l) cudaMemcpyAsync(fw.U[l], u0, sizeof(float) * slot, cudaMemcpyDeviceToDevice, s);
+  Setup setup(s);
+  zero_guess(fw.U[0], c, hr, slot, &setup);
+  for (int l = 0; l < hr.L; ++l) setup.copy(fw.U[l], u0, slot);
   LstmFwdCycle cy;
   cy.c = &c; cy.hr = hr; cy.s = s; cy.U = fw.U; cy.G = fw.G; cy.res_acc = fw.res_acc; cy.BH = slot;
   cy.p = p; cy.gi = gi; cy.fw = &fw;
-  rc = cy.solve();
+  rc = cy.solve(&setup);
   if (rc) return rc;
   cudaMemcpyAsync(u, fw.U[0] + slot, sizeof(float) * (size_t)c.T * slot, cudaMemcpyDeviceToDevice, s);
   if (resnorm && hr.L > 1 && c.iters > 0) {
@@ -1624,23 +1640,30 @@ int lstm_adjoint_impl(const mgrit_gru_cfg* cfg, const gru_params* p, const float
     else if (bf) { rc = lstmbf_linearise(a, &aw.bf, s); if (rc) return rc; }
     else simt_lstm_linearise(a, s);
   }
-  cudaMemsetAsync(aw.U[0], 0, sizeof(float) * slot, s);
-  zero_guess(aw.U[0], c, hr, slot, s);
+  Setup setup(s);
+  zero_guess(aw.U[0], c, hr, slot, &setup);
   float* Gl[kMaxLevels];
   for (int l = 0; l < hr.L; ++l) Gl[l] = aw.G[l];
   if (!du_seed) Gl[0] = nullptr;
+  const float* const last = du_seed ? du_seed + (size_t)(T - 1) * slot : nullptr;
+  for (int l = 0; l < hr.L; ++l) {      // cell part, hidden part; dhT: loss on the last hidden state
+    if (last) {
+      setup.copy(aw.U[l], last, bh);
+      setup.copy(aw.U[l] + bh, last + bh, bh, dhT);
+    } else {
+      setup.zero(aw.U[l], sizeof(float) * bh);
+      setup.copy(aw.U[l] + bh, dhT, bh);
+    }
+  }
   if (du_seed) {
-    cudaMemcpyAsync(aw.U[0], du_seed + (size_t)(T - 1) * slot, sizeof(float) * slot, cudaMemcpyDeviceToDevice, s);
-    cudaMemsetAsync(aw.G[0] + (size_t)T * slot, 0, sizeof(float) * slot, s);
+    setup.zero(aw.G[0] + (size_t)T * slot, sizeof(float) * slot);
     if (T > 1) stream_gather_rows(aw.G[0] + slot, (i64)slot, du_seed + (size_t)(T - 2) * slot, -(i64)slot, T - 1, (i64)slot, s);
   }
-  if (dhT) stream_add_rows(aw.U[0] + bh, dhT, (i64)bh, s);      // loss on the last hidden state
-  for (int l = 1; l < hr.L; ++l) cudaMemcpyAsync(aw.U[l], aw.U[0], sizeof(float) * slot, cudaMemcpyDeviceToDevice, s);
   LstmAdjCycle cy;
   cy.homog = !du_seed;
   cy.c = &c; cy.hr = hr; cy.s = s; cy.U = aw.U; cy.G = Gl; cy.res_acc = aw.res_acc; cy.BH = slot;
   cy.p = p; cy.w = &aw;
-  rc = cy.solve();
+  rc = cy.solve(&setup);
   if (rc) return rc;
   if (du) stream_gather_rows(du, (i64)slot, aw.U[0] + (size_t)(T - 1) * slot, -(i64)slot, T, (i64)slot, s);
   cudaMemcpyAsync(du0, aw.U[0] + (size_t)T * slot, sizeof(float) * slot, cudaMemcpyDeviceToDevice, s);

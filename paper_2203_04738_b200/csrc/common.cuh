@@ -201,6 +201,29 @@ void simt_lstm_adj_step(const LstmAdjArgs& a, cudaStream_t s);
 void simt_lstm_form_dA(const float* lc, const float* lh, i64 lam_ts, int B, const float* p, const float* ci, const float* cf,
                        const float* cg, const float* co, float* dA, i64 M, int H, cudaStream_t s);
 
+// What a solve clears and copies before its first step, collected and done in one launch: a handful of small memory operations cost
+// 1.6 us each and a gap behind each, up to 16 us of a solve that takes 80.
+struct SetupJob { void* dst; const float *src, *add; i64 rows, n4, pitch4; int bf16; };      // rows of n4 16-byte (bf16: 8-byte) words
+struct SetupArgs { static constexpr int kMax = 40; SetupJob job[kMax]; int n; };
+class Setup {
+ public:
+  explicit Setup(cudaStream_t s) : s_(s) { a_.n = 0; }
+  // rows of `bytes`, `pitch` apart; counts of bytes are rounded up to 16 (the arrays of a workspace are padded to 256)
+  void zero(void* dst, size_t bytes, size_t rows = 1, size_t pitch = 0) { put(SetupJob{dst, nullptr, nullptr, (i64)rows, (i64)(bytes + 15) / 16, (i64)(pitch / 16), 0}); }
+  // dst = src (+ add), n a multiple of 4
+  void copy(float* dst, const float* src, size_t n, const float* add = nullptr) { put(SetupJob{dst, src, add, 1, (i64)n / 4, 0, 0}); }
+  void to_bf16(__nv_bfloat16* dst, const float* src, size_t n) { put(SetupJob{dst, src, nullptr, 1, (i64)n / 4, 0, 1}); }
+  bool run();
+ private:
+  void put(const SetupJob& j) {
+    if (j.rows <= 0 || j.n4 <= 0) return;
+    if (a_.n == SetupArgs::kMax) run();
+    a_.job[a_.n++] = j;
+  }
+  SetupArgs a_;
+  cudaStream_t s_;
+};
+
 // SIMT (fp32 FFMA) engine
 void simt_project(const float* x, const float* W_ih, const float* b_ih, float* gi, int M, int I, int H3, cudaStream_t s);
 void simt_fwd_step(const FwdStepArgs& a, cudaStream_t s);
@@ -226,7 +249,6 @@ void stream_restrict_residual(const float* uf, int cf, const float* v, float* uc
 void stream_correct(float* uf, __nv_bfloat16* ufb, int cf, const float* uc, int nc, i64 rowlen, cudaStream_t s);
 // dst[k] = src[k*src_ks], k = 0..nk-1, rows of rowlen floats (src_ks in elements, may be negative)
 void stream_gather_rows(float* dst, i64 dst_ks, const float* src, i64 src_ks, int nk, i64 rowlen, cudaStream_t s);
-void stream_add_rows(float* dst, const float* src, i64 n, cudaStream_t s);
 // dst[k] = a[k*a_ks] + b[k*b_ks], k = 0..nk-1, rows of rowlen floats (dst contiguous)
 void stream_sum_rows(float* dst, const float* a, i64 a_ks, const float* b, i64 b_ks, int nk, i64 rowlen, cudaStream_t s);
 // stacked layers.  Row j - 1 = U[j] (V[j / cf] at the C-points when V is given) minus G[j] (when G is given), j = 1..N, to

@@ -760,7 +760,6 @@ bool launch_solve(bool adj, F32Args& a, const Shape& q, cudaStream_t s) {
     if (nb > blocks) blocks = nb;
   }
   if (blocks > ncl) blocks = ncl;
-  if (cudaMemsetAsync(a.bar, 0, sizeof(unsigned), s) != cudaSuccess) return false;
   cfg.gridDim = dim3(blocks * q.NC); cfg.dynamicSmemBytes = fix + row * rmax; cfg.stream = s; cfg.numAttrs = 2;
   if (cudaLaunchKernelEx(&cfg, kern, a, q.NC, q.U, rmax, st) != cudaSuccess) { cudaGetLastError(); return false; }
   count_launch();

@@ -36,7 +36,7 @@ struct F32Args {
   const float* W;                          // [3H, H]
   const float *gi, *b_hh;                  // forward
   const float* coef[kF32Levels][4];        // adjoint: a, c_r, c_z, c_n of every level
-  unsigned* bar;                           // barrier counter (scratch)
+  unsigned* bar;                           // barrier counter, cleared by the caller
   F32Phase ph[kF32MaxPhases];
 };
 // does a solve over rows of this width fit (weights of a cluster of CTAs resident in shared memory)?

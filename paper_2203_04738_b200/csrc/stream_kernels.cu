@@ -111,12 +111,6 @@ __global__ void __launch_bounds__(kThreads) combine_rows_kernel(const float4* __
   }
 }
 
-__global__ void __launch_bounds__(kThreads) add_rows_kernel(float4* __restrict__ dst, const float4* __restrict__ src, i64 n4) {
-  for (i64 e = (i64)blockIdx.x * blockDim.x + threadIdx.x; e < n4; e += (i64)gridDim.x * blockDim.x) {
-    float4 a = dst[e], b = src[e];
-    dst[e] = make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w);
-  }
-}
 
 __device__ __forceinline__ float4 sub4(float4 a, float4 b) { return make_float4(a.x - b.x, a.y - b.y, a.z - b.z, a.w - b.w); }
 __device__ __forceinline__ float4 sum4(float4 a, float4 b) { return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); }
@@ -365,6 +359,42 @@ void stream_correct(float* uf, __nv_bfloat16* ufb, int cf, const float* uc, int 
   count_launch();
 }
 
+namespace {
+__global__ void __launch_bounds__(kThreads) setup_kernel(const __grid_constant__ SetupArgs a) {
+  pdl_wait();
+  pdl_trigger();
+  const i64 t0 = (i64)blockIdx.x * blockDim.x + threadIdx.x, step = (i64)gridDim.x * blockDim.x;
+  for (int q = 0; q < a.n; ++q) {
+    const SetupJob& j = a.job[q];
+    const i64 total = j.rows * j.n4;
+    for (i64 e = t0; e < total; e += step) {
+      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (j.src) v = reinterpret_cast<const float4*>(j.src)[e];
+      if (j.add) {
+        const float4 w = reinterpret_cast<const float4*>(j.add)[e];
+        v = make_float4(v.x + w.x, v.y + w.y, v.z + w.z, v.w + w.w);
+      }
+      if (j.bf16) {
+        const __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y), hi = __floats2bfloat162_rn(v.z, v.w);
+        reinterpret_cast<uint2*>(j.dst)[e] = make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
+      } else {
+        const i64 r = j.rows > 1 ? e / j.n4 : 0;
+        reinterpret_cast<float4*>(j.dst)[r * j.pitch4 + (e - r * j.n4)] = v;
+      }
+    }
+  }
+}
+}  // namespace
+bool Setup::run() {
+  if (a_.n == 0) return true;
+  i64 most = 1;
+  for (int q = 0; q < a_.n; ++q) { const i64 t = a_.job[q].rows * a_.job[q].n4; if (t > most) most = t; }
+  const bool ok = launch_pdl(setup_kernel, dim3(stream_grid(most)), dim3(kThreads), 0, s_, a_) == cudaSuccess;
+  if (ok) count_launch();
+  a_.n = 0;
+  return ok;
+}
+
 void stream_gather_rows(float* dst, i64 dst_ks, const float* src, i64 src_ks, int nk, i64 rowlen, cudaStream_t s) {
   if (nk <= 0) return;
   i64 row4 = rowlen / 4;
@@ -376,11 +406,6 @@ void stream_gather_rows(float* dst, i64 dst_ks, const float* src, i64 src_ks, in
 void stream_combine_rows(const float* tmp, const float* g, i64 g_ks, float* dst, i64 dst_ks, int B, int H, i64 M, int mode, cudaStream_t s) {
   combine_rows_kernel<<<stream_grid(M * (H / 4)), kThreads, 0, s>>>(reinterpret_cast<const float4*>(tmp), reinterpret_cast<const float4*>(g),
                                                                    g_ks / 4, reinterpret_cast<float4*>(dst), dst_ks / 4, B, H / 4, M, mode);
-  count_launch();
-}
-
-void stream_add_rows(float* dst, const float* src, i64 n, cudaStream_t s) {
-  add_rows_kernel<<<stream_grid(n / 4), kThreads, 0, s>>>(reinterpret_cast<float4*>(dst), reinterpret_cast<const float4*>(src), n / 4);
   count_launch();
 }
 

@@ -41,7 +41,8 @@ def test_solve_against_the_oracle(c):
         cfg = Bd.make_cfg(T, B, 16, H, iters=iters, operands=op, flags=fl, **kw)
         n0 = Bd.kernel_launches()
         h, gi, rn = Bd.mgrit_gru_forward(cfg, p, x, h0, want_resnorm=L > 1)
-        assert Bd.kernel_launches() - n0 <= 6          # projection (and its operand splits) + at most three solve launches
+        # the projection (tf32: and its operand splits, two), one launch that clears and copies, one solve per 40 phases: at most five here
+        assert Bd.kernel_launches() - n0 <= 7
         r = Bd.mgrit_gru_adjoint(cfg, p, x, h0, gi, h, dh_seed=to_dev(seed), want_resnorm=L > 1)
         if L == 1:
             href = O.serial_forward(*P, xr, h0r)
