@@ -200,7 +200,7 @@ __global__ void sqrt_to_float_kernel(const double* acc, float* out, int n) {
 // A label outside [0, C) marks a row without a target: it adds nothing to the loss and its one-hot term is absent.
 // Few blocks (B) read a few rows of W_c each: bound by the latency of those reads, so a warp of the sixteen keeps four
 // classes' 16-byte loads in flight at once and the hidden row sits in shared memory (one class at a time with 4-byte loads
-// took 103 us for 8 rows and 51 classes of 1024 units; both passes together now take 87 us less, B200).
+// took 103 us for 8 rows and 51 classes of 1024 units, now 10.4).
 constexpr int kHeadThreads = 512, kHeadRowFloats = 4096;
 template <bool VEC>      // VEC: H is a multiple of 4 (16-byte aligned rows) and a row fits the shared array
 __global__ void __launch_bounds__(kHeadThreads) xent_rows_kernel(int B, int H, int C, const float* __restrict__ hT,
@@ -266,45 +266,55 @@ __global__ void __launch_bounds__(kHeadThreads) xent_rows_kernel(int B, int H, i
 }
 
 // pass 2: dhT = dlogits Wc ; dWc = dlogits^T hT ; dbc = column sums of dlogits ; loss = sum of the row terms (one warp, fixed
-// order: the same bits on every run; one thread walking the rows took 13 us at B = 100).  Each output is a short sum whose
-// terms are independent loads: eight in flight.
+// order: the same bits on every run; one thread walking the rows took 13 us at B = 100).
+// Short sums over C or B of operands that lie in L2: bound by the latency of their loads.  A block has a tile of 4 rows x 32 columns,
+// its eight warps split the terms, every one of 4 terms of a warp in flight feeds four rows (one thread per output walking all its
+// terms: 25 us for 100 rows, 6 classes and 104 units, 10.2 for 16 rows, 51 classes and 256 units; now 6.4 and 4.8).
+constexpr int kGradRows = 4;
 __global__ void __launch_bounds__(kThreads) xent_grads_kernel(int B, int H, int C, const float* __restrict__ hT,
                                                               const float* __restrict__ Wc,
                                                               const float* __restrict__ dlogits, const float* __restrict__ rowloss,
                                                               float* __restrict__ loss, float* __restrict__ dhT,
                                                               float* __restrict__ dWc, float* __restrict__ dbc) {
+  constexpr int NW = kThreads / 32;
+  __shared__ float part[NW][kGradRows][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   pdl_wait();
   pdl_trigger();
-  if (blockIdx.x == 0 && threadIdx.x < 32) {
+  if (blockIdx.x == 0 && warp == 0) {
     float s = 0.f;
-    for (int b = threadIdx.x; b < B; b += 32) s += rowloss[b];
+    for (int b = lane; b < B; b += 32) s += rowloss[b];
     s = warp_sum(s);
-    if (threadIdx.x == 0) *loss = s;
+    if (lane == 0) *loss = s;
   }
-  i64 nBH = (i64)B * H, nCH = (i64)C * H;
-  for (i64 e = (i64)blockIdx.x * blockDim.x + threadIdx.x; e < nBH + nCH + C; e += (i64)gridDim.x * blockDim.x) {
-    float s = 0.f;
-    if (e < nBH) {
-      int b = (int)(e / H), i = (int)(e % H);
-      const float* __restrict__ d = dlogits + (i64)b * C;
-      const float* __restrict__ w = Wc + i;
-#pragma unroll 8
-      for (int c = 0; c < C; ++c) s = fmaf(d[c], w[(i64)c * H], s);
-      dhT[e] = s;
-    } else if (e < nBH + nCH) {
-      i64 f = e - nBH;
-      int c = (int)(f / H), i = (int)(f % H);
-      const float* __restrict__ d = dlogits + c;
-      const float* __restrict__ h = hT + i;
-#pragma unroll 8
-      for (int b = 0; b < B; ++b) s = fmaf(d[(i64)b * C], h[(i64)b * H], s);
-      dWc[f] = s;
-    } else {
-      int c = (int)(e - nBH - nCH);
-#pragma unroll 8
-      for (int b = 0; b < B; ++b) s += dlogits[(i64)b * C + c];
-      dbc[c] = s;
+  const int nh = (H + 31) / 32, nb = (B + kGradRows - 1) / kGradRows, nc = (C + kGradRows - 1) / kGradRows, tiles = (nb + nc) * nh + (C + 31) / 32;
+  for (int t = blockIdx.x; t < tiles; t += gridDim.x) {
+    const bool bias = t >= (nb + nc) * nh, dh = t < nb * nh;      // (the bias row: the term's operand is one)
+    const int r0 = bias ? 0 : (dh ? t / nh : (t - nb * nh) / nh) * kGradRows, rows = bias ? 1 : min(kGradRows, (dh ? B : C) - r0);
+    const int col = (bias ? t - (nb + nc) * nh : t % nh) * 32 + lane, terms = dh ? C : B;
+    float s[kGradRows] = {0.f, 0.f, 0.f, 0.f};
+    if (col < (bias ? C : H)) {
+      const float* __restrict__ x = bias ? dlogits + col : (dh ? Wc : hT) + col;
+      const i64 xs = bias ? C : H, ds = dh ? 1 : C, dr = dh ? C : 1;
+      const float* __restrict__ d = dlogits + (i64)r0 * dr;
+#pragma unroll 4
+      for (int k = warp; k < terms; k += NW) {
+        const float v = x[(i64)k * xs];
+#pragma unroll
+        for (int q = 0; q < kGradRows; ++q)
+          if (q < rows) s[q] = bias ? s[q] + v : fmaf(d[(i64)k * ds + (i64)q * dr], v, s[q]);
+      }
     }
+#pragma unroll
+    for (int q = 0; q < kGradRows; ++q) part[warp][q][lane] = s[q];
+    __syncthreads();
+    if (warp < rows && col < (bias ? C : H)) {
+      float v = 0.f;
+#pragma unroll
+      for (int w = 0; w < NW; ++w) v += part[w][warp][lane];
+      *(bias ? dbc + col : (dh ? dhT : dWc) + (i64)(r0 + warp) * H + col) = v;
+    }
+    __syncthreads();
   }
 }
 
@@ -452,6 +462,10 @@ void stream_sqrt_to_float(const double* acc, float* out, int n, cudaStream_t s) 
   count_launch();
 }
 
+static int xent_grads_grid(int B, int H, int C) {
+  const i64 tiles = ((i64)(B + kGradRows - 1) / kGradRows + (C + kGradRows - 1) / kGradRows) * ((H + 31) / 32) + (C + 31) / 32;
+  return tiles < 1184 ? (int)tiles : 1184;      // at most the eight blocks that fit an SM
+}
 void stream_xent(int B, int H, int C, const float* hT, const float* Wc, const float* bc, const int32_t* labels, float* loss,
                  float* dhT, float* dWc, float* dbc, float* dlogits, cudaStream_t s) {
   float* rowloss = dlogits + (size_t)B * C;      // the scratch holds [B, C] derivatives followed by B row terms
@@ -460,7 +474,7 @@ void stream_xent(int B, int H, int C, const float* hT, const float* Wc, const fl
     launch_pdl(xent_rows_kernel<true>, dim3(B), dim3(kHeadThreads), (size_t)(H + C) * sizeof(float), s, B, H, C, hT, Wc, bc, labels, rowloss, dlogits);
   else
     launch_pdl(xent_rows_kernel<false>, dim3(B), dim3(kHeadThreads), (size_t)C * sizeof(float), s, B, H, C, hT, Wc, bc, labels, rowloss, dlogits);
-  launch_pdl(xent_grads_kernel, dim3(stream_grid((i64)B * H + (i64)C * H + C)), dim3(kThreads), 0, s, B, H, C, hT, Wc,
+  launch_pdl(xent_grads_kernel, dim3(xent_grads_grid(B, H, C)), dim3(kThreads), 0, s, B, H, C, hT, Wc,
              (const float*)dlogits, (const float*)rowloss, loss, dhT, dWc, dbc);
   count_launch(2);
 }
