@@ -1672,7 +1672,7 @@ int lstm_adjoint_impl(const mgrit_gru_cfg* cfg, const gru_params* p, const float
   const float* lam_c = aw.U[0] + (size_t)(T - 1) * slot;
   if (bf) {
     // bf16 operands: dA is formed as bf16 together with the bias sums, the hidden states are packed straight from u
-    rc = lstmbf_gradients(&c, lam_c, lam_c + bh, -(i64)slot, aw.p[0], aw.cib[0], aw.cfb[0], aw.cgb[0], aw.cob[0], x, u0 + bh, u + bh, (i64)slot, g,
+    rc = lstmbf_gradients(&c, lam_c, lam_c + bh, -(i64)slot, aw.p[0], aw.cib[0], aw.cfb[0], aw.cgb[0], aw.cob[0], x, g,
                           dx, &aw.bf, s);
     if (rc) return rc;
   } else {

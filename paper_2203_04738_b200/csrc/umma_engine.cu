@@ -1887,23 +1887,25 @@ int lstmbf_fwd_step(const LstmFwdArgs& a, LstmBfWs* w, cudaStream_t s) {
 int lstmbf_linearise(const LstmLinArgs& a, LstmBfWs* w, cudaStream_t s) {
   const int N = a.M / a.B;
   const i64 BH = (i64)a.B * a.H;
+  // the finest level's rows are h_0 .. h_{T-1} as the gradient pass needs them: kept for it
+  bf16* const rows = a.t0 == 0 && a.stride_t == 1 ? w->hb0 : w->Apack;
   int done = 0;
   if (a.t0 == 0) {
-    if (!pack_rows(a.h0, 0, a.B, a.H, a.B, w->Apack, s)) return MGRIT_CUDA_ERROR;
+    if (!pack_rows(a.h0, 0, a.B, a.H, a.B, rows, s)) return MGRIT_CUDA_ERROR;
     done = 1;
   }
   if (N > done) {
     const i64 t1 = a.t0 + (i64)done * a.stride_t;
-    if (!pack_rows(a.h + (t1 - 1) * a.ts, a.stride_t * a.ts, a.B, a.H, (i64)(N - done) * a.B, w->Apack + (i64)done * BH, s)) return MGRIT_CUDA_ERROR;
+    if (!pack_rows(a.h + (t1 - 1) * a.ts, a.stride_t * a.ts, a.B, a.H, (i64)(N - done) * a.B, rows + (i64)done * BH, s)) return MGRIT_CUDA_ERROR;
   }
   if (lstm_pair(a.M)) {
     EpiLstmStaged<true> epi{};
     epi.l = a;
-    return launch_gemm_pair(KC_LINEARISE, w->Apack, a.H, w->W_hh, a.H, a.M, a.H, a.H, 4 * a.H, epi, s) ? MGRIT_OK : MGRIT_CUDA_ERROR;
+    return launch_gemm_pair(KC_LINEARISE, rows, a.H, w->W_hh, a.H, a.M, a.H, a.H, 4 * a.H, epi, s) ? MGRIT_OK : MGRIT_CUDA_ERROR;
   }
   EpiLstm<true, true> epi{};
   epi.l = a;
-  return launch_gemm<256, 4>(KC_LINEARISE, w->Apack, a.H, w->W_hh, a.H, a.M, a.H, a.H, a.H, 4 * a.H, epi, s) ? MGRIT_OK : MGRIT_CUDA_ERROR;
+  return launch_gemm<256, 4>(KC_LINEARISE, rows, a.H, w->W_hh, a.H, a.M, a.H, a.H, a.H, 4 * a.H, epi, s) ? MGRIT_OK : MGRIT_CUDA_ERROR;
 }
 
 int lstmbf_adj_step(const LstmAdjArgs& a, LstmBfWs* w, cudaStream_t s) {
@@ -1985,9 +1987,9 @@ __global__ void __launch_bounds__(kPT) lstm_sum_db_kernel(const float* __restric
 }  // namespace
 
 // All gradients of the LSTM parameters (and dx) from the step-output sensitivities (lc, lh; rows (t, b) at + t*lam_ts + b*H),
-// the level-0 coefficients and the hidden states entering each step (h0, then h_rows + (t-1)*h_ts).
+// the level-0 coefficients and the hidden states entering each step (w->hb0: packed by the linearisation of the finest level).
 int lstmbf_gradients(const mgrit_gru_cfg* c, const float* lc, const float* lh, i64 lam_ts, const float* p, const bf16* ci, const bf16* cf,
-                     const bf16* cg, const bf16* co, const float* x, const float* h0, const float* h_rows, i64 h_ts, const gru_grads* g,
+                     const bf16* cg, const bf16* co, const float* x, const gru_grads* g,
                      float* dx, LstmBfWs* w, cudaStream_t s) {
   const int H = c->H, I = c->I, B = c->B;
   const i64 M = (i64)c->T * B;
@@ -2001,8 +2003,6 @@ int lstmbf_gradients(const mgrit_gru_cfg* c, const float* lc, const float* lh, i
   lstm_sum_db_kernel<<<pgrid(4 * H), kPT, 0, s>>>(w->scratch, (int)grid.x, H, g->db_hh, g->db_ih);
   count_launch(2);
   convert(x, w->xb, M * I, s);
-  convert(h0, w->hb0, (i64)B * H, s);
-  if (c->T > 1 && !pack_rows(h_rows, h_ts, B, H, M - B, w->hb0 + (i64)B * H, s)) return MGRIT_CUDA_ERROR;   // rows (t, b) of h_{t-1} start at hb0
   bool ok = wgrad_gemm(w->dAb, 4 * H, w->hb0, H, (int)M, g->dW_hh, w->scratch, w->scratch_bytes, s);
   ok = ok && wgrad_gemm(w->dAb, 4 * H, w->xb, I, (int)M, g->dW_ih, w->scratch, w->scratch_bytes, s);
   const EpiStore st{dx, I, (int)M, I, 0};
