@@ -200,7 +200,7 @@ int gru_serial_backward(const mgrit_gru_cfg* cfg, const gru_params* p, const flo
  *   state at the step's arrival time (restriction by injection for inputs as for states).
  *   dh_seed[T,n_layers,B,H] or NULL; dhT[B,H] or NULL: loss derivative w.r.t. the TOP layer's last state; dh (optional)
  *   and dh0 have the shapes of h and h0: the sensitivities of the states as step outputs; dx[T,B,I] or NULL;
- *   grads: HOST array of n_layers gru_grads.  The coarsest level is advanced step by step (no persistent chain). */
+ *   grads: HOST array of n_layers gru_grads. */
 int mgrit_gru_stack_workspace_bytes(const mgrit_gru_cfg* cfg, int32_t n_layers, size_t* fwd_bytes, size_t* adj_bytes);
 int mgrit_gru_stack_forward(const mgrit_gru_cfg* cfg, int32_t n_layers, const gru_params* layers, const float* x, const float* h0,
                             float* gi0, float* h, float* resnorm, void* ws, size_t ws_bytes, mgrit_stream_t stream);

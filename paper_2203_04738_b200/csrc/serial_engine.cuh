@@ -91,7 +91,7 @@ struct LstmChainAdjArgs {
   const __nv_bfloat16* WT;       // [H][4H] = W_hh^T
   uint4* xw; size_t xw_bytes;    // exchange words, serial_xw_bytes(B, H, 4)
 };
-// false: shape not supported (forward: H % 128 != 0; adjoint: H not in {128, 256, 512, 1024}; too many CTAs for one wave)
+// false: shape not supported (H % 64 != 0; adjoint not split by gate: H not in {128, 256, 512, 1024}; too many CTAs for one wave)
 // or the cooperative launch failed: the caller then advances step by step
 bool lstm_chain_fwd_solve(const LstmChainFwdArgs& a, cudaStream_t s);
 bool lstm_chain_adj_solve(const LstmChainAdjArgs& a, cudaStream_t s);
