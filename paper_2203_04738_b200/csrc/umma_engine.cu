@@ -1511,6 +1511,7 @@ struct EpiLstmStaged {
   static constexpr int kGates = 4, kSlot = 32 * 32, kSlice = (COMB ? 7 : 5) * kSlot, kWarpBytes = 2 * kSlice + 2 * kSlot;
   LstmFwdArgs f;      // !LIN
   LstmLinArgs l;      // LIN
+  bf16* hb;           // !LIN: the new hidden rows once more as bf16, contiguous [M, H], for the step that continues from them (or null)
   // 16-byte chunk `c` of row `r`: chunks trade places so that eight rows lie in different banks
   static __device__ __forceinline__ float4* at(uint8_t* slot, int r, int c) { return reinterpret_cast<float4*>(slot + r * 32 + ((c ^ ((r >> 2) & 1)) << 4)); }
   static __device__ __forceinline__ void copy(void* dst, const float* src) {
@@ -1655,6 +1656,7 @@ struct EpiLstmStaged {
           } else if (update) {
             *reinterpret_cast<float4*>(f.up.out + o) = c;
             *reinterpret_cast<float4*>(f.up.out + f.up.part + o) = h;
+            if (hb) *reinterpret_cast<uint2*>(hb + (i64)(row0 + r) * H + col0 + s * 8 + chunk * 4) = pack4(h);
           } else {
             *reinterpret_cast<float4*>(f.cout + o) = c;
             *reinterpret_cast<float4*>(f.hout + o) = h;
@@ -1822,6 +1824,7 @@ void lstmbf_plan_fwd(const mgrit_gru_cfg* c, size_t max_rows, char* base, size_t
   o->W_ih = take<bf16>(base, off, 4 * H * I);
   o->apack_elems = max_rows * H > TB * I ? max_rows * H : TB * I;      // a step's rows, or x for the projection
   o->Apack = take<bf16>(base, off, o->apack_elems);
+  o->Apack2 = o->Apack && o->apack_elems >= 2 * max_rows * H ? o->Apack + max_rows * H : nullptr;
 }
 
 void lstmbf_plan_adj(const mgrit_gru_cfg* c, size_t max_rows, char* base, size_t* off, LstmBfWs* o) {
@@ -1870,19 +1873,24 @@ static bool lstm_pair(int M) {
   return v == 1 && M > BM;
 }
 
-int lstmbf_fwd_step(const LstmFwdArgs& a, LstmBfWs* w, cudaStream_t s) {
-  if (!pack_rows(a.hin, a.in_ks, a.B, a.H, a.M, w->Apack, s)) return MGRIT_CUDA_ERROR;
+int lstmbf_fwd_step(const LstmFwdArgs& a, const bf16* rows, bf16* next, LstmBfWs* w, cudaStream_t s) {
+  if (!rows) {
+    if (!pack_rows(a.hin, a.in_ks, a.B, a.H, a.M, w->Apack, s)) return MGRIT_CUDA_ERROR;
+    rows = w->Apack;
+  }
   if (lstm_pair(a.M)) {
     auto launch = [&](auto epi) {
       epi.f = a;
-      return launch_gemm_pair(KC_FWD_STEP, w->Apack, a.H, w->W_hh, a.H, a.M, a.H, a.H, 4 * a.H, epi, s) ? MGRIT_OK : MGRIT_CUDA_ERROR;
+      epi.hb = next;
+      return launch_gemm_pair(KC_FWD_STEP, rows, a.H, w->W_hh, a.H, a.M, a.H, a.H, 4 * a.H, epi, s) ? MGRIT_OK : MGRIT_CUDA_ERROR;
     };
     return a.up.out && (a.up.mode == 1 || a.up.g) ? launch(EpiLstmStaged<false, true>{}) : launch(EpiLstmStaged<false>{});
   }
   EpiLstm<false, true> epi{};
   epi.f = a;
-  return launch_gemm<256, 4>(KC_FWD_STEP, w->Apack, a.H, w->W_hh, a.H, a.M, a.H, a.H, a.H, 4 * a.H, epi, s) ? MGRIT_OK : MGRIT_CUDA_ERROR;
+  return launch_gemm<256, 4>(KC_FWD_STEP, rows, a.H, w->W_hh, a.H, a.M, a.H, a.H, a.H, 4 * a.H, epi, s) ? MGRIT_OK : MGRIT_CUDA_ERROR;
 }
+bool lstmbf_leaves_rows(int M) { return lstm_pair(M); }
 
 int lstmbf_linearise(const LstmLinArgs& a, LstmBfWs* w, cudaStream_t s) {
   const int N = a.M / a.B;

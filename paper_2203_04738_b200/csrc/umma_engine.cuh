@@ -64,6 +64,7 @@ struct LstmBfWs {
   __nv_bfloat16 *W_hhT, *W_ihT;   // [H,4H], [I,4H]   (adjoint call)
   __nv_bfloat16* Apack;           // A side of the current product
   size_t apack_elems;
+  __nv_bfloat16* Apack2;          // forward: a second set of rows where Apack has room for it (else null)
   __nv_bfloat16 *xb, *hb0, *dAb;  // [T*B,I]; [(T+1)*B,H] = [h_0; h]; [T*B,4H]   (gradient pass)
   float* scratch; size_t scratch_bytes;   // partial products of the split weight-gradient reductions
 };
@@ -71,7 +72,9 @@ void lstmbf_plan_fwd(const mgrit_gru_cfg* c, size_t max_rows, char* base, size_t
 void lstmbf_plan_adj(const mgrit_gru_cfg* c, size_t max_rows, char* base, size_t* off, LstmBfWs* o);
 int lstmbf_prepare_fwd(const mgrit_gru_cfg* c, const gru_params* p, const float* x, float* gi, LstmBfWs* w, cudaStream_t s);
 int lstmbf_prepare_adj(const mgrit_gru_cfg* c, const gru_params* p, LstmBfWs* w, cudaStream_t s);
-int lstmbf_fwd_step(const LstmFwdArgs& a, LstmBfWs* w, cudaStream_t s);
+// rows: the hidden rows of this step as bf16 (null: packed into w->Apack first); next: where to leave those of its result (or null)
+int lstmbf_fwd_step(const LstmFwdArgs& a, const __nv_bfloat16* rows, __nv_bfloat16* next, LstmBfWs* w, cudaStream_t s);
+bool lstmbf_leaves_rows(int M);      // can a step of M rows leave its result as bf16?
 int lstmbf_linearise(const LstmLinArgs& a, LstmBfWs* w, cudaStream_t s);
 int lstmbf_adj_step(const LstmAdjArgs& a, LstmBfWs* w, cudaStream_t s);
 // dW_hh, dW_ih (and dx) from dA[T*B,4H] fp32; hidden states h0 [B,H] and hk [T,B,H] fp32
