@@ -1491,7 +1491,7 @@ struct LstmFwdCycle : Cycle {
   const gru_params* p; const float* gi; LstmFwdWs* fw;
   // bf16: a step that ends at F-points leaves its hidden rows as bf16 for the next one, which reads the same slots (rows `left` in
   // the order of the step's rows).  Nothing else writes F-points between two steps of a relaxation.  Packing 16384 rows of 1024
-  // units in front of a step takes 26 us, leaving them 8.
+  // units in front of a step takes 26 us; a training step at T = 2048, B = 32, H = 1024 13.88 -> 13.67 ms.
   __nv_bfloat16* left = nullptr; const float* left_of = nullptr; i64 left_ks = 0; int left_nk = 0;
   bool chain(int l) override {
     if (c->operands != MGRIT_OPERANDS_BF16 || !fw->chain_xw) return false;
