@@ -205,11 +205,11 @@ __device__ __forceinline__ void fwd_sums(const float* S, const FwdWeights<KC>& q
 }
 
 __device__ __forceinline__ void block_rows(const F32Args& a, const F32Phase& p, int r0, int* rk, int* rb) {
-  if ((int)threadIdx.x < p.R) {
-    const int m = r0 + threadIdx.x;
+  for (int i = threadIdx.x; i < p.R; i += blockDim.x) {      // (a block may have more rows than threads: H = 8 runs on 32)
+    const int m = r0 + i;
     const bool v = m < p.nk * a.B;
-    rk[threadIdx.x] = v ? m / a.B : -1;
-    rb[threadIdx.x] = v ? m % a.B : 0;
+    rk[i] = v ? m / a.B : -1;
+    rb[i] = v ? m % a.B : 0;
   }
 }
 __device__ __forceinline__ void add_norm(float norm, double* acc) {

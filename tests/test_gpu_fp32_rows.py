@@ -1,0 +1,50 @@
+"""The persistent fp32 solve with many rows: row blocks with more rows than a block has threads (H = 8 runs on 32).  Forward,
+adjoint and gradients against the fp64 oracle at the same cycle count."""
+import numpy as np
+import pytest
+
+from oracle import mgrit_gru_oracle as O
+from paper_2203_04738_b200.synthetic import Workload, make_inputs
+from tests.gpu_util import oracle_params, to_dev, upload
+
+pytestmark = pytest.mark.gpu
+
+
+def norm(a, b):
+    return np.linalg.norm(a - b) / max(np.linalg.norm(b), 1e-30)
+
+
+def solve_against_the_oracle(T, B, H, cf, L, rf, rc, iters):
+    from paper_2203_04738_b200 import binding as Bd
+    ragged = T % cf ** (L - 1) != 0
+    w = Workload("rows", T=T, B=B, I=16, H=H, cf=cf, levels=L, iters_fwd=iters, iters_adj=iters, relax_fine=rf, relax_coarse=rc,
+                 operands=0, classes=4, relu=False, seed=T + H)
+    d = make_inputs(w)
+    d["h0"] = (np.random.default_rng(1).standard_normal(d["h0"].shape) * 0.3).astype(np.float32)
+    p, x, h0 = upload(d)
+    P = oracle_params(d)
+    kw = dict(cf=cf, levels=L, relax_fine=rf, relax_coarse=rc)
+    cfg = Bd.make_cfg(T, B, 16, H, iters=iters, operands=0, flags=Bd.FLAG_RAGGED_T if ragged else 0, **kw)
+    xr, h0r = d["x"].astype(np.float64), d["h0"].astype(np.float64)
+    seed = np.random.default_rng(2).standard_normal((T, B, H)).astype(np.float32)
+    h, gi, rn = Bd.mgrit_gru_forward(cfg, p, x, h0, want_resnorm=True)
+    r = Bd.mgrit_gru_adjoint(cfg, p, x, h0, gi, h, dh_seed=to_dev(seed))
+    assert Bd.last_device_status() == 0
+    href, rref = O.mgrit_forward(*P, xr, h0r, iters=iters, ragged=ragged, **kw)
+    # 2^-24 per operation through at most T dependent steps of a contraction; the gates keep the factor near one
+    assert norm(h.cpu().numpy(), href) < 5e-6
+    assert np.allclose(rn, rref, rtol=1e-3, atol=1e-5 * rref[0] + 1e-6)
+    lam, lam0, g, _ = O.mgrit_adjoint(*P, xr, h0r, h.cpu().numpy().astype(np.float64), seed.astype(np.float64), iters=iters, ragged=ragged, **kw)
+    assert norm(r.dh.cpu().numpy(), lam) < 5e-6 and norm(r.dh0.cpu().numpy(), lam0) < 2e-5
+    # (sums of T*B terms of either sign: 2^-24 of the running sum per addition, over at most some thousand additions a range)
+    for k in ("dx", "dW_ih", "dW_hh", "db_ih", "db_hh"):
+        assert norm(getattr(r, k).cpu().numpy(), g[k]) < 1e-5, k
+
+
+#        T    B    H   cf L  rf rc iters     rows of the largest phase: 6500 and 12800, blocks of 44 rows and more
+MORE_ROWS_THAN_THREADS = [(258, 100, 8, 4, 2, 0, 1, 2), (512, 100, 8, 4, 3, 1, 1, 1), (1024, 32, 8, 4, 2, 0, 1, 2), (258, 100, 16, 4, 2, 1, 0, 2)]
+
+
+@pytest.mark.parametrize("c", MORE_ROWS_THAN_THREADS, ids=lambda c: "T{}B{}H{}cf{}L{}r{}{}i{}".format(*c))
+def test_blocks_with_more_rows_than_threads(c):
+    solve_against_the_oracle(*c)
