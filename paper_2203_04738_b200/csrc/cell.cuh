@@ -28,9 +28,15 @@ __device__ __forceinline__ float rcp_newton(float x) {
   const float y = rcp_approx(x);
   return fmaf(fmaf(-x, y, 1.0f), y, y);
 }
+// the smaller one, or NaN where one of them is (fminf would drop it, and a diverged run would pass for a sound one)
+__device__ __forceinline__ float min_nan(float a, float b) {
+  float y;
+  asm("min.NaN.f32 %0, %1, %2;" : "=f"(y) : "f"(a), "f"(b));
+  return y;
+}
 template <bool FAST> __device__ __forceinline__ float sigmoid_t(float x) {
   if (FAST) return fmaf(tanh_approx(0.5f * x), 0.5f, 0.5f);
-  return rcp_newton(1.0f + __expf(fminf(-x, 80.0f)));      // (below -80 the result is 1.8e-35 instead of less)
+  return rcp_newton(1.0f + __expf(min_nan(-x, 80.0f)));      // (below -80 the result is 1.8e-35 instead of less)
 }
 template <bool FAST> __device__ __forceinline__ float tanh_t(float x) { return FAST ? tanh_approx(x) : tanhf(x); }
 template <bool FAST> __device__ __forceinline__ float inv_t(float x) { return FAST ? rcp_approx(x) : rcp_newton(x); }
