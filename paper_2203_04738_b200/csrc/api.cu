@@ -529,7 +529,7 @@ struct AdjCycle : Cycle {
 struct F32Cycle {
   const mgrit_gru_cfg* c; const Hier* hr; bool adjoint; cudaStream_t s;
   float** U; float** G; double* res_acc; F32Args a;
-  bool ok = true, fcycle_leg = true;
+  bool ok = true, fcycle_leg = true, started = false;      // started: a launch of this solve went out
   bool homog = false;      // as Cycle::homog
   int cycle_idx = 0;
   i64 bh() const { return (i64)c->B * c->H; }
@@ -540,6 +540,7 @@ struct F32Cycle {
       if (bars_left > 0) { a.bar = bars++; --bars_left; }
       else ok = cudaMemsetAsync(own, 0, sizeof(unsigned), s) == cudaSuccess;
       ok = ok && f32_solve(adjoint, a, s);
+      started = started || ok;
       a.bar = own;
     }
     a.nph = 0;
@@ -613,12 +614,13 @@ struct F32Cycle {
       fcycle_leg = true;
     }
   }
-  bool solve(Setup* q) {      // q: what the caller has collected
+  // MGRIT_UNSUPPORTED: the first launch was refused and the arrays are as the set-up left them; the caller advances step by step
+  int solve(Setup* q) {      // q: what the caller has collected
     a.nph = 0;
     bars = a.bar + 1; bars_left = 15;
     q->zero(bars - 1, 16 * sizeof(unsigned));
     if (hr->L == 1) {
-      ok = q->run();
+      if (!q->run()) return MGRIT_CUDA_ERROR;
       cycle(0, false, false);
     } else {
       q->zero(res_acc, sizeof(double) * (size_t)(c->iters > 0 ? c->iters : 1));
@@ -627,12 +629,12 @@ struct F32Cycle {
         q->zero(U[l] + bh(), sizeof(float) * (size_t)hr->N[l] * bh());
         q->zero(G[l] + bh(), sizeof(float) * (size_t)hr->N[l] * bh());
       }
-      ok = q->run();
+      if (!q->run()) return MGRIT_CUDA_ERROR;
       for (cycle_idx = 0; cycle_idx < c->iters; ++cycle_idx)
         cycle(0, cycle_idx > 0 && (c->flags & MGRIT_FLAG_SKIP_DUPLICATE_FRELAX), true);
     }
     flush();
-    return ok;
+    return ok ? MGRIT_OK : started ? MGRIT_CUDA_ERROR : MGRIT_UNSUPPORTED;
   }
 };
 
@@ -743,15 +745,15 @@ int forward_impl(const mgrit_gru_cfg* cfg_in, bool serial, const gru_params* p, 
   cy.Ub = shadows ? fw.Ub : nullptr;
   cy.gib = shadows ? fw.um.gib : nullptr;
   cy.gi_f32 = gi_f32;
+  rc = MGRIT_UNSUPPORTED;
   if (use_f32_solve(&c, hr)) {
     F32Cycle fc;
     fc.c = &c; fc.hr = &hr; fc.adjoint = false; fc.s = s; fc.U = fw.U; fc.G = fw.G; fc.res_acc = fw.res_acc;
     fc.a.B = c.B; fc.a.H = c.H; fc.a.cell = c.cell; fc.a.W = p->W_hh; fc.a.gi = gi; fc.a.b_hh = p->b_hh; fc.a.bar = fw.chain_bar;
-    if (!fc.solve(&setup)) return MGRIT_CUDA_ERROR;
-  } else {
-    rc = cy.solve(&setup);
-    if (rc) return rc;
+    rc = fc.solve(&setup);
   }
+  if (rc == MGRIT_UNSUPPORTED) rc = cy.solve(&setup);
+  if (rc) return rc;
   if (!h_in_place) cudaMemcpyAsync(h, fw.U[0] + BH, sizeof(float) * (size_t)c.T * BH, cudaMemcpyDeviceToDevice, s);
   if (resnorm && hr.L > 1 && c.iters > 0) {
     rc = fetch_resnorm(fw.res_acc, resnorm, c.iters, s);
@@ -801,7 +803,6 @@ int adjoint_impl(const mgrit_gru_cfg* cfg_in, bool serial, const gru_params* p, 
     if (rc) return rc;
   }
   // adjoint coefficients of every level's steps at the given states (restricted by injection)
-  const bool lin32 = use_f32_lin(&c, hr);
   LinArgs lins[kMaxLevels];
   for (int l = 0; l < hr.L; ++l) {
     LinArgs& a = lins[l];
@@ -812,18 +813,16 @@ int adjoint_impl(const mgrit_gru_cfg* cfg_in, bool serial, const gru_params* p, 
     a.a = aw.a[l]; a.cr = aw.cr[l]; a.cz = aw.cz[l]; a.cn = aw.cn[l]; a.cnp = l == 0 ? aw.cnp : nullptr;
     a.crb = aw.crb[l]; a.czb = aw.czb[l]; a.cnb = aw.cnb[l]; a.cnpb = l == 0 ? aw.cnpb : nullptr;
     a.gi_b = (bf16 && copies) ? aw.um.gib : nullptr;
-    if (lin32) continue;
-    if (bf16) {
-      rc = umma_linearise(a, &aw.um, s);
+  }
+  if (!(use_f32_lin(&c, hr) && f32_linearise(lins, hr.L, s))) {
+    for (int l = 0; l < hr.L; ++l) {
+      rc = MGRIT_OK;
+      if (bf16) rc = umma_linearise(lins[l], &aw.um, s);
+      else if (tf32) rc = tf32_linearise(lins[l], &aw.tf, s);
+      else simt_linearise(lins[l], s);
       if (rc) return rc;
-    } else if (tf32) {
-      rc = tf32_linearise(a, &aw.tf, s);
-      if (rc) return rc;
-    } else {
-      simt_linearise(a, s);
     }
   }
-  if (lin32 && !f32_linearise(lins, hr.L, s)) return MGRIT_CUDA_ERROR;
   // mu_0 = lambda_T; zero initial guess elsewhere; fine-level source = reversed dh_seed
   Setup setup(s);
   zero_guess(aw.U[0], c, hr, BH, &setup);        // (slot 0 is set below)
@@ -842,17 +841,17 @@ int adjoint_impl(const mgrit_gru_cfg* cfg_in, bool serial, const gru_params* p, 
   cy.c = &c; cy.hr = hr; cy.s = s; cy.U = aw.U; cy.G = Gl; cy.res_acc = aw.res_acc; cy.BH = BH;
   cy.p = p; cy.w = &aw;
   cy.homog = !dh_seed;
+  rc = MGRIT_UNSUPPORTED;
   if (use_f32_solve(&c, hr)) {
     F32Cycle fc;
     fc.homog = !dh_seed;
     fc.c = &c; fc.hr = &hr; fc.adjoint = true; fc.s = s; fc.U = aw.U; fc.G = Gl; fc.res_acc = aw.res_acc;
     fc.a.B = c.B; fc.a.H = c.H; fc.a.cell = c.cell; fc.a.W = p->W_hh; fc.a.bar = aw.chain_bar;
     for (int l = 0; l < hr.L; ++l) { fc.a.coef[l][0] = aw.a[l]; fc.a.coef[l][1] = aw.cr[l]; fc.a.coef[l][2] = aw.cz[l]; fc.a.coef[l][3] = aw.cn[l]; }
-    if (!fc.solve(&setup)) return MGRIT_CUDA_ERROR;
-  } else {
-    rc = cy.solve(&setup);
-    if (rc) return rc;
+    rc = fc.solve(&setup);
   }
+  if (rc == MGRIT_UNSUPPORTED) rc = cy.solve(&setup);
+  if (rc) return rc;
 
   // dh[k] = lambda_{k+1} = mu_{T-1-k} (optional output);  dh0 = lambda_0 = mu_T
   if (dh) stream_gather_rows(dh, (i64)BH, aw.U[0] + (size_t)(T - 1) * BH, -(i64)BH, T, (i64)BH, s);
@@ -1024,6 +1023,7 @@ struct StackFwdCycle : StackCycle {
                     bf ? fw->L[k + 1].um.xb : nullptr, s);
     project(k, l, fw->raw, hr.N[l]);
   }
+  // false: not available here, nothing has been enqueued
   bool run_fp32(FwdCycle& q, int k, int l, int kz, bool f, int last) {
     if (c->operands != MGRIT_OPERANDS_FP32 || !f32_solve_fits(c->H)) return false;
     F32Cycle fc;
@@ -1045,8 +1045,7 @@ struct StackFwdCycle : StackCycle {
     }
     fc.add(ph);
     fc.flush();
-    if (!fc.ok) rc = MGRIT_CUDA_ERROR;
-    return true;
+    return fc.ok;
   }
   void segment(int l, int kz, bool f, int last) override {
     int kinds[32], n = 0;
@@ -1277,8 +1276,7 @@ struct StackAdjCycle : StackCycle {
     fc.a.nph = 0;
     fc.cycle(l, false, false);       // (the coarsest level: one phase)
     fc.flush();
-    if (!fc.ok) rc = MGRIT_CUDA_ERROR;
-    return true;
+    return fc.ok || y[k].chain_on(l, mu, g);
   }
   // Below the top layer mu_s = step(mu_{s-1} + d_{s-1}) + g_s: a chain in nu_s = mu_s + d_s with the source g_s + d_s.
   void coarsest(int l) override {

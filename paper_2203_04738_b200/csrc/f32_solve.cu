@@ -24,6 +24,8 @@
 // us a step, forward / adjoint, weights in shared memory -> in registers:
 //   H = 32, 2 rows 1.4 / 1.9 -> 0.87 / 1.2; H = 104, 3300 rows 15 / 16 -> 12.3 / 11.5; H = 256, 16 rows 3.3 / 3.2 -> 2.9 / 2.0,
 //   500 rows 14.7 / 11.8 -> 11.1 / 8.4 (18 and 24 TFLOP/s); H = 320, 16 rows 4.1 / 4.4 -> 4.4 / 3.5, 700 rows 28 / 23 -> 23 / 26.
+#include <stdlib.h>
+
 #include "cell.cuh"
 #include "f32_solve.cuh"
 
@@ -678,6 +680,14 @@ __global__ void __launch_bounds__(fwd_most(KC), 1) f32_lin_kernel(const __grid_c
   }
 }
 
+// MGRIT_GRU_F32_SOLVE=0 in the environment answers as where the cooperative cluster launch is refused: the callers then advance step
+// by step, as at widths that do not fit.
+bool solve_enabled() {
+  static int v = -1;
+  if (v < 0) { const char* e = getenv("MGRIT_GRU_F32_SOLVE"); v = (e && e[0] == '0') ? 0 : 1; }
+  return v == 1;
+}
+
 int* status_ptr() {
   const int dev = current_device_slot();
   if (dev < 0) return nullptr;
@@ -774,7 +784,7 @@ bool f32_solve_fits(int H) {
 
 bool f32_solve(bool adjoint, F32Args& a, cudaStream_t s) {
   Shape q;
-  if (!pick_shape(a.H, &q)) return false;
+  if (!solve_enabled() || !pick_shape(a.H, &q)) return false;
   if (adjoint) {
     if (q.adj_kp == 32)
       return q.adj_kc == 1   ? launch_solve<f32_adj_kernel<false, 32, 1, 384>>(true, a, q, s)
