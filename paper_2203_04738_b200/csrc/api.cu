@@ -537,6 +537,7 @@ struct F32Cycle {
   void flush() {
     if (a.nph > 0 && ok) {
       unsigned* const own = a.bar;
+      a.progress = own + 16;            // (behind the counters of the launches)
       if (bars_left > 0) { a.bar = bars++; --bars_left; }
       else ok = cudaMemsetAsync(own, 0, sizeof(unsigned), s) == cudaSuccess;
       ok = ok && f32_solve(adjoint, a, s);

@@ -36,7 +36,6 @@ namespace {
 __host__ __device__ constexpr int fwd_most(int KC) { return KC == 4 || KC == 7 || KC == 8 ? 256 : 384; }
 constexpr int kMaxRows = 64;
 constexpr size_t kSmemMax = 227 * 1024 - 2048;     // dynamic part: the kernels hold under 1 KiB of static shared memory
-constexpr uint64_t kWaitLimitNs = 2000000000ull;
 
 __device__ int g_f32_status = 0;
 int* g_f32_status_ptrs[kMaxDevices] = {nullptr};
@@ -57,24 +56,34 @@ template <bool MULTI> __device__ __forceinline__ void block_sync() { if (MULTI) 
 __device__ __forceinline__ uint64_t now_ns() { uint64_t t; asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t)); return t; }
 
 // All clusters have finished the phase.  The leader CTA arrives and polls (bounded); its verdict reaches the whole cluster, so
-// either every CTA of a cluster goes on or every one leaves.
+// either every CTA of a cluster goes on or every one leaves.  A phase may be a whole serial chain of millions of steps, so what is
+// bounded is the time without progress: a working cluster reports every kReport-th step (report()), and with the blocks of a phase
+// dealt out evenly no wait sees more than one block's shorter chain unreported.
+constexpr int kReport = 256;
+__device__ __forceinline__ void report(const F32Args& a, int j, int rank) {
+  if ((j & (kReport - 1)) == kReport - 1 && threadIdx.x == 0 && rank == 0)
+    asm volatile("red.relaxed.gpu.global.add.u32 [%0], 1;" ::"l"(a.progress) : "memory");
+}
 template <bool MULTI>
-__device__ bool grid_barrier(unsigned* bar, unsigned target, int nc, int* status, int* verdict) {
+__device__ bool grid_barrier(const F32Args& a, unsigned target, int nc, int* status, int* verdict) {
   block_sync<MULTI>();
   if (ctarank() == 0 && threadIdx.x == 0) {
-    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(a.bar) : "memory");
     int ok = 1;
-    unsigned spins = 0, v;
+    unsigned spins = 0, v, seen = 0;
     uint64_t t0 = 0;
     while (true) {
-      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(a.bar) : "memory");
       if (v >= target) break;
       if ((++spins & 127u) == 0) {
         int st;
+        unsigned done;
         asm volatile("ld.relaxed.gpu.global.s32 %0, [%1];" : "=r"(st) : "l"(status) : "memory");
-        if (t0 == 0) t0 = now_ns();
+        asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(done) : "l"(a.progress) : "memory");
         if (st != 0) { ok = 0; break; }
-        if (now_ns() - t0 > kWaitLimitNs) { atomicCAS(status, 0, 41); ok = 0; break; }
+        const uint64_t t = now_ns();
+        if (t0 == 0 || done != seen) { t0 = t; seen = done; }
+        if (t - t0 > a.limit_ns) { atomicCAS(status, 0, 41); ok = 0; break; }
       }
     }
     for (int c = 0; c < nc; ++c) asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(peer_addr(verdict, c)), "r"(ok) : "memory");
@@ -364,6 +373,7 @@ __global__ void __launch_bounds__(fwd_most(KC), 1) f32_fwd_kernel(const __grid_c
           }
         }
         if (!closing) block_sync<MULTI>();
+        report(a, j, rank);
       }
       if (coarse) {
         float *S = S0 + ((steps - 1) & 1) * sstride, *N = S0 + (steps & 1) * sstride;
@@ -393,7 +403,7 @@ __global__ void __launch_bounds__(fwd_most(KC), 1) f32_fwd_kernel(const __grid_c
     if (p.acc) add_norm(norm, p.acc);
     if (ip + 1 < a.nph) {
       target += ncl;
-      if (!grid_barrier<MULTI>(a.bar, target, NC, status, &verdict)) return;
+      if (!grid_barrier<MULTI>(a, target, NC, status, &verdict)) return;
     }
   }
 }
@@ -578,6 +588,7 @@ __global__ void __launch_bounds__(T, 1) f32_adj_kernel(const __grid_constant__ F
           if (!closing || coarse) form(row, u, o, m);
         });
         par ^= 1;
+        report(a, j, rank);
       }
       if (coarse) {
         __syncthreads();
@@ -598,7 +609,7 @@ __global__ void __launch_bounds__(T, 1) f32_adj_kernel(const __grid_constant__ F
     if (p.acc) add_norm(norm, p.acc);
     if (ip + 1 < a.nph) {
       target += ncl;
-      if (!grid_barrier<MULTI>(a.bar, target, NC, status, &verdict)) return;
+      if (!grid_barrier<MULTI>(a, target, NC, status, &verdict)) return;
     }
   }
   block_sync<MULTI>();      // no CTA leaves while a peer may still write its partial sums
@@ -678,6 +689,17 @@ __global__ void __launch_bounds__(fwd_most(KC), 1) f32_lin_kernel(const __grid_c
       __syncwarp();
     }
   }
+}
+
+// How long a barrier waits without progress: 2 s, or MGRIT_GRU_TEST_F32_WAIT_US microseconds from the environment.
+unsigned long long wait_limit_ns() {
+  static unsigned long long v = 0;
+  if (v == 0) {
+    const char* e = getenv("MGRIT_GRU_TEST_F32_WAIT_US");
+    const long long us = e ? atoll(e) : 0;
+    v = us > 0 && us <= 2000000 ? 1000ull * (unsigned long long)us : 2000000000ull;
+  }
+  return v;
 }
 
 // MGRIT_GRU_F32_SOLVE=0 in the environment answers as where the cooperative cluster launch is refused: the callers then advance step
@@ -761,6 +783,7 @@ bool launch_solve(bool adj, F32Args& a, const Shape& q, cudaStream_t s) {
   }
   const int ncl = clusters;
   if (ncl <= 0) return false;
+  a.limit_ns = wait_limit_ns();
   int rmax = 4, blocks = 1;
   for (int i = 0; i < a.nph; ++i) {
     F32Phase& p = a.ph[i];

@@ -37,6 +37,8 @@ struct F32Args {
   const float *gi, *b_hh;                  // forward
   const float* coef[kF32Levels][4];        // adjoint: a, c_r, c_z, c_n of every level
   unsigned* bar;                           // barrier counter, cleared by the caller
+  unsigned* progress;                      // counts up while a phase lasts (any start value)
+  unsigned long long limit_ns;             // longest wait without progress: set by the launcher
   F32Phase ph[kF32MaxPhases];
 };
 // does a solve over rows of this width fit (weights of a cluster of CTAs resident in shared memory)?
