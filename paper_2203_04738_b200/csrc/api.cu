@@ -128,9 +128,11 @@ GiTail gi_tail(const mgrit_gru_cfg* c, float* gi) {
   t.total_bytes = off;
   return t;
 }
-// the copies exist when the tensor-core engine keeps bf16 shadows of the level states (B <= 128) in an MGRIT solve
+// The copies exist when the tensor-core engine keeps bf16 shadows of the level states in an MGRIT solve and B divides 128: for other
+// batch sizes the flag's contract says that it is ignored, so that a buffer of the projection's size and one that another call
+// filled (gru_input_projection, the serial sweep) serve there.
 bool carries_copies(const mgrit_gru_cfg* c, bool serial) {
-  return !serial && (c->flags & MGRIT_FLAG_GI_CARRIES_COPIES) && c->operands == MGRIT_OPERANDS_BF16 && c->B <= 128 && c->levels > 1;
+  return !serial && (c->flags & MGRIT_FLAG_GI_CARRIES_COPIES) && c->operands == MGRIT_OPERANDS_BF16 && 128 % c->B == 0 && c->levels > 1;
 }
 
 // MGRIT_GRU_GI_BF16=0 in the environment keeps the fused kernels on the fp32 input projection (A/B measurements).
@@ -718,8 +720,7 @@ int forward_impl(const mgrit_gru_cfg* cfg_in, bool serial, const gru_params* p, 
   // (the projection is staged as bf16 where B divides 128; other batch sizes keep its fp32 values, as they always have)
   if (!gi_bf16_enabled() || 128 % c.B != 0) fw.um.gib = nullptr;
   // the caller does not read the fp32 projection and every kernel of this solve reads its bf16 copy: do not write it
-  // (where B divides 128, as the flag's contract says)
-  const bool gi_f32 = !((c.flags & MGRIT_FLAG_GI_F32_UNUSED) && carries_copies(&c, serial) && 128 % c.B == 0 && fw.um.gib);
+  const bool gi_f32 = !((c.flags & MGRIT_FLAG_GI_F32_UNUSED) && carries_copies(&c, serial) && fw.um.gib);
 
   if (c.operands == MGRIT_OPERANDS_BF16) {
     rc = umma_prepare_fwd(&c, p, x, gi_f32 ? gi : nullptr, &fw.um, s);
@@ -791,8 +792,7 @@ int adjoint_impl(const mgrit_gru_cfg* cfg_in, bool serial, const gru_params* p, 
     aw.um.xb = t.xb;
     aw.um.hb0 = t.hb0;
     aw.um.hb = t.hb0 + BH;
-    // (where B does not divide 128 the flags change no bit: the linearisation stays on the fp32 projection)
-    aw.um.gib = gi_bf16_enabled() && 128 % c.B == 0 ? t.gib : nullptr;
+    aw.um.gib = gi_bf16_enabled() ? t.gib : nullptr;
   }
   if (bf16) {
     rc = umma_prepare_adj(&c, p, h0, h, &aw.um, copies, s);
