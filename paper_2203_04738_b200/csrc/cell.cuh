@@ -1,10 +1,11 @@
 // Device arithmetic of one GRU cell evaluation and of its transposed Jacobian.
 //
-// FAST = false: precise expf/tanhf/division, used by the fp32 operand mode.
-// FAST = true : MUFU approximations (tanh.approx, rcp.approx; absolute error about 5e-4 on a gate),
-//               used by the bf16 operand mode, whose operand rounding is coarser than that.  At
-//               H = 1024 the gate arithmetic of a tile costs as many issue slots as its tensor-core
-//               main loop, so the instruction count per element matters.
+// FAST = 0: __expf, tanhf and the language's division, used by the step and chain kernels of the fp32 and tf32 operand modes.
+// FAST = 1: MUFU approximations (tanh.approx, rcp.approx; absolute error about 5e-4 on a gate),
+//           used by the bf16 operand mode, whose operand rounding is coarser than that.  At
+//           H = 1024 the gate arithmetic of a tile costs as many issue slots as its tensor-core
+//           main loop, so the instruction count per element matters.
+// FAST = 2: as 0 with a reciprocal without branches, used by the persistent fp32 solve.
 #pragma once
 #include "common.cuh"
 
@@ -23,7 +24,9 @@ __device__ __forceinline__ float rcp_approx(float x) {
 
 // 1 / x for 1 <= x < 2^125 by one Newton-Raphson step on the hardware's approximation (relative error 2^-23 before, below 2^-23
 // after it: the step squares the error, what remains is its rounding).  A division of the language brings a branch for the
-// operands it cannot take; four gates side by side have to be branch-free to hide each other's latency.
+// operands it cannot take; where a lane has four gates side by side they have to be branch-free to hide each other's latency.
+// Kernels with one gate at a time keep the division: without its branch the compiler gives the fp32 step kernel 40 instead of 52
+// registers and fewer loads in flight (forward solve at H = 512, T = 512, B = 16: 4.86 ms against 4.43).
 __device__ __forceinline__ float rcp_newton(float x) {
   const float y = rcp_approx(x);
   return fmaf(fmaf(-x, y, 1.0f), y, y);
@@ -34,17 +37,18 @@ __device__ __forceinline__ float min_nan(float a, float b) {
   asm("min.NaN.f32 %0, %1, %2;" : "=f"(y) : "f"(a), "f"(b));
   return y;
 }
-template <bool FAST> __device__ __forceinline__ float sigmoid_t(float x) {
-  if (FAST) return fmaf(tanh_approx(0.5f * x), 0.5f, 0.5f);
+template <int FAST> __device__ __forceinline__ float sigmoid_t(float x) {
+  if (FAST == 1) return fmaf(tanh_approx(0.5f * x), 0.5f, 0.5f);
+  if (FAST == 0) return 1.0f / (1.0f + __expf(-x));
   return rcp_newton(1.0f + __expf(min_nan(-x, 80.0f)));      // (below -80 the result is 1.8e-35 instead of less)
 }
-template <bool FAST> __device__ __forceinline__ float tanh_t(float x) { return FAST ? tanh_approx(x) : tanhf(x); }
-template <bool FAST> __device__ __forceinline__ float inv_t(float x) { return FAST ? rcp_approx(x) : rcp_newton(x); }
+template <int FAST> __device__ __forceinline__ float tanh_t(float x) { return FAST == 1 ? tanh_approx(x) : tanhf(x); }
+template <int FAST> __device__ __forceinline__ float inv_t(float x) { return FAST == 1 ? rcp_approx(x) : FAST == 0 ? 1.0f / x : rcp_newton(x); }
 
 // Phi_gamma(x_t, h_{t-1}) given the pre-activations: gi_* = W_i* x + b_i*, gh_* = W_h* h + b_h*.
 // classic  (Eq. "gru-classic"): h + gamma(1-z)(n - h)
 // implicit (Eq. "gru-imap")   : (h + gamma(1-z) n) / (1 + gamma(1-z))
-template <bool FAST = false>
+template <int FAST = 0>
 __device__ __forceinline__ float cell_forward(float gir, float giz, float gin, float ghr, float ghz, float ghn,
                                               float hp, float gamma, int cell) {
   float r = sigmoid_t<FAST>(gir + ghr);
@@ -58,7 +62,7 @@ struct CellLin { float a, cr, cz, cn, cnp; };
 
 // Entries of the transposed Jacobian of one step: lambda_prev = a*lam + [cr*lam|cz*lam|cn*lam] W_hh,
 // d(gi) = [cr*lam|cz*lam|cnp*lam].
-template <bool FAST = false>
+template <int FAST = 0>
 __device__ __forceinline__ CellLin cell_linearise(float gir, float giz, float gin, float ghr, float ghz, float ghn,
                                                   float hp, float gamma, int cell) {
   float r = sigmoid_t<FAST>(gir + ghr);
@@ -85,7 +89,7 @@ __device__ __forceinline__ CellLin cell_linearise(float gir, float giz, float gi
 // (implicit) or explicit (classic; gamma = 1 is the textbook LSTM); h = o tanh(c) is re-evaluated from the new c.
 // Pre-activations: gi_* = W_i* x + b_i*, gh_* = W_h* h + b_h*, gate order i | f | g | o.
 struct LstmOut { float c, h; };
-template <bool FAST = false>
+template <int FAST = 0>
 __device__ __forceinline__ LstmOut lstm_forward(float gii, float gif, float gig, float gio, float ghi, float ghf, float ghg, float gho,
                                                 float cp, float gamma, int cell) {
   float i = sigmoid_t<FAST>(gii + ghi), f = sigmoid_t<FAST>(gif + ghf), g = tanh_t<FAST>(gig + ghg), o = sigmoid_t<FAST>(gio + gho);
@@ -99,7 +103,7 @@ __device__ __forceinline__ LstmOut lstm_forward(float gii, float gif, float gig,
 // Transposed Jacobian of one LSTM step: with (L_c, L_h) the sensitivities of the outputs,
 //   dc = L_c + p*L_h;  d(pre-activations) = [ci*dc | cf*dc | cg*dc | co*L_h];  L_c_in = a*dc;  L_h_in = d(pre) W_hh
 struct LstmLin { float a, p, ci, cf, cg, co; };
-template <bool FAST = false>
+template <int FAST = 0>
 __device__ __forceinline__ LstmLin lstm_linearise(float gii, float gif, float gig, float gio, float ghi, float ghf, float ghg, float gho,
                                                   float cp, float gamma, int cell) {
   float i = sigmoid_t<FAST>(gii + ghi), f = sigmoid_t<FAST>(gif + ghf), g = tanh_t<FAST>(gig + ghg), o = sigmoid_t<FAST>(gio + gho);

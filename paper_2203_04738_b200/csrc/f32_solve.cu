@@ -243,8 +243,8 @@ __device__ __forceinline__ Pre4 fwd_parked(const float* P, float4 br, float4 bz,
   return Pre4{add4(lds4(P + l), br), add4(lds4(P + 128 + l), bz), add4(lds4(P + 256 + l), bn)};
 }
 __device__ __forceinline__ float4 cell_forward4(float4 gr, float4 gz, float4 gn, const Pre4& q, float4 h, float gamma, int cell) {
-  return make_float4(cell_forward(gr.x, gz.x, gn.x, q.r.x, q.z.x, q.n.x, h.x, gamma, cell), cell_forward(gr.y, gz.y, gn.y, q.r.y, q.z.y, q.n.y, h.y, gamma, cell),
-                     cell_forward(gr.z, gz.z, gn.z, q.r.z, q.z.z, q.n.z, h.z, gamma, cell), cell_forward(gr.w, gz.w, gn.w, q.r.w, q.z.w, q.n.w, h.w, gamma, cell));
+  return make_float4(cell_forward<2>(gr.x, gz.x, gn.x, q.r.x, q.z.x, q.n.x, h.x, gamma, cell), cell_forward<2>(gr.y, gz.y, gn.y, q.r.y, q.z.y, q.n.y, h.y, gamma, cell),
+                     cell_forward<2>(gr.z, gz.z, gn.z, q.r.z, q.z.z, q.n.z, h.z, gamma, cell), cell_forward<2>(gr.w, gz.w, gn.w, q.r.w, q.z.w, q.n.w, h.w, gamma, cell));
 }
 
 // shared: S[2][R][LD] (the whole state of the rows, this step's and the next), O[2][R][op_row] (operands of this step and the next),
@@ -327,7 +327,7 @@ __global__ void __launch_bounds__(fwd_most(KC), 1) f32_fwd_kernel(const __grid_c
           if (!closing || coarse) fetch(j + 1, closing);
           if (u < Un) {
             const float* o = O + rl * OR + u;
-            float v = cell_forward(o[0], o[U], o[2 * U], pre[0] + Bs[u], pre[1] + Bs[U + u], pre[2] + Bs[2 * U + u], S[rl * LD + c], p.gamma, a.cell);
+            float v = cell_forward<2>(o[0], o[U], o[2 * U], pre[0] + Bs[u], pre[1] + Bs[U + u], pre[2] + Bs[2 * U + u], S[rl * LD + c], p.gamma, a.cell);
             if (p.g) v += o[3 * U];
             float* n = N + rl * LD + c;
             *n = v;
@@ -675,10 +675,10 @@ __global__ void __launch_bounds__(fwd_most(KC), 1) f32_lin_kernel(const __grid_c
         const float* g = O + row * OR;
         const Pre4 t = fwd_parked(P, lds4(Bs + qu), lds4(Bs + U + qu), lds4(Bs + 2 * U + qu));
         const float4 gr = lds4(g), gz = lds4(g + U), gn = lds4(g + 2 * U), h = lds4(S + row * LD + u0 + qu);
-        const CellLin x = cell_linearise(gr.x, gz.x, gn.x, t.r.x, t.z.x, t.n.x, h.x, a.gamma, a.cell);
-        const CellLin y = cell_linearise(gr.y, gz.y, gn.y, t.r.y, t.z.y, t.n.y, h.y, a.gamma, a.cell);
-        const CellLin z = cell_linearise(gr.z, gz.z, gn.z, t.r.z, t.z.z, t.n.z, h.z, a.gamma, a.cell);
-        const CellLin w = cell_linearise(gr.w, gz.w, gn.w, t.r.w, t.z.w, t.n.w, h.w, a.gamma, a.cell);
+        const CellLin x = cell_linearise<2>(gr.x, gz.x, gn.x, t.r.x, t.z.x, t.n.x, h.x, a.gamma, a.cell);
+        const CellLin y = cell_linearise<2>(gr.y, gz.y, gn.y, t.r.y, t.z.y, t.n.y, h.y, a.gamma, a.cell);
+        const CellLin z = cell_linearise<2>(gr.z, gz.z, gn.z, t.r.z, t.z.z, t.n.z, h.z, a.gamma, a.cell);
+        const CellLin w = cell_linearise<2>(gr.w, gz.w, gn.w, t.r.w, t.z.w, t.n.w, h.w, a.gamma, a.cell);
         const i64 o = (i64)(r0 + row) * H + u0 + qu;
         *reinterpret_cast<float4*>(a.a + o) = make_float4(x.a, y.a, z.a, w.a);
         *reinterpret_cast<float4*>(a.cr + o) = make_float4(x.cr, y.cr, z.cr, w.cr);
