@@ -364,7 +364,8 @@ struct FwdCycle : Cycle {
       a.B = c->B; a.H = c->H; a.nsteps = hr.N[l]; a.u = U[l];
       const i64 st = gi_stride(l); const float* gi = gi_of(l);
       a.gi = gi + (st - 1) * (i64)BH * 3; a.gi_step = st * (i64)BH * 3;
-      a.g = G[l]; a.W = p->W_hh; a.b_hh = p->b_hh; a.gamma = hr.gamma[l]; a.cell = c->cell; a.bar = fw->chain_bar;
+      a.g = G[l]; a.W = p->W_hh; a.b_hh = p->b_hh; a.gamma = hr.gamma[l]; a.cell = c->cell;
+      a.bar = fw->chain_bar + 32;       // (the words in front are the persistent solve's)
       return serial32_fwd_solve(a, s);
     }
     if (!fw->chain_ub) return false;
@@ -524,6 +525,21 @@ struct AdjCycle : Cycle {
   }
 };
 
+// fp32 forward steps that depend on one another: the chain kernel (W_hh spread over up to 148 CTAs, 16 rows each) or a phase of the
+// persistent solve (a cluster per rows, weights in registers; above H = 256 a third of them in shared memory)?  us a step, chain /
+// persistent: 16 rows, H = 160 2.97 / 2.82, 192 3.14 / 3.17 (one row 2.90 / 3.13), 224 3.28 / 2.73, 256 3.56 / 3.00, 288 3.60 / 4.50,
+// 320 3.89 / 4.55, 352 3.92 / 4.71; where eight units a CTA do not fit one wave the chain loses (64 rows, H = 320 5.23 / 4.63)
+// until the rows take the persistent clusters of eight a second wave (128 rows, H = 224 4.43 / 4.80, 288 5.12 / 8.26).  Inside a
+// solve the chain is two more launches, 25 us.  Two levels, T = 2048, cf = 2, one row, a forward solve of two cycles: H = 192 6.49 ->
+// 5.91 ms, 288 9.23 -> 6.90, 352 9.72 -> 7.23.  (Adjoint phases win but for single cells of H = 288: H = 256, 16 rows 4.65 / 2.78.)
+bool chain32_wins(const mgrit_gru_cfg* c, int nsteps, bool alone) {
+  const int units = serial32_fwd_units(c->B, c->H);
+  int gain_ns = 0;
+  if (units == 8) gain_ns = c->H > 256 ? 800 : c->H == 192 ? 150 : 0;
+  else if (units > 0 && c->H > 192 && c->B > 120) gain_ns = 400;
+  return gain_ns > 0 && (alone || (i64)nsteps * gain_ns >= 25000);
+}
+
 // The whole solve of an fp32-state GRU recurrence as phases of the persistent kernels in f32_solve.cu.  The same cycle as
 // Cycle::cycle, phase by phase; what differs is where C-points travel: a C-relaxation of level l leaves its results in the
 // coarse array U[l+1] (which the restriction would fill with them anyway) and the next one back in U[l], so that no row of
@@ -536,6 +552,7 @@ struct F32Cycle {
   int cycle_idx = 0;
   i64 bh() const { return (i64)c->B * c->H; }
   unsigned* bars = nullptr; int bars_left = 0;      // cleared barrier counters, one per launch
+  Cycle* by_steps = nullptr;                        // forward: its chain serves the coarsest level where that is faster
   void flush() {
     if (a.nph > 0 && ok) {
       unsigned* const own = a.bar;
@@ -569,10 +586,14 @@ struct F32Cycle {
     const i64 BH = bh();
     const int cf = c->cf, N = hr->N[l];
     if (l == hr->L - 1) {
+      homog = false;
+      if (by_steps && chain32_wins(c, N, l == 0)) {
+        flush();
+        if (ok && by_steps->chain(l)) { started = true; return; }
+      }
       F32Phase p = phase(l, U[l], 0, 0);
       p.nk = p.nfull = 1; p.n = N;
       add(p);
-      homog = false;
       return;
     }
     const int nc = hr->N[l + 1], tail = N % cf, relax = l == 0 ? c->relax_fine : c->relax_coarse;
@@ -752,6 +773,7 @@ int forward_impl(const mgrit_gru_cfg* cfg_in, bool serial, const gru_params* p, 
     F32Cycle fc;
     fc.c = &c; fc.hr = &hr; fc.adjoint = false; fc.s = s; fc.U = fw.U; fc.G = fw.G; fc.res_acc = fw.res_acc;
     fc.a.B = c.B; fc.a.H = c.H; fc.a.cell = c.cell; fc.a.W = p->W_hh; fc.a.gi = gi; fc.a.b_hh = p->b_hh; fc.a.bar = fw.chain_bar;
+    fc.by_steps = &cy;
     rc = fc.solve(&setup);
   }
   if (rc == MGRIT_UNSUPPORTED) rc = cy.solve(&setup);
@@ -1078,7 +1100,8 @@ struct StackFwdCycle : StackCycle {
   void coarsest(int l) override {
     for (int k = 0; k < nl && status() == MGRIT_OK; ++k) {
       FwdCycle& q = y[k];
-      if (!run_fp32(q, k, l, 1, false, kNone) && !q.chain(l))
+      const bool chain_first = c->operands == MGRIT_OPERANDS_FP32 && chain32_wins(c, hr.N[l], true);
+      if (!(chain_first && q.chain(l)) && !run_fp32(q, k, l, 1, false, kNone) && !q.chain(l))
         for (int j = 1; j <= hr.N[l]; ++j) q.step(StepDesc{l, 1, j - 1, 1, q.U[l], j, 1, q.G[l], j, 1, j, 1, 0});
       feed(k, l, false);
     }

@@ -57,6 +57,7 @@ struct Serial32AdjArgs {
   const float* W;                // [3H][H] fp32 (W_hh as given)
   unsigned* bar;
 };
+int serial32_fwd_units(int B, int H);      // hidden units per CTA of the forward chain, 0: not available
 bool serial32_fwd_solve(const Serial32FwdArgs& a, cudaStream_t s);
 bool serial32_adj_solve(const Serial32AdjArgs& a, cudaStream_t s);
 

@@ -1442,8 +1442,9 @@ static bool chain32_enabled() {
   return v == 1;
 }
 
+int serial32_fwd_units(int B, int H) { return chain32_enabled() ? pick_unc32(B, H, false) : 0; }
 bool serial32_fwd_solve(const Serial32FwdArgs& a, cudaStream_t s) {
-  const int unc = chain32_enabled() ? pick_unc32(a.B, a.H, false) : 0;
+  const int unc = serial32_fwd_units(a.B, a.H);
   if (unc == 0 || a.nsteps <= 0 || !a.bar || !status_ptr()) return false;
   const size_t smem = fwd32_smem(unc, a.H);
   prof_begin(KC_FWD_SERIAL, 2.0 * a.B * 3.0 * a.H * a.H * a.nsteps, s);
