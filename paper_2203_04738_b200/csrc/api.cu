@@ -527,11 +527,12 @@ struct AdjCycle : Cycle {
 
 // fp32 forward steps that depend on one another: the chain kernel (W_hh spread over up to 148 CTAs, 16 rows each) or a phase of the
 // persistent solve (a cluster per rows, weights in registers; above H = 256 a third of them in shared memory)?  us a step, chain /
-// persistent: 16 rows, H = 160 2.97 / 2.82, 192 3.14 / 3.17 (one row 2.90 / 3.13), 224 3.28 / 2.73, 256 3.56 / 3.00, 288 3.60 / 4.50,
-// 320 3.89 / 4.55, 352 3.92 / 4.71; where eight units a CTA do not fit one wave the chain loses (64 rows, H = 320 5.23 / 4.63)
-// until the rows take the persistent clusters of eight a second wave (128 rows, H = 224 4.43 / 4.80, 288 5.12 / 8.26).  Inside a
+// persistent: 16 rows, H = 160 2.97 / 2.82, 192 3.14 / 3.17 (one row 2.90 / 3.13), 224 3.28 / 2.73, 256 3.56 / 3.00, 288 3.59 / 4.03,
+// 320 3.88 / 4.17, 352 3.94 / 4.70; where eight units a CTA do not fit one wave the chain loses (64 rows, H = 320 5.23 / 4.24)
+// until the rows take the persistent clusters of eight a second wave (128 rows, H = 224 4.43 / 4.80, 288 5.12 / 6.96).  Inside a
 // solve the chain is two more launches, 25 us.  Two levels, T = 2048, cf = 2, one row, a forward solve of two cycles: H = 192 6.49 ->
-// 5.91 ms, 288 9.23 -> 6.90, 352 9.72 -> 7.23.  (Adjoint phases win but for single cells of H = 288: H = 256, 16 rows 4.65 / 2.78.)
+// 5.91 ms, 304 (no multiple of 32: no chain) 8.66, 320 7.0, 352 9.72 -> 7.23.  (Adjoint phases win everywhere: H = 288, 16 rows
+// 5.17 / 3.94.)
 bool chain32_wins(const mgrit_gru_cfg* c, int nsteps, bool alone) {
   const int units = serial32_fwd_units(c->B, c->H);
   int gain_ns = 0;
@@ -664,9 +665,9 @@ struct F32Cycle {
 
 // Which fp32-state solves run there: every one of the fp32 mode whose weights fit, and those of the tf32 split whose steps are
 // too small for the tensor cores (rows of the largest step x H^2).  Forward and adjoint us a step there: H = 256 500 rows 11.1 and
-// 8.4, 1200 rows 22 and 18, 1700 rows 32 and 26; H = 320 700 rows 23 and 26, 1100 rows 41 and 44.  The tensor-core step takes
+// 8.4, 1200 rows 22 and 18, 1700 rows 32 and 26; H = 320 700 rows 25 and 25, 1100 rows 41 and 39.  The tensor-core step takes
 // 27 + 6 and 24 + 4 us (product and operand split, one wave of tiles) at 512 rows and hardly more at 2000.  They meet at
-// 900 (H = 320) to 1700 rows (H = 256); the line is the lower one.  Linearisation at H = 256: 2560 rows 45 against 58 us, 5120 rows 84.
+// 800 to 900 (H = 320) and 1700 rows (H = 256); the line is the lower one.  Linearisation at H = 256: 2560 rows 45 against 58 us, 5120 rows 84.
 constexpr double kF32TfStep = 9e7, kF32TfLin = 2.2e8;
 bool use_f32_solve(const mgrit_gru_cfg* c, const Hier& hr) {
   if (!f32_solve_fits(c->H)) return false;

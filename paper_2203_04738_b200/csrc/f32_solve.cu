@@ -23,7 +23,9 @@
 // latency: a CTA has the registers for 6 to 12 warps, two or three per scheduler, which issue in half of the cycles.
 // us a step, forward / adjoint, weights in shared memory -> in registers:
 //   H = 32, 2 rows 1.4 / 1.9 -> 0.87 / 1.2; H = 104, 3300 rows 15 / 16 -> 12.3 / 11.5; H = 256, 16 rows 3.3 / 3.2 -> 2.9 / 2.0,
-//   500 rows 14.7 / 11.8 -> 11.1 / 8.4 (18 and 24 TFLOP/s); H = 320, 16 rows 4.1 / 4.4 -> 4.4 / 3.5, 700 rows 28 / 23 -> 23 / 26.
+//   500 rows 14.7 / 11.8 -> 11.1 / 8.4 (18 and 24 TFLOP/s); H = 320, 16 rows 4.1 / 4.4 -> 4.4 / 3.6, 700 rows 28 / 23 -> 29 / 32.
+// There every width above 256 was padded to 352 columns; padded to the next 32 (adjoint: its own operand words) H = 320 takes
+// 4.0 / 3.1 and 25 / 25, H = 288, 700 rows 27 / 32 -> 22 / 25.
 #include <stdlib.h>
 
 #include "cell.cuh"
@@ -725,14 +727,14 @@ int* status_ptr() {
 struct Shape { int NC, U, KC, fwd_threads, adj_kp, adj_kc, adj_threads; size_t fwd_row, fwd_fix, adj_row, adj_fix; };
 bool pick_shape(int H, Shape* q) {
   if (H % 8 != 0 || H > 352) return false;
-  q->KC = H <= 256 ? (H + 31) / 32 : 11;
+  q->KC = (H + 31) / 32;
   const int nc = H <= 96 ? 1 : H <= 128 ? 2 : H <= 192 ? 4 : 8;      // at most 96 (NU = 2) or 48 (NU = 1) units per CTA: 384 threads
   q->U = ((H + nc - 1) / nc + 3) / 4 * 4;
   q->NC = (H + q->U - 1) / q->U;
   const int nu = q->KC <= 4 ? 2 : 1;
   q->fwd_threads = ((q->U + nu - 1) / nu * 8 + 31) / 32 * 32;
   q->adj_kp = H <= 96 ? 32 : H <= 192 ? 16 : 8;
-  q->adj_kc = H <= 256 ? (3 * q->U / 4 + q->adj_kp - 1) / q->adj_kp : 5;
+  q->adj_kc = (3 * q->U / 4 + q->adj_kp - 1) / q->adj_kp;
   q->adj_threads = (H / 8 * q->adj_kp + 31) / 32 * 32;
   const int lda = 3 * q->U > 4 * q->adj_kp * q->adj_kc ? 3 * q->U : 4 * q->adj_kp * q->adj_kc, pad = nu == 2 ? 8 : 4;
   q->fwd_row = (size_t)2 * (32 * q->KC + pad + 4 * q->U + pad) * 4;
@@ -817,7 +819,9 @@ bool f32_solve(bool adjoint, F32Args& a, cudaStream_t s) {
       return q.adj_kc == 2             ? launch_solve<f32_adj_kernel<true, 16, 2, 384>>(true, a, q, s)
              : q.adj_threads <= 256 ? launch_solve<f32_adj_kernel<true, 16, 3, 256>>(true, a, q, s)
                                     : launch_solve<f32_adj_kernel<true, 16, 3, 384>>(true, a, q, s);
-    return q.adj_kc == 3 ? launch_solve<f32_adj_kernel<true, 8, 3, 256>>(true, a, q, s) : launch_solve<f32_adj_kernel<true, 8, 5, 384>>(true, a, q, s);
+    return q.adj_kc == 3   ? launch_solve<f32_adj_kernel<true, 8, 3, 256>>(true, a, q, s)
+           : q.adj_kc == 4 ? launch_solve<f32_adj_kernel<true, 8, 4, 384>>(true, a, q, s)
+                           : launch_solve<f32_adj_kernel<true, 8, 5, 384>>(true, a, q, s);
   }
   switch (q.KC) {
     case 1: return launch_solve<f32_fwd_kernel<false, 1>>(false, a, q, s);
@@ -828,6 +832,8 @@ bool f32_solve(bool adjoint, F32Args& a, cudaStream_t s) {
     case 6: return launch_solve<f32_fwd_kernel<true, 6>>(false, a, q, s);
     case 7: return launch_solve<f32_fwd_kernel<true, 7>>(false, a, q, s);
     case 8: return launch_solve<f32_fwd_kernel<true, 8>>(false, a, q, s);
+    case 9: return launch_solve<f32_fwd_kernel<true, 9>>(false, a, q, s);
+    case 10: return launch_solve<f32_fwd_kernel<true, 10>>(false, a, q, s);
     default: return launch_solve<f32_fwd_kernel<true, 11>>(false, a, q, s);
   }
 }
@@ -867,6 +873,8 @@ bool f32_linearise(const LinArgs* levels, int n, cudaStream_t s) {
     case 6: return launch_lin<6>(ls, q, gx, gy, R, s);
     case 7: return launch_lin<7>(ls, q, gx, gy, R, s);
     case 8: return launch_lin<8>(ls, q, gx, gy, R, s);
+    case 9: return launch_lin<9>(ls, q, gx, gy, R, s);
+    case 10: return launch_lin<10>(ls, q, gx, gy, R, s);
     default: return launch_lin<11>(ls, q, gx, gy, R, s);
   }
 }
