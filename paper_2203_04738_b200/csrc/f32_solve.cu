@@ -787,8 +787,11 @@ bool launch_solve(bool adj, F32Args& a, const Shape& q, cudaStream_t s) {
   if (ncl <= 0) return false;
   a.limit_ns = wait_limit_ns();
   int rmax = 4, blocks = 1;
+  double steps = 0;       // cell evaluations of all phases, in rows
   for (int i = 0; i < a.nph; ++i) {
     F32Phase& p = a.ph[i];
+    const int full = p.nk < p.nfull ? p.nk : p.nfull;
+    steps += ((double)full * (p.n + p.last_kind) + (double)(p.nk - full) * p.ntail) * a.B;      // (kLastStore one step more, kLastCoarse two)
     tune(adj, p, q, ncl, p.nk * a.B);
     if (p.R > rmax) rmax = p.R;
     const int nb = (p.nk * a.B + p.R - 1) / p.R;
@@ -796,6 +799,7 @@ bool launch_solve(bool adj, F32Args& a, const Shape& q, cudaStream_t s) {
   }
   if (blocks > ncl) blocks = ncl;
   cfg.gridDim = dim3(blocks * q.NC); cfg.dynamicSmemBytes = fix + row * rmax; cfg.stream = s; cfg.numAttrs = 2;
+  ProfScope prof(adj ? KC_ADJ_STEP : KC_FWD_STEP, 6.0 * steps * a.H * a.H, s);
   if (cudaLaunchKernelEx(&cfg, kern, a, q.NC, q.U, rmax, st) != cudaSuccess) { cudaGetLastError(); return false; }
   count_launch();
   return true;
