@@ -1,5 +1,5 @@
-"""The persistent fp32 solve: row blocks with more rows than a block has threads (H = 8 runs on 32), and the sizes around which the
-coarsest level of the forward solve goes to the chain kernel.  Forward, adjoint and gradients against the fp64 oracle at the same
+"""The persistent fp32 solve: row blocks with more rows than a block has threads (H = 8 runs on 32), several row blocks per cluster,
+and the sizes around which the coarsest level of the forward solve goes to the chain kernel.  Forward, adjoint and gradients against the fp64 oracle at the same
 cycle count."""
 import numpy as np
 import pytest
@@ -60,4 +60,15 @@ CHAIN_OR_PHASE = [(7, 64, 192, 2, 1, 0, 0, 1), (7, 100, 192, 2, 1, 0, 0, 1), (9,
 
 @pytest.mark.parametrize("c", CHAIN_OR_PHASE, ids=lambda c: "T{}B{}H{}cf{}L{}r{}{}i{}".format(*c))
 def test_coarsest_level_on_the_chain_or_as_a_phase(c):
+    solve_against_the_oracle(*c)
+
+
+# more rows than one wave of row blocks holds, for every size of cluster (148, 74, some 35 and some 16 of them with up to 64 rows each; H = 96
+# and above 256 fewer): clusters take a second and a third block, whose buffers their peers have to be done with
+SEVERAL_BLOCKS = [(1024, 48, 32, 4, 2, 0, 1, 1), (512, 64, 96, 4, 2, 1, 0, 1), (515, 44, 104, 4, 2, 1, 1, 1), (259, 50, 136, 4, 3, 0, 1, 2),
+                  (256, 50, 192, 4, 2, 1, 0, 1), (131, 50, 224, 4, 2, 1, 1, 1), (128, 50, 256, 4, 2, 0, 1, 1), (128, 50, 288, 4, 2, 1, 0, 1), (130, 30, 352, 4, 2, 0, 1, 1)]
+
+
+@pytest.mark.parametrize("c", SEVERAL_BLOCKS, ids=lambda c: "T{}B{}H{}cf{}L{}r{}{}i{}".format(*c))
+def test_clusters_with_several_row_blocks(c):
     solve_against_the_oracle(*c)
