@@ -1224,6 +1224,10 @@ bool serial_fwd_supported(int B, int H) { return pick_unc(B, H, false) != 0; }
 bool serial_adj_supported(int B, int H) { return pick_unc(B, H, true) != 0; }
 
 // MGRIT_GRU_CHAIN_WREG=0 in the environment keeps the chains' weight fragments in shared memory (same results).
+// The fragments' count, H / 128 (adjoint 3H / 128, the LSTM's 4H / 128) k-steps per warp, is a template argument, so every width costs
+// kernels of its own.  They exist for H = 512 and 1024; us a step, registers / shared memory, forward and unsplit adjoint: H = 512,
+// 8 rows 1.72 / 1.86 and 1.70 / 1.90, 32 rows 2.07 / 2.21 and 2.01 / 2.20; H = 1024, 8 rows 1.94 / 2.25 and 2.08 / 2.40, 32 rows
+// 2.66 / 3.00 and 4.67 / 4.96.  Other widths read them from shared memory: H = 256, 8 rows 1.72 and 1.58, H = 768 2.06 and 2.22.
 static bool chain_wreg_enabled() {
   static int v = -1;
   if (v < 0) { const char* e = getenv("MGRIT_GRU_CHAIN_WREG"); v = (e && e[0] == '0') ? 0 : 1; }
@@ -1233,6 +1237,8 @@ static bool chain_wreg_enabled() {
 namespace {
 // Rows that travel between the CTAs of a row group: with few batch rows most of a sixteen-row block would be zeros, and every
 // CTA polls every block (8 rows at H = 1024: forward 2.05 -> 1.88 us a step, adjoint 3.43 -> 2.00).
+// Kernels that no shape reaches are not instantiated (every one of them is loaded code): up to eight rows are one row group, whose
+// slices are 8 units wide up to H = 1184 and 16 above; 32 units and the register-resident weights of 16 come with more rows.
 template <class F> bool by_rows(int B, F f) {
   if (B <= 4) return f(std::integral_constant<int, 4>());
   if (B <= 8) return f(std::integral_constant<int, 8>());
@@ -1255,10 +1261,13 @@ bool serial_fwd_solve(const SerialFwdArgs& a, cudaStream_t s) {
       constexpr int RL = decltype(rl)::value;
       auto go = [&](auto kern) { return launch_coop(kern, a, unc, RL, smem, true, 1, s); };
       if (wreg && a.H == 1024 && unc == 8) return go(serial_fwd_kernel<8, true, RL, 8>);
-      if (wreg && a.H == 1024 && unc == 16) return go(serial_fwd_kernel<16, true, RL, 8>);
       if (wreg && a.H == 512 && unc == 8) return go(serial_fwd_kernel<8, true, RL, 4>);
-      if (wreg && a.H == 512 && unc == 16) return go(serial_fwd_kernel<16, true, RL, 4>);
-      return unc == 8 ? go(serial_fwd_kernel<8, true, RL>) : unc == 16 ? go(serial_fwd_kernel<16, true, RL>) : go(serial_fwd_kernel<32, true, RL>);
+      if constexpr (RL == kRows) {
+        if (wreg && a.H == 1024 && unc == 16) return go(serial_fwd_kernel<16, true, RL, 8>);
+        if (wreg && a.H == 512 && unc == 16) return go(serial_fwd_kernel<16, true, RL, 4>);
+        if (unc == 32) return go(serial_fwd_kernel<32, true, RL>);
+      }
+      return unc == 8 ? go(serial_fwd_kernel<8, true, RL>) : unc == 16 ? go(serial_fwd_kernel<16, true, RL>) : false;
     });
   }
   prof_end(s);
@@ -1304,8 +1313,18 @@ bool launch_adj_split(const typename AdjChainArgs<NG>::type& a, cudaStream_t s) 
 }
 template <int NG, int RL>
 bool adj_split_solve(const typename AdjChainArgs<NG>::type& a, bool wreg, cudaStream_t s) {
-  if (wreg && a.H == 1024) return launch_adj_split<NG, 8, RL, 8>(a, s) || launch_adj_split<NG, 16, RL, 8>(a, s);
-  if (wreg && a.H == 512) return launch_adj_split<NG, 8, RL, 4>(a, s) || launch_adj_split<NG, 16, RL, 4>(a, s);
+  // (what split_pays() lets through: at H = 1024 the GRU with more than eight rows and the LSTM with more than four, at H = 512 the
+  // LSTM with more than eight)
+  if constexpr (RL == kRows || (NG == 4 && RL == 8)) {
+    if (wreg && a.H == 1024) {
+      if (launch_adj_split<NG, 8, RL, 8>(a, s)) return true;
+      if constexpr (RL == kRows) return launch_adj_split<NG, 16, RL, 8>(a, s);
+      return false;
+    }
+  }
+  if constexpr (NG == 4 && RL == kRows) {
+    if (wreg && a.H == 512) return launch_adj_split<NG, 8, RL, 4>(a, s) || launch_adj_split<NG, 16, RL, 4>(a, s);
+  }
   return launch_adj_split<NG, 8, RL>(a, s) || launch_adj_split<NG, 16, RL>(a, s);
 }
 // Splitting costs a cluster barrier and the exchange of the sums (about 0.6 us a step) and pays where the unsplit kernel's words
@@ -1345,10 +1364,13 @@ bool serial_adj_solve(const SerialAdjArgs& a, cudaStream_t s) {
       constexpr int RL = decltype(rl)::value;
       auto go = [&](auto kern) { return launch_coop(kern, a, unc, RL, smem, true, 3, s); };
       if (wreg && a.H == 1024 && unc == 8) return go(serial_adj_kernel<8, true, RL, 24>);
-      if (wreg && a.H == 1024 && unc == 16) return go(serial_adj_kernel<16, true, RL, 24>);
       if (wreg && a.H == 512 && unc == 8) return go(serial_adj_kernel<8, true, RL, 12>);
-      if (wreg && a.H == 512 && unc == 16) return go(serial_adj_kernel<16, true, RL, 12>);
-      return unc == 8 ? go(serial_adj_kernel<8, true, RL>) : unc == 16 ? go(serial_adj_kernel<16, true, RL>) : go(serial_adj_kernel<32, true, RL>);
+      if constexpr (RL == kRows) {
+        if (wreg && a.H == 1024 && unc == 16) return go(serial_adj_kernel<16, true, RL, 24>);
+        if (wreg && a.H == 512 && unc == 16) return go(serial_adj_kernel<16, true, RL, 12>);
+        if (unc == 32) return go(serial_adj_kernel<32, true, RL>);
+      }
+      return unc == 8 ? go(serial_adj_kernel<8, true, RL>) : unc == 16 ? go(serial_adj_kernel<16, true, RL>) : false;
     });
   }
   prof_end(s);
@@ -1410,7 +1432,11 @@ bool lstm_chain_fwd_solve(const LstmChainFwdArgs& a, cudaStream_t s) {
   const bool ok = by_rows(a.B, [&](auto rl) {
     constexpr int RL = decltype(rl)::value;
     auto go = [&](auto kern) { return launch_lstm_chain(kern, a, unc, RL, smem, 1, s); };
-    return unc == 8 ? go(lstm_fwd_chain_kernel<8, RL>) : unc == 16 ? go(lstm_fwd_chain_kernel<16, RL>) : go(lstm_fwd_chain_kernel<32, RL>);
+    if constexpr (RL == kRows) {
+      if (unc == 16) return go(lstm_fwd_chain_kernel<16, RL>);
+      if (unc == 32) return go(lstm_fwd_chain_kernel<32, RL>);
+    }
+    return unc == 8 ? go(lstm_fwd_chain_kernel<8, RL>) : false;      // (four slices of 16 units do not fit shared memory above H = 1184)
   });
   prof_end(s);
   return ok;
@@ -1429,7 +1455,10 @@ bool lstm_chain_adj_solve(const LstmChainAdjArgs& a, cudaStream_t s) {
   prof_begin(KC_ADJ_SERIAL, 2.0 * a.B * 4.0 * a.H * a.H * a.nsteps, s);
   const bool ok = by_rows(a.B, [&](auto rl) {
     constexpr int RL = decltype(rl)::value;
-    return unc == 8 ? launch_lstm_adj<8, RL>(a, smem, s) : launch_lstm_adj<16, RL>(a, smem, s);
+    if constexpr (RL == kRows) {
+      if (unc == 16) return launch_lstm_adj<16, RL>(a, smem, s);
+    }
+    return unc == 8 ? launch_lstm_adj<8, RL>(a, smem, s) : false;
   });
   prof_end(s);
   return ok;
