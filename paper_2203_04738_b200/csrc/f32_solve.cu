@@ -705,7 +705,7 @@ unsigned long long wait_limit_ns() {
 }
 
 // MGRIT_GRU_F32_SOLVE=0 in the environment answers as where the cooperative cluster launch is refused: the callers then advance step
-// by step, as at widths that do not fit.
+// by step, as at widths that do not fit (the linearisation, which is no cooperative launch, goes with it).
 bool solve_enabled() {
   static int v = -1;
   if (v < 0) { const char* e = getenv("MGRIT_GRU_F32_SOLVE"); v = (e && e[0] == '0') ? 0 : 1; }
@@ -855,7 +855,7 @@ template <int KC> bool launch_lin(const LinSet& ls, const Shape& q, int gx, int 
 bool f32_linearise(const LinArgs* levels, int n, cudaStream_t s) {
   Shape q;
   const int H = levels[0].H;
-  if (!pick_shape(H, &q)) return false;
+  if (!solve_enabled() || !pick_shape(H, &q)) return false;
   LinSet ls;
   ls.n = n;
   i64 rows = 0;
