@@ -145,6 +145,7 @@ bool gi_bf16_enabled() {
 struct FwdWs {
   float* U[kMaxLevels]; float* G[kMaxLevels]; double* res_acc; UmmaFwdWs um; Tf32Ws tf;
   __nv_bfloat16* chain_ub; unsigned* chain_bar; uint4* chain_xw; size_t chain_xw_bytes;   // scratch of the persistent serial-chain kernel
+  unsigned chain_steps;                           // steps of its chains so far (the words are cleared once per call)
   __nv_bfloat16* Ub[kMaxLevels];                  // bf16 copies of the level states (tensor-core A operands)
   int* sweep_ctr; size_t sweep_ctr_n, sweep_ctr_used;   // progress counters of the multi-step relaxation launches (zeroed per call)
 };
@@ -154,7 +155,7 @@ struct AdjWs {
   __nv_bfloat16 *crb[kMaxLevels], *czb[kMaxLevels], *cnb[kMaxLevels], *cnpb;       // ... tensor-core engine (bf16)
   float *dA_h, *dA_i, *lam_tmp; double* res_acc; UmmaAdjWs um; Tf32Ws tf;
   float* grad_scratch;      // fp32 engine: partial weight gradients
-  __nv_bfloat16* chain_dAb; unsigned* chain_bar; uint4* chain_xw; size_t chain_xw_bytes;
+  __nv_bfloat16* chain_dAb; unsigned* chain_bar; uint4* chain_xw; size_t chain_xw_bytes; unsigned chain_steps;
   float* chain_dA32;        // fp32 chain: [2][B][3H] operand exchange
 };
 
@@ -165,7 +166,7 @@ void plan_fwd(const mgrit_gru_cfg* c, const Hier& hr, Ws& w, FwdWs* o) {
     o->G[l] = l == 0 ? nullptr : w.take<float>((size_t)(hr.N[l] + 1) * BH);
   }
   o->res_acc = w.take<double>((size_t)(c->iters > 0 ? c->iters : 1));
-  o->chain_ub = nullptr; o->chain_bar = nullptr; o->chain_xw = nullptr; o->chain_xw_bytes = 0;
+  o->chain_ub = nullptr; o->chain_bar = nullptr; o->chain_xw = nullptr; o->chain_xw_bytes = 0; o->chain_steps = 0;
   o->sweep_ctr = nullptr; o->sweep_ctr_n = o->sweep_ctr_used = 0;
   for (int l = 0; l < kMaxLevels; ++l) o->Ub[l] = nullptr;
   if (c->operands == MGRIT_OPERANDS_BF16) {
@@ -204,6 +205,7 @@ void plan_adj(const mgrit_gru_cfg* c, const Hier& hr, Ws& w, AdjWs* o) {
   if (c->operands == MGRIT_OPERANDS_BF16) { o->cnp = nullptr; o->cnpb = w.take<__nv_bfloat16>((size_t)hr.N[0] * BH); }
   else { o->cnpb = nullptr; o->cnp = w.take<float>((size_t)hr.N[0] * BH); }
   o->res_acc = w.take<double>((size_t)(c->iters > 0 ? c->iters : 1));
+  o->chain_steps = 0;
   if (c->operands == MGRIT_OPERANDS_BF16) {
     o->dA_h = o->dA_i = o->lam_tmp = o->grad_scratch = nullptr;
     umma_plan_adj(c, hr.N, hr.L, w.base, &w.off, &o->um);
@@ -378,7 +380,7 @@ struct FwdCycle : Cycle {
     a.gi_as_bf16 = (gib && hr.L > 1) ? 1 : 0;
     if (!gi_f32) { a.gi_b = gib + (st - 1) * (i64)BH * 3; a.gi = nullptr; }
     a.g = G[l]; a.W = um->W_hh; a.b_hh = p->b_hh; a.gamma = hr.gamma[l]; a.cell = c->cell; a.bar = fw->chain_bar;
-    a.xw = fw->chain_xw; a.xw_bytes = fw->chain_xw_bytes;
+    a.xw = fw->chain_xw; a.xw_bytes = fw->chain_xw_bytes; a.step0 = fw->chain_steps; fw->chain_steps += hr.N[l];
     return serial_fwd_solve(a, s) || chain_by_sweeps(l);
   }
   // The dependent steps of a level whose rows and weights do not fit the chain kernel (many batch rows at a large width): sweeps
@@ -485,14 +487,14 @@ struct AdjCycle : Cycle {
       return serial32_adj_solve(a, s);
     }
     if (!w->chain_dAb) return false;
-    SerialAdjArgs a;
+    SerialAdjArgs a{};
     a.B = c->B; a.H = c->H; a.nsteps = hr.N[l];
     a.mu = mu; a.dAb = w->chain_dAb;
     i64 row0 = (i64)(hr.N[l] - 1) * BH;        // step s = 1 applies forward step N_l, stored at row N_l - 1
     a.a = w->a[l] + row0; a.cr = w->crb[l] + row0; a.cz = w->czb[l] + row0; a.cn = w->cnb[l] + row0;
     a.coef_step = -(i64)BH;
     a.g = g; a.WT = w->um.W_hhT; a.bar = w->chain_bar;
-    a.xw = w->chain_xw; a.xw_bytes = w->chain_xw_bytes;
+    a.xw = w->chain_xw; a.xw_bytes = w->chain_xw_bytes; a.step0 = w->chain_steps; w->chain_steps += hr.N[l];
     return serial_adj_solve(a, s);
   }
   int launch_step(const StepDesc& d) override {
@@ -756,6 +758,7 @@ int forward_impl(const mgrit_gru_cfg* cfg_in, bool serial, const gru_params* p, 
   Setup setup(s);
   zero_guess(fw.U[0], c, hr, BH, &setup);
   for (int l = 0; l < hr.L; ++l) setup.copy(fw.U[l], h0, BH);
+  if (fw.chain_xw) setup.zero(fw.chain_xw, fw.chain_xw_bytes);
   const bool shadows = c.operands == MGRIT_OPERANDS_BF16 && c.B <= 128;
   if (shadows && fw.sweep_ctr) setup.zero(fw.sweep_ctr, sizeof(int) * fw.sweep_ctr_n);
   if (shadows) {
@@ -852,6 +855,7 @@ int adjoint_impl(const mgrit_gru_cfg* cfg_in, bool serial, const gru_params* p, 
   zero_guess(aw.U[0], c, hr, BH, &setup);        // (slot 0 is set below)
   const float* const last = dh_seed ? dh_seed + (size_t)(T - 1) * BH : dhT;
   for (int l = 0; l < hr.L; ++l) setup.copy(aw.U[l], last, BH, dh_seed ? dhT : nullptr);
+  if (aw.chain_xw) setup.zero(aw.chain_xw, aw.chain_xw_bytes);
   if (dh_seed) {
     setup.zero(aw.G[0], sizeof(float) * BH);
     setup.zero(aw.G[0] + (size_t)T * BH, sizeof(float) * BH);
@@ -1152,6 +1156,7 @@ int stack_forward_impl(const mgrit_gru_cfg* cfg, int nl, const gru_params* p, co
     ck[k] = layer_cfg(c, k);
     zero_guess(q.U[0], c, hr, bh, &setup);
     for (int l = 0; l < hr.L; ++l) setup.copy(q.U[l], h0 + k * bh, bh);
+    if (q.chain_xw) setup.zero(q.chain_xw, q.chain_xw_bytes);
     if (fused) {
       setup.zero(q.sweep_ctr, sizeof(int) * q.sweep_ctr_n);
       zero_guess(q.Ub[0], c, hr, bh, &setup);
@@ -1400,6 +1405,7 @@ int stack_adjoint_impl(const mgrit_gru_cfg* cfg, int nl, const gru_params* p, co
     AdjWs& q = aw.L[k].w;
     ck[k] = layer_cfg(c, k);
     zero_guess(q.U[0], c, hr, bh, &setup);
+    if (q.chain_xw) setup.zero(q.chain_xw, q.chain_xw_bytes);
     for (int l = 0; l < hr.L; ++l) Gl[k][l] = q.G[l];
     if (!dh_seed) Gl[k][0] = nullptr;
     const float* const seed = dh_seed ? dh_seed + (size_t)(T - 1) * slot + k * bh : nullptr;
@@ -1449,14 +1455,14 @@ int stack_adjoint_impl(const mgrit_gru_cfg* cfg, int nl, const gru_params* p, co
 // the same Cycle drives them.  fp32 engine only (four-gate FFMA products).
 struct LstmFwdWs {
   float* U[kMaxLevels]; float* G[kMaxLevels]; double* res_acc; float *tmpC, *tmpH; size_t maxM; Tf32Ws tf; LstmBfWs bf;
-  uint4* chain_xw; size_t chain_xw_bytes;      // exchange words of the persistent chain kernel (bf16 operands)
+  uint4* chain_xw; size_t chain_xw_bytes; unsigned chain_steps;      // exchange words of the persistent chain kernel (bf16 operands)
 };
 struct LstmAdjWs {
   float* U[kMaxLevels]; float* G[kMaxLevels]; double* res_acc;
   float *a[kMaxLevels], *p[kMaxLevels], *ci[kMaxLevels], *cf[kMaxLevels], *cg[kMaxLevels], *co[kMaxLevels];
   __nv_bfloat16 *cib[kMaxLevels], *cfb[kMaxLevels], *cgb[kMaxLevels], *cob[kMaxLevels];    // bf16 operands: the gate coefficients as bf16 instead
   float *tmpC, *tmpH, *hk, *dA, *grad_scratch; size_t maxM; Tf32Ws tf; LstmBfWs bf;
-  uint4* chain_xw; size_t chain_xw_bytes;
+  uint4* chain_xw; size_t chain_xw_bytes; unsigned chain_steps;
 };
 
 void plan_lstm_fwd(const mgrit_gru_cfg* c, const Hier& hr, Ws& w, LstmFwdWs* o) {
@@ -1471,7 +1477,7 @@ void plan_lstm_fwd(const mgrit_gru_cfg* c, const Hier& hr, Ws& w, LstmFwdWs* o) 
   o->tmpH = w.take<float>(o->maxM * c->H);
   if (is_tf32(c)) tf32_plan_fwd(c, hr.N, hr.L, w.base, &w.off, &o->tf, 4);
   if (c->operands == MGRIT_OPERANDS_BF16) lstmbf_plan_fwd(c, o->maxM, w.base, &w.off, &o->bf);
-  o->chain_xw = nullptr; o->chain_xw_bytes = 0;
+  o->chain_xw = nullptr; o->chain_xw_bytes = 0; o->chain_steps = 0;
   if (c->operands == MGRIT_OPERANDS_BF16) {
     o->chain_xw_bytes = serial_xw_bytes(c->B, c->H, 1);
     o->chain_xw = reinterpret_cast<uint4*>(w.take<char>(o->chain_xw_bytes));
@@ -1503,7 +1509,7 @@ void plan_lstm_adj(const mgrit_gru_cfg* c, const Hier& hr, Ws& w, LstmAdjWs* o) 
   o->grad_scratch = c->operands == MGRIT_OPERANDS_FP32 ? w.take<float>(simt_gradients_scratch((int)TB, 4 * c->H, c->H, c->I)) : nullptr;
   if (is_tf32(c)) tf32_plan_adj(c, hr.N, hr.L, w.base, &w.off, &o->tf, 4);
   if (c->operands == MGRIT_OPERANDS_BF16) lstmbf_plan_adj(c, o->maxM, w.base, &w.off, &o->bf);
-  o->chain_xw = nullptr; o->chain_xw_bytes = 0;
+  o->chain_xw = nullptr; o->chain_xw_bytes = 0; o->chain_steps = 0;
   if (c->operands == MGRIT_OPERANDS_BF16) {
     o->chain_xw_bytes = serial_xw_bytes(c->B, c->H, 4);
     o->chain_xw = reinterpret_cast<uint4*>(w.take<char>(o->chain_xw_bytes));
@@ -1523,7 +1529,7 @@ struct LstmFwdCycle : Cycle {
     a.B = c->B; a.H = c->H; a.nsteps = hr.N[l]; a.u = U[l];
     a.gi = gi + (st - 1) * bh * 4; a.gi_step = st * bh * 4;
     a.g = G[l]; a.W = fw->bf.W_hh; a.b_hh = p->b_hh; a.gamma = hr.gamma[l]; a.cell = c->cell;
-    a.xw = fw->chain_xw; a.xw_bytes = fw->chain_xw_bytes;
+    a.xw = fw->chain_xw; a.xw_bytes = fw->chain_xw_bytes; a.step0 = fw->chain_steps; fw->chain_steps += hr.N[l];
     return lstm_chain_fwd_solve(a, s);
   }
   int launch_step(const StepDesc& d) override {
@@ -1571,7 +1577,7 @@ struct LstmAdjCycle : Cycle {
     a.a = w->a[l] + row0; a.p = w->p[l] + row0; a.ci = w->cib[l] + row0; a.cf = w->cfb[l] + row0; a.cg = w->cgb[l] + row0;
     a.co = w->cob[l] + row0; a.coef_step = -bh;
     a.g = G[l]; a.WT = w->bf.W_hhT;
-    a.xw = w->chain_xw; a.xw_bytes = w->chain_xw_bytes;
+    a.xw = w->chain_xw; a.xw_bytes = w->chain_xw_bytes; a.step0 = w->chain_steps; w->chain_steps += hr.N[l];
     return lstm_chain_adj_solve(a, s);
   }
   int launch_step(const StepDesc& d) override {
@@ -1629,6 +1635,7 @@ int lstm_forward_impl(const mgrit_gru_cfg* cfg, const gru_params* p, const float
   Setup setup(s);
   zero_guess(fw.U[0], c, hr, slot, &setup);
   for (int l = 0; l < hr.L; ++l) setup.copy(fw.U[l], u0, slot);
+  if (fw.chain_xw) setup.zero(fw.chain_xw, fw.chain_xw_bytes);
   LstmFwdCycle cy;
   cy.c = &c; cy.hr = hr; cy.s = s; cy.U = fw.U; cy.G = fw.G; cy.res_acc = fw.res_acc; cy.BH = slot;
   cy.p = p; cy.gi = gi; cy.fw = &fw;
@@ -1676,6 +1683,7 @@ int lstm_adjoint_impl(const mgrit_gru_cfg* cfg, const gru_params* p, const float
   }
   Setup setup(s);
   zero_guess(aw.U[0], c, hr, slot, &setup);
+  if (aw.chain_xw) setup.zero(aw.chain_xw, aw.chain_xw_bytes);
   float* Gl[kMaxLevels];
   for (int l = 0; l < hr.L; ++l) Gl[l] = aw.G[l];
   if (!du_seed) Gl[0] = nullptr;

@@ -19,6 +19,7 @@ struct SerialFwdArgs {
   float gamma; int cell;
   unsigned* bar;                 // [ceil(B/16)] barrier counters (scratch)
   uint4* xw; size_t xw_bytes;    // exchange words of the flag-in-data hand-over (scratch, serial_xw_bytes()), or nullptr
+  unsigned step0;                // the words carry step0 + 1 .. step0 + nsteps; none of them may hold one of these numbers yet
 };
 
 // mu_s = a_s*mu_{s-1} + ([cr_s|cz_s|cn_s]*mu_{s-1}) W_hh + g_s,  s = 1..nsteps
@@ -32,7 +33,7 @@ struct SerialAdjArgs {
   const float* g;                // [nsteps+1][B][H] or nullptr
   const __nv_bfloat16* WT;       // [H][3H] = W_hh^T
   unsigned* bar;
-  uint4* xw; size_t xw_bytes;    // as in SerialFwdArgs (three gate blocks per producer)
+  uint4* xw; size_t xw_bytes; unsigned step0;    // as in SerialFwdArgs (three gate blocks per producer)
 };
 
 // The same chains in fp32 arithmetic (FFMA, precise gate math) for the fp32 and tf32 operand modes: fp32 weights in
@@ -80,7 +81,7 @@ struct LstmChainFwdArgs {
   const __nv_bfloat16* W;        // [4H][H]
   const float* b_hh;
   float gamma; int cell;
-  uint4* xw; size_t xw_bytes;    // exchange words, serial_xw_bytes(B, H, 1)
+  uint4* xw; size_t xw_bytes; unsigned step0;    // exchange words, serial_xw_bytes(B, H, 1)
 };
 struct LstmChainAdjArgs {
   int B, H, nsteps;
@@ -90,7 +91,7 @@ struct LstmChainAdjArgs {
   i64 coef_step;
   const float* g;
   const __nv_bfloat16* WT;       // [H][4H] = W_hh^T
-  uint4* xw; size_t xw_bytes;    // exchange words, serial_xw_bytes(B, H, 4)
+  uint4* xw; size_t xw_bytes; unsigned step0;    // exchange words, serial_xw_bytes(B, H, 4)
 };
 // false: shape not supported (H % 64 != 0; adjoint not split by gate: H not in {128, 256, 512, 1024}; too many CTAs for one wave)
 // or the cooperative launch failed: the caller then advances step by step

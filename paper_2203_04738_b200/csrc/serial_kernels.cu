@@ -80,7 +80,9 @@ __device__ __forceinline__ void cp_async_wait_all() {
 // number sees the six values too.  Readers poll the words they need directly: one trip to L2 once the data is
 // there, instead of an arrival counter, a poll of that counter and a reload.  Two buffers alternate by step
 // parity: a CTA writes step j + 2 only after it has read all of step j + 1, which nobody could produce before
-// reading all of step j.  The host clears the words before every launch (step numbers start at 1).
+// reading all of step j.  Step numbers start at step0 + 1: the caller clears the words once per solve and numbers the steps of its
+// chains on from one another, so that no word carries a number that a later chain waits for (clearing in front of every launch was
+// two memory operations and the gaps behind them, 8 us a chain: four chains in a 2.3 ms training step at H = 512).
 constexpr int kValsPerWord = 6;
 __device__ __forceinline__ uint4 ld_word(const uint4* p) {
   uint4 v;
@@ -330,7 +332,7 @@ __global__ void __launch_bounds__(kThreads, 1) serial_fwd_kernel(SerialFwdArgs a
     if (j == a.nsteps) break;
     if (LL) {
       __syncthreads();
-      publish_block(xstage, kBlockVals, a.xw + ((i64)(rg * 2 + (j & 1)) * gridDim.x + blockIdx.x) * kBlockWords, (unsigned)j);
+      publish_block(xstage, kBlockVals, a.xw + ((i64)(rg * 2 + (j & 1)) * gridDim.x + blockIdx.x) * kBlockWords, a.step0 + (unsigned)j);
     }
     // operands of the next step that do not depend on other CTAs
 #pragma unroll
@@ -346,7 +348,7 @@ __global__ void __launch_bounds__(kThreads, 1) serial_fwd_kernel(SerialFwdArgs a
     }
     if (LL) {
       // the full new state of this row group, as the bf16 A operand: every producer's words, polled in place
-      const bool ok = gather_blocks<UNC, 1, RL>(a.xw + (i64)(rg * 2 + (j & 1)) * gridDim.x * kBlockWords, (int)gridDim.x, (unsigned)j, As, ldk,
+      const bool ok = gather_blocks<UNC, 1, RL>(a.xw + (i64)(rg * 2 + (j & 1)) * gridDim.x * kBlockWords, (int)gridDim.x, a.step0 + (unsigned)j, As, ldk,
                                             H, status);
       if (!ok) ok_smem = 0;
       __syncthreads();
@@ -456,7 +458,7 @@ __global__ void __launch_bounds__(kThreads, 1) serial_adj_kernel(SerialAdjArgs a
     if (s == a.nsteps) break;
     if (LL) {
       __syncthreads();
-      publish_block(xstage, kBlockVals, a.xw + ((i64)(rg * 2 + (s & 1)) * gridDim.x + blockIdx.x) * kBlockWords, (unsigned)s);
+      publish_block(xstage, kBlockVals, a.xw + ((i64)(rg * 2 + (s & 1)) * gridDim.x + blockIdx.x) * kBlockWords, a.step0 + (unsigned)s);
     }
 #pragma unroll
     for (int o = 0; o < OPT; ++o) {
@@ -472,7 +474,7 @@ __global__ void __launch_bounds__(kThreads, 1) serial_adj_kernel(SerialAdjArgs a
       }
     }
     if (LL) {
-      const bool ok = gather_blocks<UNC, 3, RL>(a.xw + (i64)(rg * 2 + (s & 1)) * gridDim.x * kBlockWords, (int)gridDim.x, (unsigned)s, As, ldk,
+      const bool ok = gather_blocks<UNC, 3, RL>(a.xw + (i64)(rg * 2 + (s & 1)) * gridDim.x * kBlockWords, (int)gridDim.x, a.step0 + (unsigned)s, As, ldk,
                                             H, status);
       if (!ok) ok_smem = 0;
       __syncthreads();
@@ -570,7 +572,7 @@ __global__ void __launch_bounds__(kThreads, 1) lstm_fwd_chain_kernel(LstmChainFw
     }
     if (j == a.nsteps) break;
     __syncthreads();
-    publish_block(xstage, kBlockVals, a.xw + ((i64)(rg * 2 + (j & 1)) * gridDim.x + blockIdx.x) * kBlockWords, (unsigned)j);
+    publish_block(xstage, kBlockVals, a.xw + ((i64)(rg * 2 + (j & 1)) * gridDim.x + blockIdx.x) * kBlockWords, a.step0 + (unsigned)j);
     // operands of the next step that do not depend on other CTAs (nothing may depend on these loads before the exchange)
 #pragma unroll
     for (int o = 0; o < OPT; ++o) {
@@ -585,7 +587,7 @@ __global__ void __launch_bounds__(kThreads, 1) lstm_fwd_chain_kernel(LstmChainFw
         }
       }
     }
-    const bool ok = gather_blocks<UNC, 1, RL>(a.xw + (i64)(rg * 2 + (j & 1)) * gridDim.x * kBlockWords, (int)gridDim.x, (unsigned)j, As, ldk, H,
+    const bool ok = gather_blocks<UNC, 1, RL>(a.xw + (i64)(rg * 2 + (j & 1)) * gridDim.x * kBlockWords, (int)gridDim.x, a.step0 + (unsigned)j, As, ldk, H,
                                           status);
     if (!ok) ok_smem = 0;
     __syncthreads();
@@ -698,7 +700,7 @@ __global__ void __launch_bounds__(kThreads, 1) lstm_adj_chain_kernel(LstmChainAd
     }
     if (s == a.nsteps) break;
     __syncthreads();
-    publish_block(xstage, kBlockVals, a.xw + ((i64)(rg * 2 + (s & 1)) * gridDim.x + blockIdx.x) * kBlockWords, (unsigned)s);
+    publish_block(xstage, kBlockVals, a.xw + ((i64)(rg * 2 + (s & 1)) * gridDim.x + blockIdx.x) * kBlockWords, a.step0 + (unsigned)s);
 #pragma unroll
     for (int o = 0; o < OPT; ++o) {             // operands of the steps to come that do not depend on other CTAs
       int idx = tid + o * kThreads, r = idx / UNC, i = idx % UNC;
@@ -714,7 +716,7 @@ __global__ void __launch_bounds__(kThreads, 1) lstm_adj_chain_kernel(LstmChainAd
         }
       }
     }
-    const bool ok = gather_blocks<UNC, 4, RL>(a.xw + (i64)(rg * 2 + (s & 1)) * gridDim.x * kBlockWords, (int)gridDim.x, (unsigned)s, As, ldk, H,
+    const bool ok = gather_blocks<UNC, 4, RL>(a.xw + (i64)(rg * 2 + (s & 1)) * gridDim.x * kBlockWords, (int)gridDim.x, a.step0 + (unsigned)s, As, ldk, H,
                                           status);
     if (!ok) ok_smem = 0;
     __syncthreads();
@@ -869,7 +871,7 @@ __global__ void __launch_bounds__(kThreads, 1) adj_split_chain_kernel(typename A
         v.x = 6 * k < kBlockVals ? s32[0] : 0u;
         v.y = 6 * k + 2 < kBlockVals ? s32[1] : 0u;
         v.z = 6 * k + 4 < kBlockVals ? s32[2] : 0u;
-        v.w = (unsigned)s;
+        v.w = a.step0 + (unsigned)s;
         st_word(a.xw + xbase + ((i64)q * nprod + blockIdx.x) * kBlockWords + k, v);
       }
     }
@@ -886,7 +888,7 @@ __global__ void __launch_bounds__(kThreads, 1) adj_split_chain_kernel(typename A
       }
       load_coefs(o, (i64)(s + 1) * a.coef_step + off, s + 1 < a.nsteps);
     }
-    if (waits && !gather_blocks<UF, 1, RL>(a.xw + xbase + (i64)g * nprod * kBlockWords, H / UF, (unsigned)s, As, ldk, H, status)) ok_smem = 0;
+    if (waits && !gather_blocks<UF, 1, RL>(a.xw + xbase + (i64)g * nprod * kBlockWords, H / UF, a.step0 + (unsigned)s, As, ldk, H, status)) ok_smem = 0;
     __syncthreads();
     waits = ok_smem != 0;
   }
@@ -1160,11 +1162,11 @@ template <class Args, class Kern>
 bool launch_coop(Kern kern, const Args& a, int unc, int RL, size_t smem, bool ll, int gates, cudaStream_t s) {
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return false;
   int rgs = (a.B + kRows - 1) / kRows;
-  if (cudaMemsetAsync(a.bar, 0, sizeof(unsigned) * rgs, s) != cudaSuccess) return false;
-  if (ll) {   // no word may carry a step number of an earlier launch
+  if (ll) {
     const size_t words = (size_t)rgs * 2 * (a.H / unc) * ((size_t)(gates * RL * unc + kValsPerWord - 1) / kValsPerWord);
     if (words * sizeof(uint4) > a.xw_bytes) return false;
-    if (cudaMemsetAsync(a.xw, 0, words * sizeof(uint4), s) != cudaSuccess) return false;
+  } else if (cudaMemsetAsync(a.bar, 0, sizeof(unsigned) * rgs, s) != cudaSuccess) {
+    return false;
   }
   Args args = a;
   int* st = status_ptr();
@@ -1305,7 +1307,7 @@ bool launch_adj_split(const typename AdjChainArgs<NG>::type& a, cudaStream_t s) 
   const size_t words = (size_t)rgs * 2 * NG * NG * clusters * ((size_t)(RL * UF + kValsPerWord - 1) / kValsPerWord);
   if (words * sizeof(uint4) > a.xw_bytes) return false;
   int* st = status_ptr();
-  if (!st || cudaMemsetAsync(a.xw, 0, words * sizeof(uint4), s) != cudaSuccess) return false;
+  if (!st) return false;
   cfg.gridDim = dim3(NG * clusters, rgs); cfg.dynamicSmemBytes = smem; cfg.stream = s; cfg.numAttrs = 2;
   if (cudaLaunchKernelEx(&cfg, kern, a, st) != cudaSuccess) { cudaGetLastError(); return false; }
   count_launch();
@@ -1397,10 +1399,8 @@ template <class Args, class Kern>
 bool launch_lstm_chain(Kern kern, const Args& a, int unc, int RL, size_t smem, int gates, cudaStream_t s) {
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return false;
   const int rgs = (a.B + kRows - 1) / kRows;
-  // no exchange word may carry a step number of an earlier launch
   const size_t words = (size_t)rgs * 2 * (a.H / unc) * ((size_t)(gates * RL * unc + kValsPerWord - 1) / kValsPerWord);
   if (words * sizeof(uint4) > a.xw_bytes) return false;
-  if (cudaMemsetAsync(a.xw, 0, words * sizeof(uint4), s) != cudaSuccess) return false;
   Args args = a;
   int* st = status_ptr();
   if (!st) return false;
