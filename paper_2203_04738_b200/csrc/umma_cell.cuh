@@ -202,19 +202,23 @@ constexpr int kOpBytes = BM * CH * 4;   // one epilogue operand chunk: 128 rows 
 constexpr int kCoefBytes = BM * CH * 2;   // one coefficient chunk: 128 rows x 16 bf16
 // SMALL: 32 units per tile, for steps whose 64-unit tiles would leave half of the SMs without one: a step is then bound by what
 // one CTA takes in (28 instead of 40 KiB per k-block) and by its epilogue (half the chunks).
-template <bool PAIR, bool SMALL = false> struct Geo {
+template <bool PAIR, bool SMALL = false, bool GIB = false> struct Geo {
   static constexpr int UN = PAIR ? 80 : (SMALL ? 32 : 64);   // hidden units per tile
   static constexpr int BN = 3 * UN;                 // accumulator columns: r | z | n
   static constexpr int NCH = UN / CH;
   static constexpr int kBox = PAIR ? 40 : UN;       // weight rows per TMA box
   static constexpr int kBBytes = (PAIR ? BN / 2 : BN) * BK * 2;   // weight bytes staged per CTA and k-block
-  static constexpr int kStageBytes = kABytes + kBBytes;           // 31 KiB / 40 KiB (multiples of 1 KiB)
+  // Small tiles: two k-blocks per stage.  The thread that waits for a stage, issues its MMAs and commits needs 470 to 580 cycles a
+  // stage whatever the MMAs take, and four of 128 x 96 x 16 take 192.
+  static constexpr int KG = SMALL && GIB ? 2 : 1;
+  static constexpr int kBlockBytes = kABytes + kBBytes;           // 31 KiB / 40 KiB / 28 KiB (multiples of 1 KiB)
+  static constexpr int kStageBytes = KG * kBlockBytes;
 };
 // GIB: the input projection is staged from its bf16 copy (rows of 32 bytes, 32-byte swizzle) instead of fp32: 10 instead of
 // 16 bytes per element of epilogue operands, and a third operand buffer fits.  What hides the latency of those loads is
 // the bytes in flight, and shared memory bounds them: a tile needs 128 x UN x (bytes per element) per main-loop time.
 template <bool HAS_G, bool LIN = false, bool PAIR = false, bool GIB = false, bool SMALL = false> struct CellCfg {
-  using G = Geo<PAIR, SMALL>;
+  using G = Geo<PAIR, SMALL, GIB>;
 #ifndef CELL_PAIR_STAGES_PLAIN
 #define CELL_PAIR_STAGES_PLAIN 5
 #endif
@@ -224,7 +228,7 @@ template <bool HAS_G, bool LIN = false, bool PAIR = false, bool GIB = false, boo
 #ifndef CELL_PAIR_EBUFS
 #define CELL_PAIR_EBUFS 2
 #endif
-  static constexpr int kStages = PAIR ? CELL_PAIR_STAGES : SMALL ? 5 : ((HAS_G || LIN) ? 3 : 4);
+  static constexpr int kStages = PAIR ? CELL_PAIR_STAGES : SMALL ? (GIB ? 3 : 5) : ((HAS_G || LIN) ? 3 : 4);
 #ifndef CELL_GIB_EBUFS
 #define CELL_GIB_EBUFS 3
 #endif
@@ -248,8 +252,8 @@ umma_cell_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   using namespace cellk;
   using C = CellCfg<HAS_G, LIN, PAIR, GIB, SMALL>;
   constexpr int kGi = C::kGiBytes;
-  using G = Geo<PAIR, SMALL>;
-  constexpr int UN = G::UN, BN = G::BN, NCH = G::NCH, kStageBytes = G::kStageBytes;
+  using G = Geo<PAIR, SMALL, GIB>;
+  constexpr int UN = G::UN, BN = G::BN, NCH = G::NCH, kStageBytes = G::kStageBytes, kBlockBytes = G::kBlockBytes, KG = G::KG;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t tiles_base = (raw + 1023u) & ~1023u;
@@ -273,8 +277,8 @@ umma_cell_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   const int cta = PAIR ? (int)(blockIdx.x >> 1) : (int)blockIdx.x, ncta = PAIR ? (int)(gridDim.x >> 1) : (int)gridDim.x;
   const int tile_k = PAIR ? 2 * p.kt : p.kt, rt = p.kt * p.B;        // k's per tile, rows per CTA
   const int m_tiles = (p.nk + tile_k - 1) / tile_k, n_tiles = (H + UN - 1) / UN, tiles = m_tiles * n_tiles;
-  const int k_blocks = (H + BK - 1) / BK;
-  const uint32_t stage_tx = (uint32_t)(rt * BK * 2 + G::kBBytes), epi_tx = (uint32_t)(C::kEpiBytes / BM * rt);   // bytes that really arrive
+  const int k_blocks = (H + BK - 1) / BK, k_groups = (k_blocks + KG - 1) / KG;      // (the last group may be short)
+  const uint32_t block_tx = (uint32_t)(rt * BK * 2 + G::kBBytes), epi_tx = (uint32_t)(C::kEpiBytes / BM * rt);   // bytes that really arrive
   auto row_tile = [&](int t) { return PAIR ? 2 * (t / n_tiles) + (int)rank : t / n_tiles; };
   // forward: items (step, tile); the linearisation is a single step
   const int n_items = LIN ? tiles : tiles * swp.n_steps;
@@ -333,9 +337,11 @@ umma_cell_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         const int in_s = LIN ? 0 : swp.st[sg].in_s;
         const CUtensorMap* mapA = !LIN && swp.st[sg].ext ? &tmCR : &tmA;
         // The weight tiles of the first stages do not depend on the step before: they are requested before the wait for it.
-        const int ahead = k_blocks < C::kStages ? k_blocks : C::kStages;
-        auto load_w = [&](int st, int kb) {
+        const int ahead = k_groups < C::kStages ? k_groups : C::kStages;
+        auto load_w = [&](int st, int kg) {
+          const int kb = kg * KG;
           const uint32_t b_dst = tiles_base + st * kStageBytes + kABytes;
+          const uint32_t stage_tx = KG == 1 || kb + KG <= k_blocks ? KG * block_tx : (uint32_t)(k_blocks - kb) * block_tx;
           if (PAIR) {
             // The accumulator columns r | z | n (80 each) split into two halves of 120: CTA 0 stages the weight rows
             // of r and of the first 40 units of z, CTA 1 the rest -- six 40-row boxes, three per CTA.
@@ -349,18 +355,26 @@ umma_cell_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
           } else {
             mbar_expect_tx(full_bar(st), stage_tx);
 #pragma unroll
-            for (int g = 0; g < 3; ++g) tma_load_2d(b_dst + g * (G::kBBytes / 3), &tmB, full_bar(st), kb * BK, g * H + nt * UN);
+            for (int j = 0; j < KG; ++j)
+              if (KG == 1 || kb + j < k_blocks)
+#pragma unroll
+                for (int g = 0; g < 3; ++g) tma_load_2d(b_dst + j * kBlockBytes + g * (G::kBBytes / 3), &tmB, full_bar(st), (kb + j) * BK, g * H + nt * UN);
           }
         };
-        auto load_state = [&](int st, int kb) {
+        auto load_state = [&](int st, int kg) {
+          const int kb = kg * KG;
           const uint32_t a_dst = tiles_base + st * kStageBytes;
           if (PAIR) {
             const uint32_t fullL = mapa_shared(full_bar(st), 0);
             if (LIN) tma_load_3d_pair(a_dst, &tmA, fullL, kb * BK, 0, mt * p.kt);
             else tma_load_4d_pair(a_dst, mapA, fullL, kb * BK, 0, in_s, mt * p.kt);
           } else {
-            if (LIN) tma_load_3d(a_dst, &tmA, full_bar(st), kb * BK, 0, mt * p.kt);
-            else tma_load_4d(a_dst, mapA, full_bar(st), kb * BK, 0, in_s, mt * p.kt);
+#pragma unroll
+            for (int j = 0; j < KG; ++j)
+              if (KG == 1 || kb + j < k_blocks) {
+                if (LIN) tma_load_3d(a_dst + j * kBlockBytes, &tmA, full_bar(st), (kb + j) * BK, 0, mt * p.kt);
+                else tma_load_4d(a_dst + j * kBlockBytes, mapA, full_bar(st), (kb + j) * BK, 0, in_s, mt * p.kt);
+              }
           }
         };
         int st = stage; uint32_t ph = phase;
@@ -370,7 +384,7 @@ umma_cell_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
           if (++st == C::kStages) { st = 0; ph ^= 1u; }
         }
         if (!ok || !deps_ready(sg, t / n_tiles, 17)) { ok = false; break; }
-        for (int kb = 0; kb < k_blocks; ++kb) {
+        for (int kb = 0; kb < k_groups; ++kb) {
           if (kb >= ahead) {
             if (!mbar_wait(empty_bar(stage), phase ^ 1u, abortp, status, 11)) { ok = false; break; }
             load_w(stage, kb);
@@ -391,15 +405,19 @@ umma_cell_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         if (!mbar_wait(tempty_bar(as), aphase ^ 1u, abortp, status, 12)) { ok = false; break; }
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + (uint32_t)(as * BN);
-        for (int kb = 0; kb < k_blocks; ++kb) {
+        for (int kg = 0; kg < k_groups; ++kg) {
           if (!mbar_wait(full_bar(stage), phase, abortp, status, 13)) { ok = false; break; }
           tc_fence_after();
-          const uint32_t a_src = tiles_base + stage * kStageBytes;
-          const uint64_t adesc = smem_desc_sw128(a_src), bdesc = smem_desc_sw128(a_src + kABytes);
 #pragma unroll
-          for (int k = 0; k < BK / 16; ++k) {
-            if (PAIR) mma_bf16_pair(d_tmem, adesc + (uint64_t)(k * 2), bdesc + (uint64_t)(k * 2), idesc, (kb | k) != 0 ? 1u : 0u);
-            else mma_bf16(d_tmem, adesc + (uint64_t)(k * 2), bdesc + (uint64_t)(k * 2), idesc, (kb | k) != 0 ? 1u : 0u);
+          for (int j = 0; j < KG; ++j) {
+            if (KG > 1 && kg * KG + j >= k_blocks) break;
+            const uint32_t a_src = tiles_base + stage * kStageBytes + j * kBlockBytes;
+            const uint64_t adesc = smem_desc_sw128(a_src), bdesc = smem_desc_sw128(a_src + kABytes);
+#pragma unroll
+            for (int k = 0; k < BK / 16; ++k) {
+              if (PAIR) mma_bf16_pair(d_tmem, adesc + (uint64_t)(k * 2), bdesc + (uint64_t)(k * 2), idesc, (kg | j | k) != 0 ? 1u : 0u);
+              else mma_bf16(d_tmem, adesc + (uint64_t)(k * 2), bdesc + (uint64_t)(k * 2), idesc, (kg | j | k) != 0 ? 1u : 0u);
+            }
           }
           if (PAIR) {   // the stage is free again in both CTAs
             mma_commit_pair(mapa_shared(empty_bar(stage), 0));

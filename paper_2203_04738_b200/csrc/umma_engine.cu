@@ -330,7 +330,7 @@ struct CellFwdOperands {
 template <bool HAS_G, bool PAIR, bool GIB, bool SMALL = false>
 bool launch_fwd_geo(int kc, const CellFwdOperands& o, int nk, int nk_ext, const bf16* W, CellArgs ca, const SweepArgs& sw, cudaStream_t s) {
   using C = cellk::CellCfg<HAS_G, false, PAIR, GIB, SMALL>;
-  using G = cellk::Geo<PAIR, SMALL>;
+  using G = cellk::Geo<PAIR, SMALL, GIB>;
   if (nk <= 0) return true;
   int* const status = status_ptr();
   if (!status) return false;
