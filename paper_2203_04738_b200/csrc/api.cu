@@ -257,9 +257,10 @@ struct Cycle {
   virtual bool chain(int l) { (void)l; return false; }
   // A relaxation sweep of level l in one launch: kinds[i] = s in 1..cf-1: F-step to slot s of every interval;
   // cf: C-step; cf + 1: the step that evaluates v at the C-points into G[l+1].  false = not available here.
-  virtual bool launch_sweep(int l, const int* kinds, int n) { (void)l; (void)kinds; (void)n; return false; }
+  // kz: the first intervals that take part (one more after every C-step while `homog`).
+  virtual bool launch_sweep(int l, const int* kinds, int n, int kz) { (void)l; (void)kinds; (void)n; (void)kz; return false; }
   // F (CF)^relax (the opening F optional), optionally followed by the evaluation of v at the C-points
-  bool relax_sweep(int l, bool first_f, int relax, bool with_v) {
+  bool relax_sweep(int l, bool first_f, int relax, bool with_v, int kz = INT_MAX) {
     if (rc != MGRIT_OK) return true;
     int kinds[64], n = 0;
     const int cf = c->cf;
@@ -268,7 +269,7 @@ struct Cycle {
     for (int r = 0; r < relax; ++r) { kinds[n++] = cf; for (int sI = 1; sI < cf; ++sI) kinds[n++] = sI; }
     if (with_v) kinds[n++] = cf + 1;
     if (n < 2) return false;
-    return launch_sweep(l, kinds, n);
+    return launch_sweep(l, kinds, n, kz);
   }
   virtual ~Cycle() {}
 
@@ -309,7 +310,9 @@ struct Cycle {
     }
     int relax = l == 0 ? c->relax_fine : c->relax_coarse;       // n: F (CF)^n
     int nc = hr.N[l + 1], kz = homog ? live / cf + 1 : INT_MAX;
-    if (homog || !relax_sweep(l, !skip_first_f, relax, true)) {
+    if (relax_sweep(l, !skip_first_f, relax, true, kz)) {
+      if (homog) kz += relax;
+    } else {
       if (!skip_first_f) frelax(l, kz);
       for (int n = 0; n < relax; ++n) { crelax(l, kz); if (homog) ++kz; frelax(l, kz); }
       // v_k = step_l(u_{cf k - 1}) + g_{cf k}  ->  G[l+1][k]
@@ -410,7 +413,7 @@ struct FwdCycle : Cycle {
     }
     return true;
   }
-  bool launch_sweep(int l, const int* kinds, int n) override {
+  bool launch_sweep(int l, const int* kinds, int n, int) override {      // (a forward solve has source terms: every interval takes part)
     const int cf = c->cf;
     const int tail = hr.N[l] % cf;      // F-points behind the last C-point (ragged levels): a shorter last interval
     if (c->operands != MGRIT_OPERANDS_BF16 || !Ub || c->B > 128 || hr.N[l] < cf || n > kMaxFwdSweepSteps) return false;
@@ -496,6 +499,58 @@ struct AdjCycle : Cycle {
     a.g = g; a.WT = w->um.W_hhT; a.bar = w->chain_bar;
     a.xw = w->chain_xw; a.xw_bytes = w->chain_xw_bytes; a.step0 = w->chain_steps; w->chain_steps += hr.N[l];
     return serial_adj_solve(a, s);
+  }
+  // n dependent steps over the same rows (each starts where its predecessor ended): one launch where that is available.
+  // ladds: the rows that join each step's incoming sensitivities (stacked layers), `ladds_ks` apart by k; null: none
+  void run_steps(const StepDesc* d, int n, const float* const* ladds = nullptr, i64 ladds_ks = 0) {
+    for (int i0 = 0; i0 < n && rc == MGRIT_OK; i0 += kMaxAdjSweepSteps) {
+      const int m = n - i0 < kMaxAdjSweepSteps ? n - i0 : kMaxAdjSweepSteps;
+      int r = MGRIT_UNSUPPORTED;
+      if (c->operands == MGRIT_OPERANDS_BF16) {
+        const StepDesc& f = d[i0];
+        AdjSweepArgs a{};
+        a.B = c->B; a.H = c->H; a.n = m; a.mode = f.mode;
+        a.lin = U[f.l] + (size_t)f.in_slot * BH; a.lin_ks = (i64)f.in_stride * BH;
+        a.a = w->a[f.l]; a.cr = w->crb[f.l]; a.cz = w->czb[f.l]; a.cn = w->cnb[f.l]; a.coef_ks = -(i64)f.tgt_stride * BH;
+        for (int i = 0; i < m; ++i) {
+          const StepDesc& e = d[i0 + i];
+          AdjSweepStep& q = a.st[i];
+          q.out = e.out + (size_t)e.out_slot * BH; q.out_ks = (i64)e.out_stride * BH;
+          q.g = e.gadd ? e.gadd + (size_t)e.gadd_slot * BH : nullptr; q.g_ks = (i64)e.gadd_stride * BH;
+          q.coff = (i64)(hr.N[e.l] - e.tgt_slot) * BH;      // (as in launch_step)
+          q.ladd = ladds ? ladds[i0 + i] : nullptr; q.ladd_ks = ladds_ks;
+          q.nk = e.nk;
+        }
+        r = umma_adj_sweep(a, &w->um, s);
+      }
+      if (r == MGRIT_UNSUPPORTED) {
+        for (int i = i0; i < i0 + m; ++i) {
+          if (ladds) { ladd = ladds[i]; ladd_ks = ladds_ks; }
+          step(d[i]);
+        }
+        if (ladds) ladd = nullptr;
+      } else {
+        rc = r;
+      }
+    }
+  }
+  bool launch_sweep(int l, const int* kinds, int n, int kz) override {
+    const int cf = c->cf, nki = hr.N[l] / cf, tail = hr.N[l] % cf;
+    if (c->operands != MGRIT_OPERANDS_BF16) return false;
+    StepDesc d[64];      // (relax_sweep() lists at most 64 steps)
+    int m = 0;
+    for (int i = 0; i < n; ++i) {
+      const int kd = kinds[i], nk = nki + (kd < cf && kd <= tail ? 1 : 0), live = nk < kz ? nk : kz;
+      if (kd < cf) d[m++] = StepDesc{l, live, kd - 1, cf, U[l], kd, cf, G[l], kd, cf, kd, cf, 0};
+      else if (kd == cf) d[m++] = StepDesc{l, live, cf - 1, cf, U[l], cf, cf, G[l], cf, cf, cf, cf, 0};
+      else d[m++] = StepDesc{l, live, cf - 1, cf, G[l + 1], 1, 1, G[l], cf, cf, cf, cf, 0};
+      if (kd == cf || i + 1 == n) {      // (the steps behind a C-step start from what it left in the neighbouring interval)
+        run_steps(d, m);
+        m = 0;
+        if (homog) ++kz;
+      }
+    }
+    return true;
   }
   int launch_step(const StepDesc& d) override {
     AdjStepArgs a{};
@@ -856,6 +911,7 @@ int adjoint_impl(const mgrit_gru_cfg* cfg_in, bool serial, const gru_params* p, 
   const float* const last = dh_seed ? dh_seed + (size_t)(T - 1) * BH : dhT;
   for (int l = 0; l < hr.L; ++l) setup.copy(aw.U[l], last, BH, dh_seed ? dhT : nullptr);
   if (aw.chain_xw) setup.zero(aw.chain_xw, aw.chain_xw_bytes);
+  if (bf16) setup.zero(aw.um.sweep_ctr, sizeof(int) * aw.um.sweep_ctr_n);
   if (dh_seed) {
     setup.zero(aw.G[0], sizeof(float) * BH);
     setup.zero(aw.G[0] + (size_t)T * BH, sizeof(float) * BH);
@@ -1082,7 +1138,7 @@ struct StackFwdCycle : StackCycle {
     if (last == kC) kinds[n++] = cf;
     if (last == kV) kinds[n++] = cf + 1;
     for (int k = 0; k < nl && status() == MGRIT_OK; ++k) {
-      if (!(cf <= kMaxFwdSweepSteps && y[k].launch_sweep(l, kinds, n))) {
+      if (!(cf <= kMaxFwdSweepSteps && y[k].launch_sweep(l, kinds, n, INT_MAX))) {
         // (fp32 phases: the C-step overwrites what other rows of a phase read, so it is a launch of its own)
         const bool part = last == kC && f;
         if (part && run_fp32(y[k], k, l, kz, true, kNone)) steps(y[k], l, kz, false, kC);
@@ -1259,20 +1315,22 @@ struct StackAdjCycle : StackCycle {
       AdjCycle& q = y[k];
       const i64 bh = (i64)q.BH;
       q.lsum = w->lsum;
+      std::vector<StepDesc> d;
+      std::vector<const float*> la;
       if (f) {
         const int nki = nc, tail = N % cf;
         for (int sI = 1; sI < cf; ++sI) {
-          q.ladd = k == nl - 1 ? nullptr : w->dx + (i64)(sI - 1) * bh; q.ladd_ks = (i64)cf * bh;
           const int nk = nki + (sI <= tail ? 1 : 0);
-          q.step(StepDesc{l, nk < kz ? nk : kz, sI - 1, cf, q.U[l], sI, cf, q.G[l], sI, cf, sI, cf, 0});
+          d.push_back(StepDesc{l, nk < kz ? nk : kz, sI - 1, cf, q.U[l], sI, cf, q.G[l], sI, cf, sI, cf, 0});
+          la.push_back(w->dx + (i64)(sI - 1) * bh);
         }
       }
       if (last != kNone) {
-        q.ladd = k == nl - 1 ? nullptr : f ? w->dx + (i64)(cf - 1) * bh : w->dx; q.ladd_ks = f ? (i64)cf * bh : bh;
         float* out = last == kV ? q.G[l + 1] : q.U[l];
-        q.step(StepDesc{l, nc < kz ? nc : kz, cf - 1, cf, out, last == kV ? 1 : cf, last == kV ? 1 : cf, q.G[l], cf, cf, cf, cf, 0});
+        d.push_back(StepDesc{l, nc < kz ? nc : kz, cf - 1, cf, out, last == kV ? 1 : cf, last == kV ? 1 : cf, q.G[l], cf, cf, cf, cf, 0});
+        la.push_back(f ? w->dx + (i64)(cf - 1) * bh : w->dx);
       }
-      q.ladd = nullptr;
+      q.run_steps(d.data(), (int)d.size(), k == nl - 1 ? nullptr : la.data(), f ? (i64)cf * bh : bh);
       if (f) send(k, l, 0, 1, kz < nc ? kz * cf : N);
       else send(k, l, cf - 1, cf, nc < kz ? nc : kz);
     }
@@ -1406,6 +1464,7 @@ int stack_adjoint_impl(const mgrit_gru_cfg* cfg, int nl, const gru_params* p, co
     ck[k] = layer_cfg(c, k);
     zero_guess(q.U[0], c, hr, bh, &setup);
     if (q.chain_xw) setup.zero(q.chain_xw, q.chain_xw_bytes);
+    if (c.operands == MGRIT_OPERANDS_BF16) setup.zero(q.um.sweep_ctr, sizeof(int) * q.um.sweep_ctr_n);
     for (int l = 0; l < hr.L; ++l) Gl[k][l] = q.G[l];
     if (!dh_seed) Gl[k][0] = nullptr;
     const float* const seed = dh_seed ? dh_seed + (size_t)(T - 1) * slot + k * bh : nullptr;

@@ -158,6 +158,23 @@ struct AdjStepArgs {
   int mode;                         // as FwdStepArgs
 };
 
+// ---- n dependent adjoint steps over the same rows (k, b) in ONE launch (bf16 operands); step 0 starts from the rows lin, every
+// other one from its predecessor's results.  No row may read what another row of the launch writes.
+struct AdjSweepStep {
+  float* out; i64 out_ks;          // result rows (+ k*out_ks + b*H)
+  const float* g; i64 g_ks;        // optional source rows
+  i64 coff;                        // coefficient rows of k = 0 (offset into the level's arrays)
+  const float* ladd; i64 ladd_ks;  // optional rows that join the incoming sensitivities (stacked layers)
+  int nk;                          // rows with k < nk take the step; never more than the step before
+};
+constexpr int kMaxAdjSweepSteps = 20;
+struct AdjSweepArgs {
+  int B, H, n, mode;               // mode 1 (one step): out = out - result
+  const float* lin; i64 lin_ks;
+  const float* a; const __nv_bfloat16 *cr, *cz, *cn; i64 coef_ks;
+  AdjSweepStep st[kMaxAdjSweepSteps];
+};
+
 // ---- Implicit LSTM steps (state of a point = (c, h), 4H gate rows i | f | g | o); rows m = (k, b) as above ----
 // Level-array update formed by the step kernel itself (tensor-core engines): the raw result of row (k, b) goes to
 // out + k*out_ks + b*H (cell part; hidden part at + part) as raw + g (mode 0; g optional, same indexing with g_ks) or as

@@ -7,6 +7,7 @@
 #include "umma_engine.cuh"
 #include "umma_cell.cuh"
 #include "umma_adj.cuh"
+#include "umma_adj_sweep.cuh"
 #include "umma_gemm.cuh"
 #include "umma_gemm_pair.cuh"
 #include "umma_split.cuh"
@@ -861,6 +862,12 @@ void umma_plan_adj(const mgrit_gru_cfg* c, const int* N, int L, char* base, size
   o->Apack = take<bf16>(base, off, apack);
   o->apack_elems = apack;
   o->dA4 = take<bf16>(base, off, 4 * H * TB);
+  o->op2 = o->dA4;
+  const size_t rows2 = o->maxM * 3 * H, all = 4 * H * TB;      // (3 maxM <= 3 (T / 2 + 1) B <= 4 T B but for T = 1)
+  o->sweep_ctr_n = rows2 + 128 < all ? (all - rows2) / 2 : 0;
+  if (o->sweep_ctr_n > 1 << 16) o->sweep_ctr_n = 1 << 16;
+  o->sweep_ctr = o->dA4 ? reinterpret_cast<int*>(o->dA4 + rows2) : nullptr;
+  o->sweep_ctr_used = 0;
   o->xb = take<bf16>(base, off, I * TB);
   o->hb0 = take<bf16>(base, off, (size_t)c->B * H + TB * H);   // [h_0; h] contiguous: rows (t, b) of h_{t-1} start at hb0
   o->hb = o->hb0 ? o->hb0 + (size_t)c->B * H : nullptr;
@@ -1063,6 +1070,87 @@ static bool few_row_adj(const AdjStepArgs& a, const bf16* Apack, const bf16* WT,
     case 12808: return launch_split<128, 8>(KC_ADJ_STEP, Apack, K, WT, K, a.M, a.H, K, a.H, EpiAdjSplit<8>{a}, s);
     default: return launch_gemm<64, 0>(KC_ADJ_STEP, Apack, K, WT, K, a.M, a.H, K, 0, a.H, EpiAdj<64>{a}, s);
   }
+}
+
+// MGRIT_GRU_ADJ_SWEEP=0 in the environment launches every adjoint step by itself.
+static bool adj_sweep_enabled() {
+  static int v = -1;
+  if (v < 0) { const char* e = getenv("MGRIT_GRU_ADJ_SWEEP"); v = (e && e[0] == '0') ? 0 : 1; }
+  return v == 1;
+}
+// Clusters of S CTAs of the kernel that are resident at the same time (0: none).
+template <int NR, int S> static int adj_sweep_resident() {
+  static int cache[kMaxDevices] = {0};
+  const int dev = current_device_slot();
+  if (dev < 0) return 0;
+  if (cache[dev] == 0) {
+    auto kern = umma_adj_sweep_kernel<NR, S>;
+    int n = 0;
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = S; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3(S); cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = AdjSweepCfg<NR, S>::kSmemBytes; cfg.attrs = at; cfg.numAttrs = 1;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, AdjSweepCfg<NR, S>::kSmemBytes) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess) { cudaGetLastError(); n = 0; }
+    if (n > kSMs / S) n = kSMs / S;
+    cache[dev] = n > 0 ? n : -1;
+  }
+  return cache[dev] > 0 ? cache[dev] : 0;
+}
+template <int NR, int S>
+static int launch_adj_sweep(const AdjSweepArgs& a, int M, UmmaAdjWs* w, cudaStream_t s) {
+  using C = AdjSweepCfg<NR, S>;
+  int* const status = status_ptr();
+  if (!status) return MGRIT_CUDA_ERROR;
+  AdjSweepK k{};
+  k.q = a; k.op[0] = w->Apack; k.op[1] = w->op2;
+  k.mt = (M + NR - 1) / NR; k.ncol = (a.H + 127) / 128;
+  const int resident = adj_sweep_resident<NR, S>();
+  k.lanes = resident / k.ncol;
+  if (k.lanes > k.mt) k.lanes = k.mt;
+  const size_t need = (size_t)k.mt * k.ncol;
+  if (k.lanes < 1 || w->sweep_ctr_used + need > w->sweep_ctr_n) return MGRIT_UNSUPPORTED;
+  k.ctr = w->sweep_ctr + w->sweep_ctr_used;
+  CUtensorMap t0, t1, tw;
+  if (!make_map(&t0, k.op[0], (uint64_t)3 * a.H, (uint64_t)M, (uint64_t)3 * a.H, NR) ||
+      !make_map(&t1, k.op[1], (uint64_t)3 * a.H, (uint64_t)M, (uint64_t)3 * a.H, NR) ||
+      !make_map(&tw, w->W_hhT, (uint64_t)3 * a.H, (uint64_t)a.H, (uint64_t)3 * a.H, BM)) return MGRIT_CUDA_ERROR;
+  double rows = 0;
+  for (int i = 0; i < a.n; ++i) rows += (double)a.st[i].nk * a.B;
+  ProfScope prof(KC_ADJ_STEP, 2.0 * rows * 3.0 * a.H * a.H, s);
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = S; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+  at[1].id = cudaLaunchAttributeCooperative;      // clusters wait for one another: all of them resident
+  at[1].val.cooperative = 1;
+  cfg.gridDim = dim3(S * k.ncol * k.lanes); cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = C::kSmemBytes; cfg.stream = s;
+  cfg.attrs = at; cfg.numAttrs = 2;
+  if (cudaLaunchKernelEx(&cfg, umma_adj_sweep_kernel<NR, S>, t0, t1, tw, k, status) != cudaSuccess) { cudaGetLastError(); return MGRIT_UNSUPPORTED; }
+  w->sweep_ctr_used += need;
+  count_launch();
+  return MGRIT_OK;
+}
+int umma_adj_sweep(const AdjSweepArgs& a, UmmaAdjWs* w, cudaStream_t s) {
+  if (!adj_sweep_enabled() || a.n < 1 || a.n > kMaxAdjSweepSteps) return MGRIT_UNSUPPORTED;
+  const int M = a.st[0].nk * a.B, nb = a.H / 64;
+  if (M < 1 || (size_t)M > w->maxM) return MGRIT_UNSUPPORTED;
+  auto fits = [](i64 ks) { return ks > -(1ll << 31) && ks < (1ll << 31); };      // (the kernel's strides are 32-bit)
+  if (!fits(a.lin_ks) || !fits(a.coef_ks)) return MGRIT_UNSUPPORTED;
+  for (int i = 0; i < a.n; ++i)
+    if (!fits(a.st[i].out_ks) || !fits(a.st[i].g_ks) || !fits(a.st[i].ladd_ks)) return MGRIT_UNSUPPORTED;
+  // A launch costs about 9 us (weights, first operand, filling), so it takes steps enough to spread that over, and rows enough that a
+  // step by itself is far from what its products take, or so few that it is all latency; many rows per lane group, and the single
+  // steps with their larger tiles win again.  us an adjoint cycle of a two-level solve (11 to 23 such steps), step by step / here:
+  // H = 1024, 64 rows 174 / 151 (S = 8), 256 rows 249 / 260, 512 366 / 352, 768 317 / 276, 1024 666 / 553, 2048 877 / 824,
+  // 4096 1804 / 1961; H = 768, 1024 rows 357 / 330, 2048 652 / 624, 4096 1020 / 1129; H = 640, 256 rows 202 / 227, 2048 597 / 556;
+  // H = 512, 1024 rows 164 / 188 (S = 2), 2048 281 / 275, 4096 487 / 463; H = 384, 2048 rows 373 / 364; H = 192, 1488 rows 176 / 207.
+  if (a.n < 3) return MGRIT_UNSUPPORTED;
+  if (nb == 16 && M <= 64) return launch_adj_sweep<64, 8>(a, M, w, s);
+  if (nb >= 9 && nb <= 16 && M >= 512 && M <= 2048) return launch_adj_sweep<128, 4>(a, M, w, s);
+  if (nb >= 5 && nb <= 8 && M >= 1536 && M <= 4096) return launch_adj_sweep<128, 2>(a, M, w, s);
+  return MGRIT_UNSUPPORTED;
 }
 
 int umma_adj_step(const AdjStepArgs& in, UmmaAdjWs* w, cudaStream_t s) {

@@ -25,6 +25,10 @@ struct UmmaAdjWs {
   __nv_bfloat16* hb;      // = hb0 + B*H: the given states
   const __nv_bfloat16* gib;  // bf16 copy of the input projection left by the forward call, or nullptr
   size_t maxM;
+  // adjoint sweeps, inside dA4 (which only the gradient pass uses): a second operand buffer of maxM rows, and counters that the
+  // caller clears once per solve
+  __nv_bfloat16* op2;
+  int* sweep_ctr; size_t sweep_ctr_n, sweep_ctr_used;
 };
 
 // TF32 operand modes (same GEMM kernel, `.kind::tf32`): operands are fp32 arrays of tf32 values, split in S = 3 parts
@@ -100,6 +104,8 @@ int umma_fwd_step(const FwdStepArgs& a, UmmaFwdWs* w, cudaStream_t s);
 int umma_fwd_sweep(const FwdSweepArgs& a, UmmaFwdWs* w, cudaStream_t s);
 int umma_linearise(const LinArgs& a, UmmaAdjWs* w, cudaStream_t s);
 int umma_adj_step(const AdjStepArgs& a, UmmaAdjWs* w, cudaStream_t s);
+// all steps of a relaxation between two C-points in one launch; MGRIT_UNSUPPORTED = not available for this shape
+int umma_adj_sweep(const AdjSweepArgs& a, UmmaAdjWs* w, cudaStream_t s);
 int umma_gradients(const mgrit_gru_cfg* c, const gru_params* p, const float* x, const float* h0, const float* h,
                    const float* lam, i64 lam_ts, const __nv_bfloat16* cr, const __nv_bfloat16* cz, const __nv_bfloat16* cn,
                    const __nv_bfloat16* cnp, float* dx,
