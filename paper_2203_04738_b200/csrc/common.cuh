@@ -8,10 +8,9 @@
 #include <stddef.h>
 
 #include "../../include/mgrit_gru.h"
+#include "adj_sweep.h"
 
 namespace mg {
-
-typedef long long i64;
 
 // Every launch goes through this counter (reported by mgrit_gru_kernel_launches()).
 extern std::atomic<unsigned long long> g_kernel_launches;
@@ -156,23 +155,6 @@ struct AdjStepArgs {
   const float* ladd; i64 ladd_ks; float* lsum;
   const float* W_hh;                // [3H,H] fp32
   int mode;                         // as FwdStepArgs
-};
-
-// ---- n dependent adjoint steps over the same rows (k, b) in ONE launch (bf16 operands); step 0 starts from the rows lin, every
-// other one from its predecessor's results.  No row may read what another row of the launch writes.
-struct AdjSweepStep {
-  float* out; i64 out_ks;          // result rows (+ k*out_ks + b*H)
-  const float* g; i64 g_ks;        // optional source rows
-  i64 coff;                        // coefficient rows of k = 0 (offset into the level's arrays)
-  const float* ladd; i64 ladd_ks;  // optional rows that join the incoming sensitivities (stacked layers)
-  int nk;                          // rows with k < nk take the step; never more than the step before
-};
-constexpr int kMaxAdjSweepSteps = 20;
-struct AdjSweepArgs {
-  int B, H, n, mode;               // mode 1 (one step): out = out - result
-  const float* lin; i64 lin_ks;
-  const float* a; const __nv_bfloat16 *cr, *cz, *cn; i64 coef_ks;
-  AdjSweepStep st[kMaxAdjSweepSteps];
 };
 
 // ---- Implicit LSTM steps (state of a point = (c, h), 4H gate rows i | f | g | o); rows m = (k, b) as above ----

@@ -2,7 +2,8 @@
 //
 //   lambda_{s+1}[m, n] = a_s[m, n] * lambda_s[m, n] + sum_j dA_s[m, j] * W_hhT[n, j] (+ g_s[m, n])      dA_s = [c_r | c_z | c_n]_s * lambda_s
 //
-// for the steps of a relaxation between two C-points (rows m = (k, b): interval k, batch row b; no row reads another one's).
+// for the steps of a relaxation between two C-points (rows m = (k, b): interval k, batch row b).  No row reads another one's, but the
+// last step may replace the rows that the next interval started from (a C-step).
 //
 // Step by step (packing kernel, then a product) such a step costs 8.5 us at 64 rows and 12.5 at 512 (H = 1024), of which the tensor
 // cores need 0.3 and 2.3: two launches, their first loads, and all of W_hhT from L2 each time.  Here
@@ -15,6 +16,9 @@
 //    pass disappears.  (Finished in the accumulator's own layout, a lane per column with 64-byte stores of bf16: 0.27 us a row and CTA.)
 //  * clusters hand a row tile's operand on through L2: a CTA's producer waits until the column tiles of its units have counted the
 //    step (red.release / ld.acquire, then the TMA loads).
+//  * lane groups are not ordered against one another, but for a C-step: before its results are stored, the tiles of the rows that
+//    started from what they replace have counted their first step, in front of which they read it (both as that step's operand and
+//    as its incoming rows).  No step in front of the C-step waits for another group, so these counts always come.
 // A lane group of clusters covers all columns and takes every `lanes`-th row tile.  All CTAs are resident (cooperative launch).
 // The operand of step s + 1 goes to the buffer that step s - 1 was read from: its writer holds sums of step s, which every slice
 // of every column tile of step s - 1 went into.
@@ -205,6 +209,17 @@ umma_adj_sweep_kernel(const __grid_constant__ CUtensorMap tm0, const __grid_cons
       if (++b == B) { b = 0; ++k; }
     }
   };
+  // The rows that started from what rows r0 .. r0 + 3 replace are `ahead` behind them, in at most two tiles: a lane polls for each.
+  auto starts_read = [&](int r0, int M, int ahead) {
+    int lo, hi;
+    tiles_ahead(r0, M, ahead, NR, &lo, &hi);
+    const int mine = lo + lane;
+    bool done = true;
+    if (mine <= hi && mine < p.mt) done = sweep_wait(p.ctr + mine * p.ncol + ct, 2 * AW * S, abortp, status, 68);
+    done = __all_sync(0xffffffffu, done);
+    __syncwarp();      // (orders what the polling lanes acquired in front of every lane's stores)
+    return done;
+  };
   bool ok = true;
   if (warp >= 2) {
     // the operand of the first step, while the weights arrive
@@ -376,6 +391,8 @@ umma_adj_sweep_kernel(const __grid_constant__ CUtensorMap tm0, const __grid_cons
               if (col && r0 + i < Mn) put_operand(p.op[(s + 1) & 1], r0 + i, cy[i], o.cr[i], o.cz[i], o.cn[i]);
           }
           if (j == QW - 1 && s + 1 < q.n) count(m);
+          if (t.ahead > 0 && ok) ok = starts_read(r0, M, t.ahead);
+          if (!ok) continue;
           int k = r0 / B, b = r0 - k * B;
 #pragma unroll
           for (int i = 0; i < 4; ++i) {

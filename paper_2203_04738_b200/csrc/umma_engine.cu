@@ -1132,8 +1132,9 @@ static int launch_adj_sweep(const AdjSweepArgs& a, int M, UmmaAdjWs* w, cudaStre
   count_launch();
   return MGRIT_OK;
 }
-int umma_adj_sweep(const AdjSweepArgs& a, UmmaAdjWs* w, cudaStream_t s) {
-  if (!adj_sweep_enabled() || a.n < 1 || a.n > kMaxAdjSweepSteps) return MGRIT_UNSUPPORTED;
+int umma_adj_sweep(const AdjSweepArgs& in, UmmaAdjWs* w, cudaStream_t s) {
+  if (!adj_sweep_enabled() || in.n < 1 || in.n > kMaxAdjSweepSteps) return MGRIT_UNSUPPORTED;
+  AdjSweepArgs a = in;
   const int M = a.st[0].nk * a.B, nb = a.H / 64;
   if (M < 1 || (size_t)M > w->maxM) return MGRIT_UNSUPPORTED;
   auto fits = [](i64 ks) { return ks > -(1ll << 31) && ks < (1ll << 31); };      // (the kernel's strides are 32-bit)
@@ -1146,11 +1147,9 @@ int umma_adj_sweep(const AdjSweepArgs& a, UmmaAdjWs* w, cudaStream_t s) {
   // H = 1024, 64 rows 174 / 151 (S = 8), 256 rows 249 / 260, 512 366 / 352, 768 317 / 276, 1024 666 / 553, 2048 877 / 824,
   // 4096 1804 / 1961; H = 768, 1024 rows 357 / 330, 2048 652 / 624, 4096 1020 / 1129; H = 640, 256 rows 202 / 227, 2048 597 / 556;
   // H = 512, 1024 rows 164 / 188 (S = 2), 2048 281 / 275, 4096 487 / 463; H = 384, 2048 rows 373 / 364; H = 192, 1488 rows 176 / 207.
-  if (a.n < 3) return MGRIT_UNSUPPORTED;
-  if (nb == 16 && M <= 64) return launch_adj_sweep<64, 8>(a, M, w, s);
-  if (nb >= 9 && nb <= 16 && M >= 512 && M <= 2048) return launch_adj_sweep<128, 4>(a, M, w, s);
-  if (nb >= 5 && nb <= 8 && M >= 1536 && M <= 4096) return launch_adj_sweep<128, 2>(a, M, w, s);
-  return MGRIT_UNSUPPORTED;
+  const int S = nb == 16 && M <= 64 ? 8 : nb >= 9 && nb <= 16 && M >= 512 && M <= 2048 ? 4 : nb >= 5 && nb <= 8 && M >= 1536 && M <= 4096 ? 2 : 0;
+  if (a.n < 3 || S == 0 || !plan_adj_sweep(&a)) return MGRIT_UNSUPPORTED;
+  return S == 8 ? launch_adj_sweep<64, 8>(a, M, w, s) : S == 4 ? launch_adj_sweep<128, 4>(a, M, w, s) : launch_adj_sweep<128, 2>(a, M, w, s);
 }
 
 int umma_adj_step(const AdjStepArgs& in, UmmaAdjWs* w, cudaStream_t s) {
