@@ -270,6 +270,7 @@ umma_adj_sweep_kernel(const __grid_constant__ CUtensorMap tm0, const __grid_cons
       for (int m = group; m < p.mt && ok; m += p.lanes) {
         if (lane < cts) ok = sweep_wait(p.ctr + m * p.ncol + first_ct + lane, AW * S * (s + 1), abortp, status, 61);
         ok = __all_sync(0xffffffffu, ok);
+        __syncwarp();      // (a vote orders no memory: what the polling lanes acquired comes before lane 0's loads by this barrier)
         for (int ub = b0; ub < b1 && ok; ++ub) {
           ok = __all_sync(0xffffffffu, mbar_wait(empty_bar(stage), phase ^ 1u, abortp, status, 62));
           if (!ok) break;
