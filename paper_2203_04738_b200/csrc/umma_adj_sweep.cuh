@@ -24,7 +24,7 @@
 // of every column tile of step s - 1 went into.
 //
 // Warps: 0 = TMA producer, 1 = MMA issuer and TMEM owner, 2..9 = epilogue.  Every wait is bounded; a CTA whose wait ran out skips to
-// the closing cluster barrier.
+// the closing cluster barrier, behind its own loads and products in flight.
 #pragma once
 #include "umma_cell.cuh"
 #include "umma_split.cuh"
@@ -94,6 +94,12 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity,
     }
   }
 }
+// bounded wait for the CTA's own loads and products when a launch ends, whether a wait ran out before or not
+__device__ __forceinline__ void mbar_drain(uint32_t bar, uint32_t parity) {
+  const uint64_t t0 = global_ns();
+  while (!mbar_try(bar, parity))
+    if (global_ns() - t0 > kWaitLimitNs) return;
+}
 // element k * ks + off of rows: strides fit 32 bits (checked by the host), so an address is two multiply-adds
 template <class T> __device__ __forceinline__ T* at(T* base, int k, int ks, int off) { return base + ((i64)k * ks + off); }
 __device__ __forceinline__ float4 ld_f4(const float* p) {      // (rows that this launch writes too: not through the read-only path)
@@ -127,7 +133,7 @@ umma_adj_sweep_kernel(const __grid_constant__ CUtensorMap tm0, const __grid_cons
   auto empty_bar = [&](int s) { return bars + 8u * (C::kStages + s); };
   auto tfull_bar = [&](int a) { return bars + 8u * (2 * C::kStages + a); };
   auto tempty_bar = [&](int a) { return bars + 8u * (2 * C::kStages + 2 + a); };
-  const uint32_t xfull = bars + 8u * (2 * C::kStages + 4), xempty = xfull + 8u, wfull = xfull + 16u;
+  const uint32_t xfull = bars + 8u * (2 * C::kStages + 4), xempty = xfull + 8u, wfull = xfull + 16u, mma_done = xfull + 24u;
   __shared__ uint32_t tmem_base_smem;
   __shared__ int abort_flag;
 
@@ -145,6 +151,7 @@ umma_adj_sweep_kernel(const __grid_constant__ CUtensorMap tm0, const __grid_cons
     mbar_init(xfull, 1);
     mbar_init(xempty, AW * S);
     mbar_init(wfull, 1);
+    mbar_init(mma_done, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     mbar_expect_tx(wfull, (uint32_t)(3 * (b1 - b0) * C::kWBytes));
     for (int x = 0; x < 3 * (b1 - b0); ++x) tma_load_2d(tiles_base + x * C::kWBytes, &tmW, wfull, (x % 3) * H + (b0 + x / 3) * 64, ct * 128);
@@ -263,7 +270,7 @@ umma_adj_sweep_kernel(const __grid_constant__ CUtensorMap tm0, const __grid_cons
   if (warp == 0) {
     // ------------------------------------------------------------ producer: the operand rows of this CTA's units (a lane polls for
     // each column tile that they come from)
-    int stage = 0; uint32_t phase = 0;
+    int stage = 0, loads = 0; uint32_t phase = 0;
     const int first_ct = b0 >> 1, cts = ((b1 - 1) >> 1) - first_ct + 1;
     for (int s = 0; s < q.n && ok; ++s) {
       const CUtensorMap* tm = (s & 1) ? &tm1 : &tm0;
@@ -281,10 +288,16 @@ umma_adj_sweep_kernel(const __grid_constant__ CUtensorMap tm0, const __grid_cons
             for (int g = 0; g < 3; ++g) tma_load_2d(tiles_base + stage * C::kStageBytes + g * C::kBoxBytes, tm, full_bar(stage), g * H + ub * 64, m * NR);
           }
           __syncwarp();
+          ++loads;
           if (++stage == C::kStages) { stage = 0; phase ^= 1u; }
         }
       }
     }
+    if (lane == 0) {      // (after an aborted loop too, nothing leaves before its loads have landed)
+      mbar_drain(wfull, 0u);
+      for (int x = loads > C::kStages ? loads - C::kStages : 0; x < loads; ++x) mbar_drain(full_bar(x % C::kStages), (uint32_t)(x / C::kStages) & 1u);
+    }
+    __syncwarp();
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
     if (lane == 0) {
@@ -312,6 +325,8 @@ umma_adj_sweep_kernel(const __grid_constant__ CUtensorMap tm0, const __grid_cons
           }
           if (ok) mma_commit(tfull_bar(as));
         }
+      mma_commit(mma_done);
+      mbar_drain(mma_done, 0u);
     }
     __syncwarp();
   } else {
@@ -410,6 +425,10 @@ umma_adj_sweep_kernel(const __grid_constant__ CUtensorMap tm0, const __grid_cons
   tc_fence_before();
   __syncthreads();
   if (S > 1) cluster_sync_all();
+  if (abort_flag != 0) {      // partial sums of peers may still be on their way to a CTA that stopped waiting for them
+    const uint64_t t0 = global_ns();
+    while (global_ns() - t0 < 100000) __nanosleep(1000);
+  }
   tc_fence_after();
   if (warp == 1) {
     __syncwarp();
