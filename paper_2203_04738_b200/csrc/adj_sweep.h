@@ -27,7 +27,7 @@ struct AdjSweepStep {
 };
 constexpr int kMaxAdjSweepSteps = 20;
 struct AdjSweepArgs {
-  int B, H, n, mode;               // mode 1 (one step): out = out - result
+  int B, H, n;
   const float* lin; i64 lin_ks;
   const float* a; const __nv_bfloat16 *cr, *cz, *cn; i64 coef_ks;
   AdjSweepStep st[kMaxAdjSweepSteps];

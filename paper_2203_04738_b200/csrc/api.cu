@@ -508,8 +508,9 @@ struct AdjCycle : Cycle {
       int r = MGRIT_UNSUPPORTED;
       if (c->operands == MGRIT_OPERANDS_BF16) {
         const StepDesc& f = d[i0];
+        bool sums = true;      // (residuals are single steps)
         AdjSweepArgs a{};
-        a.B = c->B; a.H = c->H; a.n = m; a.mode = f.mode;
+        a.B = c->B; a.H = c->H; a.n = m;
         a.lin = U[f.l] + (size_t)f.in_slot * BH; a.lin_ks = (i64)f.in_stride * BH;
         a.a = w->a[f.l]; a.cr = w->crb[f.l]; a.cz = w->czb[f.l]; a.cn = w->cnb[f.l]; a.coef_ks = -(i64)f.tgt_stride * BH;
         for (int i = 0; i < m; ++i) {
@@ -520,8 +521,9 @@ struct AdjCycle : Cycle {
           q.coff = (i64)(hr.N[e.l] - e.tgt_slot) * BH;      // (as in launch_step)
           q.ladd = ladds ? ladds[i0 + i] : nullptr; q.ladd_ks = ladds_ks;
           q.nk = e.nk;
+          sums = sums && e.mode == 0;
         }
-        r = umma_adj_sweep(a, &w->um, s);
+        if (sums) r = umma_adj_sweep(a, &w->um, s);
       }
       if (r == MGRIT_UNSUPPORTED) {
         for (int i = i0; i < i0 + m; ++i) {

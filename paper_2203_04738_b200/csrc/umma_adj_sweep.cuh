@@ -139,7 +139,7 @@ umma_adj_sweep_kernel(const __grid_constant__ CUtensorMap tm0, const __grid_cons
 
   const AdjSweepArgs& q = p.q;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int rank = S > 1 ? (int)cluster_ctarank() : 0, cid = blockIdx.x / S, group = cid / p.ncol, ct = cid - group * p.ncol;
+  const int rank = (int)cluster_ctarank(), cid = blockIdx.x / S, group = cid / p.ncol, ct = cid - group * p.ncol;
   const int H = q.H, B = q.B, nb = H / 64, b0 = nb * rank / S, b1 = nb * (rank + 1) / S;
   // tensor memory: one or two accumulators of NR columns, then the weights (room for the largest share of any CTA)
   const int wmax = 3 * ((nb + S - 1) / S) * 32, accs = wmax + 2 * NR <= 512 ? 2 : 1, wcol = accs * NR;
@@ -189,8 +189,8 @@ umma_adj_sweep_kernel(const __grid_constant__ CUtensorMap tm0, const __grid_cons
     const int M = t.nk * B, Mn = s + 1 < q.n ? nx.nk * B : 0, c_ks = (int)q.coef_ks;
     const float* const in = s > 0 ? q.st[s - 1].out : q.lin;
     const int in_ks = (int)(s > 0 ? q.st[s - 1].out_ks : q.lin_ks);
-    const float* const gp = q.mode == 1 ? t.out : t.g;
-    const int g_ks = (int)(q.mode == 1 ? t.out_ks : t.g_ks);
+    const float* const gp = t.g;
+    const int g_ks = (int)t.g_ks;
     int k = r0 / B, b = r0 - k * B;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
@@ -264,7 +264,7 @@ umma_adj_sweep_kernel(const __grid_constant__ CUtensorMap tm0, const __grid_cons
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");      // (TMA writes the same memory next)
   }
   __syncthreads();
-  if (S > 1) cluster_sync_all();      // every CTA of the cluster is past its weights before anything is written into its shared memory
+  cluster_sync_all();      // every CTA of the cluster is past its weights before anything is written into its shared memory
   tc_fence_after();
 
   if (warp == 0) {
@@ -395,7 +395,7 @@ umma_adj_sweep_kernel(const __grid_constant__ CUtensorMap tm0, const __grid_cons
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
             const float4 u = make_float4(o.a[i].x * o.l[i].x + v[i].x, o.a[i].y * o.l[i].y + v[i].y, o.a[i].z * o.l[i].z + v[i].z, o.a[i].w * o.l[i].w + v[i].w);
-            v[i] = q.mode == 1 ? make_float4(o.g[i].x - u.x, o.g[i].y - u.y, o.g[i].z - u.z, o.g[i].w - u.w) : add4f(u, o.g[i]);
+            v[i] = add4f(u, o.g[i]);
           }
           if (Mn > 0) {      // the operand first: it is what the other clusters wait for
             float4 cy[4];
@@ -424,7 +424,7 @@ umma_adj_sweep_kernel(const __grid_constant__ CUtensorMap tm0, const __grid_cons
   // ------------------------------------------------------------ teardown: nobody leaves while a peer may still signal it
   tc_fence_before();
   __syncthreads();
-  if (S > 1) cluster_sync_all();
+  cluster_sync_all();
   if (abort_flag != 0) {      // partial sums of peers may still be on their way to a CTA that stopped waiting for them
     const uint64_t t0 = global_ns();
     while (global_ns() - t0 < 100000) __nanosleep(1000);
