@@ -1141,13 +1141,8 @@ int umma_adj_sweep(const AdjSweepArgs& in, UmmaAdjWs* w, cudaStream_t s) {
   if (!fits(a.lin_ks) || !fits(a.coef_ks)) return MGRIT_UNSUPPORTED;
   for (int i = 0; i < a.n; ++i)
     if (!fits(a.st[i].out_ks) || !fits(a.st[i].g_ks) || !fits(a.st[i].ladd_ks)) return MGRIT_UNSUPPORTED;
-  // A launch costs about 9 us (weights, first operand, filling), so it takes steps enough to spread that over, and rows enough that a
-  // step by itself is far from what its products take, or so few that it is all latency; many rows per lane group, and the single
-  // steps with their larger tiles win again.  us an adjoint cycle of a two-level solve (11 to 23 such steps), step by step / here:
-  // H = 1024, 64 rows 174 / 151 (S = 8), 256 rows 249 / 260, 512 366 / 352, 768 317 / 276, 1024 666 / 553, 2048 877 / 824,
-  // 4096 1804 / 1961; H = 768, 1024 rows 357 / 330, 2048 652 / 624, 4096 1020 / 1129; H = 640, 256 rows 202 / 227, 2048 597 / 556;
-  // H = 512, 1024 rows 164 / 188 (S = 2), 2048 281 / 275, 4096 487 / 463; H = 384, 2048 rows 373 / 364; H = 192, 1488 rows 176 / 207.
-  const int S = nb == 16 && M <= 64 ? 8 : nb >= 9 && nb <= 16 && M >= 512 && M <= 2048 ? 4 : nb >= 5 && nb <= 8 && M >= 1536 && M <= 4096 ? 2 : 0;
+  // A launch costs about 9 us (weights, first operand, filling), so it takes three steps and more.
+  const int S = adj_sweep_split(a.H, M, adj_sweep_resident<128, 4>(), adj_sweep_resident<128, 2>());
   if (a.n < 3 || S == 0 || !plan_adj_sweep(&a)) return MGRIT_UNSUPPORTED;
   return S == 8 ? launch_adj_sweep<64, 8>(a, M, w, s) : S == 4 ? launch_adj_sweep<128, 4>(a, M, w, s) : launch_adj_sweep<128, 2>(a, M, w, s);
 }
