@@ -913,7 +913,7 @@ int adjoint_impl(const mgrit_gru_cfg* cfg_in, bool serial, const gru_params* p, 
   const float* const last = dh_seed ? dh_seed + (size_t)(T - 1) * BH : dhT;
   for (int l = 0; l < hr.L; ++l) setup.copy(aw.U[l], last, BH, dh_seed ? dhT : nullptr);
   if (aw.chain_xw) setup.zero(aw.chain_xw, aw.chain_xw_bytes);
-  if (bf16) setup.zero(aw.um.sweep_ctr, sizeof(int) * aw.um.sweep_ctr_n);
+  if (bf16 && hr.L > 1) setup.zero(aw.um.sweep_ctr, sizeof(int) * aw.um.sweep_ctr_n);
   if (dh_seed) {
     setup.zero(aw.G[0], sizeof(float) * BH);
     setup.zero(aw.G[0] + (size_t)T * BH, sizeof(float) * BH);
@@ -1466,7 +1466,7 @@ int stack_adjoint_impl(const mgrit_gru_cfg* cfg, int nl, const gru_params* p, co
     ck[k] = layer_cfg(c, k);
     zero_guess(q.U[0], c, hr, bh, &setup);
     if (q.chain_xw) setup.zero(q.chain_xw, q.chain_xw_bytes);
-    if (c.operands == MGRIT_OPERANDS_BF16) setup.zero(q.um.sweep_ctr, sizeof(int) * q.um.sweep_ctr_n);
+    if (c.operands == MGRIT_OPERANDS_BF16 && hr.L > 1) setup.zero(q.um.sweep_ctr, sizeof(int) * q.um.sweep_ctr_n);
     for (int l = 0; l < hr.L; ++l) Gl[k][l] = q.G[l];
     if (!dh_seed) Gl[k][0] = nullptr;
     const float* const seed = dh_seed ? dh_seed + (size_t)(T - 1) * slot + k * bh : nullptr;
