@@ -369,6 +369,11 @@ __global__ void __launch_bounds__(kThreads, 1) serial_fwd_kernel(SerialFwdArgs a
 // ------------------------------------------------------------------------------------------------
 // adjoint chain:  mu_s = a_s * mu_{s-1} + [cr_s|cz_s|cn_s]*mu_{s-1} W_hh + g_s ,  s = 1..nsteps
 // The bf16 operand copy carries dA_{s+1} = [cr|cz|cn]_{s+1} * mu_s, formed by the CTA that produced mu_s.
+// In the kernels of eight units per CTA the steps are counted by the number that their words carry (from step0 + 1 to nsteps, which
+// the launch raises by step0; the rows' addresses are lowered to match): with the sum of both in the loop the compiler's schedule of
+// the polls came out 0.03 us a step longer (H = 512, 8 rows: 1.700 against 1.669).  The wider kernels are the other way round
+// (H = 512, 64 rows: 2.726 counted by word, 2.692 with the sum).
+__host__ __device__ constexpr bool adj_words_number_steps(int unc, bool ll) { return ll && unc == 8; }
 template <int UNC, bool LL, int RL, int KS = 0>     // KS > 0: weight fragments in registers, KS = 3H / 128
 __global__ void __launch_bounds__(kThreads, 1) serial_adj_kernel(SerialAdjArgs a, int* status) {
   constexpr int NT = UNC / 8, OPT = (RL * UNC + kThreads - 1) / kThreads;
@@ -385,6 +390,8 @@ __global__ void __launch_bounds__(kThreads, 1) serial_adj_kernel(SerialAdjArgs a
   const int nrows = min(kRows, a.B - row0);
   const unsigned ncta_rg = gridDim.x;
   const i64 BH = (i64)a.B * H;
+  const int first = adj_words_number_steps(UNC, LL) ? (int)a.step0 + 1 : 1;
+  const unsigned tag0 = adj_words_number_steps(UNC, LL) ? 0u : a.step0;
 
   for (int e = tid; e < UNC * (K / 8); e += kThreads) {
     int r = e / (K / 8), c = e % (K / 8);
@@ -394,10 +401,11 @@ __global__ void __launch_bounds__(kThreads, 1) serial_adj_kernel(SerialAdjArgs a
   if (tid == 0) ok_smem = 1;
   __syncthreads();
   // step 1: dA_1 = c_1 * mu_0 for all 3H columns of this row group
+  const i64 m0 = (i64)(first - 1) * BH, k0 = (i64)(first - 1) * a.coef_step;      // slot and coefficient rows that the chain starts from
   for (int e = tid; e < nrows * H; e += kThreads) {
     int r = e / H, i = e % H;
-    i64 off = (i64)(row0 + r) * H + i;
-    float m = __ldcg(a.mu + off);
+    i64 off = k0 + (i64)(row0 + r) * H + i;
+    float m = __ldcg(a.mu + m0 + (off - k0));
     As[r * ldk + i] = __float2bfloat16(__bfloat162float(a.cr[off]) * m);
     As[r * ldk + H + i] = __float2bfloat16(__bfloat162float(a.cz[off]) * m);
     As[r * ldk + 2 * H + i] = __float2bfloat16(__bfloat162float(a.cn[off]) * m);
@@ -409,21 +417,21 @@ __global__ void __launch_bounds__(kThreads, 1) serial_adj_kernel(SerialAdjArgs a
     int idx = tid + o * kThreads, r = idx / UNC, i = idx % UNC;
     bool v = idx < RL * UNC && r < nrows;
     i64 off = (i64)(row0 + r) * H + u0 + i;
-    mp[o] = v ? __ldcg(a.mu + off) : 0.f;
-    pa[o] = v ? a.a[off] : 0.f;
-    pg[o] = (v && a.g) ? a.g[BH + off] : 0.f;
-    bool more = v && a.nsteps > 1;
+    mp[o] = v ? __ldcg(a.mu + m0 + off) : 0.f;
+    pa[o] = v ? a.a[k0 + off] : 0.f;
+    pg[o] = (v && a.g) ? a.g[m0 + BH + off] : 0.f;
+    bool more = v && a.nsteps > first;
     const bf16 zero = __float2bfloat16(0.f);
-    ncr[o] = more ? a.cr[a.coef_step + off] : zero;
-    ncz[o] = more ? a.cz[a.coef_step + off] : zero;
-    ncn[o] = more ? a.cn[a.coef_step + off] : zero;
+    ncr[o] = more ? a.cr[k0 + a.coef_step + off] : zero;
+    ncz[o] = more ? a.cz[k0 + a.coef_step + off] : zero;
+    ncn[o] = more ? a.cn[k0 + a.coef_step + off] : zero;
   }
   __syncthreads();
 
   const int kw = K / kWarps;
   uint32_t wreg[KS > 0 ? KS : 1][NT][2];
   if (KS > 0) load_wregs<NT, (KS > 0 ? KS : 1)>(Ws, ldk, warp * kw, wreg);
-  for (int s = 1; s <= a.nsteps; ++s) {
+  for (int s = first; s <= a.nsteps; ++s) {
     float acc[NT][4];
 #pragma unroll
     for (int nt = 0; nt < NT; ++nt) acc[nt][0] = acc[nt][1] = acc[nt][2] = acc[nt][3] = 0.f;
@@ -458,7 +466,7 @@ __global__ void __launch_bounds__(kThreads, 1) serial_adj_kernel(SerialAdjArgs a
     if (s == a.nsteps) break;
     if (LL) {
       __syncthreads();
-      publish_block(xstage, kBlockVals, a.xw + ((i64)(rg * 2 + (s & 1)) * gridDim.x + blockIdx.x) * kBlockWords, a.step0 + (unsigned)s);
+      publish_block(xstage, kBlockVals, a.xw + ((i64)(rg * 2 + (s & 1)) * gridDim.x + blockIdx.x) * kBlockWords, tag0 + (unsigned)s);
     }
 #pragma unroll
     for (int o = 0; o < OPT; ++o) {
@@ -474,7 +482,7 @@ __global__ void __launch_bounds__(kThreads, 1) serial_adj_kernel(SerialAdjArgs a
       }
     }
     if (LL) {
-      const bool ok = gather_blocks<UNC, 3, RL>(a.xw + (i64)(rg * 2 + (s & 1)) * gridDim.x * kBlockWords, (int)gridDim.x, a.step0 + (unsigned)s, As, ldk,
+      const bool ok = gather_blocks<UNC, 3, RL>(a.xw + (i64)(rg * 2 + (s & 1)) * gridDim.x * kBlockWords, (int)gridDim.x, tag0 + (unsigned)s, As, ldk,
                                             H, status);
       if (!ok) ok_smem = 0;
       __syncthreads();
@@ -660,7 +668,9 @@ __global__ void __launch_bounds__(kThreads, 1) lstm_adj_chain_kernel(LstmChainAd
   }
   __syncthreads();
 
+  unsigned tag = a.step0;
   for (int s = 1; s <= a.nsteps; ++s) {
+    ++tag;
     float acc[NT][4];
 #pragma unroll
     for (int nt = 0; nt < NT; ++nt) acc[nt][0] = acc[nt][1] = acc[nt][2] = acc[nt][3] = 0.f;
@@ -700,7 +710,7 @@ __global__ void __launch_bounds__(kThreads, 1) lstm_adj_chain_kernel(LstmChainAd
     }
     if (s == a.nsteps) break;
     __syncthreads();
-    publish_block(xstage, kBlockVals, a.xw + ((i64)(rg * 2 + (s & 1)) * gridDim.x + blockIdx.x) * kBlockWords, a.step0 + (unsigned)s);
+    publish_block(xstage, kBlockVals, a.xw + ((i64)(rg * 2 + (s & 1)) * gridDim.x + blockIdx.x) * kBlockWords, tag);
 #pragma unroll
     for (int o = 0; o < OPT; ++o) {             // operands of the steps to come that do not depend on other CTAs
       int idx = tid + o * kThreads, r = idx / UNC, i = idx % UNC;
@@ -716,7 +726,7 @@ __global__ void __launch_bounds__(kThreads, 1) lstm_adj_chain_kernel(LstmChainAd
         }
       }
     }
-    const bool ok = gather_blocks<UNC, 4, RL>(a.xw + (i64)(rg * 2 + (s & 1)) * gridDim.x * kBlockWords, (int)gridDim.x, a.step0 + (unsigned)s, As, ldk, H,
+    const bool ok = gather_blocks<UNC, 4, RL>(a.xw + (i64)(rg * 2 + (s & 1)) * gridDim.x * kBlockWords, (int)gridDim.x, tag, As, ldk, H,
                                           status);
     if (!ok) ok_smem = 0;
     __syncthreads();
@@ -811,7 +821,9 @@ __global__ void __launch_bounds__(kThreads, 1) adj_split_chain_kernel(typename A
   uint32_t wreg[KS > 0 ? KS : 1][NT][2];
   if (KS > 0) load_wregs<NT, (KS > 0 ? KS : 1)>(Ws, ldk, warp * (H / kWarps), wreg);
   bool waits = true;
+  unsigned tag = a.step0;
   for (int s = 1; s <= a.nsteps; ++s) {
+    ++tag;
     float acc[NT][4];
 #pragma unroll
     for (int nt = 0; nt < NT; ++nt) acc[nt][0] = acc[nt][1] = acc[nt][2] = acc[nt][3] = 0.f;
@@ -871,7 +883,7 @@ __global__ void __launch_bounds__(kThreads, 1) adj_split_chain_kernel(typename A
         v.x = 6 * k < kBlockVals ? s32[0] : 0u;
         v.y = 6 * k + 2 < kBlockVals ? s32[1] : 0u;
         v.z = 6 * k + 4 < kBlockVals ? s32[2] : 0u;
-        v.w = a.step0 + (unsigned)s;
+        v.w = tag;
         st_word(a.xw + xbase + ((i64)q * nprod + blockIdx.x) * kBlockWords + k, v);
       }
     }
@@ -888,7 +900,7 @@ __global__ void __launch_bounds__(kThreads, 1) adj_split_chain_kernel(typename A
       }
       load_coefs(o, (i64)(s + 1) * a.coef_step + off, s + 1 < a.nsteps);
     }
-    if (waits && !gather_blocks<UF, 1, RL>(a.xw + xbase + (i64)g * nprod * kBlockWords, H / UF, a.step0 + (unsigned)s, As, ldk, H, status)) ok_smem = 0;
+    if (waits && !gather_blocks<UF, 1, RL>(a.xw + xbase + (i64)g * nprod * kBlockWords, H / UF, tag, As, ldk, H, status)) ok_smem = 0;
     __syncthreads();
     waits = ok_smem != 0;
   }
@@ -1362,9 +1374,17 @@ bool serial_adj_solve(const SerialAdjArgs& a, cudaStream_t s) {
     auto go = [&](auto kern) { return launch_coop(kern, a, unc, kRows, smem, false, 3, s); };
     ok = unc == 8 ? go(serial_adj_kernel<8, false, kRows>) : unc == 16 ? go(serial_adj_kernel<16, false, kRows>) : go(serial_adj_kernel<32, false, kRows>);
   } else {
+    SerialAdjArgs b = a;
+    if (adj_words_number_steps(unc, true)) {
+      if (a.step0 > 0x7fffffffu - (unsigned)a.nsteps) { prof_end(s); return false; }
+      const i64 c0 = (i64)a.step0 * a.coef_step, m0 = (i64)a.step0 * a.B * a.H;
+      b.nsteps += (int)a.step0;
+      b.mu -= m0; b.a -= c0; b.cr -= c0; b.cz -= c0; b.cn -= c0;
+      if (b.g) b.g -= m0;
+    }
     ok = by_rows(a.B, [&](auto rl) {
       constexpr int RL = decltype(rl)::value;
-      auto go = [&](auto kern) { return launch_coop(kern, a, unc, RL, smem, true, 3, s); };
+      auto go = [&](auto kern) { return launch_coop(kern, b, unc, RL, smem, true, 3, s); };
       if (wreg && a.H == 1024 && unc == 8) return go(serial_adj_kernel<8, true, RL, 24>);
       if (wreg && a.H == 512 && unc == 8) return go(serial_adj_kernel<8, true, RL, 12>);
       if constexpr (RL == kRows) {
