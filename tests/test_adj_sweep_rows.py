@@ -1,6 +1,7 @@
 """Which rows of one launch of adjoint steps read what other rows of it write, on the CPU: the plan that the library makes for every
 such launch (csrc/adj_sweep.h) against a row by row enumeration.  A C-step behind F-steps replaces what the next interval started
-from; the launch has to say so, and the tiles that the kernel then waits for have to hold those rows."""
+from; the launch has to say so, and the tiles that the kernel then waits for have to hold those rows.  And the sizes at which such
+a launch is taken at all."""
 import os
 import subprocess
 
@@ -107,6 +108,14 @@ int main() {
           }
         }
   CHECK(ordered > 100 && plain > 100 && refused > 100);
+  // rounds of row tiles against waves of single steps, on both sides of every jump (33 clusters of four, 74 of two)
+  const int rule[][3] = {{1024, 64, 8}, {1024, 65, 0}, {960, 64, 0}, {1024, 511, 0}, {1024, 512, 4}, {1024, 1024, 4}, {1024, 1025, 0}, {1024, 1153, 4},
+                         {1024, 2048, 4}, {1024, 2049, 0}, {640, 512, 0}, {640, 896, 0}, {640, 897, 4}, {640, 1537, 0}, {704, 640, 4}, {704, 641, 0},
+                         {576, 1024, 0}, {576, 1025, 4}, {576, 1537, 0}, {512, 1535, 0}, {512, 1536, 2}, {512, 4096, 2}, {512, 4097, 0}, {448, 2304, 2},
+                         {448, 2305, 0}, {448, 2688, 0}, {448, 2689, 2}, {448, 2816, 2}, {320, 1792, 0}, {320, 1793, 2}, {320, 3072, 2}, {320, 3073, 0}, {256, 2048, 0},
+                         {1088, 1024, 0}};
+  for (const auto& r : rule) CHECK(adj_sweep_split(r[0], r[1], 33, 74) == r[2]);
+  for (int M = 65; M <= 4096; ++M) CHECK(adj_sweep_split(1024, M, 7, 74) == 0 && adj_sweep_split(512, M, 33, 3) == 0);      // (no room for one group)
   printf("ok\n");
   return 0;
 }
